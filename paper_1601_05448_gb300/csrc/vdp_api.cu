@@ -325,7 +325,7 @@ bool ensure_while_graph(vdp_ctx* c, int prec) {
 int ensure_scaled(vdp_ctx* c, int prec) {
   if (c->scaled_prec == prec) return VDP_OK;
   VDP_CK(launch_scaled(prec, c->bx, c->by, c->bz, c->sinv, c->nx, c->ny, c->nz, c->sx, c->sy,
-                       c->sz, c->sd, c->stream));
+                       c->sz, c->sd, nullptr, 0, c->stream));
   c->scaled_prec = prec;
   return VDP_OK;
 }
@@ -431,7 +431,7 @@ int prepare_spectral_solve(vdp_ctx* c) {
   if (c->hdesc.pc == PC_MG) {
     if (!c->mg) return VDP_EINVAL;
     if (!c->omega_valid) {
-      VDP_CK(launch_omega(c->sinv, c->n, c->omega, c->stream));
+      VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
       c->omega_valid = true;
     }
     if (!c->mg_valid) {
@@ -442,7 +442,7 @@ int prepare_spectral_solve(vdp_ctx* c) {
   }
   if (c->hdesc.pc == PC_FIXED && !c->rho_w_valid) return VDP_EINVAL;
   if (!c->omega_valid) {
-    VDP_CK(launch_omega(c->sinv, c->n, c->omega, c->stream));
+    VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
     c->omega_valid = true;
   }
   return VDP_OK;
@@ -495,19 +495,22 @@ int vdp_create_bc(int nx, int ny, int nz, double Lx, double Ly, double Lz, int b
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->desc, sizeof(InstDesc));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->units, sizeof(UnitRef) * (maxunits + kSMs * 8));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->flag, sizeof(int));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hstate, 2 * sizeof(InstState));
+  // pinned: two states and the density verdict
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hstate, 2 * sizeof(InstState) + sizeof(int));
   if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->evs[0], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->evs[1], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMemset(c->ticket, 0, sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMemset(c->flag, 0, sizeof(int));
   if (e != cudaSuccess) {
     int s = cuda_fail(e, "vdp_create");
     free_ctx(c);
     return s;
   }
-  std::memset(c->hstate, 0, 2 * sizeof(InstState));
+  std::memset(c->hstate, 0, 2 * sizeof(InstState) + sizeof(int));
+  c->hflag = reinterpret_cast<int*>(c->hstate + 2);
   Layout lay;
   if (choose_layout(c, c->opts.precision, &lay) != VDP_OK) {  // rows too long for any stage
     free_ctx(c);
@@ -608,26 +611,24 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
     VDP_CK(cudaMemcpyAsync(c->stage_a, rho, bytes, cudaMemcpyHostToDevice, c->stream));
     src = c->stage_a;
   }
-  VDP_CK(cudaMemsetAsync(c->flag, 0, sizeof(int), c->stream));
-  VDP_CK(launch_check_density(src, c->n, c->flag, c->stream));
-  int bad = 0;
-  VDP_CK(cudaMemcpyAsync(&bad, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  VDP_CK(cudaStreamSynchronize(c->stream));
-  if (bad) return VDP_EDENSITY;
+  // the check and everything built from rho are launched together; the kernels after the check
+  // write nothing when it fails, and the host waits once
+  const int gen = ++c->density_gen, prec = c->opts.precision;
+  VDP_CK(launch_check_density(src, c->n, gen, c->flag, c->stream));
   VDP_CK(launch_build_coefficients(src, c->nx, c->ny, c->nz, c->Lx / c->nx, c->Ly / c->ny,
                                    c->Lz / c->nz, c->bc_x == VDP_BC_DUCT, c->bx, c->by, c->bz,
-                                   c->sinv, c->dg, c->stream));
-  c->scaled_prec = -1;
-  c->omega_valid = false;
-  c->rho_w_valid = false;
-  c->mg_valid = false;
-  if (c->rho_w) {  // the fixed-point iteration's weight needs rho itself
-    VDP_CK(launch_rho_weight(src, c->sinv, c->n, c->rho_w, c->stream));
-    c->rho_w_valid = true;
-  }
-  int s = ensure_scaled(c, c->opts.precision);
-  if (s != VDP_OK) return s;
+                                   c->sinv, c->dg, c->flag, gen, c->stream));
+  if (c->rho_w)  // the fixed-point iteration's weight needs rho itself
+    VDP_CK(launch_rho_weight(src, c->dg, c->sinv, c->n, c->rho_w, c->flag, gen, c->stream));
+  VDP_CK(launch_scaled(prec, c->bx, c->by, c->bz, c->sinv, c->nx, c->ny, c->nz, c->sx, c->sy, c->sz,
+                       c->sd, c->flag, gen, c->stream));
+  VDP_CK(cudaMemcpyAsync(c->hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   VDP_CK(cudaStreamSynchronize(c->stream));
+  if (*c->hflag == gen) return VDP_EDENSITY;
+  c->scaled_prec = prec;
+  c->omega_valid = false;
+  c->rho_w_valid = c->rho_w != nullptr;
+  c->mg_valid = false;
   c->has_density = true;
   return VDP_OK;
 }
@@ -774,7 +775,7 @@ int vdp_mg_apply(vdp_ctx* c, const double* g, double* out) {
   int s;
   if ((s = ensure_mg(c)) != VDP_OK) return s;
   if (!c->omega_valid) {
-    VDP_CK(launch_omega(c->sinv, c->n, c->omega, c->stream));
+    VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
     c->omega_valid = true;
   }
   if (!c->mg_valid) {

@@ -17,7 +17,7 @@
 // vdp_spectral.cu) replaces rt as the stencil sweep's source; the paper's fixed-point iteration
 // runs as the same sweeps with beta = 0 and alpha = 1.
 //
-// Kernels: the coefficient builders (set-up) and three sweep kernels, each advancing every
+// Kernels (the coefficient builders are in vdp_setup.cu): three sweep kernels, each advancing every
 // instance whose phase is of its kind (see vdp_internal.cuh): k_res64_direct (FP64 residual),
 // k_stencil_direct (search direction, stencil product and <d, q>; Chebyshev sweeps in its
 // CHEBOK variant) and k_flat (element-wise phases).  The direct sweeps march each work unit
@@ -1322,123 +1322,7 @@ __global__ void k_init(InstDesc* desc, const double* rhs, double* p, double tol,
   *desc->ticket = 0u;
 }
 
-// ---- coefficient set-up -----------------------------------------------------------------------
-
-__global__ void k_check_density(const double* __restrict__ rho, long long n, int* bad) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x) {
-    const double v = rho[c];
-    if (!(v > 0.0) || !isfinite(v)) atomicOr(bad, 1);
-  }
-}
-
-// b_d[c] = 2 / (rho[c - e_d] + rho[c]) / h_d^2 on the low d-face of every cell
-// duct: the face at the x ends (slot x = 0, shared by x = 0 and x = Lx) carries no flux
-__global__ void k_faces(const double* __restrict__ rho, int nx, int ny, int nz, double ihx2,
-                        double ihy2, double ihz2, int duct, double* bx, double* by, double* bz) {
-  const long long n = (long long)nx * ny * nz;
-  const long long plane = (long long)nx * ny;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx);
-    const int y = (int)((c / nx) % ny);
-    const int z = (int)(c / plane);
-    const long long cxm = c - x + (x == 0 ? nx - 1 : x - 1);
-    const long long cym = c + (long long)((y == 0 ? ny - 1 : y - 1) - y) * nx;
-    const long long czm = c + (long long)((z == 0 ? nz - 1 : z - 1) - z) * plane;
-    const double rc = rho[c];
-    bx[c] = (duct && x == 0) ? 0.0 : 2.0 / (rho[cxm] + rc) * ihx2;
-    by[c] = 2.0 / (rho[cym] + rc) * ihy2;
-    bz[c] = 2.0 / (rho[czm] + rc) * ihz2;
-  }
-}
-
-// sinv = D^-1/2 with D = sum of the six face coefficients of the cell
-__global__ void k_diag(const double* __restrict__ bx, const double* __restrict__ by,
-                       const double* __restrict__ bz, int nx, int ny, int nz, double* sinv,
-                       double* dg) {
-  const long long n = (long long)nx * ny * nz;
-  const long long plane = (long long)nx * ny;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx);
-    const int y = (int)((c / nx) % ny);
-    const int z = (int)(c / plane);
-    const long long cxp = c - x + (x == nx - 1 ? 0 : x + 1);
-    const long long cyp = c + (long long)((y == ny - 1 ? 0 : y + 1) - y) * nx;
-    const long long czp = c + (long long)((z == nz - 1 ? 0 : z + 1) - z) * plane;
-    const double D = bx[c] + bx[cxp] + by[c] + by[cyp] + bz[c] + bz[czp];
-    sinv[c] = 1.0 / sqrt(D);
-    dg[c] = D;
-  }
-}
-
-// Rounded to nearest: the rounding errors of the stored off-diagonals have no common sign, so
-// they do not add up to a spurious diagonal shift that would swamp the operator's smallest
-// eigenvalues (a directed rounding would, at BF16 precision).
-template <class BT> __device__ __forceinline__ BT to_coef(double v);
-template <> __device__ __forceinline__ double to_coef<double>(double v) { return v; }
-template <> __device__ __forceinline__ float to_coef<float>(double v) { return __double2float_rn(v); }
-template <> __device__ __forceinline__ __nv_bfloat16 to_coef<__nv_bfloat16>(double v) {
-  return __double2bfloat16(v);
-}
-
-// bt_d[c] = b_d[c] sinv[c - e_d] sinv[c]
-template <class BT>
-__global__ void k_scaled(const double* __restrict__ bx, const double* __restrict__ by,
-                         const double* __restrict__ bz, const double* __restrict__ sinv, int nx,
-                         int ny, int nz, BT* sx, BT* sy, BT* sz) {
-  const long long n = (long long)nx * ny * nz;
-  const long long plane = (long long)nx * ny;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx);
-    const int y = (int)((c / nx) % ny);
-    const int z = (int)(c / plane);
-    const long long cxm = c - x + (x == 0 ? nx - 1 : x - 1);
-    const long long cym = c + (long long)((y == 0 ? ny - 1 : y - 1) - y) * nx;
-    const long long czm = c + (long long)((z == 0 ? nz - 1 : z - 1) - z) * plane;
-    const double s = sinv[c];
-    sx[c] = to_coef<BT>(bx[c] * sinv[cxm] * s);
-    sy[c] = to_coef<BT>(by[c] * sinv[cym] * s);
-    sz[c] = to_coef<BT>(bz[c] * sinv[czm] * s);
-  }
-}
-
-// BF16 coefficients: the rounded off-diagonals no longer sum (with the weights sqrt(D)) to the
-// unit diagonal, and at BF16 precision that inconsistency is large enough to create spurious
-// near-zero or negative eigenvalues.  The correction dg = sum_faces bt' s_nb / s_c - 1 (s =
-// sqrt(D), bt' the stored BF16 values) restores sqrt(D) as an exact null vector of the stored
-// inner operator  (1 + dg) I - offdiag(bt'), which is then congruent to a graph Laplacian with
-// non-negative weights, i.e. symmetric positive semi-definite.
-__global__ void k_diag_correction(const __nv_bfloat16* __restrict__ sx,
-                                  const __nv_bfloat16* __restrict__ sy,
-                                  const __nv_bfloat16* __restrict__ sz,
-                                  const double* __restrict__ sinv, int nx, int ny, int nz,
-                                  __nv_bfloat16* dg) {
-  const long long n = (long long)nx * ny * nz;
-  const long long plane = (long long)nx * ny;
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(c % nx);
-    const int y = (int)((c / nx) % ny);
-    const int z = (int)(c / plane);
-    const long long cxm = c - x + (x == 0 ? nx - 1 : x - 1), cxp = c - x + (x == nx - 1 ? 0 : x + 1);
-    const long long cym = c + (long long)((y == 0 ? ny - 1 : y - 1) - y) * nx;
-    const long long cyp = c + (long long)((y == ny - 1 ? 0 : y + 1) - y) * nx;
-    const long long czm = c + (long long)((z == 0 ? nz - 1 : z - 1) - z) * plane;
-    const long long czp = c + (long long)((z == nz - 1 ? 0 : z + 1) - z) * plane;
-    // s_nb / s_c = sinv_c / sinv_nb
-    const double sc = sinv[c];
-    double g = (double)__bfloat162float(sx[c]) * sc / sinv[cxm] +
-               (double)__bfloat162float(sx[cxp]) * sc / sinv[cxp] +
-               (double)__bfloat162float(sy[c]) * sc / sinv[cym] +
-               (double)__bfloat162float(sy[cyp]) * sc / sinv[cyp] +
-               (double)__bfloat162float(sz[c]) * sc / sinv[czm] +
-               (double)__bfloat162float(sz[czp]) * sc / sinv[czp];
-    dg[c] = __double2bfloat16(g - 1.0);
-  }
-}
+// ---- one operator application -----------------------------------------------------------------------
 
 // out = A p (FP64)
 __global__ void k_apply(const double* __restrict__ bx, const double* __restrict__ by,
@@ -1469,43 +1353,6 @@ static int grid_for(long long n) {
   if (b > 152 * 16) b = 152 * 16;
   if (b < 1) b = 1;
   return (int)b;
-}
-
-cudaError_t launch_check_density(const double* rho, long long n, int* bad, cudaStream_t s) {
-  k_check_density<<<grid_for(n), 256, 0, s>>>(rho, n, bad);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
-                                      double hy, double hz, int duct, double* bx, double* by,
-                                      double* bz, double* sinv, double* dg, cudaStream_t s) {
-  const long long n = (long long)nx * ny * nz;
-  k_faces<<<grid_for(n), 256, 0, s>>>(rho, nx, ny, nz, 1.0 / (hx * hx), 1.0 / (hy * hy),
-                                      1.0 / (hz * hz), duct, bx, by, bz);
-  k_diag<<<grid_for(n), 256, 0, s>>>(bx, by, bz, nx, ny, nz, sinv, dg);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scaled(int prec, const double* bx, const double* by, const double* bz,
-                          const double* sinv, int nx, int ny, int nz, void* sx, void* sy, void* sz,
-                          void* sd, cudaStream_t s) {
-  const long long n = (long long)nx * ny * nz;
-  if (prec == PREC_FP64)
-    k_scaled<double><<<grid_for(n), 256, 0, s>>>(bx, by, bz, sinv, nx, ny, nz, (double*)sx,
-                                                 (double*)sy, (double*)sz);
-  else if (prec == PREC_MIXED)
-    k_scaled<float><<<grid_for(n), 256, 0, s>>>(bx, by, bz, sinv, nx, ny, nz, (float*)sx,
-                                                (float*)sy, (float*)sz);
-  else {
-    k_scaled<__nv_bfloat16><<<grid_for(n), 256, 0, s>>>(bx, by, bz, sinv, nx, ny, nz,
-                                                        (__nv_bfloat16*)sx, (__nv_bfloat16*)sy,
-                                                        (__nv_bfloat16*)sz);
-    k_diag_correction<<<grid_for(n), 256, 0, s>>>((const __nv_bfloat16*)sx,
-                                                  (const __nv_bfloat16*)sy,
-                                                  (const __nv_bfloat16*)sz, sinv, nx, ny, nz,
-                                                  (__nv_bfloat16*)sd);
-  }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_apply(const double* bx, const double* by, const double* bz, const double* p,

@@ -1,4 +1,4 @@
-// vdp_launch.h -- host-side launchers of the kernels in vdp_kernels.cu (internal to libvdp).
+// vdp_launch.h -- host-side launchers of the kernels in vdp_kernels.cu and vdp_setup.cu (internal to libvdp).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -7,14 +7,22 @@
 
 namespace vdp {
 
-cudaError_t launch_check_density(const double* rho, long long n, int* bad, cudaStream_t s);
-// face coefficients on the low faces (spacings h_d; duct: no flux through the x ends) and D^-1/2
+// vdp_setup.cu.  The check stores gen in *bad when an entry is <= 0 or not finite; the launches
+// that take (bad, gen) then write nothing (null: not gated).
+cudaError_t launch_check_density(const double* rho, long long n, int gen, int* bad, cudaStream_t s);
+// face coefficients on the low faces (spacings h_d; duct: no flux through the x ends), D^-1/2, D
 cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
                                       double hy, double hz, int duct, double* bx, double* by,
-                                      double* bz, double* sinv, double* dg, cudaStream_t s);
+                                      double* bz, double* sinv, double* dg, const int* bad,
+                                      int gen, cudaStream_t s);
 cudaError_t launch_scaled(int prec, const double* bx, const double* by, const double* bz,
                           const double* sinv, int nx, int ny, int nz, void* sx, void* sy, void* sz,
-                          void* sd, cudaStream_t s);
+                          void* sd, const int* bad, int gen, cudaStream_t s);
+// W = D^1/2, and rho W (the fixed-point iteration's input weight)
+cudaError_t launch_omega(const double* dg, const double* sinv, long long n, float* omega,
+                         cudaStream_t s);
+cudaError_t launch_rho_weight(const double* rho, const double* dg, const double* sinv, long long n,
+                              float* out, const int* bad, int gen, cudaStream_t s);
 cudaError_t launch_apply(const double* bx, const double* by, const double* bz, const double* p,
                          int nx, int ny, int nz, double* out, cudaStream_t s);
 cudaError_t launch_init(InstDesc* desc, const double* rhs, double* p, double tol, double inner_tol,

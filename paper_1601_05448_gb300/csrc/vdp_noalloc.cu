@@ -191,13 +191,14 @@ extern "C" int vdp_solve_noalloc(int nx, int ny, int nz, double L, const double*
   // density check, then the coefficients (the flag must start at zero on every call)
   int bad = 0;
   NA_CK(cudaMemsetAsync(flag, 0, sizeof(int), s));
-  NA_CK(launch_check_density(rho, n, flag, s));
+  NA_CK(launch_check_density(rho, n, 1, flag, s));
   NA_CK(cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, s));
   NA_CK(cudaStreamSynchronize(s));
   if (bad) return VDP_EDENSITY;
   double* dg = f64[12];
-  NA_CK(launch_build_coefficients(rho, nx, ny, nz, L / nx, L / ny, L / nz, 0, bx, by, bz, sinv, dg, s));
-  NA_CK(launch_scaled(precision, bx, by, bz, sinv, nx, ny, nz, sx, sy, sz, sd, s));
+  NA_CK(launch_build_coefficients(rho, nx, ny, nz, L / nx, L / ny, L / nz, 0, bx, by, bz, sinv, dg,
+                                  nullptr, 0, s));
+  NA_CK(launch_scaled(precision, bx, by, bz, sinv, nx, ny, nz, sx, sy, sz, sd, nullptr, 0, s));
 
   // the default unit layout of vdp_solve
   Layout lay;

@@ -992,28 +992,4 @@ int spectral_units(int nx, int ny, int nz) {  // CTAs of the Z pass (they store 
   return (int)line_grid(2, nz, (long long)(spectral_pitch(nx) / kTX) * ny);
 }
 
-__global__ void k_omega(const double* __restrict__ sinv, long long n, float* __restrict__ omega) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x)
-    omega[c] = (float)(1.0 / sinv[c]);
-}
-
-cudaError_t launch_omega(const double* sinv, long long n, float* omega, cudaStream_t s) {
-  k_omega<<<152 * 8, 256, 0, s>>>(sinv, n, omega);
-  return cudaGetLastError();
-}
-
-__global__ void k_rho_weight(const double* __restrict__ rho, const double* __restrict__ sinv,
-                             long long n, float* __restrict__ out) {
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x)
-    out[c] = (float)(rho[c] / sinv[c]);
-}
-
-cudaError_t launch_rho_weight(const double* rho, const double* sinv, long long n, float* out,
-                              cudaStream_t s) {
-  k_rho_weight<<<152 * 8, 256, 0, s>>>(rho, sinv, n, out);
-  return cudaGetLastError();
-}
-
 }  // namespace vdp

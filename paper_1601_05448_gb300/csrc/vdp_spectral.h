@@ -69,9 +69,5 @@ int spectral_xinv_units(int prec, const SpecArgs& a, int slab);
 SpecArgs spectral_launch_args(int prec, const SpecArgs& a, const SpecLaunch& l, int slab);
 // All launches of one application, in order.
 cudaError_t launch_spectral_apply(int prec, const SpecArgs& a, int slab, cudaStream_t s);
-cudaError_t launch_omega(const double* sinv, long long n, float* omega, cudaStream_t s);
-// out = rho / sinv (the fixed-point iteration's input weight)
-cudaError_t launch_rho_weight(const double* rho, const double* sinv, long long n, float* out,
-                              cudaStream_t s);
 
 }  // namespace vdp
