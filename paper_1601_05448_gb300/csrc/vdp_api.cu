@@ -112,7 +112,7 @@ void free_ctx(vdp_ctx* c) {
     delete c->mg;
   }
   void* bufs[] = {c->bx, c->by, c->bz, c->sinv, c->dg, c->f0, c->sx, c->sy, c->sz, c->sd, c->x, c->r, c->d0, c->d1,
-                  c->za, c->zb, c->dch, c->spec, c->omega, c->sptab, c->rho_w, c->d_rounds,
+                  c->za, c->zb, c->dch, c->spec, c->omega, c->sptab, c->rho_w, c->rho32, c->dsc, c->d_rounds,
                   c->q, c->part, c->ticket, c->st, c->desc, c->units, c->flag, c->stage_a,
                   c->stage_b, c->proj_f};
   for (void* b : bufs)
@@ -155,6 +155,13 @@ int configure_layout(vdp_ctx* c, int prec) {
   d.stages = lay.stages;
   d.zc = lay.zc;
   d.mode = lay.mode;
+  d.form = density_form(c, prec) ? 1 : 0;
+  d.duct = c->bc_x == VDP_BC_DUCT;
+  const double hx = c->Lx / c->nx, hy = c->Ly / c->ny, hz = c->Lz / c->nz;
+  d.cy = (float)(2.0 * (hx / hy) * (hx / hy));
+  d.cz = (float)(2.0 * (hx / hz) * (hx / hz));
+  d.rho32 = c->rho32;
+  d.dsc = c->dsc;
   d.ncell = c->n;
   d.bx = c->bx;
   d.by = c->by;
@@ -218,7 +225,7 @@ int steps_per_sync(const vdp_ctx* c) {
 cudaError_t launch_round(vdp_ctx* c, int prec, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   if (c->lay.mode == 0)  // the residual sweep has its own kernel in the direct mode
-    e = launch_res64(prec, c->desc, c->units, c->lay.nunits, c->lay.threads, s);
+    e = launch_res64(prec, c->hdesc.form, c->desc, c->units, c->lay.nunits, c->lay.threads, s);
   if (e == cudaSuccess && c->hdesc.pc == PC_MG) {  // z = W M W rt by one V-cycle
     const MgArgs a{c->r, c->za, c->omega, c->st, c->desc};
     e = launch_mg_vcycle(*c->mg, prec, a, s);
@@ -228,7 +235,7 @@ cudaError_t launch_round(vdp_ctx* c, int prec, cudaStream_t s) {
     e = launch_spectral_apply(prec, a, spec_slab(c), s);
   }
   if (e == cudaSuccess)
-    e = launch_stencil(prec, c->lay.mode, stencil_kind(c->hdesc.pc), c->desc, c->units,
+    e = launch_stencil(prec, c->lay.mode, stencil_kind(c->hdesc), c->desc, c->units,
                        c->lay.nunits, c->lay.threads, c->lay.smem, s);
   if (e == cudaSuccess) e = launch_flat(prec, c->desc, c->units + c->lay.nunits, c->lay.nunits_f, s);
   return e;
@@ -322,11 +329,36 @@ bool ensure_while_graph(vdp_ctx* c, int prec) {
   return true;
 }
 
+bool density_form(const vdp_ctx* c, int prec) {
+  return prec == PREC_MIXED && c->rho32_valid &&
+         (c->opts.method == VDP_METHOD_FIXED_POINT || c->opts.precond == VDP_PRECOND_SPECTRAL);
+}
+
+int ensure_sinv(vdp_ctx* c) {
+  if (c->sinv_valid) return VDP_OK;
+  VDP_CK(launch_sinv(c->dg, c->n, c->sinv, c->stream));
+  c->sinv_valid = true;
+  return VDP_OK;
+}
+
 int ensure_scaled(vdp_ctx* c, int prec) {
-  if (c->scaled_prec == prec) return VDP_OK;
+  if (c->scaled_prec == prec || density_form(c, prec)) return VDP_OK;
+  const int s = ensure_sinv(c);
+  if (s != VDP_OK) return s;
   VDP_CK(launch_scaled(prec, c->bx, c->by, c->bz, c->sinv, c->nx, c->ny, c->nz, c->sx, c->sy,
                        c->sz, c->sd, nullptr, 0, c->stream));
   c->scaled_prec = prec;
+  return VDP_OK;
+}
+
+// W = D^1/2 (the scaled spectral passes and the V-cycle)
+static int ensure_omega(vdp_ctx* c) {
+  if (c->omega_valid) return VDP_OK;
+  const int s = ensure_sinv(c);
+  if (s != VDP_OK) return s;
+  if (!c->omega) VDP_CK(cudaMalloc((void**)&c->omega, sizeof(float) * (size_t)c->n));
+  VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
+  c->omega_valid = true;
   return VDP_OK;
 }
 
@@ -349,18 +381,16 @@ int ensure_spectral(vdp_ctx* c) {
   cudaError_t e = cudaSuccess;
   if (!c->za) e = cudaMalloc(&c->za, sizeof(double) * (size_t)c->n);
   if (e == cudaSuccess && !c->spec) e = cudaMalloc((void**)&c->spec, spec_bytes);
-  if (e == cudaSuccess && !c->omega) e = cudaMalloc((void**)&c->omega, sizeof(float) * (size_t)c->n);
   if (e == cudaSuccess && !c->sptab) e = cudaMalloc((void**)&c->sptab, sizeof(float) * tab.size());
   if (e == cudaSuccess)
     e = cudaMemcpy(c->sptab, tab.data(), sizeof(float) * tab.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
-    for (void** b : {(void**)&c->spec, (void**)&c->omega, (void**)&c->sptab}) {
+    for (void** b : {(void**)&c->spec, (void**)&c->sptab}) {
       if (*b) cudaFree(*b);
       *b = nullptr;
     }
     return cuda_fail(e, "spectral buffers");
   }
-  c->omega_valid = false;
   return VDP_OK;
 }
 
@@ -374,8 +404,11 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   // paper's update p += damping L_h^-1 (rho r) (applied as p -= D^-1/2 x, x the sum of the z)
   a->out = c->za;
   a->out_f32 = fixed ? 1 : 0;  // the fixed-point sweep reads z as FP32
-  a->omega_in = fixed ? c->rho_w : c->omega;
-  a->omega_out = c->omega;
+  // density form: the stored residual is g = rho' r (fixed point) or r (CG), z is unscaled, and
+  // the inverse is that of hx^2 L_h: no weights
+  const bool dens = density_form(c, prec);
+  a->omega_in = dens ? nullptr : fixed ? c->rho_w : c->omega;
+  a->omega_out = dens ? nullptr : c->omega;
   a->spec = c->spec;
   a->tw = reinterpret_cast<const float2*>(c->sptab);
   a->lam = c->sptab + 2 * (2 * m + 1 + c->ny + c->nz);
@@ -386,7 +419,9 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   a->nxd = c->nx;
   a->mirror = c->bc_x == VDP_BC_DUCT;
   a->ewt = a->mirror ? 0.5f : 1.f;
-  a->scale = (float)((fixed ? c->opts.damping : 1.0) / ((double)nxt * c->ny * c->nz));
+  const double hx = c->Lx / c->nx;
+  a->scale = (float)((fixed ? c->opts.damping : 1.0) / ((double)nxt * c->ny * c->nz) /
+                     (dens ? hx * hx : 1.0));
   a->st = c->st;
   a->I = c->desc;
   a->zunits = spectral_units(nxt, c->ny, c->nz);
@@ -428,22 +463,25 @@ int precond_launches(const vdp_ctx* c) {
 
 int prepare_spectral_solve(vdp_ctx* c) {
   if (c->hdesc.pc < PC_SPECTRAL) return VDP_OK;
+  int s;
   if (c->hdesc.pc == PC_MG) {
     if (!c->mg) return VDP_EINVAL;
-    if (!c->omega_valid) {
-      VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
-      c->omega_valid = true;
-    }
+    if ((s = ensure_omega(c)) != VDP_OK) return s;
     if (!c->mg_valid) {
       VDP_CK(mg_setup(c->mg, c->bx, c->by, c->bz, c->sinv, c->stream));
       c->mg_valid = true;
     }
     return VDP_OK;
   }
-  if (c->hdesc.pc == PC_FIXED && !c->rho_w_valid) return VDP_EINVAL;
-  if (!c->omega_valid) {
-    VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
-    c->omega_valid = true;
+  const bool fixed = c->hdesc.pc == PC_FIXED;
+  if (fixed && !c->rho32_valid) return VDP_EINVAL;
+  if (c->hdesc.form) return VDP_OK;
+  if ((s = ensure_omega(c)) != VDP_OK) return s;
+  if (fixed && !c->rho_w_valid) {
+    if (!c->rho_w) VDP_CK(cudaMalloc((void**)&c->rho_w, sizeof(float) * (size_t)c->n));
+    const double hx = c->Lx / c->nx;
+    VDP_CK(launch_rho_weight(c->rho32, c->dsc, hx * hx, c->dg, c->sinv, c->n, c->rho_w, c->stream));
+    c->rho_w_valid = true;
   }
   return VDP_OK;
 }
@@ -582,14 +620,16 @@ int vdp_set_options(vdp_ctx* c, const vdp_opts* o) {
       return mres;
     }
   }
-  if (o->method == VDP_METHOD_FIXED_POINT && !c->rho_w) {
-    cudaError_t e = cudaMalloc((void**)&c->rho_w, sizeof(float) * (size_t)c->n);
+  if ((o->method == VDP_METHOD_FIXED_POINT || o->precond == VDP_PRECOND_SPECTRAL) && !c->rho32) {
+    cudaError_t e = cudaMalloc((void**)&c->rho32, sizeof(float) * (size_t)c->n);
+    if (e == cudaSuccess && !c->dsc) e = cudaMalloc((void**)&c->dsc, sizeof(double));
     if (e != cudaSuccess) {
-      c->rho_w = nullptr;
+      if (c->rho32) cudaFree(c->rho32);
+      c->rho32 = nullptr;
       c->opts = old;
       return cuda_fail(e, "vdp_set_options (density weight)");
     }
-    c->rho_w_valid = false;
+    c->rho32_valid = false;
   }
   c->stream = (cudaStream_t)o->stream;
   c->layout_dirty = true;
@@ -614,21 +654,28 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
   // the check and everything built from rho are launched together; the kernels after the check
   // write nothing when it fails, and the host waits once
   const int gen = ++c->density_gen, prec = c->opts.precision;
+  const bool kept = c->rho32_valid;
+  c->rho32_valid = c->rho32 != nullptr;  // as it will be (density_form looks at it)
+  const bool scaled = !density_form(c, prec);
+  c->rho32_valid = kept;
   VDP_CK(launch_check_density(src, c->n, gen, c->flag, c->stream));
   VDP_CK(launch_build_coefficients(src, c->nx, c->ny, c->nz, c->Lx / c->nx, c->Ly / c->ny,
                                    c->Lz / c->nz, c->bc_x == VDP_BC_DUCT, c->bx, c->by, c->bz,
-                                   c->sinv, c->dg, c->flag, gen, c->stream));
-  if (c->rho_w)  // the fixed-point iteration's weight needs rho itself
-    VDP_CK(launch_rho_weight(src, c->dg, c->sinv, c->n, c->rho_w, c->flag, gen, c->stream));
-  VDP_CK(launch_scaled(prec, c->bx, c->by, c->bz, c->sinv, c->nx, c->ny, c->nz, c->sx, c->sy, c->sz,
-                       c->sd, c->flag, gen, c->stream));
+                                   scaled ? c->sinv : nullptr, c->dg, c->rho32, c->dsc, c->flag,
+                                   gen, c->stream));
+  if (scaled)
+    VDP_CK(launch_scaled(prec, c->bx, c->by, c->bz, c->sinv, c->nx, c->ny, c->nz, c->sx, c->sy,
+                         c->sz, c->sd, c->flag, gen, c->stream));
   VDP_CK(cudaMemcpyAsync(c->hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   VDP_CK(cudaStreamSynchronize(c->stream));
   if (*c->hflag == gen) return VDP_EDENSITY;
-  c->scaled_prec = prec;
+  c->scaled_prec = scaled ? prec : -1;
+  c->sinv_valid = scaled;
   c->omega_valid = false;
-  c->rho_w_valid = c->rho_w != nullptr;
+  c->rho_w_valid = false;
+  c->rho32_valid = c->rho32 != nullptr;
   c->mg_valid = false;
+  if (c->rho32_valid != kept) c->layout_dirty = true;  // the form may change with it
   c->has_density = true;
   return VDP_OK;
 }
@@ -644,9 +691,9 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   if ((s = ensure_scaled(c, prec)) != VDP_OK) return s;
   if ((c->layout_dirty || c->layout_prec != prec) && (s = configure_layout(c, prec)) != VDP_OK)
     return s;
+  if ((s = prepare_spectral_solve(c)) != VDP_OK) return s;  // before the capture of its buffers
   const bool dev_loop = c->opts.steps_per_sync == 0 && ensure_while_graph(c, prec);
   if (!dev_loop && (s = ensure_graph(c, prec)) != VDP_OK) return s;
-  if ((s = prepare_spectral_solve(c)) != VDP_OK) return s;
   const double* drhs = rhs;
   double* dp = p;
   if (host_rhs) {
@@ -774,10 +821,7 @@ int vdp_mg_apply(vdp_ctx* c, const double* g, double* out) {
     return VDP_EINVAL;
   int s;
   if ((s = ensure_mg(c)) != VDP_OK) return s;
-  if (!c->omega_valid) {
-    VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
-    c->omega_valid = true;
-  }
+  if ((s = ensure_omega(c)) != VDP_OK) return s;
   if (!c->mg_valid) {
     VDP_CK(mg_setup(c->mg, c->bx, c->by, c->bz, c->sinv, c->stream));
     c->mg_valid = true;

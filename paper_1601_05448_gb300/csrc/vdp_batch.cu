@@ -151,15 +151,27 @@ int capture(vdp_batch* b, int pairs) {
   } else {
     // one stencil kernel for all members: the fixed-point variant if every member uses that
     // method, the variant with Chebyshev sweeps if any member needs it (it also runs the
-    // fixed-point sweep), the CG variant otherwise
-    int nfixed = 0, ncheb = 0;
+    // fixed-point sweep), the CG variant otherwise; the members in the density form have their own
+    // residual and sweep kernels (each kernel leaves the other forms' units alone)
+    int nscaled = 0, nfixed = 0, ncheb = 0, ndfixed = 0, ndcg = 0;
     for (int k : b->active) {
-      nfixed += b->members[k].ctx->hdesc.pc == PC_FIXED;
-      ncheb += b->members[k].ctx->hdesc.pc == PC_CHEB;
+      const InstDesc& d = b->members[k].ctx->hdesc;
+      if (d.form) {
+        ++(d.pc == PC_FIXED ? ndfixed : ndcg);
+        continue;
+      }
+      ++nscaled;
+      nfixed += d.pc == PC_FIXED;
+      ncheb += d.pc == PC_CHEB;
     }
-    const int kind = nfixed == (int)b->active.size() ? 2 : (ncheb || nfixed) ? 1 : 0;
+    const int kind = nfixed == nscaled ? 2 : (ncheb || nfixed) ? 1 : 0;
+    auto sweeps = [&](int k) {
+      return launch_stencil(b->prec, 0, k, b->d_desc, b->d_units, b->ns, kDirectThreads, 0, b->cap);
+    };
     for (int i = 0; i < pairs && e == cudaSuccess; ++i) {
-      e = launch_res64(b->prec, b->d_desc, b->d_units, b->ns, kDirectThreads, b->cap);
+      if (nscaled) e = launch_res64(b->prec, 0, b->d_desc, b->d_units, b->ns, kDirectThreads, b->cap);
+      if (e == cudaSuccess && ndfixed + ndcg)
+        e = launch_res64(b->prec, 1, b->d_desc, b->d_units, b->ns, kDirectThreads, b->cap);
       // members with the spectral passes or the V-cycle: their kernels (each gated on its own
       // member's phase), between the residual and the stencil sweeps as in a solve alone.  The
       // members' chains are independent, so they go to up to four graph branches that the GPU
@@ -187,9 +199,9 @@ int capture(vdp_batch* b, int pairs) {
         e = cudaEventRecord(b->join[j], b->aux[j]);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->join[j], 0);
       }
-      if (e == cudaSuccess)
-        e = launch_stencil(b->prec, 0, kind, b->d_desc, b->d_units, b->ns, kDirectThreads, 0,
-                           b->cap);
+      if (e == cudaSuccess && nscaled) e = sweeps(kind);
+      if (e == cudaSuccess && ndfixed) e = sweeps(kSweepDensityFixed);
+      if (e == cudaSuccess && ndcg) e = sweeps(kSweepDensityCg);
       if (e == cudaSuccess) e = launch_flat(b->prec, b->d_desc, b->d_units + b->ns, b->nf, b->cap);
     }
   }

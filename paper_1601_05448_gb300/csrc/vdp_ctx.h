@@ -46,8 +46,12 @@ struct vdp_ctx {
   float* omega = nullptr;          // D^1/2 per cell (FP32)
   float* sptab = nullptr;          // twiddle and eigenvalue tables
   bool omega_valid = false;        // omega matches the current density
-  float* rho_w = nullptr;          // fixed-point iteration: rho D^1/2 per cell (FP32)
+  float* rho_w = nullptr;          // scaled fixed-point iteration: rho D^1/2 per cell (FP32)
   bool rho_w_valid = false;        // rho_w was computed from the current density
+  float* rho32 = nullptr;          // rho / 2^e0 (FP32), kept once a spectral method is selected
+  double* dsc = nullptr;           // kappa = 2^e0 hx^2
+  bool rho32_valid = false;        // rho32 and dsc hold the current density
+  bool sinv_valid = false;         // sinv was computed from the current density
   vdp::MgHier* mg = nullptr;       // multigrid levels (VDP_PRECOND_MG, vdp_mg_apply)
   bool mg_valid = false;           // the levels were built from the current density
   int scaled_prec = -1;            // precision the scaled coefficients were built for
@@ -88,7 +92,12 @@ namespace vdp {
 // Make the context ready to run in precision `prec`: scaled coefficients built and the unit
 // layout (and its device description) configured.
 int configure_layout(vdp_ctx* c, int prec);
-int ensure_scaled(vdp_ctx* c, int prec);
+int ensure_scaled(vdp_ctx* c, int prec);  // no-op in the density form, which has none
+int ensure_sinv(vdp_ctx* c);
+// The inner solve runs in the density form (vdp_density.cu): the spectral inverse is its
+// preconditioner or iteration, the coefficients are FP32, and the FP32 density is at hand (a
+// density that was set before the method was selected is not: CG then runs in the scaled form).
+bool density_form(const vdp_ctx* c, int prec);
 // length of the x transform of the spectral passes: nx, or 2 nx in the duct (even extension)
 inline int spectral_nx(const vdp_ctx* c) { return c->bc_x == VDP_BC_DUCT ? 2 * c->nx : c->nx; }
 // allocate the spectral buffers and tables (no-op when present); VDP_EINVAL for unsupported grids

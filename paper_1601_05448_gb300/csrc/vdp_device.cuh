@@ -30,7 +30,22 @@ __device__ __forceinline__ double widen(float v) {
   const unsigned lo = e == 0 ? 0u : (frac << 29);
   return __hiloint2double((int)hi, (int)lo);
 }
+// to binary32 of v times 2^p, the same way
+__device__ __forceinline__ float narrow_pow2(double v, int p) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const unsigned sign = hi & 0x80000000u;
+  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127 + p;
+  const unsigned frac = ((hi & 0xfffffu) << 3) | (lo >> 29);
+  const unsigned bits = e <= 0 ? sign : (e >= 255 ? (sign | 0x7f800000u) : (sign | ((unsigned)e << 23) | frac));
+  return __uint_as_float(bits);
+}
 
+// approximate reciprocal (1 ulp)
+__device__ __forceinline__ float rcp_approx(float s) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s));
+  return y;
+}
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

@@ -257,12 +257,14 @@ __device__ void sweep_meanf(const InstDesc& I, long long c0, long long c1, doubl
   sum = s[0] + s[1];
 }
 
-// p -= D^-1/2 x (x in the inner type); sums the new p (the final gauge needs its mean).  fresh:
-// p is still the zero start (never written), so p = -D^-1/2 x without reading it.
-template <class T>
+// p -= D^-1/2 x (x in the inner type; DENS, the density form: p -= kappa x); sums the new p (the
+// final gauge needs its mean).  fresh: p is still the zero start (never written), so it is not
+// read.
+template <class T, bool DENS>
 __device__ void sweep_correct(const InstDesc& I, long long c0, long long c1, bool fresh,
                               double& psum) {
   const T* x = static_cast<const T*>(I.x);
+  const double kappa = DENS ? I.dsc[0] : 0.0;
   double s = 0.0;
   const long long step = 2LL * blockDim.x;
   constexpr int U = kFlatU / 2;  // four operands per vector: half the vectors in flight
@@ -273,7 +275,7 @@ __device__ void sweep_correct(const InstDesc& I, long long c0, long long c1, boo
     for (int u = 0; u < U; ++u) {
       const long long c = cb + u * step;
       if (c < c1) {
-        sv[u] = __ldg(reinterpret_cast<const double2*>(I.sinv + c));
+        sv[u] = DENS ? make_double2(kappa, kappa) : __ldg(reinterpret_cast<const double2*>(I.sinv + c));
         pv[u] = fresh ? make_double2(0.0, 0.0) : *reinterpret_cast<const double2*>(I.p + c);
         xa[u] = x[c];
         xb[u] = x[c + 1];
@@ -854,7 +856,26 @@ __device__ void sweep_stencil_direct(const InstDesc& I, const InstState* st, int
 // diagonal form r = (f - <f>) + D p_c - sum of b_face p_neighbour (D stored per cell): one FMA
 // per term, 8 FP64 operations per cell against 13 for the face-difference form; in the mixed
 // precisions the scaling rt = D^-1/2 r is an FP32 product; the norms are summed in FP32.
-template <class T, bool FIRST, bool F0 = false>
+// What the residual sweep hands to the inner solve in the density form (DENS), from the FP64
+// residual of a cell: fixed point g = rho' r and r^2 / D' (D' = kappa D), CG r and r^2.
+struct DensityResidual {
+  bool fixed;
+  int ek;      // kappa = 2^ek x mk
+  float mk;
+  const float* rho;
+  __device__ __forceinline__ DensityResidual() : fixed(false), ek(0), mk(0.f), rho(nullptr) {}
+  __device__ __forceinline__ explicit DensityResidual(const InstDesc& I)
+      : fixed(I.pc == PC_FIXED), rho(I.rho32) {
+    const double k = I.dsc[0];
+    ek = ((__double2hiint(k) >> 20) & 0x7ff) - 1023;
+    mk = narrow_pow2(k, -ek);
+  }
+  __device__ __forceinline__ float inv_diag(double D) const {
+    return rcp_approx(narrow_pow2(D, ek) * mk);
+  }
+};
+
+template <class T, bool FIRST, bool DENS, bool F0 = false>
 __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* st, int unit,
                                             double (&acc)[kSlots]) {
   constexpr int VR = VecW<T>::V;  // cells per thread (4 for FP32 inner, 2 for FP64)
@@ -874,6 +895,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
   const double mu = st->mu_f;
   const double* p = I.p;
   T* rt = static_cast<T*>(I.r);
+  const DensityResidual dr = DENS ? DensityResidual(I) : DensityResidual();
   auto at = [&](int z, int yy) -> long long {
     const int zz = z < 0 ? z + nz : (z >= nz ? z - nz : z);
     return ((long long)zz * ny + yy) * nx;
@@ -916,7 +938,10 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       const double2 dg = *reinterpret_cast<const double2*>(I.dg + o);
       // F0: f - <f> as the first residual stored it (one FP64 operation fewer per cell)
       const double2 f = *reinterpret_cast<const double2*>((F0 ? I.f0 : I.rhs) + o);
-      const double2 si = *reinterpret_cast<const double2*>(I.sinv + o);
+      double2 si = make_double2(0.0, 0.0);
+      float2 rh = make_float2(1.f, 1.f);
+      if (!DENS) si = *reinterpret_cast<const double2*>(I.sinv + o);
+      if (DENS && dr.fixed) rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o));
       const double l0 = h == 0 ? left : pc[h - 1];
       const double r1 = h + 2 == VR ? right : pc[h + 2];
       const double br1 = h + 2 == VR ? bxr : I.bx[o + 2];
@@ -939,7 +964,12 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       res1 = fma(-bzp.y, pp[h + 1], res1);
       T t0, t1;
       float r0f = narrow(res0), r1f = narrow(res1), t0f, t1f;
-      if constexpr (IsF64<T>::value) {
+      if constexpr (DENS) {
+        t0 = rh.x * r0f;
+        t1 = rh.y * r1f;
+        t0f = dr.fixed ? r0f * r0f * dr.inv_diag(dg.x) : r0f * r0f;  // the norm's terms
+        t1f = dr.fixed ? r1f * r1f * dr.inv_diag(dg.y) : r1f * r1f;
+      } else if constexpr (IsF64<T>::value) {
         t0 = si.x * res0;
         t1 = si.y * res1;
         t0f = narrow(t0);
@@ -953,7 +983,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
         rt[o] = t0;
         rt[o + 1] = t1;
         a0 = fmaf(r0f, r0f, fmaf(r1f, r1f, a0));
-        a1 = fmaf(t0f, t0f, fmaf(t1f, t1f, a1));
+        a1 = DENS ? a1 + (t0f + t1f) : fmaf(t0f, t0f, fmaf(t1f, t1f, a1));
         if (FIRST) {
           const double f0 = f.x - mu, f1 = f.y - mu;
           a2 += c0 + c1;
@@ -974,7 +1004,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
 }
 
 // The first residual of a solve started from p = 0 is r = f - <f>: no stencil, no p reads.
-template <class T>
+template <class T, bool DENS>
 __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
                              double (&acc)[kSlots]) {
   constexpr int VR = VecW<T>::V;
@@ -987,6 +1017,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
   const int z0 = (int)((long long)chunk * nz / I.zc), z1 = (int)((long long)(chunk + 1) * nz / I.zc);
   const double mu = st->mu_f;
   T* rt = static_cast<T*>(I.r);
+  const DensityResidual dr = DENS ? DensityResidual(I) : DensityResidual();
   double a0 = 0;
   T a1 = 0;
   if (row < I.ty && yr < ny) {
@@ -995,10 +1026,23 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
 #pragma unroll
       for (int h = 0; h < VR; h += 2) {
         const double2 f = *reinterpret_cast<const double2*>(I.rhs + o + h);
-        const double2 si = *reinterpret_cast<const double2*>(I.sinv + o + h);
+        double2 si = make_double2(0.0, 0.0);
+        if (!DENS) si = *reinterpret_cast<const double2*>(I.sinv + o + h);
         const double f0 = f.x - mu, f1 = f.y - mu;
         if (I.f0) *reinterpret_cast<double2*>(I.f0 + o + h) = make_double2(f0, f1);
-        if constexpr (IsF64<T>::value) {
+        if constexpr (DENS) {
+          const float r0 = narrow(f0), r1 = narrow(f1);
+          float2 rh = make_float2(1.f, 1.f), d = make_float2(1.f, 1.f);
+          if (dr.fixed) {
+            rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o + h));
+            const double2 D = *reinterpret_cast<const double2*>(I.dg + o + h);
+            d = make_float2(dr.inv_diag(D.x), dr.inv_diag(D.y));
+          }
+          rt[o + h] = rh.x * r0;
+          rt[o + h + 1] = rh.y * r1;
+          a0 = fma(f0, f0, fma(f1, f1, a0));
+          a1 = fmaf(r0 * d.x, r0, fmaf(r1 * d.y, r1, a1));
+        } else if constexpr (IsF64<T>::value) {
           const T t0 = si.x * f0, t1 = si.y * f1;
           rt[o + h] = t0;
           rt[o + h + 1] = t1;
@@ -1022,17 +1066,17 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
   acc[3] = a0;          // ||f - <f>||^2 (this is the first residual)
 }
 
-template <class T>
+template <class T, bool DENS = false>
 __device__ void sweep_res64_direct(const InstDesc& I, const InstState* st, int unit,
                                    double (&acc)[kSlots]) {
   if (st->first_res != 0 && !st->use_guess)
-    res64_zero_p<T>(I, st, unit, acc);
+    res64_zero_p<T, DENS>(I, st, unit, acc);
   else if (st->first_res != 0)
-    res64_march<T, true>(I, st, unit, acc);
+    res64_march<T, true, DENS>(I, st, unit, acc);
   else if (I.f0 && !st->use_guess)  // f - <f> stored by the first residual
-    res64_march<T, false, true>(I, st, unit, acc);
+    res64_march<T, false, DENS, true>(I, st, unit, acc);
   else
-    res64_march<T, false>(I, st, unit, acc);
+    res64_march<T, false, DENS>(I, st, unit, acc);
 }
 
 // ---- the FP64 residual sweep (a few times per solve): z march through a three-plane ring ---------
@@ -1130,6 +1174,7 @@ __device__ __forceinline__ void stencil_kind_unit(const InstDesc& I, int unit,
   if (phase != PH_RES64 && phase != PH_STENCIL && phase != PH_CHEB) return;
   if ((WHICH == 1 && phase == PH_RES64) || (WHICH == 2 && phase != PH_RES64)) return;
   if ((MODE != 0 || KIND != 1) && phase == PH_CHEB) return;  // direct form, KIND 1 only
+  if (I.form != 0) return;  // the density form has its own kernels
   const InstState sn = snapshot(st);
   if (WHICH != 1 && phase == PH_RES64) {
     double acc[kSlots] = {0.0, 0.0, 0.0, 0.0};
@@ -1182,7 +1227,10 @@ __device__ __forceinline__ void flat_kind_unit(const InstDesc& I, int unit) {
     }
     case PH_CORRECT: {
       double ps[1] = {0.0};
-      sweep_correct<T>(I, c0, c1, sn.p_set == 0, ps[0]);
+      if (I.form)
+        sweep_correct<T, true>(I, c0, c1, sn.p_set == 0, ps[0]);
+      else
+        sweep_correct<T, false>(I, c0, c1, sn.p_set == 0, ps[0]);
       store_partials<1, double>(ps, I.part, I.nunits_f, unit);
       break;
     }
@@ -1219,6 +1267,21 @@ __global__ void __launch_bounds__(kDirectThreads, Res64Occ<T>::kMinBlocks) k_res
     const InstDesc* __restrict__ insts, const UnitRef* __restrict__ units) {
   const UnitRef ur = units[blockIdx.x];
   stencil_kind_unit<T, T, 0, 2>(insts[ur.inst], ur.unit, nullptr);
+}
+
+// The same for the instances in the density form.
+template <class T>
+__global__ void __launch_bounds__(kDirectThreads, Res64Occ<T>::kMinBlocks) k_res64_density(
+    const InstDesc* __restrict__ insts, const UnitRef* __restrict__ units) {
+  const UnitRef ur = units[blockIdx.x];
+  const InstDesc& I = insts[ur.inst];
+  InstState* st = I.st;
+  if (__ldcg(&st->phase) != PH_RES64 || I.form == 0) return;
+  const InstState sn = snapshot(st);
+  double acc[kSlots] = {0.0, 0.0, 0.0, 0.0};
+  sweep_res64_direct<T, true>(I, &sn, ur.unit, acc);
+  store_partials<kSlots, double>(acc, I.part, I.nunits, ur.unit);
+  finish_sweep(I, st, PH_RES64, I.nunits);
 }
 
 // TMA-staged pipeline
@@ -1390,9 +1453,11 @@ cudaError_t prepare_step(int prec, int mode, size_t smem_bytes) {
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
 }
 
-cudaError_t launch_res64(int prec, const InstDesc* desc, const UnitRef* units, int nunits,
+cudaError_t launch_res64(int prec, int form, const InstDesc* desc, const UnitRef* units, int nunits,
                          int threads, cudaStream_t s) {
-  if (prec == PREC_FP64)
+  if (form)
+    k_res64_density<float><<<nunits, threads, 0, s>>>(desc, units);
+  else if (prec == PREC_FP64)
     k_res64_direct<double><<<nunits, threads, 0, s>>>(desc, units);
   else
     k_res64_direct<float><<<nunits, threads, 0, s>>>(desc, units);
@@ -1402,6 +1467,7 @@ cudaError_t launch_res64(int prec, const InstDesc* desc, const UnitRef* units, i
 cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
                            const UnitRef* units, int nunits, int threads, size_t smem_bytes,
                            cudaStream_t s) {
+  if (kind >= kSweepDensityCg) return launch_density(kind, desc, units, nunits, threads, s);
   void* fn = stencil_fn(prec, mode, kind);
   void* args[] = {(void*)&desc, (void*)&units};
   return cudaLaunchKernel(fn, dim3(nunits), dim3(threads), args, smem_bytes, s);

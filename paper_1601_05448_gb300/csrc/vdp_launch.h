@@ -1,4 +1,5 @@
-// vdp_launch.h -- host-side launchers of the kernels in vdp_kernels.cu and vdp_setup.cu (internal to libvdp).
+// vdp_launch.h -- host-side launchers of the kernels in vdp_kernels.cu, vdp_setup.cu
+// and vdp_density.cu (internal to libvdp).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -10,31 +11,41 @@ namespace vdp {
 // vdp_setup.cu.  The check stores gen in *bad when an entry is <= 0 or not finite; the launches
 // that take (bad, gen) then write nothing (null: not gated).
 cudaError_t launch_check_density(const double* rho, long long n, int gen, int* bad, cudaStream_t s);
-// face coefficients on the low faces (spacings h_d; duct: no flux through the x ends), D^-1/2, D
+// face coefficients on the low faces (spacings h_d; duct: no flux through the x ends) and D; with
+// sinv also D^-1/2, with rho32 the density form's FP32 density and dsc[0] = kappa
 cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
                                       double hy, double hz, int duct, double* bx, double* by,
-                                      double* bz, double* sinv, double* dg, const int* bad,
-                                      int gen, cudaStream_t s);
+                                      double* bz, double* sinv, double* dg, float* rho32,
+                                      double* dsc, const int* bad, int gen, cudaStream_t s);
+cudaError_t launch_sinv(const double* dg, long long n, double* sinv, cudaStream_t s);
 cudaError_t launch_scaled(int prec, const double* bx, const double* by, const double* bz,
                           const double* sinv, int nx, int ny, int nz, void* sx, void* sy, void* sz,
                           void* sd, const int* bad, int gen, cudaStream_t s);
-// W = D^1/2, and rho W (the fixed-point iteration's input weight)
+// W = D^1/2, and rho W (the scaled fixed-point iteration's input weight) from rho32 and kappa
 cudaError_t launch_omega(const double* dg, const double* sinv, long long n, float* omega,
                          cudaStream_t s);
-cudaError_t launch_rho_weight(const double* rho, const double* dg, const double* sinv, long long n,
-                              float* out, const int* bad, int gen, cudaStream_t s);
+cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double hx2, const double* dg,
+                              const double* sinv, long long n, float* out, cudaStream_t s);
 cudaError_t launch_apply(const double* bx, const double* by, const double* bz, const double* p,
                          int nx, int ny, int nz, double* out, cudaStream_t s);
 cudaError_t launch_init(InstDesc* desc, const double* rhs, double* p, double tol, double inner_tol,
                         int max_iter, int inner_max, int use_guess, int precision,
                         cudaStream_t s);
 cudaError_t prepare_step(int prec, int mode, size_t smem_bytes);
-// mode 0 only: the FP64 residual sweep (its own kernel, launched before each stencil launch)
-cudaError_t launch_res64(int prec, const InstDesc* desc, const UnitRef* units, int nunits,
+// mode 0 only: the FP64 residual sweep (its own kernel, launched before each stencil launch) of
+// the instances in the scaled (form 0) or the density form (1)
+cudaError_t launch_res64(int prec, int form, const InstDesc* desc, const UnitRef* units, int nunits,
                          int threads, cudaStream_t s);
 // kind (direct sweep variants): 0 = CG, 1 = CG and Chebyshev preconditioner sweeps (PH_CHEB),
-// 2 = the fixed-point iteration; stencil_kind(pc) picks it for an instance's preconditioner
-inline int stencil_kind(int pc) { return pc == PC_FIXED ? 2 : (pc == PC_CHEB ? 1 : 0); }
+// 2 = the fixed-point iteration; the density form's sweeps (vdp_density.cu); stencil_kind(d)
+// picks it for an instance
+constexpr int kSweepDensityCg = 3, kSweepDensityFixed = 4;
+inline int stencil_kind(const InstDesc& d) {
+  if (d.form) return d.pc == PC_FIXED ? kSweepDensityFixed : kSweepDensityCg;
+  return d.pc == PC_FIXED ? 2 : (d.pc == PC_CHEB ? 1 : 0);
+}
+cudaError_t launch_density(int kind, const InstDesc* desc, const UnitRef* units, int nunits,
+                           int threads, cudaStream_t s);
 cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
                            const UnitRef* units, int nunits, int threads, size_t smem_bytes,
                            cudaStream_t s);

@@ -197,7 +197,7 @@ extern "C" int vdp_solve_noalloc(int nx, int ny, int nz, double L, const double*
   if (bad) return VDP_EDENSITY;
   double* dg = f64[12];
   NA_CK(launch_build_coefficients(rho, nx, ny, nz, L / nx, L / ny, L / nz, 0, bx, by, bz, sinv, dg,
-                                  nullptr, 0, s));
+                                  nullptr, nullptr, nullptr, 0, s));
   NA_CK(launch_scaled(precision, bx, by, bz, sinv, nx, ny, nz, sx, sy, sz, sd, nullptr, 0, s));
 
   // the default unit layout of vdp_solve
@@ -252,7 +252,7 @@ extern "C" int vdp_solve_noalloc(int nx, int ny, int nz, double L, const double*
   long long rounds = 0;
   while (!done && rounds < max_rounds) {
     for (int i = 0; i < m; ++i) {
-      NA_CK(launch_res64(precision, desc, units, nunits, lay.threads, s));
+      NA_CK(launch_res64(precision, 0, desc, units, nunits, lay.threads, s));
       NA_CK(launch_stencil(precision, lay.mode, 0, desc, units, nunits, lay.threads, lay.smem, s));
       NA_CK(launch_flat(precision, desc, units + nunits, nunits_f, s));
     }

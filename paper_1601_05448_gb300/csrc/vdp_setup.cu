@@ -1,6 +1,7 @@
 // vdp_setup.cu -- what vdp_set_density builds from rho: the FP64 face coefficients
 // b_d = 2 / (rho_l + rho_r) / h_d^2 on the low faces, the diagonal D (sum of the six faces of a
-// cell), the Jacobi scaling D^-1/2, the scaled inner coefficients and the spectral weights.
+// cell), the Jacobi scaling D^-1/2, the scaled inner coefficients, and the FP32 density of the
+// density-form sweeps (vdp_density.cu).
 //
 // What bounds these kernels.  The FP64 pipe of this GPU issues 2 FMA per clock and SM, 1/64 of the
 // FP32 rate: an IEEE double division costs about ten such instructions and a reciprocal square
@@ -69,6 +70,15 @@ __device__ __forceinline__ double inv_sqrt(double D) {
   return fma(Y * e, fma(e, 0.375, 0.5), Y);
 }
 
+// A positive normal v times 2^p as FP32, rounded to nearest, by integer operations.
+__device__ __forceinline__ float narrow_rn_pow2(double v, int p) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127 + p;
+  if (e <= 0) return 0.f;
+  if (e >= 255) return __uint_as_float(0x7f800000u);
+  return __uint_as_float((((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29)) + ((lo >> 28) & 1u));
+}
+
 // Thread geometry of the set-up kernels: pair q = two cells of a row, z chunk [z0, z1).
 struct PairMarch {
   int x, y, z0, z1;
@@ -120,14 +130,18 @@ __global__ void k_check_density(const double* __restrict__ rho, long long n, int
   if (!ok) *bad = gen;
 }
 
-// b_d[c] = 2 / (rho[c - e_d] + rho[c]) / h_d^2 on the low d-face of every cell.
+// b_d[c] = 2 / (rho[c - e_d] + rho[c]) / h_d^2 on the low d-face of every cell; with rho32 also the
+// FP32 density, scaled by the power of two of the first cell's (2^-e0), and dsc[0] = 2^e0 hx^2, the
+// factor between the density-form operator and A (vdp_density.cu).
 // duct: the face at the x ends (slot x = 0, shared by x = 0 and x = Lx) carries no flux.
 __global__ void __launch_bounds__(kSetupThreads)
     k_faces(const double* __restrict__ rho, int nx, int ny, int nz, double cx, double cy, double cz,
             int duct, double* __restrict__ bx, double* __restrict__ by, double* __restrict__ bz,
-            const int* bad, int gen) {
+            float* __restrict__ rho32, double* dsc, double hx2, const int* bad, int gen) {
   if (rejected(bad, gen)) return;
   const PairMarch m = pair_march(nx, ny, nz);
+  const int e0 = exponent_of(__ldg(rho)) - 1023;
+  if (dsc && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) dsc[0] = ldexp(hx2, e0);
   if (!m.on) return;
   const bool wide = ((uintptr_t)rho & 15) == 0;  // 16-byte loads of the caller's array
   auto load = [&](long long o) {
@@ -152,11 +166,14 @@ __global__ void __launch_bounds__(kSetupThreads)
     *reinterpret_cast<double2*>(bx + c) = vx;
     *reinterpret_cast<double2*>(by + c) = vy;
     *reinterpret_cast<double2*>(bz + c) = vz;
+    if (rho32)
+      *reinterpret_cast<float2*>(rho32 + c) =
+          make_float2(narrow_rn_pow2(r.x, -e0), narrow_rn_pow2(r.y, -e0));
     lo = r;
   }
 }
 
-// sinv = D^-1/2 with D = sum of the six face coefficients of the cell
+// D = sum of the six face coefficients of the cell; with sinv also D^-1/2
 __global__ void __launch_bounds__(kSetupThreads)
     k_diag(const double* __restrict__ bx, const double* __restrict__ by,
            const double* __restrict__ bz, int nx, int ny, int nz, double* __restrict__ sinv,
@@ -177,9 +194,16 @@ __global__ void __launch_bounds__(kSetupThreads)
     D.x = x.x + x.y + y.x + yp.x + z_lo.x + z_hi.x;
     D.y = x.y + xr + y.y + yp.y + z_lo.y + z_hi.y;
     *reinterpret_cast<double2*>(dg + c) = D;
-    *reinterpret_cast<double2*>(sinv + c) = make_double2(inv_sqrt(D.x), inv_sqrt(D.y));
+    if (sinv) *reinterpret_cast<double2*>(sinv + c) = make_double2(inv_sqrt(D.x), inv_sqrt(D.y));
     z_lo = z_hi;
   }
+}
+
+// D^-1/2 alone, for a context whose density was set for the density form
+__global__ void k_sinv(const double* __restrict__ dg, long long n, double* __restrict__ sinv) {
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
+       c += (long long)gridDim.x * blockDim.x)
+    sinv[c] = inv_sqrt(dg[c]);
 }
 
 // Rounded to nearest: the rounding errors of the stored off-diagonals have no common sign, so
@@ -272,13 +296,13 @@ __global__ void k_omega(const double* __restrict__ dg, const double* __restrict_
     omega[c] = __double2float_rn(dg[c] * sinv[c]);
 }
 
-__global__ void k_rho_weight(const double* __restrict__ rho, const double* __restrict__ dg,
-                             const double* __restrict__ sinv, long long n, float* __restrict__ out,
-                             const int* bad, int gen) {
-  if (rejected(bad, gen)) return;
+__global__ void k_rho_weight(const float* __restrict__ rho32, const double* __restrict__ dsc,
+                             double ihx2, const double* __restrict__ dg,
+                             const double* __restrict__ sinv, long long n, float* __restrict__ out) {
+  const double scale = dsc[0] * ihx2;  // 2^e0
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
        c += (long long)gridDim.x * blockDim.x)
-    out[c] = __double2float_rn(rho[c] * (dg[c] * sinv[c]));
+    out[c] = __double2float_rn((double)rho32[c] * scale * (dg[c] * sinv[c]));
 }
 
 // ---- host launchers ---------------------------------------------------------------------------
@@ -308,12 +332,18 @@ cudaError_t launch_check_density(const double* rho, long long n, int gen, int* b
 
 cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
                                       double hy, double hz, int duct, double* bx, double* by,
-                                      double* bz, double* sinv, double* dg, const int* bad,
-                                      int gen, cudaStream_t s) {
+                                      double* bz, double* sinv, double* dg, float* rho32,
+                                      double* dsc, const int* bad, int gen, cudaStream_t s) {
   const dim3 g = pair_grid(nx, ny, nz);
   k_faces<<<g, kSetupThreads, 0, s>>>(rho, nx, ny, nz, 2.0 / (hx * hx), 2.0 / (hy * hy),
-                                      2.0 / (hz * hz), duct, bx, by, bz, bad, gen);
+                                      2.0 / (hz * hz), duct, bx, by, bz, rho32, dsc, hx * hx, bad,
+                                      gen);
   k_diag<<<g, kSetupThreads, 0, s>>>(bx, by, bz, nx, ny, nz, sinv, dg, bad, gen);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sinv(const double* dg, long long n, double* sinv, cudaStream_t s) {
+  k_sinv<<<flat_grid(n), 256, 0, s>>>(dg, n, sinv);
   return cudaGetLastError();
 }
 
@@ -344,9 +374,9 @@ cudaError_t launch_omega(const double* dg, const double* sinv, long long n, floa
   return cudaGetLastError();
 }
 
-cudaError_t launch_rho_weight(const double* rho, const double* dg, const double* sinv, long long n,
-                              float* out, const int* bad, int gen, cudaStream_t s) {
-  k_rho_weight<<<flat_grid(n), 256, 0, s>>>(rho, dg, sinv, n, out, bad, gen);
+cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double hx2, const double* dg,
+                              const double* sinv, long long n, float* out, cudaStream_t s) {
+  k_rho_weight<<<flat_grid(n), 256, 0, s>>>(rho32, dsc, 1.0 / hx2, dg, sinv, n, out);
   return cudaGetLastError();
 }
 

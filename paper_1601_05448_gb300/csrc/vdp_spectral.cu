@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(M1 * rows_per_block<M1, M2>(), 768 / (M1 * row
 // The X- transform of one row per group of M1 threads: `src` is the row of the half spectrum
 // (global or shared memory), `rb` the group's shared exchange buffer; z = W x is stored to row
 // `row` of a.out.  Every thread of the block calls it (barrier).
-template <class T, int M1, int M2, bool MIRROR>
+template <class T, int M1, int M2, bool MIRROR, bool WEIGHT>
 __device__ __forceinline__ void x_inv_rows(const SpecArgs& a, const Tables& tb, float2* rb,
                                            const float2* src, long long row, bool live, int t) {
   constexpr int m = M1 * M2;
@@ -369,17 +369,19 @@ __device__ __forceinline__ void x_inv_rows(const SpecArgs& a, const Tables& tb, 
   // the transforms (cells 2l, 2l + 1 with l = k2 + M2 k1, k2 = t, t + M1, ...)
   constexpr int R = (M2 + M1 - 1) / M1;
   float2 wv[R][M1];
-  const float* om = a.omega_out ? a.omega_out + row * a.nxd : nullptr;
+  if constexpr (WEIGHT) {
+    const float* om = a.omega_out + row * a.nxd;
 #pragma unroll
-  for (int rr = 0; rr < R; ++rr)
+    for (int rr = 0; rr < R; ++rr)
 #pragma unroll
-    for (int k1 = 0; k1 < M1; ++k1) {
-      const int k2 = t + M1 * rr;
-      const int l = k2 + M2 * k1;
-      wv[rr][k1] = make_float2(1.f, 1.f);
-      if (live && om && k2 < M2 && (!MIRROR || 2 * l < a.nxd))
-        wv[rr][k1] = *reinterpret_cast<const float2*>(om + 2 * l);
-    }
+      for (int k1 = 0; k1 < M1; ++k1) {
+        const int k2 = t + M1 * rr;
+        const int l = k2 + M2 * k1;
+        wv[rr][k1] = make_float2(1.f, 1.f);
+        if (live && k2 < M2 && (!MIRROR || 2 * l < a.nxd))
+          wv[rr][k1] = *reinterpret_cast<const float2*>(om + 2 * l);
+      }
+  }
   // Z'[k] = (X[k] + conj X[m-k]) + i conj(W_nx^k) (X[k] - conj X[m-k]); inverse M2-point DFTs.
   // Both X[k] and X[m-k] are read straight from the spectrum: for a fixed j2 the lanes of a row
   // read consecutive values, ascending and descending.
@@ -420,8 +422,8 @@ __device__ __forceinline__ void x_inv_rows(const SpecArgs& a, const Tables& tb, 
       for (int k1 = 0; k1 < M1; ++k1) {
         const int l = k2 + M2 * k1;  // cells 2l, 2l + 1 of the row
         if (MIRROR && 2 * l >= a.nxd) continue;  // the second half is the reflection
-        const float2 z = make_float2(o[k1].x * wv[rr][k1].x, o[k1].y * wv[rr][k1].y);
-        Pair<T>::st(out + 2 * l, z);
+        Pair<T>::st(out + 2 * l, WEIGHT ? make_float2(o[k1].x * wv[rr][k1].x, o[k1].y * wv[rr][k1].y)
+                                        : o[k1]);
       }
     }
   }
@@ -431,7 +433,7 @@ __device__ __forceinline__ void x_inv_rows(const SpecArgs& a, const Tables& tb, 
 // shared memory.  The 512^3 mixed solve: 33.6 ms against 34.1 ms with one row group per block
 // and the tables read through L1; and a launch in another phase of the solve exits after 3 us
 // instead of 29 us.
-template <class T, int M1, int M2, bool MIRROR>
+template <class T, int M1, int M2, bool MIRROR, bool WEIGHT>
 __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>())
     k_spec_x_inv_persistent(SpecArgs a) {
   constexpr int RY = inv_rows_per_block<M1, M2>();
@@ -445,7 +447,7 @@ __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>())
   for (long long g = blockIdx.x; g * RY < rows; g += gridDim.x) {
     const long long row = (long long)a.z0 * a.ny + g * RY + r;
     const bool live = g * RY + r < rows;
-    x_inv_rows<T, M1, M2, MIRROR>(a, tb, sb + r * SB, a.spec + row * a.nxp, row, live, t);
+    x_inv_rows<T, M1, M2, MIRROR, WEIGHT>(a, tb, sb + r * SB, a.spec + row * a.nxp, row, live, t);
     __syncthreads();  // the exchange buffers are reused by the next group
   }
   if (a.st) {  // the solve: the last block of the application's X- launches completes the
@@ -702,15 +704,18 @@ void factor(int n, int* m1, int* m2) {
 using SpecKernel = void (*)(SpecArgs);
 
 template <class T>
-SpecKernel x_kernel(int m, bool inverse, bool mirror, int* threads) {
+SpecKernel x_kernel(int m, bool inverse, bool mirror, bool weight, int* threads) {
   int m1, m2;
   factor(m, &m1, &m2);
 #define VDP_X(M1, M2)                                                                       \
   if (m1 == M1 && m2 == M2) {                                                               \
     *threads = M1 * (inverse ? inv_rows_per_block<M1, M2>() : rows_per_block<M1, M2>());     \
+    if (inverse && weight)                                                                  \
+      return mirror ? k_spec_x_inv_persistent<T, M1, M2, true, true>                        \
+                    : k_spec_x_inv_persistent<T, M1, M2, false, true>;                      \
     if (inverse)                                                                            \
-      return mirror ? k_spec_x_inv_persistent<T, M1, M2, true>                              \
-                    : k_spec_x_inv_persistent<T, M1, M2, false>;                            \
+      return mirror ? k_spec_x_inv_persistent<T, M1, M2, true, false>                       \
+                    : k_spec_x_inv_persistent<T, M1, M2, false, false>;                     \
     if constexpr (sizeof(T) == 8 || kXFwdF32Persistent)                                     \
       return mirror ? k_spec_x_fwd_persistent<T, M1, M2, true>                              \
                     : k_spec_x_fwd_persistent<T, M1, M2, false>;                            \
@@ -782,8 +787,9 @@ bool x_f64(int prec, bool inv, const SpecArgs& a) { return prec == PREC_FP64 && 
 
 SpecKernel x_pass_kernel(int prec, bool inv, const SpecArgs& a, int* threads) {
   const int m = a.nx / 2;
-  return x_f64(prec, inv, a) ? x_kernel<double>(m, inv, a.mirror != 0, threads)
-                             : x_kernel<float>(m, inv, a.mirror != 0, threads);
+  const bool weight = inv && a.omega_out;
+  return x_f64(prec, inv, a) ? x_kernel<double>(m, inv, a.mirror != 0, weight, threads)
+                             : x_kernel<float>(m, inv, a.mirror != 0, weight, threads);
 }
 
 // Grid of an X pass over `rows` rows: a persistent grid for the persistent forms (0 if not
@@ -815,7 +821,7 @@ long long line_grid(int which, int n, long long tiles) {
 bool x_supported(int nx) {
   if (nx % 2) return false;
   int threads = 0;
-  return x_kernel<float>(nx / 2, false, false, &threads) != nullptr;
+  return x_kernel<float>(nx / 2, false, false, false, &threads) != nullptr;
 }
 
 bool yz_supported(int n) {
@@ -889,11 +895,12 @@ cudaError_t spectral_upload_roots() {
   // the X kernels (static shared memory): resident blocks per SM, for the persistent grids
   g_x_per_sm[dev < 0 ? 0 : dev].clear();
   for (const int m : kXHalfLengths)
-    for (int v = 0; v < 8 && e == cudaSuccess; ++v) {
-      const bool f64 = v & 1, inv = v & 2, mirror = v & 4;
+    for (int v = 0; v < 16 && e == cudaSuccess; ++v) {
+      const bool f64 = v & 1, inv = v & 2, mirror = v & 4, weight = v & 8;
+      if (weight && !inv) continue;
       int threads = 0, per_sm = 0;
-      const SpecKernel k = f64 ? x_kernel<double>(m, inv, mirror, &threads)
-                               : x_kernel<float>(m, inv, mirror, &threads);
+      const SpecKernel k = f64 ? x_kernel<double>(m, inv, mirror, weight, &threads)
+                               : x_kernel<float>(m, inv, mirror, weight, &threads);
       if (!k) continue;
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, 0);
       if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;

@@ -42,11 +42,11 @@ cudaError_t launch_for_phase(vdp_ctx* c, int prec, int phase, cudaStream_t s) {
   const Layout& l = c->lay;
   switch (phase) {
     case PH_RES64:
-      if (l.mode == 0) return launch_res64(prec, c->desc, c->units, l.nunits, l.threads, s);
+      if (l.mode == 0) return launch_res64(prec, c->hdesc.form, c->desc, c->units, l.nunits, l.threads, s);
       return launch_stencil(prec, l.mode, 0, c->desc, c->units, l.nunits, l.threads, l.smem, s);
     case PH_STENCIL:
     case PH_CHEB:
-      return launch_stencil(prec, l.mode, stencil_kind(c->hdesc.pc), c->desc, c->units, l.nunits,
+      return launch_stencil(prec, l.mode, stencil_kind(c->hdesc), c->desc, c->units, l.nunits,
                             l.threads, l.smem, s);
     default:
       return launch_flat(prec, c->desc, c->units + l.nunits, l.nunits_f, s);
