@@ -201,6 +201,7 @@ int configure_layout(vdp_ctx* c, int prec) {
   VDP_CK(cudaMemcpyAsync(c->desc, &d, sizeof(d), cudaMemcpyHostToDevice, c->stream));
   VDP_CK(cudaStreamSynchronize(c->stream));
   VDP_CK(prepare_step(prec, lay.mode, lay.smem));
+  if (d.form) VDP_CK(prepare_density());
   if (c->gexec) {
     cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;

@@ -187,8 +187,12 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 
 // Unit layout for an nx x ny x nz grid in precision `prec`; zero arguments pick the defaults.
 // mode 0 (direct, default): units of up to 256 threads (whole rows, whole warps), one thread per
-// 16-byte vector of a row tile of threads * V / nx rows (V = 4 FP32, 2 FP64), about 12 units per
-// SM worth of z chunks.
+// 16-byte vector of a row tile of threads * V / nx rows (V = 4 FP32, 2 FP64); a unit per 12288
+// cells, at least 3 and at most 12 per SM.  A unit reloads two planes at its start and adds a slot
+// to the sweep's final sum, so small grids want few units, large ones enough for several waves
+// (sweep and residual, us: 112 x 100 x 90 FP64 46.5 and 68 with 1824 units, 34.8 and 45 with 456;
+// 96^3 FP32 26.2 and 56 against 19.4 and 42; 256^3 FP32 93.6 and 265 with 1824, 89.9 and 246 with
+// 1368; 512^3 550 with 1824, 598 with 456).
 // mode 1 (TMA pipeline): FP64 512-thread units with about 2048 cells per plane, FP32/BF16 256
 // threads with about 1024; the row tile shrinks until four pipeline stages fit; stages default to
 // what fits (at most 6), or to 4 when that lets two units share an SM; about four waves.
@@ -245,11 +249,15 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
   }
   if (ty > ny) ty = ny;
   const int uy = (ny + ty - 1) / ty;
-  const long long want = units > 0 ? units : 2LL * kSMs * per_sm;
+  const long long ncell = (long long)nx * ny * nz;
+  long long want = units > 0 ? units : 2LL * kSMs * per_sm;
+  if (units <= 0 && mode == 0) {
+    const long long by_cells = ncell / 12288 > 3LL * kSMs ? ncell / 12288 : 3LL * kSMs;
+    if (by_cells < want) want = by_cells;
+  }
   long long zc = (want + uy - 1) / uy;
   if (zc > nz) zc = nz;
   if (zc < 1) zc = 1;
-  const long long ncell = (long long)nx * ny * nz;
   long long nf = ncell / 4096;
   if (nf > kSMs * 8) nf = kSMs * 8;
   if (nf < 1) nf = 1;

@@ -44,6 +44,7 @@ inline int stencil_kind(const InstDesc& d) {
   if (d.form) return d.pc == PC_FIXED ? kSweepDensityFixed : kSweepDensityCg;
   return d.pc == PC_FIXED ? 2 : (d.pc == PC_CHEB ? 1 : 0);
 }
+cudaError_t prepare_density();  // shared-memory limits on the current device
 cudaError_t launch_density(int kind, const InstDesc* desc, const UnitRef* units, int nunits,
                            int threads, cudaStream_t s);
 cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
