@@ -322,8 +322,8 @@ __global__ void __launch_bounds__(kDirectThreads, 2)
   const UnitRef ur = units[blockIdx.x];
   const InstDesc& I = insts[ur.inst];
   InstState* st = I.st;
-  if (__ldcg(&st->phase) != PH_STENCIL || I.form == 0 || (I.pc == PC_FIXED) != FIXED) return;
-  const InstState sn = snapshot(st);
+  const InstState& sn = block_state(st);
+  if (sn.phase != PH_STENCIL || I.form == 0 || (I.pc == PC_FIXED) != FIXED) return;
   float part[1] = {0.f};
   if constexpr (FIXED) {
     sweep_density<0>(I, &sn, ur.unit, part[0], slots);

@@ -61,13 +61,17 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-// Block reduction of NS per-thread partials of type A (float partials stay FP32 within a warp;
-// the warp totals are combined in FP64) into slot k of this unit: part[k * nunits + unit].
-// Fixed shuffle tree and fixed warp order: deterministic.
+// Block reduction of NS per-thread partials of type A into slot k of this unit:
+// part[k * nunits + unit], always in the same order (threads without cells add zeros), so the
+// block size does not show.  FP32 partials, and blocks of more than kDirectThreads: a shuffle tree
+// per warp, the warp totals combined in FP64.  FP64 partials: through shared memory, a lane adding
+// its column of the block's warps before one shuffle tree -- a warp-wide FP64 addition holds this
+// GPU's FP64 pipe for 16 cycles, and a tree in every warp cost more of them than the update of
+// four cells per thread.
 template <int NS, class A>
-__device__ __forceinline__ void store_partials(const A (&v)[NS], double* part, int nunits,
-                                               int unit) {
-  __shared__ double red[kMaxThreads / 32][kSlots];
+__device__ __forceinline__ void store_partials_by_warp(const A (&v)[NS], double* part, int nunits,
+                                                       int unit) {
+  __shared__ double red[kMaxThreads / 32][NS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
   A w[NS];
@@ -89,11 +93,40 @@ __device__ __forceinline__ void store_partials(const A (&v)[NS], double* part, i
   }
 }
 
+template <int NS>
+__device__ __forceinline__ void store_partials_by_column(const double (&v)[NS], double* part,
+                                                         int nunits, int unit) {
+  static_assert(kFlatThreads <= kDirectThreads, "the columns hold one block");
+  __shared__ double col[NS][kDirectThreads];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nwarps = blockDim.x >> 5;
+  __syncthreads();  // col[] may still be read by a previous use
+#pragma unroll
+  for (int k = 0; k < NS; ++k) col[k][threadIdx.x] = v[k];
+  __syncthreads();
+  for (int k = warp; k < NS; k += nwarps) {
+    double s = 0.0;
+    for (int w = 0; w < nwarps; ++w) s += col[k][w * 32 + lane];
+    s = warp_sum(s);
+    if (lane == 0) part[k * nunits + unit] = s;
+  }
+}
+
+template <int NS, class A>
+__device__ __forceinline__ void store_partials(const A (&v)[NS], double* part, int nunits,
+                                               int unit) {
+  if constexpr (sizeof(A) == 8)
+    store_partials_by_column<NS>(v, part, nunits, unit);
+  else
+    store_partials_by_warp<NS, A>(v, part, nunits, unit);
+}
+
 // Returns true in every thread of the unit that arrives last for its instance.
 __device__ __forceinline__ bool arrive_last(unsigned int* ticket, int nunits) {
   __shared__ int last;
+  __syncthreads();  // every warp's partials are written
   if (threadIdx.x == 0) {
-    __threadfence();  // partials of this unit visible before its ticket
+    __threadfence();  // ... and visible before this unit's ticket
     unsigned t = atomicAdd(ticket, 1u);
     last = (t == (unsigned)nunits - 1u);
     if (last) __threadfence();
@@ -102,39 +135,47 @@ __device__ __forceinline__ bool arrive_last(unsigned int* ticket, int nunits) {
   return last != 0;
 }
 
-// Fixed-order sum of one slot over all units (warp 0; identical result in every lane).
-// Fixed-order sum of one slot over all units by the last unit: 64 lanes (warps 0 and 1) each
-// add the slots lane, lane + 64, ... in index order with eight loads in flight, then a fixed
-// shuffle tree per warp, warp 0's total plus warp 1's.  The order does not depend on the block
-// size, so an instance sums identically whatever launch it runs in.  Every thread returns it.
-static __device__ __noinline__ double block_sum_slot(const double* part, int nunits) {
-  __shared__ double wsum[2];
-  constexpr int U = 8, LANES = 64;
-  const int t = threadIdx.x;
-  double s = 0.0;
-  if (t < LANES) {
-    for (int i0 = t; i0 < nunits; i0 += U * LANES) {
+// Fixed-order sums of the first ns slots over all units by the last unit.  A slot is summed by 256
+// lanes, each adding the slots lane, lane + 256, ... in index order with eight loads in flight,
+// then a fixed shuffle tree per 32 lanes, then the eight totals in order.  The (slot, 32 lanes)
+// pairs are spread over the block's warps, so the slots are summed side by side; the order does
+// not depend on the block size, so an instance sums identically whatever launch it runs in.  (One
+// slot after the other over 64 lanes, the four sums of a residual took most of the 20 us that
+// sweep needs on a 32^3 grid.)  Every thread returns the sums.
+static __device__ __noinline__ void block_sum_slots(const double* part, int nunits, int ns,
+                                                    double (&S)[kSlots]) {
+  constexpr int U = 8, LANES = 256, G = LANES / 32;
+  __shared__ double wsum[kSlots][G];
+  const int lane = threadIdx.x & 31;
+  for (int q = threadIdx.x >> 5; q < ns * G; q += blockDim.x >> 5) {
+    const double* slot = part + (long long)(q / G) * nunits;
+    double s = 0.0;
+    for (int i0 = (q % G) * 32 + lane; i0 < nunits; i0 += U * LANES) {
       double v[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u * LANES;
-        v[u] = i < nunits ? __ldcg(part + i) : 0.0;
+        v[u] = i < nunits ? __ldcg(slot + i) : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) s += v[u];
     }
     s = warp_sum(s);
+    if (lane == 0) wsum[q / G][q % G] = s;
   }
-  __syncthreads();  // wsum may be in use by a previous call
-  if (t == 0 || t == 32) wsum[t >> 5] = s;
   __syncthreads();
-  return wsum[0] + wsum[1];
+  for (int k = 0; k < ns; ++k) {
+    double s = 0.0;
+#pragma unroll
+    for (int g = 0; g < G; ++g) s += wsum[k][g];
+    S[k] = s;
+  }
 }
 
 // ---- phase transitions (run by thread 0 of the last unit) -------------------------------------
 
-static __device__ void transition(const InstDesc& I, volatile InstState* st, int phase,
-                           const double (&S)[kSlots]) {
+static __device__ __noinline__ void transition(const InstDesc& I, InstState* st, int phase,
+                                               const double (&S)[kSlots]) {
   st->sweeps += 1;
   if (st->fault && phase != PH_FINAL) {  // a bounded wait expired: stop with what p holds
     st->status = 6;                      // VDP_ETIMEOUT
@@ -294,6 +335,20 @@ static __device__ void transition(const InstDesc& I, volatile InstState* st, int
   }
 }
 
+static_assert(sizeof(InstState) % 16 == 0, "the state is copied in 16-byte words");
+__device__ __forceinline__ void load_state(const InstState* st, InstState& s) {
+  const int4* a = reinterpret_cast<const int4*>(st);
+  int4* b = reinterpret_cast<int4*>(&s);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(InstState) / 16); ++i) b[i] = __ldcg(a + i);
+}
+__device__ __forceinline__ void store_state(InstState* st, const InstState& s) {
+  int4* a = reinterpret_cast<int4*>(st);
+  const int4* b = reinterpret_cast<const int4*>(&s);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(InstState) / 16); ++i) __stcg(a + i, b[i]);
+}
+
 // partial-sum slots each phase produces
 __device__ __forceinline__ int phase_slots(int phase) {
   switch (phase) {
@@ -315,33 +370,31 @@ __device__ __forceinline__ void finish_sweep(const InstDesc& I, InstState* st, i
   if (nparts <= 0) nparts = nunits;
   if (arrive_last(I.ticket, nunits)) {  // uniform in the block
     double S[kSlots] = {0.0, 0.0, 0.0, 0.0};
-    const int ns = phase_slots(phase);
-    for (int k = 0; k < ns; ++k) S[k] = block_sum_slot(I.part + k * nparts, nparts);
+    block_sum_slots(I.part, nparts, phase_slots(phase), S);
     if (threadIdx.x == 0) {
-      transition(I, st, phase, S);
+      // the whole state in one go (its words are independent loads past L1), the transition on
+      // the copy, and back: field by field it was a chain of a dozen trips to L2
+      InstState s;
+      load_state(st, s);
+      transition(I, &s, phase, S);
+      store_state(st, s);
       *I.ticket = 0u;
       __threadfence();
     }
   }
 }
 
-// Snapshot of the state fields the sweeps read.  Loaded with ld.global.cg (L2, not L1): in the
-// persistent kernel the previous phase's transition may have been written by another SM moments
-// ago, so an L1 copy must not be used; the loads are independent, so they overlap.
-__device__ __forceinline__ InstState snapshot(const InstState* st) {
-  InstState s;
-  s.phase = __ldcg(&st->phase);
-  s.inner_iters = __ldcg(&st->inner_iters);
-  s.parity = __ldcg(&st->parity);
-  s.first_res = __ldcg(&st->first_res);
-  s.zero_sol = __ldcg(&st->zero_sol);
-  s.use_guess = __ldcg(&st->use_guess);
-  s.mu_f = __ldcg(&st->mu_f);
-  s.alpha = __ldcg(&st->alpha);
-  s.beta = __ldcg(&st->beta);
-  s.sum_p = __ldcg(&st->sum_p);
-  s.cheb_j = __ldcg(&st->cheb_j);
-  s.p_set = __ldcg(&st->p_set);
+// The block's copy of an instance's state, read once per block: the words are loaded past L1 (in
+// the persistent kernel another SM may have written them moments ago) by the first threads and
+// handed on through shared memory.  When every warp of every block read the fields itself, a sweep
+// of 1000 blocks sent 100000 requests to the one L2 slice that holds them (the update of a
+// 112 x 100 x 90 grid took 25 us with 250 blocks and 32 us with 1000).  Every thread calls it.
+__device__ __forceinline__ const InstState& block_state(const InstState* st) {
+  __shared__ InstState s;
+  __syncthreads();  // a previous copy may still be in use
+  if (threadIdx.x < sizeof(InstState) / 16)
+    reinterpret_cast<int4*>(&s)[threadIdx.x] = __ldcg(reinterpret_cast<const int4*>(st) + threadIdx.x);
+  __syncthreads();
   return s;
 }
 

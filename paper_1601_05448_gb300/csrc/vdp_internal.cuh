@@ -45,7 +45,7 @@ constexpr int kDirectThreads = 256;  // threads per direct-stencil work unit, at
 constexpr int kMaxStages = 8;      // shared-memory pipeline stages of the stencil sweep
 
 // Mutable per-instance solver state (device memory).
-struct InstState {
+struct __align__(16) InstState {
   int phase;
   int status;          // vdp_status
   int iters;           // total inner iterations
@@ -196,8 +196,8 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 // mode 1 (TMA pipeline): FP64 512-thread units with about 2048 cells per plane, FP32/BF16 256
 // threads with about 1024; the row tile shrinks until four pipeline stages fit; stages default to
 // what fits (at most 6), or to 4 when that lets two units share an SM; about four waves.
-// Both: stencil units = row tiles x z chunks (chunk-major); flat units of about 4096+ cells (at
-// most 8 per SM).  In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
+// Both: stencil units = row tiles x z chunks (chunk-major); flat units of 4096+ cells
+// (at most 8 per SM), on small grids down to 1024 for two units per SM.  In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
 // Returns false when the configuration cannot run (rows too long, bad counts).
 inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, int units,
                         int stages, int threads, Layout* L) {
@@ -259,6 +259,8 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
   if (zc > nz) zc = nz;
   if (zc < 1) zc = 1;
   long long nf = ncell / 4096;
+  const long long nf_small = ncell / 1024 < 2LL * kSMs ? ncell / 1024 : 2LL * kSMs;
+  if (nf < nf_small) nf = nf_small;
   if (nf > kSMs * 8) nf = kSMs * 8;
   if (nf < 1) nf = 1;
   L->mode = mode;

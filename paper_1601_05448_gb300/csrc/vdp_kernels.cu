@@ -1170,19 +1170,22 @@ template <class T, class BT, int MODE, int WHICH = 0, int KIND = 1>
 __device__ __forceinline__ void stencil_kind_unit(const InstDesc& I, int unit,
                                                   unsigned char* smem_raw) {
   InstState* st = I.st;
-  const int phase = __ldcg(&st->phase);  // one load decides whether this unit has work
+  const InstState& sn = block_state(st);
+  const int phase = sn.phase;  // decides whether this unit has work
   if (phase != PH_RES64 && phase != PH_STENCIL && phase != PH_CHEB) return;
   if ((WHICH == 1 && phase == PH_RES64) || (WHICH == 2 && phase != PH_RES64)) return;
   if ((MODE != 0 || KIND != 1) && phase == PH_CHEB) return;  // direct form, KIND 1 only
   if (I.form != 0) return;  // the density form has its own kernels
-  const InstState sn = snapshot(st);
   if (WHICH != 1 && phase == PH_RES64) {
     double acc[kSlots] = {0.0, 0.0, 0.0, 0.0};
     if (MODE == 0)
       sweep_res64_direct<T>(I, &sn, unit, acc);
     else
       sweep_res64<T>(I, &sn, unit, acc, reinterpret_cast<double*>(smem_raw));
-    store_partials<kSlots, double>(acc, I.part, I.nunits, unit);
+    if constexpr (MODE == 0)
+      store_partials<kSlots, double>(acc, I.part, I.nunits, unit);
+    else  // blocks of up to 512 threads, and hardly any static shared memory left
+      store_partials_by_warp<kSlots, double>(acc, I.part, I.nunits, unit);
   } else if (WHICH != 2) {
     T part[1] = {0};
     if constexpr (MODE != 0) {
@@ -1199,7 +1202,10 @@ __device__ __forceinline__ void stencil_kind_unit(const InstDesc& I, int unit,
       else
         sweep_stencil_direct<T, BT, false, 0>(I, &sn, unit, part[0]);
     }
-    store_partials<1, T>(part, I.part, I.nunits, unit);
+    if constexpr (MODE == 0)
+      store_partials<1, T>(part, I.part, I.nunits, unit);
+    else
+      store_partials_by_warp<1, T>(part, I.part, I.nunits, unit);
   }
   finish_sweep(I, st, phase, I.nunits);
 }
@@ -1208,9 +1214,9 @@ __device__ __forceinline__ void stencil_kind_unit(const InstDesc& I, int unit,
 template <class T>
 __device__ __forceinline__ void flat_kind_unit(const InstDesc& I, int unit) {
   InstState* st = I.st;
-  const int phase = __ldcg(&st->phase);
+  const InstState& sn = block_state(st);
+  const int phase = sn.phase;
   if (phase != PH_MEANF && phase != PH_UPDATE && phase != PH_CORRECT && phase != PH_FINAL) return;
-  const InstState sn = snapshot(st);
   const long long c0 = flat_begin(I, unit), c1 = flat_begin(I, unit + 1);
   switch (phase) {
     case PH_MEANF: {
@@ -1276,8 +1282,8 @@ __global__ void __launch_bounds__(kDirectThreads, Res64Occ<T>::kMinBlocks) k_res
   const UnitRef ur = units[blockIdx.x];
   const InstDesc& I = insts[ur.inst];
   InstState* st = I.st;
-  if (__ldcg(&st->phase) != PH_RES64 || I.form == 0) return;
-  const InstState sn = snapshot(st);
+  const InstState& sn = block_state(st);
+  if (sn.phase != PH_RES64 || I.form == 0) return;
   double acc[kSlots] = {0.0, 0.0, 0.0, 0.0};
   sweep_res64_direct<T, true>(I, &sn, ur.unit, acc);
   store_partials<kSlots, double>(acc, I.part, I.nunits, ur.unit);

@@ -45,8 +45,9 @@ __device__ __forceinline__ float to_f(double v) { return narrow(v); }
 __device__ __forceinline__ void from_f(float v, float* out) { *out = v; }
 __device__ __forceinline__ void from_f(float v, double* out) { *out = widen(v); }
 
-__device__ __forceinline__ bool mg_active(const InstState* st) {
-  return st == nullptr || __ldcg(&st->phase) == PH_SPEC;
+__device__ __forceinline__ bool mg_active(const InstState* st) {  // one load per block
+  if (st == nullptr) return true;
+  return __syncthreads_or(threadIdx.x == 0 && __ldcg(&st->phase) == PH_SPEC) != 0;
 }
 
 struct Nbr {

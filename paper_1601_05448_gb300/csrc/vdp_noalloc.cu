@@ -27,7 +27,9 @@ using namespace vdp;
 namespace {
 
 constexpr long long kMaxCells = VDP_NOALLOC_MAX_CELLS;
-constexpr int kMaxUnits = kMaxCells / 8 + 16;  // stencil units (<= ny*nz) plus flat units (<= 16)
+// stencil units (3 per SM and one more row of tiles, of at least 256 cells each: below 1000) plus
+// flat units (<= 64); the size of the scratch array is part of the interface
+constexpr int kMaxUnits = kMaxCells / 8 + 16;
 constexpr size_t kAlign = 256;
 
 constexpr size_t align_up(size_t b) { return (b + kAlign - 1) / kAlign * kAlign; }

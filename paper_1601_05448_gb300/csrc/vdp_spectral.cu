@@ -153,9 +153,11 @@ __device__ __forceinline__ Tables tables(const SpecArgs& a) {
 }
 
 // In the solve every pass first checks that the instance is in the spectral phase (one L2
-// load); the stand-alone inverse passes st = nullptr and always runs.
+// load per block: thread 0's, handed on by the barrier); the stand-alone inverse passes
+// st = nullptr and always runs.  Every thread calls it.
 __device__ __forceinline__ bool spec_active(const SpecArgs& a) {
-  return a.st == nullptr || __ldcg(&a.st->phase) == PH_SPEC;
+  if (a.st == nullptr) return true;
+  return __syncthreads_or(threadIdx.x == 0 && __ldcg(&a.st->phase) == PH_SPEC) != 0;
 }
 
 template <class T> struct Pair;
