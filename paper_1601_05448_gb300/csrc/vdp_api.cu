@@ -112,7 +112,7 @@ void free_ctx(vdp_ctx* c) {
     delete c->mg;
   }
   void* bufs[] = {c->bx, c->by, c->bz, c->sinv, c->dg, c->f0, c->sx, c->sy, c->sz, c->sd, c->x, c->r, c->d0, c->d1,
-                  c->za, c->zb, c->dch, c->spec, c->omega, c->sptab, c->rho_w, c->rho32, c->dsc, c->d_rounds,
+                  c->za, c->zb, c->dch, c->spec, c->omega, c->sptab, c->rho_w, c->rho32, c->rho_lo, c->dsc, c->d_rounds,
                   c->q, c->part, c->ticket, c->st, c->desc, c->units, c->flag, c->stage_a,
                   c->stage_b, c->proj_f};
   for (void* b : bufs)
@@ -157,10 +157,14 @@ int configure_layout(vdp_ctx* c, int prec) {
   d.mode = lay.mode;
   d.form = density_form(c, prec) ? 1 : 0;
   d.duct = c->bc_x == VDP_BC_DUCT;
-  const double hx = c->Lx / c->nx, hy = c->Ly / c->ny, hz = c->Lz / c->nz;
-  d.cy = (float)(2.0 * (hx / hy) * (hx / hy));
-  d.cz = (float)(2.0 * (hx / hz) * (hx / hz));
+  const double h[3] = {c->Lx / c->nx, c->Ly / c->ny, c->Lz / c->nz};
+  for (int k = 0; k < 3; ++k) {
+    const double f = 2.0 * density_scale(c) / (h[k] * h[k]);
+    d.ch[k] = (float)f;
+    d.cl[k] = (float)(f - (double)d.ch[k]);
+  }
   d.rho32 = c->rho32;
+  d.rho_lo = c->rho_lo;
   d.dsc = c->dsc;
   d.ncell = c->n;
   d.bx = c->bx;
@@ -331,7 +335,7 @@ bool ensure_while_graph(vdp_ctx* c, int prec) {
 }
 
 bool density_form(const vdp_ctx* c, int prec) {
-  return prec == PREC_MIXED && c->rho32_valid &&
+  return (prec == PREC_MIXED || (prec == PREC_FP64 && c->rho_lo_valid)) && c->rho32_valid &&
          (c->opts.method == VDP_METHOD_FIXED_POINT || c->opts.precond == VDP_PRECOND_SPECTRAL);
 }
 
@@ -404,11 +408,11 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   // rho D^1/2 gives rho r, and z = damping D^1/2 (-L_h)^-1 (rho r) is the scaled form of the
   // paper's update p += damping L_h^-1 (rho r) (applied as p -= D^-1/2 x, x the sum of the z)
   a->out = c->za;
-  a->out_f32 = fixed ? 1 : 0;  // the fixed-point sweep reads z as FP32
-  // density form: the stored residual is g = rho' r (fixed point) or r (CG), z is unscaled, and
-  // the inverse is that of hx^2 L_h: no weights
+  a->out_f32 = fixed || density_form(c, prec) ? 1 : 0;  // those sweeps read z as FP32
+  // density form: the stored residual is g = rho' r (FP32 fixed point) or r, z is unscaled and
+  // FP32, and the inverse is that of s L_h: no weights but rho' on the FP64 fixed point's r
   const bool dens = density_form(c, prec);
-  a->omega_in = dens ? nullptr : fixed ? c->rho_w : c->omega;
+  a->omega_in = dens ? (fixed && prec == PREC_FP64 ? c->rho32 : nullptr) : fixed ? c->rho_w : c->omega;
   a->omega_out = dens ? nullptr : c->omega;
   a->spec = c->spec;
   a->tw = reinterpret_cast<const float2*>(c->sptab);
@@ -420,9 +424,8 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   a->nxd = c->nx;
   a->mirror = c->bc_x == VDP_BC_DUCT;
   a->ewt = a->mirror ? 0.5f : 1.f;
-  const double hx = c->Lx / c->nx;
   a->scale = (float)((fixed ? c->opts.damping : 1.0) / ((double)nxt * c->ny * c->nz) /
-                     (dens ? hx * hx : 1.0));
+                     (dens ? density_scale(c) : 1.0));
   a->st = c->st;
   a->I = c->desc;
   a->zunits = spectral_units(nxt, c->ny, c->nz);
@@ -480,8 +483,7 @@ int prepare_spectral_solve(vdp_ctx* c) {
   if ((s = ensure_omega(c)) != VDP_OK) return s;
   if (fixed && !c->rho_w_valid) {
     if (!c->rho_w) VDP_CK(cudaMalloc((void**)&c->rho_w, sizeof(float) * (size_t)c->n));
-    const double hx = c->Lx / c->nx;
-    VDP_CK(launch_rho_weight(c->rho32, c->dsc, hx * hx, c->dg, c->sinv, c->n, c->rho_w, c->stream));
+    VDP_CK(launch_rho_weight(c->rho32, c->dsc, density_scale(c), c->dg, c->sinv, c->n, c->rho_w, c->stream));
     c->rho_w_valid = true;
   }
   return VDP_OK;
@@ -632,6 +634,15 @@ int vdp_set_options(vdp_ctx* c, const vdp_opts* o) {
     }
     c->rho32_valid = false;
   }
+  if (c->rho32 && o->precision == VDP_FP64 && !c->rho_lo) {
+    const cudaError_t e = cudaMalloc((void**)&c->rho_lo, sizeof(float) * (size_t)c->n);
+    if (e != cudaSuccess) {
+      c->rho_lo = nullptr;
+      c->opts = old;
+      return cuda_fail(e, "vdp_set_options (density)");
+    }
+    c->rho_lo_valid = false;
+  }
   c->stream = (cudaStream_t)o->stream;
   c->layout_dirty = true;
   return VDP_OK;
@@ -655,15 +666,18 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
   // the check and everything built from rho are launched together; the kernels after the check
   // write nothing when it fails, and the host waits once
   const int gen = ++c->density_gen, prec = c->opts.precision;
-  const bool kept = c->rho32_valid;
-  c->rho32_valid = c->rho32 != nullptr;  // as it will be (density_form looks at it)
+  const bool kept = c->rho32_valid, kept_lo = c->rho_lo_valid;
+  float* rho_lo = prec == PREC_FP64 ? c->rho_lo : nullptr;
+  c->rho32_valid = c->rho32 != nullptr;  // as they will be (density_form looks at them)
+  c->rho_lo_valid = rho_lo != nullptr;
   const bool scaled = !density_form(c, prec);
   c->rho32_valid = kept;
+  c->rho_lo_valid = kept_lo;
   VDP_CK(launch_check_density(src, c->n, gen, c->flag, c->stream));
   VDP_CK(launch_build_coefficients(src, c->nx, c->ny, c->nz, c->Lx / c->nx, c->Ly / c->ny,
                                    c->Lz / c->nz, c->bc_x == VDP_BC_DUCT, c->bx, c->by, c->bz,
-                                   scaled ? c->sinv : nullptr, c->dg, c->rho32, c->dsc, c->flag,
-                                   gen, c->stream));
+                                   scaled ? c->sinv : nullptr, c->dg, c->rho32, rho_lo, c->dsc,
+                                   density_scale(c), c->flag, gen, c->stream));
   if (scaled)
     VDP_CK(launch_scaled(prec, c->bx, c->by, c->bz, c->sinv, c->nx, c->ny, c->nz, c->sx, c->sy,
                          c->sz, c->sd, c->flag, gen, c->stream));
@@ -675,8 +689,10 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
   c->omega_valid = false;
   c->rho_w_valid = false;
   c->rho32_valid = c->rho32 != nullptr;
+  c->rho_lo_valid = rho_lo != nullptr;
   c->mg_valid = false;
-  if (c->rho32_valid != kept) c->layout_dirty = true;  // the form may change with it
+  // the form may change with them
+  if (c->rho32_valid != kept || c->rho_lo_valid != kept_lo) c->layout_dirty = true;
   c->has_density = true;
   return VDP_OK;
 }

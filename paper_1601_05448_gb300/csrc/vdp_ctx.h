@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "vdp.h"
 #include "vdp_internal.cuh"
 #include "vdp_multigrid.h"
@@ -49,7 +51,9 @@ struct vdp_ctx {
   float* rho_w = nullptr;          // scaled fixed-point iteration: rho D^1/2 per cell (FP32)
   bool rho_w_valid = false;        // rho_w was computed from the current density
   float* rho32 = nullptr;          // rho / 2^e0 (FP32), kept once a spectral method is selected
-  double* dsc = nullptr;           // kappa = 2^e0 hx^2
+  float* rho_lo = nullptr;         // rho / 2^e0 - rho32 (FP64 solves)
+  bool rho_lo_valid = false;       // rho_lo holds the current density
+  double* dsc = nullptr;           // kappa = 2^e0 s
   bool rho32_valid = false;        // rho32 and dsc hold the current density
   bool sinv_valid = false;         // sinv was computed from the current density
   vdp::MgHier* mg = nullptr;       // multigrid levels (VDP_PRECOND_MG, vdp_mg_apply)
@@ -95,9 +99,12 @@ int configure_layout(vdp_ctx* c, int prec);
 int ensure_scaled(vdp_ctx* c, int prec);  // no-op in the density form, which has none
 int ensure_sinv(vdp_ctx* c);
 // The inner solve runs in the density form (vdp_density.cu): the spectral inverse is its
-// preconditioner or iteration, the coefficients are FP32, and the FP32 density is at hand (a
-// density that was set before the method was selected is not: CG then runs in the scaled form).
+// preconditioner or iteration, the coefficients are not BF16, and the FP32 density (for FP64 with
+// its low part) is at hand.  A density that was set before the method or the precision was
+// selected is not: the solve then runs in the scaled form.
 bool density_form(const vdp_ctx* c, int prec);
+// s of the density form: the power of 4 below hx^2
+inline double density_scale(const vdp_ctx* c) { return std::ldexp(1.0, 2 * std::ilogb(c->Lx / c->nx)); }
 // length of the x transform of the spectral passes: nx, or 2 nx in the duct (even extension)
 inline int spectral_nx(const vdp_ctx* c) { return c->bc_x == VDP_BC_DUCT ? 2 * c->nx : c->nx; }
 // allocate the spectral buffers and tables (no-op when present); VDP_EINVAL for unsupported grids

@@ -5,10 +5,10 @@
 // The spectral inverse does not: in unscaled variables its passes need no weights, and the
 // operator's three face coefficients per cell are functions of one field, the density, so a sweep
 // that reads rho (4 bytes, the neighbours' values from L1 / L2) computes them.  With
-//     rho' = rho / 2^e0 (FP32; e0 the exponent of the first cell),  kappa = 2^e0 hx^2,
-//     A' = kappa A:  face values 2 / (rho'_l + rho'_r) x (hx / h_d)^2,
+//     rho' = rho / 2^e0 (e0 the exponent of the first cell),  s = 2^(2 m), m the exponent of hx,
+//     A' = kappa A, kappa = 2^e0 s:  face values (2 s / h_d^2) / (rho'_l + rho'_r),
 // an inner solve of (-A') X = r gives the correction p -= kappa X, whatever the units of rho and
-// of the box.  Per cell and iteration of the FP32 fixed-point solve this moves
+// of the box; kappa is a power of two, so the scaling rounds nothing.  Per cell and iteration of the FP32 fixed-point solve this moves
 //     X+  g 4            (weights and rt: 8)        X-  z 4            (z and weight: 8)
 //     sweep  z, rho', g, X read, g, X written: 24   (z, three coefficients, rt, x: 32)
 // besides the half spectrum: 32 bytes instead of 48.  Fixed point: g = rho' r is the stored
@@ -128,7 +128,8 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
   const bool row_start = x0 == 0, row_end = x0 + kV == nx;
   const bool left_load = lane == 0 || row_start, right_load = lane == 31 || row_end;
   const bool wall_l = I.duct && row_start, wall_r = I.duct && row_end;
-  const f2 ny2 = pk(-I.cy, -I.cy), nz2 = pk(-I.cz, -I.cz);
+  const float nx1 = -I.ch[0];
+  const f2 ny2 = pk(-I.ch[1], -I.ch[1]), nz2 = pk(-I.ch[2], -I.ch[2]);
   const float beta = (float)st->beta;
   const f2 beta2 = pk(beta, beta);
   const bool first = st->inner_iters == 0;
@@ -219,9 +220,9 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
       rr = __ldg(rho + o + dxr);
     }
     // faces and fluxes b (u_k - u_{k-1}) through the five x faces of the four cells
-    const float b0 = wall_l ? 0.f : face(-2.f, rl, r01.x), b1 = face(-2.f, r01.x, r01.y);
-    const float b2 = face(-2.f, r01.y, r23.x), b3 = face(-2.f, r23.x, r23.y);
-    const float b4 = wall_r ? 0.f : face(-2.f, r23.y, rr);
+    const float b0 = wall_l ? 0.f : face(nx1, rl, r01.x), b1 = face(nx1, r01.x, r01.y);
+    const float b2 = face(nx1, r01.y, r23.x), b3 = face(nx1, r23.x, r23.y);
+    const float b4 = wall_r ? 0.f : face(nx1, r23.y, rr);
     const float f0 = b0 * (u01.x - ul), f1 = b1 * (u01.y - u01.x), fm = b2 * (u23.x - u01.y);
     const float f3 = b3 * (u23.y - u23.x), f4 = b4 * (ur - u23.y);
     f2 a[2] = {pk(f1 - f0, fm - f1), pk(f3 - fm, f4 - f3)};  // A' u, accumulated
@@ -305,6 +306,287 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
   part = active ? s.x + s.y : 0.f;
 }
 
+// ---- the FP64 inner solve ------------------------------------------------------------------------
+// z comes out of the FP32 transforms, so it is an FP32 field in this solve too; r, X, d and q are
+// FP64.  The product A' z in FP64 instructions bounds the sweep by the FP64 pipe (8 instructions
+// per cell at 2 per clock and SM: 282 us at 256^3, where its bytes take 109).  Here coefficients
+// and product are pairs of FP32 numbers (unevaluated sums hi + lo, about 47 bits): rho' as such a
+// pair, the quotient by a Newton step and a corrected remainder, the differences of z exact, the
+// products by FMA with their rounding errors, the six terms summed with the errors carried along.
+// Only the update of the FP64 fields is FP64: three instructions per cell (fixed point), four
+// (CG).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
+// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before.
+struct df {
+  f2 h, l;
+};
+
+__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
+
+// h + l = a + b exactly
+__device__ __forceinline__ df two_sum(f2 a, f2 b) {
+  df r;
+  r.h = add2(a, b);
+  const f2 t = sub2(r.h, a);
+  r.l = add2(sub2(a, sub2(r.h, t)), sub2(b, t));
+  return r;
+}
+__device__ __forceinline__ df two_diff(f2 a, f2 b) {
+  df r;
+  r.h = sub2(a, b);
+  const f2 t = sub2(r.h, a);
+  r.l = sub2(sub2(a, sub2(r.h, t)), add2(b, t));
+  return r;
+}
+
+// c / (a + b), c = -(nch + ncl)
+__device__ __forceinline__ df face_df(f2 nch, f2 ncl, df a, df b) {
+  df s = two_sum(a.h, b.h);
+  s.l = add2(s.l, add2(a.l, b.l));
+  const float2 v = up2(s.h);
+  f2 y = pk(rcp_approx(-v.x), rcp_approx(-v.y));  // -1 / s
+  y = fma2(y, fma2(s.h, y, pk(1.f, 1.f)), y);
+  df q;
+  q.h = mul2(nch, y);
+  const f2 t = add2(fma2(q.h, s.l, fma2(q.h, s.h, nch)), ncl);  // q s - c
+  q.l = mul2(t, y);
+  return q;
+}
+
+// -(b x difference) of a face as an unevaluated sum, from the exact difference d
+__device__ __forceinline__ df minus_flux(df b, df d) {
+  df f;
+  f.h = mul2(neg2(b.h), d.h);
+  const f2 e = fma2(b.l, d.h, fma2(b.h, d.l, fma2(b.h, d.h, f.h)));  // b d + f.h
+  f.l = neg2(e);
+  return f;
+}
+
+// acc -= f
+__device__ __forceinline__ void accumulate_minus(df& acc, df f) {
+  const df s = two_diff(acc.h, f.h);
+  acc.h = s.h;
+  acc.l = add2(acc.l, sub2(s.l, f.l));
+}
+__device__ __forceinline__ void accumulate_plus(df& acc, df f) {
+  const df s = two_sum(acc.h, f.h);
+  acc.h = s.h;
+  acc.l = add2(acc.l, add2(s.l, f.l));
+}
+
+enum Stream64 { T_UP, T_UA, T_UB, T_HP, T_HA, T_HB, T_LP, T_LA, T_LB, T_P0, T_P1, T_Q0, T_Q1, kStreams64 };
+
+// FIXED: X += z, r -= (-A') z and the sum of r^2 / D' (FP32, steers the inner stop).
+// CG: d = z + beta d_old, q = (-A') z + beta q_old, and the sum of d q.
+template <bool FIXED>
+__device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstState& st, int unit,
+                                                double& part, ulonglong2* slots) {
+  const int nx = I.nx, ny = I.ny, nz = I.nz;
+  const int tpr = nx / kV;
+  const int tile = unit % I.uy, chunk = unit / I.uy;
+  const int row = threadIdx.x / tpr;
+  const int x0 = (threadIdx.x - row * tpr) * kV;
+  const int yr = tile * I.ty + row;
+  const bool active = row < I.ty && yr < ny;
+  const int y = active ? yr : ny - 1;
+  const int z0 = (int)((long long)chunk * nz / I.zc), z1 = (int)((long long)(chunk + 1) * nz / I.zc);
+  part = 0.0;
+  if (z0 >= z1) return;
+  const int lane = threadIdx.x & 31;
+  const bool row_start = x0 == 0, row_end = x0 + kV == nx;
+  const bool left_load = lane == 0 || row_start, right_load = lane == 31 || row_end;
+  const bool wall_l = I.duct && row_start, wall_r = I.duct && row_end;
+  f2 nch[3], ncl[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    nch[d] = pk(-I.ch[d], -I.ch[d]);
+    ncl[d] = pk(-I.cl[d], -I.cl[d]);
+  }
+  const double beta = st.beta;
+  const bool first = st.inner_iters == 0;  // no X (fixed point), no history (CG) yet
+  const float* rhi = I.rho32;
+  const float* rlo = I.rho_lo;
+  const float* src = static_cast<const float*>(I.za);
+  // p, q: the two FP64 fields read and written (fixed point r, X; CG d, q)
+  const double* pin = static_cast<const double*>(FIXED ? I.r : (st.parity ? I.d1 : I.d0));
+  double* pout = static_cast<double*>(FIXED ? I.r : (st.parity ? I.d0 : I.d1));
+  double* q = static_cast<double*>(FIXED ? I.x : I.q);
+  const long long plane = (long long)nx * ny;
+  const long long dym = y == 0 ? (long long)(ny - 1) * nx : -(long long)nx;
+  const long long dyp = y == ny - 1 ? -(long long)(ny - 1) * nx : (long long)nx;
+  const int dxl = row_start ? nx - 1 : -1, dxr = row_end ? -x0 : kV;
+  const long long cell0 = (long long)y * nx + x0;
+  const long long dz_last = plane * (nz - 1);
+  auto slot = [&](int b, int k) { return slots + (b * kStreams64 + k) * blockDim.x + threadIdx.x; };
+  auto fetch = [&](int b, int z, long long o) {
+    const long long op = z == nz - 1 ? o - dz_last : o + plane;
+    fetch16(slot(b, T_UP), src + op);
+    fetch16(slot(b, T_UA), src + o + dym);
+    fetch16(slot(b, T_UB), src + o + dyp);
+    fetch16(slot(b, T_HP), rhi + op);
+    fetch16(slot(b, T_HA), rhi + o + dym);
+    fetch16(slot(b, T_HB), rhi + o + dyp);
+    fetch16(slot(b, T_LP), rlo + op);
+    fetch16(slot(b, T_LA), rlo + o + dym);
+    fetch16(slot(b, T_LB), rlo + o + dyp);
+    if (FIXED || !first) {
+      fetch16_once(slot(b, T_P0), reinterpret_cast<const float*>(pin + o));
+      fetch16_once(slot(b, T_P1), reinterpret_cast<const float*>(pin + o + 2));
+    }
+    if (!first) {
+      fetch16_once(slot(b, T_Q0), reinterpret_cast<const float*>(q + o));
+      fetch16_once(slot(b, T_Q1), reinterpret_cast<const float*>(q + o + 2));
+    }
+  };
+  auto ldg2 = [](const float* p, f2& a, f2& b) {
+    const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(p));
+    a = t.x;
+    b = t.y;
+  };
+  long long o = (long long)z0 * plane + cell0;
+  fetch(0, z0, o);
+  fetch_commit();
+  f2 u[2];
+  df r[2], bzl[2], fz[2];  // fz: minus the flux through the lower z face
+  {
+    const long long om = z0 == 0 ? o + dz_last : o - plane;
+    f2 um[2];
+    df rm[2];
+    ldg2(src + om, um[0], um[1]);
+    ldg2(src + o, u[0], u[1]);
+    ldg2(rhi + om, rm[0].h, rm[1].h);
+    ldg2(rlo + om, rm[0].l, rm[1].l);
+    ldg2(rhi + o, r[0].h, r[1].h);
+    ldg2(rlo + o, r[0].l, r[1].l);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      bzl[h] = face_df(nch[2], ncl[2], rm[h], r[h]);
+      fz[h] = minus_flux(bzl[h], two_diff(u[h], um[h]));
+    }
+  }
+  double sum = 0.0;
+  float sumf = 0.f;
+  int b = 0;
+  for (int z = z0; z < z1; ++z) {
+    if (z + 1 < z1) fetch(b ^ 1, z + 1, o + plane);
+    fetch_commit();
+    df acc[2];
+    f2 D[2];
+    {  // x: faces 0 .. 4 of the four cells, as pairs (0, 1), (2, 3) and 4
+      const float2 u01 = up2(u[0]), u23 = up2(u[1]);
+      const float2 h01 = up2(r[0].h), h23 = up2(r[1].h), l01 = up2(r[0].l), l23 = up2(r[1].l);
+      float ul = __shfl_up_sync(0xffffffffu, u23.y, 1), ur = __shfl_down_sync(0xffffffffu, u01.x, 1);
+      float hl = __shfl_up_sync(0xffffffffu, h23.y, 1), hr = __shfl_down_sync(0xffffffffu, h01.x, 1);
+      float ll = __shfl_up_sync(0xffffffffu, l23.y, 1), lr = __shfl_down_sync(0xffffffffu, l01.x, 1);
+      if (left_load) {
+        ul = __ldg(src + o + dxl);
+        hl = __ldg(rhi + o + dxl);
+        ll = __ldg(rlo + o + dxl);
+      }
+      if (right_load) {
+        ur = __ldg(src + o + dxr);
+        hr = __ldg(rhi + o + dxr);
+        lr = __ldg(rlo + o + dxr);
+      }
+      df b01 = face_df(nch[0], ncl[0], df{pk(hl, h01.x), pk(ll, l01.x)}, r[0]);
+      const df b23 = face_df(nch[0], ncl[0], df{pk(h01.y, h23.x), pk(l01.y, l23.x)}, r[1]);
+      df b44 = face_df(nch[0], ncl[0], df{pk(h23.y, h23.y), pk(l23.y, l23.y)}, df{pk(hr, hr), pk(lr, lr)});
+      if (wall_l) {
+        b01.h = pk(0.f, up2(b01.h).y);
+        b01.l = pk(0.f, up2(b01.l).y);
+      }
+      if (wall_r) b44.h = b44.l = 0ull;
+      const df f01 = minus_flux(b01, two_diff(u[0], pk(ul, u01.x)));
+      const df f23 = minus_flux(b23, two_diff(u[1], pk(u01.y, u23.x)));
+      const df f44 = minus_flux(b44, two_diff(pk(ur, ur), pk(u23.y, u23.y)));
+      const float2 fh01 = up2(f01.h), fh23 = up2(f23.h), fl01 = up2(f01.l), fl23 = up2(f23.l);
+      const df f12 = {pk(fh01.y, fh23.x), pk(fl01.y, fl23.x)};
+      const df f34 = {pk(fh23.y, up2(f44.h).x), pk(fl23.y, up2(f44.l).x)};
+      acc[0] = f01;  // A' z = sum of (upper flux - lower flux); f holds minus the flux
+      acc[1] = f23;
+      accumulate_minus(acc[0], f12);
+      accumulate_minus(acc[1], f34);
+      if (FIXED) {
+        const float2 bh01 = up2(b01.h), bh23 = up2(b23.h);
+        D[0] = add2(b01.h, pk(bh01.y, bh23.x));
+        D[1] = add2(b23.h, pk(bh23.y, up2(b44.h).x));
+      }
+    }
+    fetch_wait_previous();
+    ulonglong2 t = *slot(b, T_UP);
+    const f2 un[2] = {t.x, t.y};
+    t = *slot(b, T_HP);
+    const ulonglong2 t2 = *slot(b, T_LP);
+    const df rn[2] = {{t.x, t2.x}, {t.y, t2.y}};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const df bz = face_df(nch[2], ncl[2], r[h], rn[h]);
+      const df f = minus_flux(bz, two_diff(un[h], u[h]));
+      accumulate_plus(acc[h], fz[h]);
+      accumulate_minus(acc[h], f);
+      fz[h] = f;
+      if (FIXED) D[h] = add2(D[h], add2(bzl[h].h, bz.h));
+      bzl[h] = bz;
+    }
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      t = *slot(b, side ? T_UB : T_UA);
+      const f2 v[2] = {t.x, t.y};
+      t = *slot(b, side ? T_HB : T_HA);
+      const ulonglong2 tl = *slot(b, side ? T_LB : T_LA);
+      const df rv[2] = {{t.x, tl.x}, {t.y, tl.y}};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const df by = face_df(nch[1], ncl[1], rv[h], r[h]);
+        accumulate_minus(acc[h], minus_flux(by, two_diff(v[h], u[h])));
+        if (FIXED) D[h] = add2(D[h], by.h);
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 ah = up2(acc[h].h), al = up2(acc[h].l), uu = up2(u[h]);
+      const double2 pv = *reinterpret_cast<const double2*>(slot(b, h ? T_P1 : T_P0));
+      const double2 qv = *reinterpret_cast<const double2*>(slot(b, h ? T_Q1 : T_Q0));
+      double2 po, qo;
+      if constexpr (FIXED) {
+        po.x = (pv.x + widen(ah.x)) + widen(al.x);
+        po.y = (pv.y + widen(ah.y)) + widen(al.y);
+        qo.x = widen(uu.x);
+        qo.y = widen(uu.y);
+        if (!first) {
+          qo.x += qv.x;
+          qo.y += qv.y;
+        }
+        const float2 d = up2(D[h]);
+        const float rx = narrow(po.x), ry = narrow(po.y);
+        sumf = fmaf(rx * rcp_approx(d.x), rx, sumf);
+        sumf = fmaf(ry * rcp_approx(d.y), ry, sumf);
+      } else {
+        po.x = widen(uu.x);
+        po.y = widen(uu.y);
+        qo.x = -(widen(ah.x) + widen(al.x));
+        qo.y = -(widen(ah.y) + widen(al.y));
+        if (!first) {
+          po.x = fma(beta, pv.x, po.x);
+          po.y = fma(beta, pv.y, po.y);
+          qo.x = fma(beta, qv.x, qo.x);
+          qo.y = fma(beta, qv.y, qo.y);
+        }
+        sum = fma(po.x, qo.x, sum);
+        sum = fma(po.y, qo.y, sum);
+      }
+      if (active) {
+        *reinterpret_cast<double2*>(pout + o + 2 * h) = po;
+        *reinterpret_cast<double2*>(q + o + 2 * h) = qo;
+      }
+      u[h] = un[h];
+      r[h] = rn[h];
+    }
+    o += plane;
+    b ^= 1;
+  }
+  part = active ? (FIXED ? (double)sumf : sum) : 0.0;
+}
+
 size_t density_smem(bool fixed, int threads) {
   const int streams = fixed ? Streams<0>::kCount : Streams<2>::kCount;
   return sizeof(ulonglong2) * (size_t)kStages * streams * threads;
@@ -337,20 +619,58 @@ __global__ void __launch_bounds__(kDirectThreads, 2)
   finish_sweep(I, st, PH_STENCIL, I.nunits);
 }
 
-cudaError_t prepare_density() {
-  const cudaError_t e = cudaFuncSetAttribute(k_density<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)density_smem(true, kDirectThreads));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_density<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)density_smem(false, kDirectThreads));
+// The same in FP64: four cells per thread of the FP64 layout's two, so half its threads; three
+// blocks of 128 threads per SM (168 registers).
+constexpr int kDensity64Threads = kDirectThreads / 2;
+
+template <bool FIXED>
+__global__ void __launch_bounds__(kDensity64Threads, 3)
+    k_density64(const InstDesc* __restrict__ insts, const UnitRef* __restrict__ units) {
+  extern __shared__ __align__(16) ulonglong2 slots[];
+  const UnitRef ur = units[blockIdx.x];
+  const InstDesc& I = insts[ur.inst];
+  InstState* st = I.st;
+  const InstState& sn = block_state(st);
+  if (sn.phase != PH_STENCIL || I.form == 0 || (I.pc == PC_FIXED) != FIXED) return;
+  double part[1] = {0.0};
+  sweep_density64<FIXED>(I, sn, ur.unit, part[0], slots);
+  store_partials<1, double>(part, I.part, I.nunits, ur.unit);
+  finish_sweep(I, st, PH_STENCIL, I.nunits);
 }
 
-cudaError_t launch_density(int kind, const InstDesc* desc, const UnitRef* units, int nunits,
-                           int threads, cudaStream_t s) {
-  if (kind == kSweepDensityFixed)
+static size_t density64_smem(int threads) {
+  return sizeof(ulonglong2) * (size_t)kStages * kStreams64 * threads;
+}
+
+cudaError_t prepare_density() {
+  struct {
+    const void* fn;
+    size_t smem;
+  } const k[] = {{(const void*)k_density<true>, density_smem(true, kDirectThreads)},
+                 {(const void*)k_density<false>, density_smem(false, kDirectThreads)},
+                 {(const void*)k_density64<true>, density64_smem(kDensity64Threads)},
+                 {(const void*)k_density64<false>, density64_smem(kDensity64Threads)}};
+  for (const auto& e : k) {
+    const cudaError_t r = cudaFuncSetAttribute(e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e.smem);
+    if (r != cudaSuccess) return r;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_density(int prec, int kind, const InstDesc* desc, const UnitRef* units,
+                           int nunits, int threads, cudaStream_t s) {
+  const bool fixed = kind == kSweepDensityFixed;
+  if (prec == PREC_FP64) {
+    const int t = (threads / 2 + 31) / 32 * 32;  // whole warps; threads beyond the tile are idle
+    if (fixed)
+      k_density64<true><<<nunits, t, density64_smem(t), s>>>(desc, units);
+    else
+      k_density64<false><<<nunits, t, density64_smem(t), s>>>(desc, units);
+  } else if (fixed) {
     k_density<true><<<nunits, threads, density_smem(true, threads), s>>>(desc, units);
-  else
+  } else {
     k_density<false><<<nunits, threads, density_smem(false, threads), s>>>(desc, units);
+  }
   return cudaGetLastError();
 }
 

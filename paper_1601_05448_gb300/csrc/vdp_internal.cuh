@@ -95,7 +95,7 @@ struct InstDesc {
   int mode;            // stencil sweep: 0 = direct register march, 1 = TMA-staged pipeline
   int form;            // inner variables: 0 = Jacobi-scaled, 1 = density form (vdp_density.cu)
   int duct;            // density form: the faces at the x ends carry no coefficient
-  float cy, cz;        // density form: face factors 2 (hx / hy)^2, 2 (hx / hz)^2 (x: 2)
+  float ch[3], cl[3];  // density form: face factors 2 s / h_d^2 as FP32 pairs hi + lo
   long long ncell;
   const double* rhs;   // caller's f (set per solve)
   double* p;           // caller's p (set per solve)
@@ -111,7 +111,8 @@ struct InstDesc {
   const void* sz;
   const void* sd;      // BF16 only: diagonal correction of the stored inner operator
   const float* rho32;  // density form: rho / 2^e0 in FP32
-  const double* dsc;   // density form: kappa = 2^e0 hx^2 (the inner operator is kappa A)
+  const float* rho_lo; // density form, FP64: rho / 2^e0 - rho32
+  const double* dsc;   // density form: kappa = 2^e0 s (the inner operator is kappa A)
   void* x;             // inner solution (correction), inner type
   void* r;             // inner residual
   void* d0;            // search direction, double buffered

@@ -857,7 +857,8 @@ __device__ void sweep_stencil_direct(const InstDesc& I, const InstState* st, int
 // per term, 8 FP64 operations per cell against 13 for the face-difference form; in the mixed
 // precisions the scaling rt = D^-1/2 r is an FP32 product; the norms are summed in FP32.
 // What the residual sweep hands to the inner solve in the density form (DENS), from the FP64
-// residual of a cell: fixed point g = rho' r and r^2 / D' (D' = kappa D), CG r and r^2.
+// residual of a cell: fixed point g = rho' r (FP64 inner type: r) and r^2 / D' (D' = kappa D), CG r
+// and r^2.
 struct DensityResidual {
   bool fixed;
   int ek;      // kappa = 2^ek x mk
@@ -941,7 +942,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       double2 si = make_double2(0.0, 0.0);
       float2 rh = make_float2(1.f, 1.f);
       if (!DENS) si = *reinterpret_cast<const double2*>(I.sinv + o);
-      if (DENS && dr.fixed) rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o));
+      if (DENS && dr.fixed && !IsF64<T>::value) rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o));
       const double l0 = h == 0 ? left : pc[h - 1];
       const double r1 = h + 2 == VR ? right : pc[h + 2];
       const double br1 = h + 2 == VR ? bxr : I.bx[o + 2];
@@ -965,8 +966,13 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       T t0, t1;
       float r0f = narrow(res0), r1f = narrow(res1), t0f, t1f;
       if constexpr (DENS) {
-        t0 = rh.x * r0f;
-        t1 = rh.y * r1f;
+        if constexpr (IsF64<T>::value) {  // r itself
+          t0 = res0;
+          t1 = res1;
+        } else {
+          t0 = rh.x * r0f;
+          t1 = rh.y * r1f;
+        }
         t0f = dr.fixed ? r0f * r0f * dr.inv_diag(dg.x) : r0f * r0f;  // the norm's terms
         t1f = dr.fixed ? r1f * r1f * dr.inv_diag(dg.y) : r1f * r1f;
       } else if constexpr (IsF64<T>::value) {
@@ -1020,6 +1026,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
   const DensityResidual dr = DENS ? DensityResidual(I) : DensityResidual();
   double a0 = 0;
   T a1 = 0;
+  float a1f = 0.f;  // DENS
   if (row < I.ty && yr < ny) {
     for (int z = z0; z < z1; ++z) {
       const long long o = ((long long)z * ny + yr) * nx + x0;
@@ -1034,14 +1041,19 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
           const float r0 = narrow(f0), r1 = narrow(f1);
           float2 rh = make_float2(1.f, 1.f), d = make_float2(1.f, 1.f);
           if (dr.fixed) {
-            rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o + h));
+            if (!IsF64<T>::value) rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o + h));
             const double2 D = *reinterpret_cast<const double2*>(I.dg + o + h);
             d = make_float2(dr.inv_diag(D.x), dr.inv_diag(D.y));
           }
-          rt[o + h] = rh.x * r0;
-          rt[o + h + 1] = rh.y * r1;
+          if constexpr (IsF64<T>::value) {
+            rt[o + h] = f0;
+            rt[o + h + 1] = f1;
+          } else {
+            rt[o + h] = rh.x * r0;
+            rt[o + h + 1] = rh.y * r1;
+          }
           a0 = fma(f0, f0, fma(f1, f1, a0));
-          a1 = fmaf(r0 * d.x, r0, fmaf(r1 * d.y, r1, a1));
+          a1f = fmaf(r0 * d.x, r0, fmaf(r1 * d.y, r1, a1f));
         } else if constexpr (IsF64<T>::value) {
           const T t0 = si.x * f0, t1 = si.y * f1;
           rt[o + h] = t0;
@@ -1061,7 +1073,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
     }
   }
   acc[0] = a0;          // ||r||^2
-  acc[1] = (double)a1;  // ||rt||^2
+  acc[1] = DENS ? (dr.fixed ? (double)a1f : a0) : (double)a1;  // ||rt||^2 (density form: see above)
   acc[2] = 0.0;         // sum of p
   acc[3] = a0;          // ||f - <f>||^2 (this is the first residual)
 }
@@ -1461,7 +1473,9 @@ cudaError_t prepare_step(int prec, int mode, size_t smem_bytes) {
 
 cudaError_t launch_res64(int prec, int form, const InstDesc* desc, const UnitRef* units, int nunits,
                          int threads, cudaStream_t s) {
-  if (form)
+  if (form && prec == PREC_FP64)
+    k_res64_density<double><<<nunits, threads, 0, s>>>(desc, units);
+  else if (form)
     k_res64_density<float><<<nunits, threads, 0, s>>>(desc, units);
   else if (prec == PREC_FP64)
     k_res64_direct<double><<<nunits, threads, 0, s>>>(desc, units);
@@ -1473,7 +1487,7 @@ cudaError_t launch_res64(int prec, int form, const InstDesc* desc, const UnitRef
 cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
                            const UnitRef* units, int nunits, int threads, size_t smem_bytes,
                            cudaStream_t s) {
-  if (kind >= kSweepDensityCg) return launch_density(kind, desc, units, nunits, threads, s);
+  if (kind >= kSweepDensityCg) return launch_density(prec, kind, desc, units, nunits, threads, s);
   void* fn = stencil_fn(prec, mode, kind);
   void* args[] = {(void*)&desc, (void*)&units};
   return cudaLaunchKernel(fn, dim3(nunits), dim3(threads), args, smem_bytes, s);

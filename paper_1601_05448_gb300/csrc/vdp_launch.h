@@ -12,11 +12,13 @@ namespace vdp {
 // that take (bad, gen) then write nothing (null: not gated).
 cudaError_t launch_check_density(const double* rho, long long n, int gen, int* bad, cudaStream_t s);
 // face coefficients on the low faces (spacings h_d; duct: no flux through the x ends) and D; with
-// sinv also D^-1/2, with rho32 the density form's FP32 density and dsc[0] = kappa
+// sinv also D^-1/2, with rho32 the density form's FP32 density (with rho_lo what it rounds off)
+// and dsc[0] = kappa = 2^e0 s
 cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
                                       double hy, double hz, int duct, double* bx, double* by,
                                       double* bz, double* sinv, double* dg, float* rho32,
-                                      double* dsc, const int* bad, int gen, cudaStream_t s);
+                                      float* rho_lo, double* dsc, double s2, const int* bad,
+                                      int gen, cudaStream_t s);
 cudaError_t launch_sinv(const double* dg, long long n, double* sinv, cudaStream_t s);
 cudaError_t launch_scaled(int prec, const double* bx, const double* by, const double* bz,
                           const double* sinv, int nx, int ny, int nz, void* sx, void* sy, void* sz,
@@ -24,7 +26,7 @@ cudaError_t launch_scaled(int prec, const double* bx, const double* by, const do
 // W = D^1/2, and rho W (the scaled fixed-point iteration's input weight) from rho32 and kappa
 cudaError_t launch_omega(const double* dg, const double* sinv, long long n, float* omega,
                          cudaStream_t s);
-cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double hx2, const double* dg,
+cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double s2, const double* dg,
                               const double* sinv, long long n, float* out, cudaStream_t s);
 cudaError_t launch_apply(const double* bx, const double* by, const double* bz, const double* p,
                          int nx, int ny, int nz, double* out, cudaStream_t s);
@@ -45,7 +47,7 @@ inline int stencil_kind(const InstDesc& d) {
   return d.pc == PC_FIXED ? 2 : (d.pc == PC_CHEB ? 1 : 0);
 }
 cudaError_t prepare_density();  // shared-memory limits on the current device
-cudaError_t launch_density(int kind, const InstDesc* desc, const UnitRef* units, int nunits,
+cudaError_t launch_density(int prec, int kind, const InstDesc* desc, const UnitRef* units, int nunits,
                            int threads, cudaStream_t s);
 cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
                            const UnitRef* units, int nunits, int threads, size_t smem_bytes,

@@ -70,13 +70,14 @@ __device__ __forceinline__ double inv_sqrt(double D) {
   return fma(Y * e, fma(e, 0.375, 0.5), Y);
 }
 
-// A positive normal v times 2^p as FP32, rounded to nearest, by integer operations.
+// v times 2^p as FP32, rounded to nearest, by integer operations (below the FP32 range: 0).
 __device__ __forceinline__ float narrow_rn_pow2(double v, int p) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
   const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127 + p;
-  if (e <= 0) return 0.f;
-  if (e >= 255) return __uint_as_float(0x7f800000u);
-  return __uint_as_float((((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29)) + ((lo >> 28) & 1u));
+  const unsigned sign = hi & 0x80000000u;
+  if (e <= 0) return __uint_as_float(sign);
+  if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
+  return __uint_as_float(sign | ((((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29)) + ((lo >> 28) & 1u)));
 }
 
 // Thread geometry of the set-up kernels: pair q = two cells of a row, z chunk [z0, z1).
@@ -131,17 +132,19 @@ __global__ void k_check_density(const double* __restrict__ rho, long long n, int
 }
 
 // b_d[c] = 2 / (rho[c - e_d] + rho[c]) / h_d^2 on the low d-face of every cell; with rho32 also the
-// FP32 density, scaled by the power of two of the first cell's (2^-e0), and dsc[0] = 2^e0 hx^2, the
-// factor between the density-form operator and A (vdp_density.cu).
+// FP32 density, scaled by the power of two of the first cell's (2^-e0), with rho_lo what that
+// rounds off, and dsc[0] = 2^e0 s2, the factor between the density-form operator and A
+// (vdp_density.cu).
 // duct: the face at the x ends (slot x = 0, shared by x = 0 and x = Lx) carries no flux.
 __global__ void __launch_bounds__(kSetupThreads)
     k_faces(const double* __restrict__ rho, int nx, int ny, int nz, double cx, double cy, double cz,
             int duct, double* __restrict__ bx, double* __restrict__ by, double* __restrict__ bz,
-            float* __restrict__ rho32, double* dsc, double hx2, const int* bad, int gen) {
+            float* __restrict__ rho32, float* __restrict__ rho_lo, double* dsc, double s2,
+            const int* bad, int gen) {
   if (rejected(bad, gen)) return;
   const PairMarch m = pair_march(nx, ny, nz);
   const int e0 = exponent_of(__ldg(rho)) - 1023;
-  if (dsc && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) dsc[0] = ldexp(hx2, e0);
+  if (dsc && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) dsc[0] = ldexp(s2, e0);
   if (!m.on) return;
   const bool wide = ((uintptr_t)rho & 15) == 0;  // 16-byte loads of the caller's array
   auto load = [&](long long o) {
@@ -166,9 +169,14 @@ __global__ void __launch_bounds__(kSetupThreads)
     *reinterpret_cast<double2*>(bx + c) = vx;
     *reinterpret_cast<double2*>(by + c) = vy;
     *reinterpret_cast<double2*>(bz + c) = vz;
-    if (rho32)
-      *reinterpret_cast<float2*>(rho32 + c) =
-          make_float2(narrow_rn_pow2(r.x, -e0), narrow_rn_pow2(r.y, -e0));
+    if (rho32) {
+      const float2 h = make_float2(narrow_rn_pow2(r.x, -e0), narrow_rn_pow2(r.y, -e0));
+      *reinterpret_cast<float2*>(rho32 + c) = h;
+      if (rho_lo)
+        *reinterpret_cast<float2*>(rho_lo + c) =
+            make_float2(narrow_rn_pow2(r.x - widen_pow2(h.x, e0), -e0),
+                        narrow_rn_pow2(r.y - widen_pow2(h.y, e0), -e0));
+    }
     lo = r;
   }
 }
@@ -297,9 +305,9 @@ __global__ void k_omega(const double* __restrict__ dg, const double* __restrict_
 }
 
 __global__ void k_rho_weight(const float* __restrict__ rho32, const double* __restrict__ dsc,
-                             double ihx2, const double* __restrict__ dg,
+                             double is2, const double* __restrict__ dg,
                              const double* __restrict__ sinv, long long n, float* __restrict__ out) {
-  const double scale = dsc[0] * ihx2;  // 2^e0
+  const double scale = dsc[0] * is2;  // 2^e0
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
        c += (long long)gridDim.x * blockDim.x)
     out[c] = __double2float_rn((double)rho32[c] * scale * (dg[c] * sinv[c]));
@@ -333,11 +341,12 @@ cudaError_t launch_check_density(const double* rho, long long n, int gen, int* b
 cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
                                       double hy, double hz, int duct, double* bx, double* by,
                                       double* bz, double* sinv, double* dg, float* rho32,
-                                      double* dsc, const int* bad, int gen, cudaStream_t s) {
+                                      float* rho_lo, double* dsc, double s2, const int* bad,
+                                      int gen, cudaStream_t s) {
   const dim3 g = pair_grid(nx, ny, nz);
   k_faces<<<g, kSetupThreads, 0, s>>>(rho, nx, ny, nz, 2.0 / (hx * hx), 2.0 / (hy * hy),
-                                      2.0 / (hz * hz), duct, bx, by, bz, rho32, dsc, hx * hx, bad,
-                                      gen);
+                                      2.0 / (hz * hz), duct, bx, by, bz, rho32, rho_lo, dsc, s2,
+                                      bad, gen);
   k_diag<<<g, kSetupThreads, 0, s>>>(bx, by, bz, nx, ny, nz, sinv, dg, bad, gen);
   return cudaGetLastError();
 }
@@ -374,9 +383,9 @@ cudaError_t launch_omega(const double* dg, const double* sinv, long long n, floa
   return cudaGetLastError();
 }
 
-cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double hx2, const double* dg,
+cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double s2, const double* dg,
                               const double* sinv, long long n, float* out, cudaStream_t s) {
-  k_rho_weight<<<flat_grid(n), 256, 0, s>>>(rho32, dsc, 1.0 / hx2, dg, sinv, n, out);
+  k_rho_weight<<<flat_grid(n), 256, 0, s>>>(rho32, dsc, 1.0 / s2, dg, sinv, n, out);
   return cudaGetLastError();
 }
 
