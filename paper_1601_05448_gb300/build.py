@@ -16,8 +16,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libvdp.so")
-SOURCES = ["vdp_kernels.cu", "vdp_density.cu", "vdp_setup.cu", "vdp_api.cu", "vdp_batch.cu",
-           "vdp_noalloc.cu", "vdp_timed.cu", "vdp_spectral.cu", "vdp_projection.cu", "vdp_multigrid.cu", "vdp_probe.cu"]
+SOURCES = ["vdp_kernels.cu", "vdp_density.cu", "vdp_resident.cu", "vdp_setup.cu", "vdp_api.cu",
+           "vdp_batch.cu", "vdp_noalloc.cu", "vdp_timed.cu", "vdp_spectral.cu", "vdp_projection.cu", "vdp_multigrid.cu", "vdp_probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]

@@ -112,7 +112,7 @@ void free_ctx(vdp_ctx* c) {
     delete c->mg;
   }
   void* bufs[] = {c->bx, c->by, c->bz, c->sinv, c->dg, c->f0, c->sx, c->sy, c->sz, c->sd, c->x, c->r, c->d0, c->d1,
-                  c->za, c->zb, c->dch, c->spec, c->omega, c->sptab, c->rho_w, c->rho32, c->rho_lo, c->dsc, c->d_rounds,
+                  c->za, c->zb, c->dch, c->spec, c->omega, c->sptab, c->rho_w, c->rho32, c->rho_lo, c->dsc, c->d_rounds, c->rctl,
                   c->q, c->part, c->ticket, c->st, c->desc, c->units, c->flag, c->stage_a,
                   c->stage_b, c->proj_f};
   for (void* b : bufs)
@@ -697,6 +697,32 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
   return VDP_OK;
 }
 
+// Statistics of a finished solve (between the events ev0 and ev1) from its final state.
+static void set_stats(vdp_ctx* c, const InstState& hs, bool done, int launches) {
+  float ms = 0.f;
+  cudaEventElapsedTime(&ms, c->ev0, c->ev1);
+  c->stats.status = done ? hs.status : VDP_ETIMEOUT;
+  c->stats.iters = hs.iters;
+  c->stats.outer_iters = hs.outer;
+  c->stats.rel_res = hs.rel_res;
+  c->stats.rhs_mean = hs.mu_f;
+  c->stats.ms = ms;
+  c->stats.sweeps = hs.sweeps;
+  c->stats.launches = launches;
+}
+
+// Whether this solve runs as one cooperative launch (vdp_resident.cu); allocates its control words.
+static bool resident_solve(vdp_ctx* c, int prec) {
+  if (c->opts.steps_per_sync != 0 || !resident_supported(c->hdesc, prec)) return false;
+  if (c->hdesc.pc != PC_JACOBI && spec_slab(c) < c->nz) return false;
+  if (!c->rctl && cudaMalloc((void**)&c->rctl, sizeof(ResidentCtl)) != cudaSuccess) {
+    cudaGetLastError();
+    c->rctl = nullptr;
+    return false;
+  }
+  return true;
+}
+
 int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   if (!c || !rhs || !p || !(tol > 0.0) || !std::isfinite(tol)) return VDP_EINVAL;
   if (!c->has_density) return VDP_EINVAL;
@@ -709,8 +735,9 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   if ((c->layout_dirty || c->layout_prec != prec) && (s = configure_layout(c, prec)) != VDP_OK)
     return s;
   if ((s = prepare_spectral_solve(c)) != VDP_OK) return s;  // before the capture of its buffers
-  const bool dev_loop = c->opts.steps_per_sync == 0 && ensure_while_graph(c, prec);
-  if (!dev_loop && (s = ensure_graph(c, prec)) != VDP_OK) return s;
+  const bool resident = resident_solve(c, prec);
+  const bool dev_loop = !resident && c->opts.steps_per_sync == 0 && ensure_while_graph(c, prec);
+  if (!resident && !dev_loop && (s = ensure_graph(c, prec)) != VDP_OK) return s;
   const double* drhs = rhs;
   double* dp = p;
   if (host_rhs) {
@@ -726,7 +753,23 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   }
   VDP_CK(cudaEventRecord(c->ev0, c->stream));
   VDP_CK(launch_init(c->desc, drhs, dp, tol, c->opts.inner_tol, c->opts.max_iter,
-                     c->opts.max_iter, c->opts.use_guess ? 1 : 0, prec, c->stream));
+                     c->opts.max_iter, c->opts.use_guess ? 1 : 0, prec,
+                     resident ? c->rctl : nullptr, c->stream));
+  if (resident) {
+    SpecArgs a{};
+    if (c->hdesc.pc != PC_JACOBI) solve_spec_args(c, prec, &a);
+    // two sweeps per iteration and the outer phases; the state machine stops at max_iter itself
+    const long long bound = 3LL * c->opts.max_iter + 4096;
+    VDP_CK(launch_resident(prec, c->hdesc, c->desc, a, c->rctl,
+                           (unsigned)std::min<long long>(bound, 0x7fffffffLL), c->stream));
+    VDP_CK(cudaMemcpyAsync(&c->hstate[0], c->st, sizeof(InstState), cudaMemcpyDeviceToHost,
+                           c->stream));
+    VDP_CK(cudaEventRecord(c->ev1, c->stream));
+    if (host_p) VDP_CK(cudaMemcpyAsync(p, dp, bytes, cudaMemcpyDeviceToHost, c->stream));
+    VDP_CK(cudaStreamSynchronize(c->stream));
+    set_stats(c, c->hstate[0], c->hstate[0].phase >= PH_DONE, 2);
+    return c->stats.status;
+  }
   const int per_round = (c->lay.mode == 0 ? 3 : 2) + precond_launches(c);
   if (dev_loop) {  // the whole solve is one graph launch; the device decides when to stop
     VDP_CK(cudaMemsetAsync(c->d_rounds, 0, sizeof(unsigned), c->stream));
@@ -738,17 +781,8 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
     unsigned loops = 0;  // on the solver's stream: solves on other streams are not waited for
     VDP_CK(cudaMemcpyAsync(&loops, c->d_rounds, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     VDP_CK(cudaStreamSynchronize(c->stream));
-    const InstState& hs = c->hstate[0];
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, c->ev0, c->ev1);
-    c->stats.status = hs.phase >= PH_DONE ? hs.status : VDP_ETIMEOUT;
-    c->stats.iters = hs.iters;
-    c->stats.outer_iters = hs.outer;
-    c->stats.rel_res = hs.rel_res;
-    c->stats.rhs_mean = hs.mu_f;
-    c->stats.ms = ms;
-    c->stats.sweeps = hs.sweeps;
-    c->stats.launches = (int)(1 + (long long)loops * (per_round * kWhileRounds + 1));
+    set_stats(c, c->hstate[0], c->hstate[0].phase >= PH_DONE,
+              (int)(1 + (long long)loops * (per_round * kWhileRounds + 1)));
     return c->stats.status;
   }
   // Polling schedule: graphs of m rounds, two in flight, the host checks the state after each.
@@ -778,17 +812,7 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   VDP_CK(cudaEventRecord(c->ev1, c->stream));
   if (host_p) VDP_CK(cudaMemcpyAsync(p, dp, bytes, cudaMemcpyDeviceToHost, c->stream));
   VDP_CK(cudaStreamSynchronize(c->stream));
-  const InstState& hs = c->hstate[(checked - 1) & 1];
-  float ms = 0.f;
-  cudaEventElapsedTime(&ms, c->ev0, c->ev1);
-  c->stats.status = done ? hs.status : VDP_ETIMEOUT;
-  c->stats.iters = hs.iters;
-  c->stats.outer_iters = hs.outer;
-  c->stats.rel_res = hs.rel_res;
-  c->stats.rhs_mean = hs.mu_f;
-  c->stats.ms = ms;
-  c->stats.sweeps = hs.sweeps;
-  c->stats.launches = (int)(1 + issued * per_round * m);
+  set_stats(c, c->hstate[(checked - 1) & 1], done, (int)(1 + issued * per_round * m));
   return c->stats.status;
 }
 

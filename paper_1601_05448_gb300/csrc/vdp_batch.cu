@@ -299,7 +299,7 @@ int vdp_batch_add(vdp_batch* b, vdp_ctx* c, const double* rhs, double* p, double
   if ((s = prepare_spectral_solve(c)) != VDP_OK) return s;
   VDP_CK(cudaStreamSynchronize(c->stream));
   VDP_CK(launch_init(c->desc, rhs, p, tol, c->opts.inner_tol, c->opts.max_iter, c->opts.max_iter,
-                     c->opts.use_guess ? 1 : 0, b->prec, b->stream));
+                     c->opts.use_guess ? 1 : 0, b->prec, nullptr, b->stream));
   b->members.push_back(Member{c, rhs, p, tol, false});
   b->dirty = true;
   return VDP_OK;

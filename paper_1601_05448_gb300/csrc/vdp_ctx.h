@@ -87,6 +87,7 @@ struct vdp_ctx {
   int w_prec = -1;
   bool w_failed = false;           // the driver cannot build it: use the polling schedule
   unsigned* d_rounds = nullptr;
+  vdp::ResidentCtl* rctl = nullptr;  // resident solve (vdp_resident.cu)
   vdp_stats stats{};
 };
 

@@ -1,598 +1,9 @@
-// vdp_density.cu -- the density form of the inner iteration, used with the constant-coefficient
-// inverse (the paper's fixed-point iteration and spectrally preconditioned CG).
-//
-// The Jacobi-scaled form of vdp_kernels.cu exists for preconditioners that need a unit diagonal.
-// The spectral inverse does not: in unscaled variables its passes need no weights, and the
-// operator's three face coefficients per cell are functions of one field, the density, so a sweep
-// that reads rho (4 bytes, the neighbours' values from L1 / L2) computes them.  With
-//     rho' = rho / 2^e0 (e0 the exponent of the first cell),  s = 2^(2 m), m the exponent of hx,
-//     A' = kappa A, kappa = 2^e0 s:  face values (2 s / h_d^2) / (rho'_l + rho'_r),
-// an inner solve of (-A') X = r gives the correction p -= kappa X, whatever the units of rho and
-// of the box; kappa is a power of two, so the scaling rounds nothing.  Per cell and iteration of the FP32 fixed-point solve this moves
-//     X+  g 4            (weights and rt: 8)        X-  z 4            (z and weight: 8)
-//     sweep  z, rho', g, X read, g, X written: 24   (z, three coefficients, rt, x: 32)
-// besides the half spectrum: 32 bytes instead of 48.  Fixed point: g = rho' r is the stored
-// residual (the right side of the paper's L_h dp = rho r), so X+ reads one field.
-//
-// The march is that of sweep_stencil_direct: a thread owns 16 bytes of one row and walks a z chunk,
-// x neighbours come by shuffle, the rows above and below and the plane above by loads.  Written
-// with plain loads the sweep waited for memory (ncu at 256^3: 8.2 of 13 stall cycles per issue on
-// long-scoreboard, 47 % of the DRAM rate): each thread therefore fetches its operands of the next
-// plane by cp.async into slots of shared memory that only it reads, so no barrier is needed, no
-// registers are held while they fly, and the arithmetic of one plane covers the latency of the
-// next.  Sums, products and Newton steps of the four cells run as paired FP32 instructions, and
-// the fluxes through the x faces and the upper z face are computed once for both cells.
-#include "vdp_device.cuh"
-#include "vdp_internal.cuh"
+// vdp_density.cu -- kernels of the density form's sweeps (vdp_density.cuh says what they compute and
+// why): one launch per sweep.
+#include "vdp_density.cuh"
 #include "vdp_launch.h"
 
 namespace vdp {
-
-namespace {
-
-constexpr int kV = 4;       // cells per thread
-constexpr int kStages = 2;  // planes of operands in flight or in use
-
-using f2 = unsigned long long;  // two FP32 values
-
-__device__ __forceinline__ f2 pk(float a, float b) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 up2(f2 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-  f2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
-  f2 r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-  f2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-  f2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
-// c / (a + b) of a face: the approximate reciprocal and one Newton step (nc = -c; the reciprocal of
-// the negated sum leaves the residual 1 - s y as one FMA).  Symmetric in a and b, so the two cells
-// of a face compute the same value, and each lane of the paired form the scalar form's.
-__device__ __forceinline__ float face(float nc, float a, float b) {
-  const float s = a + b, y = rcp_approx(-s);
-  const float w = nc * y;
-  return fmaf(w, fmaf(s, y, 1.f), w);
-}
-__device__ __forceinline__ f2 face2(f2 nc, f2 a, f2 b) {
-  const f2 s = add2(a, b);
-  const float2 v = up2(s);
-  const f2 y = pk(rcp_approx(-v.x), rcp_approx(-v.y));
-  const f2 w = mul2(nc, y);
-  return fma2(w, fma2(s, y, pk(1.f, 1.f)), w);
-}
-
-__device__ __forceinline__ void fetch16(void* smem, const float* g) {  // through L1
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
-                   (unsigned)__cvta_generic_to_shared(smem)),
-               "l"(g)
-               : "memory");
-}
-__device__ __forceinline__ void fetch16_once(void* smem, const float* g) {  // L2 only
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                   (unsigned)__cvta_generic_to_shared(smem)),
-               "l"(g)
-               : "memory");
-}
-__device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// this thread's own copies: all but the newest group have landed
-__device__ __forceinline__ void fetch_wait_previous() {
-  asm volatile("cp.async.wait_group 1;" ::: "memory");
-}
-
-// Operand streams of a plane z (16 bytes per thread each): z+1 and the rows above and below of the
-// marched field and of the density, then what the kind needs besides.
-enum Stream { S_UP, S_UA, S_UB, S_RP, S_RA, S_RB, S_0, S_1, S_2 };
-template <int KIND> struct Streams { static constexpr int kCount = KIND == 0 ? 8 : (KIND == 1 ? 6 : 9); };
-
-// KIND 0: the fixed-point iteration, z = damping (-L')^-1 g: X += z, g -= rho' (-A') z and the sum
-// of r^2 / D' (the norm of the scaled residual, which steers the inner stop).
-// KIND 1, 2: CG, d = z + beta d_old (1: first iteration, d = z), q = (-A') d and the sum of d q.
-template <int KIND>
-__device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState* st, int unit,
-                                              float& part, ulonglong2* slots) {
-  constexpr bool kFixed = KIND == 0, kOld = KIND == 2;
-  constexpr int NS = Streams<KIND>::kCount;
-  const int nx = I.nx, ny = I.ny, nz = I.nz;
-  const int tpr = nx / kV;
-  const int tile = unit % I.uy, chunk = unit / I.uy;
-  const int row = threadIdx.x / tpr;
-  const int x0 = (threadIdx.x - row * tpr) * kV;
-  const int yr = tile * I.ty + row;
-  const bool active = row < I.ty && yr < ny;
-  const int y = active ? yr : ny - 1;  // idle threads follow a valid row (shuffles need them)
-  const int z0 = (int)((long long)chunk * nz / I.zc), z1 = (int)((long long)(chunk + 1) * nz / I.zc);
-  part = 0.f;
-  if (z0 >= z1) return;
-  const int lane = threadIdx.x & 31;
-  const bool row_start = x0 == 0, row_end = x0 + kV == nx;
-  const bool left_load = lane == 0 || row_start, right_load = lane == 31 || row_end;
-  const bool wall_l = I.duct && row_start, wall_r = I.duct && row_end;
-  const float nx1 = -I.ch[0];
-  const f2 ny2 = pk(-I.ch[1], -I.ch[1]), nz2 = pk(-I.ch[2], -I.ch[2]);
-  const float beta = (float)st->beta;
-  const f2 beta2 = pk(beta, beta);
-  const bool first = st->inner_iters == 0;
-  const float* rho = I.rho32;
-  const float* src = static_cast<const float*>(I.za);
-  const float* dold = static_cast<const float*>(st->parity ? I.d1 : I.d0);
-  float* dnew = static_cast<float*>(st->parity ? I.d0 : I.d1);
-  float* q = static_cast<float*>(I.q);
-  float* g = static_cast<float*>(I.r);
-  float* X = static_cast<float*>(I.x);
-  const long long plane = (long long)nx * ny;
-  const long long dym = y == 0 ? (long long)(ny - 1) * nx : -(long long)nx;
-  const long long dyp = y == ny - 1 ? -(long long)(ny - 1) * nx : (long long)nx;
-  const int dxl = row_start ? nx - 1 : -1, dxr = row_end ? -x0 : kV;
-  const long long cell0 = (long long)y * nx + x0;
-  const long long dz_last = plane * (nz - 1);  // from plane nz - 1 back to plane 0
-  // stream k of stage b of this thread
-  auto slot = [&](int b, int k) { return slots + (b * NS + k) * blockDim.x + threadIdx.x; };
-  auto fetch = [&](int b, int z, long long o) {  // the operands of plane z (cells at o)
-    const long long op = z == nz - 1 ? o - dz_last : o + plane;
-    fetch16(slot(b, S_UP), src + op);
-    fetch16(slot(b, S_UA), src + o + dym);
-    fetch16(slot(b, S_UB), src + o + dyp);
-    fetch16(slot(b, S_RP), rho + op);
-    fetch16(slot(b, S_RA), rho + o + dym);
-    fetch16(slot(b, S_RB), rho + o + dyp);
-    if (kFixed) {  // rewritten by this thread only, after this plane's copies have landed
-      fetch16_once(slot(b, S_0), g + o);
-      if (!first) fetch16_once(slot(b, S_1), X + o);
-    }
-    if (kOld) {
-      fetch16(slot(b, S_0), dold + op);
-      fetch16(slot(b, S_1), dold + o + dym);
-      fetch16(slot(b, S_2), dold + o + dyp);
-    }
-  };
-  auto ldg2 = [](const float* p, f2& a, f2& b) {
-    const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(p));
-    a = t.x;
-    b = t.y;
-  };
-  auto field1 = [&](long long o) -> float {
-    return kOld ? fmaf(beta, __ldg(dold + o), __ldg(src + o)) : __ldg(src + o);
-  };
-  long long o = (long long)z0 * plane + cell0;
-  fetch(0, z0, o);
-  fetch_commit();
-  // the field and the density of planes z0 - 1 and z0; the flux through the face between them
-  f2 u[2], r[2], bzl[2], fz[2];
-  {
-    const long long om = z0 == 0 ? o + dz_last : o - plane;
-    f2 um[2], rm[2];
-    ldg2(src + om, um[0], um[1]);
-    ldg2(src + o, u[0], u[1]);
-    ldg2(rho + om, rm[0], rm[1]);
-    ldg2(rho + o, r[0], r[1]);
-    if (kOld) {
-      f2 dm[2], dc[2];
-      ldg2(dold + om, dm[0], dm[1]);
-      ldg2(dold + o, dc[0], dc[1]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        um[h] = fma2(beta2, dm[h], um[h]);
-        u[h] = fma2(beta2, dc[h], u[h]);
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      bzl[h] = face2(nz2, rm[h], r[h]);
-      fz[h] = mul2(bzl[h], sub2(u[h], um[h]));
-    }
-  }
-  f2 sum[2] = {0ull, 0ull};
-  int b = 0;
-  for (int z = z0; z < z1; ++z) {
-    if (z + 1 < z1) fetch(b ^ 1, z + 1, o + plane);
-    fetch_commit();
-    // x neighbours: adjacent lanes, or a load at row ends and warp ends
-    const float2 u01 = up2(u[0]), u23 = up2(u[1]), r01 = up2(r[0]), r23 = up2(r[1]);
-    float ul = __shfl_up_sync(0xffffffffu, u23.y, 1), ur = __shfl_down_sync(0xffffffffu, u01.x, 1);
-    float rl = __shfl_up_sync(0xffffffffu, r23.y, 1), rr = __shfl_down_sync(0xffffffffu, r01.x, 1);
-    if (left_load) {
-      ul = field1(o + dxl);
-      rl = __ldg(rho + o + dxl);
-    }
-    if (right_load) {
-      ur = field1(o + dxr);
-      rr = __ldg(rho + o + dxr);
-    }
-    // faces and fluxes b (u_k - u_{k-1}) through the five x faces of the four cells
-    const float b0 = wall_l ? 0.f : face(nx1, rl, r01.x), b1 = face(nx1, r01.x, r01.y);
-    const float b2 = face(nx1, r01.y, r23.x), b3 = face(nx1, r23.x, r23.y);
-    const float b4 = wall_r ? 0.f : face(nx1, r23.y, rr);
-    const float f0 = b0 * (u01.x - ul), f1 = b1 * (u01.y - u01.x), fm = b2 * (u23.x - u01.y);
-    const float f3 = b3 * (u23.y - u23.x), f4 = b4 * (ur - u23.y);
-    f2 a[2] = {pk(f1 - f0, fm - f1), pk(f3 - fm, f4 - f3)};  // A' u, accumulated
-    f2 D[2] = {pk(b0 + b1, b1 + b2), pk(b2 + b3, b3 + b4)};
-    fetch_wait_previous();
-    ulonglong2 t = *slot(b, S_UP);
-    f2 un[2] = {t.x, t.y};
-    if (kOld) {
-      t = *slot(b, S_0);
-      un[0] = fma2(beta2, t.x, un[0]);
-      un[1] = fma2(beta2, t.y, un[1]);
-    }
-    t = *slot(b, S_RP);
-    const f2 rn[2] = {t.x, t.y};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {  // upper z face: its flux is the next plane's lower one
-      const f2 bz = face2(nz2, r[h], rn[h]);
-      const f2 f = mul2(bz, sub2(un[h], u[h]));
-      a[h] = add2(a[h], sub2(f, fz[h]));
-      fz[h] = f;
-      if (kFixed) D[h] = add2(D[h], add2(bzl[h], bz));
-      bzl[h] = bz;
-    }
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {  // the rows above and below
-      t = *slot(b, side ? S_UB : S_UA);
-      f2 v[2] = {t.x, t.y};
-      if (kOld) {
-        t = *slot(b, side ? S_2 : S_1);
-        v[0] = fma2(beta2, t.x, v[0]);
-        v[1] = fma2(beta2, t.y, v[1]);
-      }
-      t = *slot(b, side ? S_RB : S_RA);
-      const f2 rv[2] = {t.x, t.y};
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const f2 by = face2(ny2, rv[h], r[h]);
-        a[h] = fma2(by, sub2(v[h], u[h]), a[h]);
-        if (kFixed) D[h] = add2(D[h], by);
-      }
-    }
-    if constexpr (kFixed) {
-      t = *slot(b, S_0);
-      f2 gv[2] = {t.x, t.y}, xv[2] = {u[0], u[1]};
-      if (!first) {
-        t = *slot(b, S_1);
-        xv[0] = add2(t.x, u[0]);
-        xv[1] = add2(t.y, u[1]);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        gv[h] = fma2(r[h], a[h], gv[h]);
-        const float2 d = up2(D[h]), rv = up2(r[h]);
-        const f2 w = mul2(gv[h], pk(rcp_approx(rv.x), rcp_approx(rv.y)));
-        sum[h] = fma2(mul2(w, w), pk(rcp_approx(d.x), rcp_approx(d.y)), sum[h]);
-      }
-      if (active) {
-        *reinterpret_cast<ulonglong2*>(g + o) = make_ulonglong2(gv[0], gv[1]);
-        *reinterpret_cast<ulonglong2*>(X + o) = make_ulonglong2(xv[0], xv[1]);
-      }
-    } else {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        a[h] = sub2(0ull, a[h]);
-        sum[h] = fma2(u[h], a[h], sum[h]);
-      }
-      if (active) {
-        *reinterpret_cast<ulonglong2*>(dnew + o) = make_ulonglong2(u[0], u[1]);
-        *reinterpret_cast<ulonglong2*>(q + o) = make_ulonglong2(a[0], a[1]);
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      u[h] = un[h];
-      r[h] = rn[h];
-    }
-    o += plane;
-    b ^= 1;
-  }
-  const float2 s = up2(add2(sum[0], sum[1]));
-  part = active ? s.x + s.y : 0.f;
-}
-
-// ---- the FP64 inner solve ------------------------------------------------------------------------
-// z comes out of the FP32 transforms, so it is an FP32 field in this solve too; r, X, d and q are
-// FP64.  The product A' z in FP64 instructions bounds the sweep by the FP64 pipe (8 instructions
-// per cell at 2 per clock and SM: 282 us at 256^3, where its bytes take 109).  Here coefficients
-// and product are pairs of FP32 numbers (unevaluated sums hi + lo, about 47 bits): rho' as such a
-// pair, the quotient by a Newton step and a corrected remainder, the differences of z exact, the
-// products by FMA with their rounding errors, the six terms summed with the errors carried along.
-// Only the update of the FP64 fields is FP64: three instructions per cell (fixed point), four
-// (CG).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
-// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before.
-struct df {
-  f2 h, l;
-};
-
-__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
-
-// h + l = a + b exactly
-__device__ __forceinline__ df two_sum(f2 a, f2 b) {
-  df r;
-  r.h = add2(a, b);
-  const f2 t = sub2(r.h, a);
-  r.l = add2(sub2(a, sub2(r.h, t)), sub2(b, t));
-  return r;
-}
-__device__ __forceinline__ df two_diff(f2 a, f2 b) {
-  df r;
-  r.h = sub2(a, b);
-  const f2 t = sub2(r.h, a);
-  r.l = sub2(sub2(a, sub2(r.h, t)), add2(b, t));
-  return r;
-}
-
-// c / (a + b), c = -(nch + ncl)
-__device__ __forceinline__ df face_df(f2 nch, f2 ncl, df a, df b) {
-  df s = two_sum(a.h, b.h);
-  s.l = add2(s.l, add2(a.l, b.l));
-  const float2 v = up2(s.h);
-  f2 y = pk(rcp_approx(-v.x), rcp_approx(-v.y));  // -1 / s
-  y = fma2(y, fma2(s.h, y, pk(1.f, 1.f)), y);
-  df q;
-  q.h = mul2(nch, y);
-  const f2 t = add2(fma2(q.h, s.l, fma2(q.h, s.h, nch)), ncl);  // q s - c
-  q.l = mul2(t, y);
-  return q;
-}
-
-// -(b x difference) of a face as an unevaluated sum, from the exact difference d
-__device__ __forceinline__ df minus_flux(df b, df d) {
-  df f;
-  f.h = mul2(neg2(b.h), d.h);
-  const f2 e = fma2(b.l, d.h, fma2(b.h, d.l, fma2(b.h, d.h, f.h)));  // b d + f.h
-  f.l = neg2(e);
-  return f;
-}
-
-// acc -= f
-__device__ __forceinline__ void accumulate_minus(df& acc, df f) {
-  const df s = two_diff(acc.h, f.h);
-  acc.h = s.h;
-  acc.l = add2(acc.l, sub2(s.l, f.l));
-}
-__device__ __forceinline__ void accumulate_plus(df& acc, df f) {
-  const df s = two_sum(acc.h, f.h);
-  acc.h = s.h;
-  acc.l = add2(acc.l, add2(s.l, f.l));
-}
-
-enum Stream64 { T_UP, T_UA, T_UB, T_HP, T_HA, T_HB, T_LP, T_LA, T_LB, T_P0, T_P1, T_Q0, T_Q1, kStreams64 };
-
-// FIXED: X += z, r -= (-A') z and the sum of r^2 / D' (FP32, steers the inner stop).
-// CG: d = z + beta d_old, q = (-A') z + beta q_old, and the sum of d q.
-template <bool FIXED>
-__device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstState& st, int unit,
-                                                double& part, ulonglong2* slots) {
-  const int nx = I.nx, ny = I.ny, nz = I.nz;
-  const int tpr = nx / kV;
-  const int tile = unit % I.uy, chunk = unit / I.uy;
-  const int row = threadIdx.x / tpr;
-  const int x0 = (threadIdx.x - row * tpr) * kV;
-  const int yr = tile * I.ty + row;
-  const bool active = row < I.ty && yr < ny;
-  const int y = active ? yr : ny - 1;
-  const int z0 = (int)((long long)chunk * nz / I.zc), z1 = (int)((long long)(chunk + 1) * nz / I.zc);
-  part = 0.0;
-  if (z0 >= z1) return;
-  const int lane = threadIdx.x & 31;
-  const bool row_start = x0 == 0, row_end = x0 + kV == nx;
-  const bool left_load = lane == 0 || row_start, right_load = lane == 31 || row_end;
-  const bool wall_l = I.duct && row_start, wall_r = I.duct && row_end;
-  f2 nch[3], ncl[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    nch[d] = pk(-I.ch[d], -I.ch[d]);
-    ncl[d] = pk(-I.cl[d], -I.cl[d]);
-  }
-  const double beta = st.beta;
-  const bool first = st.inner_iters == 0;  // no X (fixed point), no history (CG) yet
-  const float* rhi = I.rho32;
-  const float* rlo = I.rho_lo;
-  const float* src = static_cast<const float*>(I.za);
-  // p, q: the two FP64 fields read and written (fixed point r, X; CG d, q)
-  const double* pin = static_cast<const double*>(FIXED ? I.r : (st.parity ? I.d1 : I.d0));
-  double* pout = static_cast<double*>(FIXED ? I.r : (st.parity ? I.d0 : I.d1));
-  double* q = static_cast<double*>(FIXED ? I.x : I.q);
-  const long long plane = (long long)nx * ny;
-  const long long dym = y == 0 ? (long long)(ny - 1) * nx : -(long long)nx;
-  const long long dyp = y == ny - 1 ? -(long long)(ny - 1) * nx : (long long)nx;
-  const int dxl = row_start ? nx - 1 : -1, dxr = row_end ? -x0 : kV;
-  const long long cell0 = (long long)y * nx + x0;
-  const long long dz_last = plane * (nz - 1);
-  auto slot = [&](int b, int k) { return slots + (b * kStreams64 + k) * blockDim.x + threadIdx.x; };
-  auto fetch = [&](int b, int z, long long o) {
-    const long long op = z == nz - 1 ? o - dz_last : o + plane;
-    fetch16(slot(b, T_UP), src + op);
-    fetch16(slot(b, T_UA), src + o + dym);
-    fetch16(slot(b, T_UB), src + o + dyp);
-    fetch16(slot(b, T_HP), rhi + op);
-    fetch16(slot(b, T_HA), rhi + o + dym);
-    fetch16(slot(b, T_HB), rhi + o + dyp);
-    fetch16(slot(b, T_LP), rlo + op);
-    fetch16(slot(b, T_LA), rlo + o + dym);
-    fetch16(slot(b, T_LB), rlo + o + dyp);
-    if (FIXED || !first) {
-      fetch16_once(slot(b, T_P0), reinterpret_cast<const float*>(pin + o));
-      fetch16_once(slot(b, T_P1), reinterpret_cast<const float*>(pin + o + 2));
-    }
-    if (!first) {
-      fetch16_once(slot(b, T_Q0), reinterpret_cast<const float*>(q + o));
-      fetch16_once(slot(b, T_Q1), reinterpret_cast<const float*>(q + o + 2));
-    }
-  };
-  auto ldg2 = [](const float* p, f2& a, f2& b) {
-    const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(p));
-    a = t.x;
-    b = t.y;
-  };
-  long long o = (long long)z0 * plane + cell0;
-  fetch(0, z0, o);
-  fetch_commit();
-  f2 u[2];
-  df r[2], bzl[2], fz[2];  // fz: minus the flux through the lower z face
-  {
-    const long long om = z0 == 0 ? o + dz_last : o - plane;
-    f2 um[2];
-    df rm[2];
-    ldg2(src + om, um[0], um[1]);
-    ldg2(src + o, u[0], u[1]);
-    ldg2(rhi + om, rm[0].h, rm[1].h);
-    ldg2(rlo + om, rm[0].l, rm[1].l);
-    ldg2(rhi + o, r[0].h, r[1].h);
-    ldg2(rlo + o, r[0].l, r[1].l);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      bzl[h] = face_df(nch[2], ncl[2], rm[h], r[h]);
-      fz[h] = minus_flux(bzl[h], two_diff(u[h], um[h]));
-    }
-  }
-  double sum = 0.0;
-  float sumf = 0.f;
-  int b = 0;
-  for (int z = z0; z < z1; ++z) {
-    if (z + 1 < z1) fetch(b ^ 1, z + 1, o + plane);
-    fetch_commit();
-    df acc[2];
-    f2 D[2];
-    {  // x: faces 0 .. 4 of the four cells, as pairs (0, 1), (2, 3) and 4
-      const float2 u01 = up2(u[0]), u23 = up2(u[1]);
-      const float2 h01 = up2(r[0].h), h23 = up2(r[1].h), l01 = up2(r[0].l), l23 = up2(r[1].l);
-      float ul = __shfl_up_sync(0xffffffffu, u23.y, 1), ur = __shfl_down_sync(0xffffffffu, u01.x, 1);
-      float hl = __shfl_up_sync(0xffffffffu, h23.y, 1), hr = __shfl_down_sync(0xffffffffu, h01.x, 1);
-      float ll = __shfl_up_sync(0xffffffffu, l23.y, 1), lr = __shfl_down_sync(0xffffffffu, l01.x, 1);
-      if (left_load) {
-        ul = __ldg(src + o + dxl);
-        hl = __ldg(rhi + o + dxl);
-        ll = __ldg(rlo + o + dxl);
-      }
-      if (right_load) {
-        ur = __ldg(src + o + dxr);
-        hr = __ldg(rhi + o + dxr);
-        lr = __ldg(rlo + o + dxr);
-      }
-      df b01 = face_df(nch[0], ncl[0], df{pk(hl, h01.x), pk(ll, l01.x)}, r[0]);
-      const df b23 = face_df(nch[0], ncl[0], df{pk(h01.y, h23.x), pk(l01.y, l23.x)}, r[1]);
-      df b44 = face_df(nch[0], ncl[0], df{pk(h23.y, h23.y), pk(l23.y, l23.y)}, df{pk(hr, hr), pk(lr, lr)});
-      if (wall_l) {
-        b01.h = pk(0.f, up2(b01.h).y);
-        b01.l = pk(0.f, up2(b01.l).y);
-      }
-      if (wall_r) b44.h = b44.l = 0ull;
-      const df f01 = minus_flux(b01, two_diff(u[0], pk(ul, u01.x)));
-      const df f23 = minus_flux(b23, two_diff(u[1], pk(u01.y, u23.x)));
-      const df f44 = minus_flux(b44, two_diff(pk(ur, ur), pk(u23.y, u23.y)));
-      const float2 fh01 = up2(f01.h), fh23 = up2(f23.h), fl01 = up2(f01.l), fl23 = up2(f23.l);
-      const df f12 = {pk(fh01.y, fh23.x), pk(fl01.y, fl23.x)};
-      const df f34 = {pk(fh23.y, up2(f44.h).x), pk(fl23.y, up2(f44.l).x)};
-      acc[0] = f01;  // A' z = sum of (upper flux - lower flux); f holds minus the flux
-      acc[1] = f23;
-      accumulate_minus(acc[0], f12);
-      accumulate_minus(acc[1], f34);
-      if (FIXED) {
-        const float2 bh01 = up2(b01.h), bh23 = up2(b23.h);
-        D[0] = add2(b01.h, pk(bh01.y, bh23.x));
-        D[1] = add2(b23.h, pk(bh23.y, up2(b44.h).x));
-      }
-    }
-    fetch_wait_previous();
-    ulonglong2 t = *slot(b, T_UP);
-    const f2 un[2] = {t.x, t.y};
-    t = *slot(b, T_HP);
-    const ulonglong2 t2 = *slot(b, T_LP);
-    const df rn[2] = {{t.x, t2.x}, {t.y, t2.y}};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const df bz = face_df(nch[2], ncl[2], r[h], rn[h]);
-      const df f = minus_flux(bz, two_diff(un[h], u[h]));
-      accumulate_plus(acc[h], fz[h]);
-      accumulate_minus(acc[h], f);
-      fz[h] = f;
-      if (FIXED) D[h] = add2(D[h], add2(bzl[h].h, bz.h));
-      bzl[h] = bz;
-    }
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      t = *slot(b, side ? T_UB : T_UA);
-      const f2 v[2] = {t.x, t.y};
-      t = *slot(b, side ? T_HB : T_HA);
-      const ulonglong2 tl = *slot(b, side ? T_LB : T_LA);
-      const df rv[2] = {{t.x, tl.x}, {t.y, tl.y}};
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const df by = face_df(nch[1], ncl[1], rv[h], r[h]);
-        accumulate_minus(acc[h], minus_flux(by, two_diff(v[h], u[h])));
-        if (FIXED) D[h] = add2(D[h], by.h);
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const float2 ah = up2(acc[h].h), al = up2(acc[h].l), uu = up2(u[h]);
-      const double2 pv = *reinterpret_cast<const double2*>(slot(b, h ? T_P1 : T_P0));
-      const double2 qv = *reinterpret_cast<const double2*>(slot(b, h ? T_Q1 : T_Q0));
-      double2 po, qo;
-      if constexpr (FIXED) {
-        po.x = (pv.x + widen(ah.x)) + widen(al.x);
-        po.y = (pv.y + widen(ah.y)) + widen(al.y);
-        qo.x = widen(uu.x);
-        qo.y = widen(uu.y);
-        if (!first) {
-          qo.x += qv.x;
-          qo.y += qv.y;
-        }
-        const float2 d = up2(D[h]);
-        const float rx = narrow(po.x), ry = narrow(po.y);
-        sumf = fmaf(rx * rcp_approx(d.x), rx, sumf);
-        sumf = fmaf(ry * rcp_approx(d.y), ry, sumf);
-      } else {
-        po.x = widen(uu.x);
-        po.y = widen(uu.y);
-        qo.x = -(widen(ah.x) + widen(al.x));
-        qo.y = -(widen(ah.y) + widen(al.y));
-        if (!first) {
-          po.x = fma(beta, pv.x, po.x);
-          po.y = fma(beta, pv.y, po.y);
-          qo.x = fma(beta, qv.x, qo.x);
-          qo.y = fma(beta, qv.y, qo.y);
-        }
-        sum = fma(po.x, qo.x, sum);
-        sum = fma(po.y, qo.y, sum);
-      }
-      if (active) {
-        *reinterpret_cast<double2*>(pout + o + 2 * h) = po;
-        *reinterpret_cast<double2*>(q + o + 2 * h) = qo;
-      }
-      u[h] = un[h];
-      r[h] = rn[h];
-    }
-    o += plane;
-    b ^= 1;
-  }
-  part = active ? (FIXED ? (double)sumf : sum) : 0.0;
-}
-
-size_t density_smem(bool fixed, int threads) {
-  const int streams = fixed ? Streams<0>::kCount : Streams<2>::kCount;
-  return sizeof(ulonglong2) * (size_t)kStages * streams * threads;
-}
-
-}  // namespace
 
 // STENCIL phase of the instances in the density form: FIXED the fixed-point iteration, else CG.
 template <bool FIXED>
@@ -621,8 +32,6 @@ __global__ void __launch_bounds__(kDirectThreads, 2)
 
 // The same in FP64: four cells per thread of the FP64 layout's two, so half its threads; three
 // blocks of 128 threads per SM (168 registers).
-constexpr int kDensity64Threads = kDirectThreads / 2;
-
 template <bool FIXED>
 __global__ void __launch_bounds__(kDensity64Threads, 3)
     k_density64(const InstDesc* __restrict__ insts, const UnitRef* __restrict__ units) {
@@ -636,10 +45,6 @@ __global__ void __launch_bounds__(kDensity64Threads, 3)
   sweep_density64<FIXED>(I, sn, ur.unit, part[0], slots);
   store_partials<1, double>(part, I.part, I.nunits, ur.unit);
   finish_sweep(I, st, PH_STENCIL, I.nunits);
-}
-
-static size_t density64_smem(int threads) {
-  return sizeof(ulonglong2) * (size_t)kStages * kStreams64 * threads;
 }
 
 cudaError_t prepare_density() {

@@ -53,6 +53,12 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+__device__ __forceinline__ uint64_t global_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 // ---- reductions: per-unit partial slots, last unit reduces them in a fixed order --------------
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -93,10 +99,19 @@ __device__ __forceinline__ void store_partials_by_warp(const A (&v)[NS], double*
   }
 }
 
+// 32 lanes' sums of a column of up to eight warps, then over the lanes
+__device__ __forceinline__ double column_sum(const double* col, int nwarps) {
+  static_assert(kDirectThreads == 256 && kFlatThreads == 256, "eight warps");
+  const int lane = threadIdx.x & 31;
+  double c[8];
+#pragma unroll
+  for (int w = 0; w < 8; ++w) c[w] = w < nwarps ? col[w * 32 + lane] : 0.0;
+  return warp_sum(((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7])));
+}
+
 template <int NS>
 __device__ __forceinline__ void store_partials_by_column(const double (&v)[NS], double* part,
                                                          int nunits, int unit) {
-  static_assert(kFlatThreads <= kDirectThreads, "the columns hold one block");
   __shared__ double col[NS][kDirectThreads];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
@@ -105,9 +120,7 @@ __device__ __forceinline__ void store_partials_by_column(const double (&v)[NS], 
   for (int k = 0; k < NS; ++k) col[k][threadIdx.x] = v[k];
   __syncthreads();
   for (int k = warp; k < NS; k += nwarps) {
-    double s = 0.0;
-    for (int w = 0; w < nwarps; ++w) s += col[k][w * 32 + lane];
-    s = warp_sum(s);
+    const double s = column_sum(col[k], nwarps);
     if (lane == 0) part[k * nunits + unit] = s;
   }
 }
@@ -135,41 +148,71 @@ __device__ __forceinline__ bool arrive_last(unsigned int* ticket, int nunits) {
   return last != 0;
 }
 
-// Fixed-order sums of the first ns slots over all units by the last unit.  A slot is summed by 256
-// lanes, each adding the slots lane, lane + 256, ... in index order with eight loads in flight,
-// then a fixed shuffle tree per 32 lanes, then the eight totals in order.  The (slot, 32 lanes)
+// Fixed-order sums of the first ns slots over all units, for thread 0.  A slot is summed by 128
+// lanes, each adding the slots lane, lane + 128, ... in index order with eight loads in flight,
+// then a fixed shuffle tree per 32 lanes, then the four totals in order.  The (slot, 32 lanes)
 // pairs are spread over the block's warps, so the slots are summed side by side; the order does
-// not depend on the block size, so an instance sums identically whatever launch it runs in.  (One
-// slot after the other over 64 lanes, the four sums of a residual took most of the 20 us that
-// sweep needs on a 32^3 grid.)  Every thread returns the sums.
+// not depend on the block size, so an instance sums identically whatever launch it runs in.  The
+// FP64 pipe takes a warp's addition in 64 cycles per scheduler: four warps, one a scheduler, and
+// only thread 0 adds the totals (eight warps and every thread: 3000 cycles instead of 1500).
 static __device__ __noinline__ void block_sum_slots(const double* part, int nunits, int ns,
                                                     double (&S)[kSlots]) {
-  constexpr int U = 8, LANES = 256, G = LANES / 32;
+  constexpr int U = 8, LANES = 128, G = LANES / 32;
   __shared__ double wsum[kSlots][G];
   const int lane = threadIdx.x & 31;
   for (int q = threadIdx.x >> 5; q < ns * G; q += blockDim.x >> 5) {
     const double* slot = part + (long long)(q / G) * nunits;
     double s = 0.0;
-    for (int i0 = (q % G) * 32 + lane; i0 < nunits; i0 += U * LANES) {
+    int i = (q % G) * 32 + lane;
+    for (; i + (U - 1) * LANES < nunits; i += U * LANES) {
       double v[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * LANES;
-        v[u] = i < nunits ? __ldcg(slot + i) : 0.0;
-      }
+      for (int u = 0; u < U; ++u) v[u] = __ldcg(slot + i + u * LANES);
 #pragma unroll
       for (int u = 0; u < U; ++u) s += v[u];
     }
+    double v[U];
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u) v[u] = i + u * LANES < nunits ? __ldcg(slot + i + u * LANES) : 0.0;
+#pragma unroll
+    for (int u = 0; u < U - 1; ++u)
+      if (i - lane + u * LANES < nunits) s += v[u];  // uniform in the warp
     s = warp_sum(s);
     if (lane == 0) wsum[q / G][q % G] = s;
   }
   __syncthreads();
-  for (int k = 0; k < ns; ++k) {
-    double s = 0.0;
-#pragma unroll
-    for (int g = 0; g < G; ++g) s += wsum[k][g];
-    S[k] = s;
-  }
+  if (threadIdx.x == 0)
+    for (int k = 0; k < ns; ++k) S[k] = (wsum[k][0] + wsum[k][1]) + (wsum[k][2] + wsum[k][3]);
+}
+
+// c / s in FP64 for s > 0 in the middle of the binary64 range: the FP32 approximation of 1/s as the
+// seed Y, e = 1 - s Y (|e| < 2^-21.4), c/s = w (1 + e + e^2), w = c Y; relative error below
+// 2^-52.  Five FP64 instructions; the division takes more than ten, each 64 cycles after the other.
+__device__ __forceinline__ int exponent_of(double v) {  // biased exponent field
+  return (__double2hiint(v) >> 20) & 0x7ff;
+}
+// Mantissa of a positive normal v as an FP32 value in [1, 2) (truncated to 23 fraction bits).
+__device__ __forceinline__ float mantissa_f(double v) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  return __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
+}
+// FP32 value y in (0, 2) times 2^p as FP64, by integer operations (no FP64 conversion).
+__device__ __forceinline__ double widen_pow2(float y, int p) {
+  const unsigned b = __float_as_uint(y);
+  const unsigned e = (b >> 23) + 1023u - 127u + (unsigned)p;
+  return __hiloint2double((int)((e << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
+}
+// Exponents that neither the seed nor the products can push out of the normal range.
+__device__ __forceinline__ bool mid_range(double v) {
+  const int e = exponent_of(v);
+  return e > 200 && e < 1846;
+}
+__device__ __forceinline__ double quotient(double c, double s) {
+  if (!mid_range(s)) return c / s;
+  const double Y = widen_pow2(rcp_approx(mantissa_f(s)), 1023 - exponent_of(s));
+  const double e = fma(-s, Y, 1.0);
+  const double w = c * Y;
+  return fma(w, fma(e, e, e), w);
 }
 
 // ---- phase transitions (run by thread 0 of the last unit) -------------------------------------
@@ -251,7 +294,7 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
         phase = PH_UPDATE;
         goto after_update;
       } else if (dq > 0.0 && isfinite(dq)) {
-        st->alpha = (I.pc != PC_JACOBI ? st->rz : st->rr) / dq;
+        st->alpha = quotient(I.pc != PC_JACOBI ? st->rz : st->rr, dq);
         st->phase = PH_UPDATE;
       } else if (st->inner_iters > 0) {
         // loss of curvature at the end of an inner solve: hand the iterate to the refinement
@@ -281,7 +324,7 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
         st->cheb_j = 1;
         st->phase = I.pc == PC_CHEB ? PH_CHEB : PH_SPEC;
       } else {
-        st->beta = rn / st->rr;
+        st->beta = quotient(rn, st->rr);
         st->rr = rn;
         st->rz = rn;
         st->parity ^= 1;
@@ -314,7 +357,7 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
       if (st->inner_iters == 0) {
         st->beta = 0.0;
       } else {
-        st->beta = rz / st->rz;
+        st->beta = quotient(rz, st->rz);
         st->parity ^= 1;
       }
       st->rz = rz;

@@ -142,6 +142,14 @@ struct BatchCtl {
   unsigned long long limit_ns;  // bound on one grid barrier wait
 };
 
+// Control words of a resident solve (vdp_resident.cu), a cache line each; zero at launch.
+struct ResidentCtl {
+  unsigned count;      // barrier arrivals
+  unsigned pad0[31];
+  int fault;           // a wait expired
+  unsigned pad1[31];
+};
+
 struct UnitRef {
   int inst;            // index into the batch's InstDesc table
   int unit;            // unit index within the instance
@@ -166,6 +174,10 @@ __host__ __device__ inline size_t ring_bytes(int nx, int ty) {
 constexpr int kSMs = 152;                 // GB300
 constexpr size_t kSmemPerSM = 227 * 1024; // shared memory per SM available to CTAs
 constexpr size_t kSmemBudget = 225 * 1024;
+
+// Largest grid that one resident launch solves (vdp_resident.cu; resident_supported() has the line
+// for each kind of solve).
+constexpr long long kResidentCells = 2500000;
 
 struct Layout {
   int mode;            // stencil sweep variant (0 direct, 1 TMA pipeline)
@@ -257,6 +269,12 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
     if (by_cells < want) want = by_cells;
   }
   long long zc = (want + uy - 1) / uy;
+  if (units <= 0 && mode == 0 && ncell <= kResidentCells) {
+    // the resident solve's blocks (two per SM) take one unit each where the planes allow it
+    want = 2LL * kSMs;
+    zc = want / uy;
+    if (zc > 0 && zc < nz) zc = (nz + (nz + zc - 1) / zc - 1) / ((nz + zc - 1) / zc);  // equal chunks
+  }
   if (zc > nz) zc = nz;
   if (zc < 1) zc = 1;
   long long nf = ncell / 4096;

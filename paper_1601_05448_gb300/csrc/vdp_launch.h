@@ -30,9 +30,10 @@ cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double s2, 
                               const double* sinv, long long n, float* out, cudaStream_t s);
 cudaError_t launch_apply(const double* bx, const double* by, const double* bz, const double* p,
                          int nx, int ny, int nz, double* out, cudaStream_t s);
+// ctl: also the control words of a resident solve (or null)
 cudaError_t launch_init(InstDesc* desc, const double* rhs, double* p, double tol, double inner_tol,
                         int max_iter, int inner_max, int use_guess, int precision,
-                        cudaStream_t s);
+                        ResidentCtl* ctl, cudaStream_t s);
 cudaError_t prepare_step(int prec, int mode, size_t smem_bytes);
 // mode 0 only: the FP64 residual sweep (its own kernel, launched before each stencil launch) of
 // the instances in the scaled (form 0) or the density form (1)
@@ -54,6 +55,13 @@ cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
                            cudaStream_t s);
 cudaError_t launch_flat(int prec, const InstDesc* desc, const UnitRef* units, int nunits,
                         cudaStream_t s);
+
+// vdp_resident.cu: the whole solve in one cooperative launch, for grids of at most kResidentCells
+// cells.  spec: the solve's spectral arguments (unused by Jacobi CG); stops after max_sweeps sweeps.
+struct SpecArgs;
+bool resident_supported(const InstDesc& d, int prec);
+cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, const SpecArgs& spec,
+                            ResidentCtl* ctl, unsigned max_sweeps, cudaStream_t s);
 
 cudaError_t persistent_grid(int prec, int* grid);
 cudaError_t launch_persistent(int prec, const InstDesc* desc, const UnitRef* sunits, int ns,

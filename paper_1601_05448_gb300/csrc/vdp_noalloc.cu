@@ -245,7 +245,7 @@ extern "C" int vdp_solve_noalloc(int nx, int ny, int nz, double L, const double*
   NA_CK(prepare_step(precision, lay.mode, lay.smem));
   // the per-solve state and the ticket are reset on the device by the init kernel
   const int max_iter = 20000;
-  NA_CK(launch_init(desc, rhs, p, tol, 1e-4, max_iter, max_iter, 0, precision, s));
+  NA_CK(launch_init(desc, rhs, p, tol, 1e-4, max_iter, max_iter, 0, precision, nullptr, s));
 
   const int m = 16;  // (stencil, flat) launch pairs per convergence check
   const long long max_rounds = (2LL * max_iter + 4096 + m - 1) / m;

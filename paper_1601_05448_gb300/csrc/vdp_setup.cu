@@ -23,41 +23,6 @@ namespace {
 
 constexpr int kSetupThreads = 256;
 
-__device__ __forceinline__ int exponent_of(double v) {  // biased exponent field
-  return (__double2hiint(v) >> 20) & 0x7ff;
-}
-
-// Mantissa of a positive normal v as an FP32 value in [1, 2) (truncated to 23 fraction bits).
-__device__ __forceinline__ float mantissa_f(double v) {
-  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  return __uint_as_float(0x3f800000u | ((hi & 0xfffffu) << 3) | (lo >> 29));
-}
-
-// FP32 value y in (0, 2) times 2^p as FP64, by integer operations (no FP64 conversion).
-__device__ __forceinline__ double widen_pow2(float y, int p) {
-  const unsigned b = __float_as_uint(y);
-  const unsigned e = (b >> 23) + 1023u - 127u + (unsigned)p;
-  return __hiloint2double((int)((e << 20) | ((b & 0x7fffffu) >> 3)), (int)(b << 29));
-}
-
-// Whether the seeded forms below apply: exponents that neither the seed nor the products can
-// push out of the normal range.
-__device__ __forceinline__ bool mid_range(double v) {
-  const int e = exponent_of(v);
-  return e > 200 && e < 1846;
-}
-
-// c / s for s > 0: seed Y0 ~ 1/s, e = 1 - s Y0 (|e| < 2^-21.4), c/s = w (1 + e + e^2), w = c Y0.
-__device__ __forceinline__ double quotient(double c, double s) {
-  if (!mid_range(s)) return c / s;
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(mantissa_f(s)));
-  const double Y = widen_pow2(y, 1023 - exponent_of(s));
-  const double e = fma(-s, Y, 1.0);
-  const double w = c * Y;
-  return fma(w, fma(e, e, e), w);
-}
-
 // D^-1/2 for D > 0: seed Y0, e = 1 - D Y0^2, Y0 (1 + e/2 + 3 e^2/8).
 __device__ __forceinline__ double inv_sqrt(double D) {
   if (!mid_range(D)) return 1.0 / sqrt(D);

@@ -152,7 +152,7 @@ extern "C" int vdp_solve_timed(vdp_ctx* c, const double* rhs, double* p, double 
   cudaError_t e;
   if ((e = cudaEventRecord(c->ev0, c->stream)) != cudaSuccess) return fail(e, "cudaEventRecord");
   e = launch_init(c->desc, rhs, p, tol, c->opts.inner_tol, c->opts.max_iter, c->opts.max_iter,
-                  c->opts.use_guess ? 1 : 0, prec, c->stream);
+                  c->opts.use_guess ? 1 : 0, prec, nullptr, c->stream);
   if (e != cudaSuccess) return fail(e, "launch_init");
   // Every launch advances the state machine by one phase; this only bounds the host loop.
   const int k = c->opts.precond == VDP_PRECOND_CHEB ? std::max(1, c->opts.cheb_degree) : 1;
