@@ -278,8 +278,6 @@ int ensure_graph(vdp_ctx* c, int prec) {
 // graph launch -- no host polling between rounds and at most kWhileRounds - 1 idle rounds at
 // the end.  Returns false (and remembers it) if the driver cannot build such a graph; the
 // solve then uses the polling schedule.
-constexpr int kWhileRounds = 2;
-
 bool ensure_while_graph(vdp_ctx* c, int prec) {
   if (c->w_failed) return false;
   if (c->wexec && c->w_prec == prec) return true;
@@ -287,7 +285,7 @@ bool ensure_while_graph(vdp_ctx* c, int prec) {
     cudaGraphExecDestroy(c->wexec);
     c->wexec = nullptr;
   }
-  if (!c->d_rounds && cudaMalloc((void**)&c->d_rounds, sizeof(unsigned)) != cudaSuccess) {
+  if (!c->d_rounds && cudaMalloc((void**)&c->d_rounds, 2 * sizeof(unsigned)) != cudaSuccess) {
     cudaGetLastError();
     c->d_rounds = nullptr;
     c->w_failed = true;
@@ -487,6 +485,18 @@ int prepare_spectral_solve(vdp_ctx* c) {
     c->rho_w_valid = true;
   }
   return VDP_OK;
+}
+
+// Whether this solve runs as one cooperative launch (vdp_resident.cu); allocates its control words.
+bool resident_solve(vdp_ctx* c, int prec) {
+  if (c->opts.steps_per_sync != 0 || !resident_supported(c->hdesc, prec)) return false;
+  if (c->hdesc.pc != PC_JACOBI && spec_slab(c) < c->nz) return false;
+  if (!c->rctl && cudaMalloc((void**)&c->rctl, sizeof(ResidentCtl)) != cudaSuccess) {
+    cudaGetLastError();
+    c->rctl = nullptr;
+    return false;
+  }
+  return true;
 }
 
 }  // namespace vdp
@@ -711,18 +721,6 @@ static void set_stats(vdp_ctx* c, const InstState& hs, bool done, int launches) 
   c->stats.launches = launches;
 }
 
-// Whether this solve runs as one cooperative launch (vdp_resident.cu); allocates its control words.
-static bool resident_solve(vdp_ctx* c, int prec) {
-  if (c->opts.steps_per_sync != 0 || !resident_supported(c->hdesc, prec)) return false;
-  if (c->hdesc.pc != PC_JACOBI && spec_slab(c) < c->nz) return false;
-  if (!c->rctl && cudaMalloc((void**)&c->rctl, sizeof(ResidentCtl)) != cudaSuccess) {
-    cudaGetLastError();
-    c->rctl = nullptr;
-    return false;
-  }
-  return true;
-}
-
 int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   if (!c || !rhs || !p || !(tol > 0.0) || !std::isfinite(tol)) return VDP_EINVAL;
   if (!c->has_density) return VDP_EINVAL;
@@ -761,7 +759,7 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
     // two sweeps per iteration and the outer phases; the state machine stops at max_iter itself
     const long long bound = 3LL * c->opts.max_iter + 4096;
     VDP_CK(launch_resident(prec, c->hdesc, c->desc, a, c->rctl,
-                           (unsigned)std::min<long long>(bound, 0x7fffffffLL), c->stream));
+                           (unsigned)std::min<long long>(bound, 0x7fffffffLL), 0, c->stream));
     VDP_CK(cudaMemcpyAsync(&c->hstate[0], c->st, sizeof(InstState), cudaMemcpyDeviceToHost,
                            c->stream));
     VDP_CK(cudaEventRecord(c->ev1, c->stream));
@@ -772,7 +770,7 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   }
   const int per_round = (c->lay.mode == 0 ? 3 : 2) + precond_launches(c);
   if (dev_loop) {  // the whole solve is one graph launch; the device decides when to stop
-    VDP_CK(cudaMemsetAsync(c->d_rounds, 0, sizeof(unsigned), c->stream));
+    VDP_CK(launch_start_rounds(c->d_rounds, 0, c->stream));
     VDP_CK(cudaGraphLaunch(c->wexec, c->stream));
     VDP_CK(cudaMemcpyAsync(&c->hstate[0], c->st, sizeof(InstState), cudaMemcpyDeviceToHost,
                            c->stream));

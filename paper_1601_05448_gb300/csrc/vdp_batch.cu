@@ -8,6 +8,13 @@
 // the equivalent sequence of ordinary launches; either is captured once into a CUDA graph per
 // membership and replayed.  Members can be added and retired between runs (continuous batching):
 // the device tables are rebuilt and the graph re-captured only when membership changes.
+//
+// A batch of ordinary launches shares launches among its Jacobi and Chebyshev members only.  The
+// others (spectral passes, V-cycle) have chains of kernels of their own anyway, so each runs as it
+// does alone -- one resident launch, or the context's device-side loop, both kept with the context
+// -- with a limit on its rounds, on one of a few streams side by side.  Capturing 64 rounds of
+// every member's passes took longer than running them, and rounds past a member's end were idle
+// launches (8 grids of 64^3 to 192^3, mixed to 1e-8 with their densities set: 20.1 -> 7.5 ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -31,6 +38,7 @@ struct Member {
   double* p;
   double tol;
   bool done;
+  bool alone;  // runs by itself, not in the shared launches
 };
 
 }  // namespace
@@ -60,8 +68,10 @@ struct vdp_batch {
   double wait_limit_s = 2.0;  // bound on each grid barrier wait of the persistent kernel
   bool inject = false;        // next persistent run: one arrival more than the grid (tests)
   bool ctl_stale = false;     // the control words must be reset before the next run
-  // graph branches for the members' spectral passes (captured from these streams)
-  static constexpr int kBranches = 4;
+  int nshared = 0;            // active members in the shared launches
+  // streams for the members that run by themselves (and graph branches for such members' passes
+  // where the driver has no device-side loops)
+  static constexpr int kBranches = 8;  // that batch of 8: 8.9, 8.6 and 7.5 ms with 2, 4 and 8
   cudaStream_t aux[kBranches] = {};
   cudaEvent_t fork = nullptr, join[kBranches] = {};
 };
@@ -85,11 +95,20 @@ int grow(X** ptr, long long* cap, long long need) {
   return VDP_OK;
 }
 
+// Whether a member runs by itself (see above) instead of in the shared launches.
+bool runs_alone(vdp_batch* b, const Member& m) {
+  vdp_ctx* c = m.ctx;
+  return !b->persistent && c->hdesc.pc >= PC_SPECTRAL &&
+         (resident_solve(c, b->prec) || ensure_while_graph(c, b->prec));
+}
+
 int rebuild(vdp_batch* b) {
   b->active.clear();
   for (size_t i = 0; i < b->members.size(); ++i)
     if (!b->members[i].done) b->active.push_back((int)i);
   const int n = (int)b->active.size();
+  b->nshared = 0;
+  for (int k : b->active) b->members[k].alone = runs_alone(b, b->members[k]);
   long long cd = b->cap_desc;
   int s;
   if ((s = grow(&b->d_desc, &cd, std::max(n, 1))) != VDP_OK) return s;
@@ -113,6 +132,8 @@ int rebuild(vdp_batch* b) {
     d.p = m.p;
     d.remaining = &b->d_ctl->remaining;
     desc[k] = d;
+    if (m.alone) continue;
+    ++b->nshared;
     for (int u = 0; u < d.nunits; ++u) su.push_back(UnitRef{k, u});
     for (int u = 0; u < d.nunits_f; ++u) fu.push_back(UnitRef{k, u});
   }
@@ -123,10 +144,12 @@ int rebuild(vdp_batch* b) {
   if (n > 0) {
     VDP_CK(cudaMemcpyAsync(b->d_desc, desc.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice,
                            b->stream));
-    VDP_CK(cudaMemcpyAsync(b->d_units, su.data(), sizeof(UnitRef) * b->ns, cudaMemcpyHostToDevice,
-                           b->stream));
-    VDP_CK(cudaMemcpyAsync(b->d_units + b->ns, fu.data(), sizeof(UnitRef) * b->nf,
-                           cudaMemcpyHostToDevice, b->stream));
+    if (b->nshared > 0) {
+      VDP_CK(cudaMemcpyAsync(b->d_units, su.data(), sizeof(UnitRef) * b->ns, cudaMemcpyHostToDevice,
+                             b->stream));
+      VDP_CK(cudaMemcpyAsync(b->d_units + b->ns, fu.data(), sizeof(UnitRef) * b->nf,
+                             cudaMemcpyHostToDevice, b->stream));
+    }
   }
   BatchCtl ctl{};
   ctl.remaining = n;
@@ -155,6 +178,7 @@ int capture(vdp_batch* b, int pairs) {
     // residual and sweep kernels (each kernel leaves the other forms' units alone)
     int nscaled = 0, nfixed = 0, ncheb = 0, ndfixed = 0, ndcg = 0;
     for (int k : b->active) {
+      if (b->members[k].alone) continue;
       const InstDesc& d = b->members[k].ctx->hdesc;
       if (d.form) {
         ++(d.pc == PC_FIXED ? ndfixed : ndcg);
@@ -177,14 +201,15 @@ int capture(vdp_batch* b, int pairs) {
       // members' chains are independent, so they go to up to four graph branches that the GPU
       // runs concurrently (small grids alone would leave most SMs idle).
       int nspec = 0;
-      for (int k : b->active) nspec += b->members[k].ctx->hdesc.pc >= PC_SPECTRAL;
+      for (int k : b->active)
+        nspec += !b->members[k].alone && b->members[k].ctx->hdesc.pc >= PC_SPECTRAL;
       const int nb = std::min(nspec, (int)vdp_batch::kBranches);
       if (nb > 0 && e == cudaSuccess) e = cudaEventRecord(b->fork, b->cap);
       for (int j = 0; j < nb && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(b->aux[j], b->fork, 0);
       int slot = 0;
       for (size_t k = 0; k < b->active.size() && e == cudaSuccess; ++k) {
         const vdp_ctx* c = b->members[b->active[k]].ctx;
-        if (c->hdesc.pc < PC_SPECTRAL) continue;
+        if (b->members[b->active[k]].alone || c->hdesc.pc < PC_SPECTRAL) continue;
         cudaStream_t br = b->aux[slot++ % nb];
         if (c->hdesc.pc == PC_MG) {
           const MgArgs a{c->r, c->za, c->omega, c->st, c->desc};
@@ -216,6 +241,43 @@ int capture(vdp_batch* b, int pairs) {
   cudaGraphDestroy(g);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate (batch)");
   b->g_pairs = pairs;
+  return VDP_OK;
+}
+
+// Launch the members that run by themselves, each for up to `pairs` rounds, on the branch streams
+// (largest first, to the stream with the fewest cells), between two points of the batch's stream.
+int launch_alone(vdp_batch* b, int pairs) {
+  std::vector<int> own;
+  for (int k : b->active)
+    if (b->members[k].alone) own.push_back(k);
+  if (own.empty()) return VDP_OK;
+  std::sort(own.begin(), own.end(), [&](int i, int j) {
+    return b->members[i].ctx->n != b->members[j].ctx->n ? b->members[i].ctx->n > b->members[j].ctx->n : i < j;
+  });
+  const int nb = std::min((int)own.size(), (int)vdp_batch::kBranches);
+  long long load[vdp_batch::kBranches] = {};
+  VDP_CK(cudaEventRecord(b->fork, b->stream));
+  for (int j = 0; j < nb; ++j) VDP_CK(cudaStreamWaitEvent(b->aux[j], b->fork, 0));
+  for (int k : own) {
+    vdp_ctx* c = b->members[k].ctx;
+    const int j = (int)(std::min_element(load, load + nb) - load);
+    load[j] += c->n;
+    if (resident_solve(c, b->prec)) {
+      SpecArgs a;
+      solve_spec_args(c, b->prec, &a);
+      VDP_CK(cudaMemsetAsync(c->rctl, 0, sizeof(ResidentCtl), b->aux[j]));
+      // a round is at most two sweeps; side by side, each member takes its share of the blocks
+      VDP_CK(launch_resident(b->prec, c->hdesc, c->desc, a, c->rctl, 2u * (unsigned)pairs,
+                             2 * kSMs / nb, b->aux[j]));
+    } else {
+      VDP_CK(launch_start_rounds(c->d_rounds, (unsigned)((pairs + kWhileRounds - 1) / kWhileRounds), b->aux[j]));
+      VDP_CK(cudaGraphLaunch(c->wexec, b->aux[j]));
+    }
+  }
+  for (int j = 0; j < nb; ++j) {
+    VDP_CK(cudaEventRecord(b->join[j], b->aux[j]));
+    VDP_CK(cudaStreamWaitEvent(b->stream, b->join[j], 0));
+  }
   return VDP_OK;
 }
 
@@ -300,7 +362,7 @@ int vdp_batch_add(vdp_batch* b, vdp_ctx* c, const double* rhs, double* p, double
   VDP_CK(cudaStreamSynchronize(c->stream));
   VDP_CK(launch_init(c->desc, rhs, p, tol, c->opts.inner_tol, c->opts.max_iter, c->opts.max_iter,
                      c->opts.use_guess ? 1 : 0, b->prec, nullptr, b->stream));
-  b->members.push_back(Member{c, rhs, p, tol, false});
+  b->members.push_back(Member{c, rhs, p, tol, false, false});
   b->dirty = true;
   return VDP_OK;
 }
@@ -314,7 +376,7 @@ int vdp_batch_run(vdp_batch* b, int max_pairs, int* active_out) {
     if (active_out) *active_out = 0;
     return VDP_OK;
   }
-  if (!b->gexec || b->g_pairs != max_pairs) {
+  if (b->nshared > 0 && (!b->gexec || b->g_pairs != max_pairs)) {
     if ((s = capture(b, max_pairs)) != VDP_OK) return s;
   }
   if (b->ctl_stale || b->inject) {  // fresh barrier words (after an expired wait, or to inject)
@@ -327,7 +389,8 @@ int vdp_batch_run(vdp_batch* b, int max_pairs, int* active_out) {
     b->ctl_stale = b->inject;  // an injected run leaves words to reset
     b->inject = false;
   }
-  VDP_CK(cudaGraphLaunch(b->gexec, b->stream));
+  if ((s = launch_alone(b, max_pairs)) != VDP_OK) return s;
+  if (b->nshared > 0) VDP_CK(cudaGraphLaunch(b->gexec, b->stream));
   VDP_CK(launch_gather(b->d_desc, n, b->d_states, b->stream));
   VDP_CK(cudaMemcpyAsync(b->h_states, b->d_states, sizeof(InstState) * n, cudaMemcpyDeviceToHost,
                          b->stream));

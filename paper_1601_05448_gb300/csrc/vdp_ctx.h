@@ -86,7 +86,7 @@ struct vdp_ctx {
   cudaGraphExec_t wexec = nullptr;
   int w_prec = -1;
   bool w_failed = false;           // the driver cannot build it: use the polling schedule
-  unsigned* d_rounds = nullptr;
+  unsigned* d_rounds = nullptr;    // rounds run, and the launch's limit
   vdp::ResidentCtl* rctl = nullptr;  // resident solve (vdp_resident.cu)
   vdp_stats stats{};
 };
@@ -117,6 +117,12 @@ int spec_slab(const vdp_ctx* c);  // planes per slab of the spectral passes
 // allocate the multigrid levels and the z and omega buffers (no-op when present); VDP_EINVAL
 // for grids the V-cycle does not support
 int ensure_mg(vdp_ctx* c);
+// The solve's device-side loop c->wexec (rounds and limit in c->d_rounds): false if the driver
+// cannot build it
+constexpr int kWhileRounds = 2;  // rounds of one loop iteration
+bool ensure_while_graph(vdp_ctx* c, int prec);
+// whether a solve runs as one cooperative launch (vdp_resident.cu); allocates its control words
+bool resident_solve(vdp_ctx* c, int prec);
 // kernel launches of one application of the solve's preconditioner (spectral passes, V-cycle)
 int precond_launches(const vdp_ctx* c);
 // before a solve that uses the spectral passes or the V-cycle: the weights (and the multigrid

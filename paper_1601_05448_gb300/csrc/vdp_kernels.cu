@@ -796,15 +796,26 @@ cudaError_t launch_persistent(int prec, const InstDesc* desc, const UnitRef* sun
 }
 
 // The body of a solve's device-side loop ends with this kernel: it keeps the loop going while
-// the solve is unfinished and the round count is below its bound.
+// the solve is unfinished and the round count rounds[0] is below its bound and the launch's own
+// limit rounds[1] (0: none).
 __global__ void k_continue(const InstState* st, cudaGraphConditionalHandle handle, unsigned* rounds,
                            unsigned max_rounds) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
-    const unsigned r = *rounds + 1u;
-    *rounds = r;
-    const bool more = __ldcg(&st->phase) < PH_DONE && r < max_rounds;
+    const unsigned r = rounds[0] + 1u, limit = rounds[1];
+    rounds[0] = r;
+    const bool more = __ldcg(&st->phase) < PH_DONE && r < max_rounds && (limit == 0u || r < limit);
     cudaGraphSetConditional(handle, more ? 1u : 0u);
   }
+}
+
+__global__ void k_start_rounds(unsigned* rounds, unsigned limit) {
+  rounds[0] = 0u;
+  rounds[1] = limit;
+}
+
+cudaError_t launch_start_rounds(unsigned* rounds, unsigned limit, cudaStream_t s) {
+  k_start_rounds<<<1, 1, 0, s>>>(rounds, limit);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_continue(const InstState* st, cudaGraphConditionalHandle handle,

@@ -434,7 +434,11 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
     }
     __syncthreads();
   }
-  // an expired wait leaves the state of the last whole sweep (the host sees an unfinished solve)
+  if (!ok && threadIdx.x == 0) {  // a wait expired: the sweep is incomplete, the solve ends
+    sn.status = 6;                  // VDP_ETIMEOUT
+    sn.phase = PH_DONE;
+  }
+  __syncthreads();
   if (blockIdx.x == 0 && threadIdx.x < sizeof(InstState) / 16)
     __stcg(reinterpret_cast<int4*>(I.st) + threadIdx.x, reinterpret_cast<const int4*>(&sn)[threadIdx.x]);
 }
@@ -496,7 +500,7 @@ bool resident_supported(const InstDesc& d, int prec) {
 }
 
 cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, const SpecArgs& spec,
-                            ResidentCtl* ctl, unsigned max_sweeps, cudaStream_t s) {
+                            ResidentCtl* ctl, unsigned max_sweeps, int max_blocks, cudaStream_t s) {
   const int kind = resident_kind(d);
   if (kind != R_JACOBI && spec.zunits > kResidentSlots) return cudaErrorInvalidValue;
   const ResidentKernel k = resident_kernel(prec, kind);
@@ -533,6 +537,7 @@ cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, c
   }
   int grid = per_sm * sms[dev];
   if (grid > most) grid = most;
+  if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kResThreads);
