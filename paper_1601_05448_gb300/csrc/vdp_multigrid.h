@@ -50,8 +50,8 @@ size_t mg_bytes(int nx, int ny, int nz);
 cudaError_t mg_alloc(MgHier* h, int nx, int ny, int nz, int wall_x);
 void mg_free(MgHier* h);
 // Build every level's coefficients from the FP64 face coefficients of the grid (level 0 scaled
-// by sinv = D^-1/2 on both sides) and the coarsest level's pseudo-inverse (host, double
-// precision); synchronises stream s.
+// by sinv = D^-1/2 on both sides) and the coarsest level's pseudo-inverse (double precision), on
+// stream s.
 cudaError_t mg_setup(MgHier* h, const double* bx, const double* by, const double* bz,
                      const double* sinv, cudaStream_t s);
 // out = in * sinv (n doubles)
