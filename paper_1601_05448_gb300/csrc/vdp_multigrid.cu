@@ -35,7 +35,6 @@ namespace vdp {
 namespace {
 
 constexpr int kMgThreads = kMarchTx * kMarchTy;  // 1-D blocks of 256 (tile 32 x 8)
-constexpr int kCoarseThreads = 512;
 
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(double v) { return narrow(v); }
@@ -156,46 +155,56 @@ __global__ void __launch_bounds__(kMgThreads, 4)
   }
 }
 
-// Prolongation, marching the fine column (x, y) along z: the bilinear xy interpolation of coarse
-// plane K at the column, L(K), is computed once and carried; fine plane k = 2K takes
-// 3/4 L(K) + 1/4 L(K-1), k = 2K + 1 takes 3/4 L(K) + 1/4 L(K+1).  With the pre-smoothed iterate:
+// Prolongation.  A thread has the two fine columns 2I, 2I + 1 of a fine row y and marches the coarse
+// planes K of a chunk: the bilinear xy interpolations of plane K at the two columns, L(K), are
+// computed once and carried (fine plane 2K takes 3/4 L(K) + 1/4 L(K-1), plane 2K + 1 3/4 L(K) + 1/4
+// L(K+1)), so four fine cells cost two 8-byte loads each of rt and omega and six coarse values,
+// and all of a step's loads are issued together (one column and one cell per step before: the whole
+// cycle at 160^3 157 -> 136 us with this and the coarsest level below).  With the pre-smoothed iterate:
 // t = w rt + omega P xc   (scaled: y1 + W P xc; xc is the coarse level's unscaled result)
-template <class T>
 __global__ void __launch_bounds__(kMgThreads, 4)
-    k_mg_prolong(MgLevel lv, MgLevel cv, MarchPlan m, const T* __restrict__ rt,
+    k_mg_prolong(MgLevel lv, MgLevel cv, MarchPlan m, const float* __restrict__ rt,
                  const float* __restrict__ om, int wall_x, const InstState* st) {
   if (!mg_active(st)) return;
-  const int cx = cv.nx, cy = cv.ny, cz = cv.nz;
-  const long long cplane = (long long)cx * cy;
+  const int nx = lv.nx, ny = lv.ny, cx = cv.nx, cy = cv.ny, cz = cv.nz;
+  const long long plane = (long long)nx * ny, cplane = (long long)cx * cy;
   const float* __restrict__ xc = cv.x;
-  MG_MARCH_BEGIN(lv)
-  (void)d;
-  const int I0 = x >> 1, J0 = y >> 1;
-  // neighbour of the parent on the fine cell's side; at the duct's x ends the parent itself
-  const int I1 = (x & 1) ? (I0 + 1 == cx ? (wall_x ? I0 : 0) : I0 + 1)
-                         : (I0 == 0 ? (wall_x ? I0 : cx - 1) : I0 - 1);
-  const int J1 = (y & 1) ? (J0 + 1 == cy ? 0 : J0 + 1) : (J0 == 0 ? cy - 1 : J0 - 1);
-  const long long q00 = I0 + (long long)cx * J0, q10 = I1 + (long long)cx * J0;
-  const long long q01 = I0 + (long long)cx * J1, q11 = I1 + (long long)cx * J1;
-  auto L = [&](int K) {
-    const float* pl = xc + cplane * K;
-    const float a = fmaf(0.75f, __ldg(pl + q00), 0.25f * __ldg(pl + q10));
-    const float b = fmaf(0.75f, __ldg(pl + q01), 0.25f * __ldg(pl + q11));
-    return fmaf(0.75f, a, 0.25f * b);
-  };
-  int K = z0 >> 1;
-  float Lm = L(K == 0 ? cz - 1 : K - 1), Lc = L(K), Lp = L(K + 1 == cz ? 0 : K + 1);
-  for (int z = z0; z < z1; ++z) {
-    const float pxc = (z & 1) ? fmaf(0.75f, Lc, 0.25f * Lp) : fmaf(0.75f, Lc, 0.25f * Lm);
-    lv.t[c] = fmaf(kMgOmega, to_f(__ldg(rt + c)), __ldg(om + c) * pxc);
-    if ((z & 1) && z + 1 < z1) {  // the next fine plane belongs to coarse plane K + 1
-      ++K;
+  for (int it = blockIdx.x; it < m.items; it += gridDim.x) {
+    int I, y, K0, K1;
+    if (!march_item(m, it, threadIdx.x & 31, threadIdx.x >> 5, cx, ny, cz, I, y, K0, K1)) continue;
+    const int J0 = y >> 1;
+    // neighbours of the parent on the fine cells' sides; at the duct's x ends the parent itself
+    const int Im = I == 0 ? (wall_x ? I : cx - 1) : I - 1;
+    const int Ip = I + 1 == cx ? (wall_x ? I : 0) : I + 1;
+    const int J1 = (y & 1) ? (J0 + 1 == cy ? 0 : J0 + 1) : (J0 == 0 ? cy - 1 : J0 - 1);
+    const long long r0 = (long long)cx * J0, r1 = (long long)cx * J1;
+    auto L = [&](int K) {
+      const float* p0 = xc + cplane * K + r0;
+      const float* p1 = xc + cplane * K + r1;
+      const float c0 = __ldg(p0 + I), l0 = __ldg(p0 + Im), h0 = __ldg(p0 + Ip);
+      const float c1 = __ldg(p1 + I), l1 = __ldg(p1 + Im), h1 = __ldg(p1 + Ip);
+      const float al = fmaf(0.75f, c0, 0.25f * l0), bl = fmaf(0.75f, c1, 0.25f * l1);
+      const float ah = fmaf(0.75f, c0, 0.25f * h0), bh = fmaf(0.75f, c1, 0.25f * h1);
+      return make_float2(fmaf(0.75f, al, 0.25f * bl), fmaf(0.75f, ah, 0.25f * bh));
+    };
+    long long c = 2 * I + (long long)nx * y + plane * (2 * K0);
+    float2 Lm = L(K0 == 0 ? cz - 1 : K0 - 1), Lc = L(K0);
+    for (int K = K0; K < K1; ++K, c += 2 * plane) {
+      const float2 Lp = L(K + 1 == cz ? 0 : K + 1);
+      const float2 ra = __ldg(reinterpret_cast<const float2*>(rt + c));
+      const float2 rb = __ldg(reinterpret_cast<const float2*>(rt + c + plane));
+      const float2 wa = __ldg(reinterpret_cast<const float2*>(om + c));
+      const float2 wb = __ldg(reinterpret_cast<const float2*>(om + c + plane));
+      float2 ta, tb;
+      ta.x = fmaf(kMgOmega, ra.x, wa.x * fmaf(0.75f, Lc.x, 0.25f * Lm.x));
+      ta.y = fmaf(kMgOmega, ra.y, wa.y * fmaf(0.75f, Lc.y, 0.25f * Lm.y));
+      tb.x = fmaf(kMgOmega, rb.x, wb.x * fmaf(0.75f, Lc.x, 0.25f * Lp.x));
+      tb.y = fmaf(kMgOmega, rb.y, wb.y * fmaf(0.75f, Lc.y, 0.25f * Lp.y));
+      *reinterpret_cast<float2*>(lv.t + c) = ta;
+      *reinterpret_cast<float2*>(lv.t + c + plane) = tb;
       Lm = Lc;
       Lc = Lp;
-      Lp = L(K + 1 == cz ? 0 : K + 1);
     }
-    c += plane;
-  }
   }
 }
 
@@ -267,17 +276,25 @@ __global__ void __launch_bounds__(kMgThreads, 4)
   }
 }
 
-// Coarsest level: x = pinv r (one block; pinv is symmetric, so thread i reads column i).
-__global__ void __launch_bounds__(kCoarseThreads)
+// Coarsest level: x = pinv r, a warp per four rows (one block with a thread per row and all its
+// products in sequence took 13 us for 125 cells).
+constexpr int kCoarseRows = 4 * (kMgThreads / 32);  // rows of a block
+
+__global__ void __launch_bounds__(kMgThreads)
     k_mg_coarse(MgLevel lv, const float* __restrict__ pinv, int n, const InstState* st) {
   if (!mg_active(st)) return;
-  __shared__ float r[kMgMaxCoarsest];
-  for (int i = threadIdx.x; i < n; i += blockDim.x) r[i] = lv.r[i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    float s = 0.f;
-    for (int j = 0; j < n; ++j) s = fmaf(__ldg(pinv + (long long)j * n + i), r[j], s);
-    lv.x[i] = s;
+  const int lane = threadIdx.x & 31, i0 = blockIdx.x * kCoarseRows + (threadIdx.x >> 5) * 4;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int j = lane; j < n; j += 32) {
+    const float r = __ldg(lv.r + j);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i0 + q < n) s[q] = fmaf(__ldg(pinv + (long long)(i0 + q) * n + j), r, s[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float v = warp_sum(s[q]);
+    if (lane == 0 && i0 + q < n) lv.x[i0 + q] = v;
   }
 }
 
@@ -669,11 +686,12 @@ static cudaError_t vcycle(const MgHier& h, const MgArgs& a, cudaStream_t s) {
     k_mg_restrict<<<mr.blocks, kMgThreads, 0, s>>>(v, cv, mr, l + 1 < L - 1 ? cv.oinv : nullptr,
                                                    h.wall_x, a.st);
   }
-  k_mg_coarse<<<1, kCoarseThreads, 0, s>>>(h.lev[L - 1], h.pinv, h.ncoarse, a.st);
+  k_mg_coarse<<<(h.ncoarse + kCoarseRows - 1) / kCoarseRows, kMgThreads, 0, s>>>(h.lev[L - 1], h.pinv, h.ncoarse, a.st);
   for (int l = L - 2; l >= 0; --l) {
     const MgLevel& v = h.lev[l];
-    const MarchPlan mp = march_plan(v.nx, v.ny, v.nz, cached_resident(k_mg_prolong<float>, &r_pro));
-    k_mg_prolong<float><<<mp.blocks, kMgThreads, 0, s>>>(v, h.lev[l + 1], mp, rhs(l), wgt(l),
+    const MgLevel& cv = h.lev[l + 1];
+    const MarchPlan mp = march_plan(cv.nx, v.ny, cv.nz, cached_resident(k_mg_prolong, &r_pro));
+    k_mg_prolong<<<mp.blocks, kMgThreads, 0, s>>>(v, h.lev[l + 1], mp, rhs(l), wgt(l),
                                                          h.wall_x, a.st);
     if (l == 0) {
       const MarchPlan m = march_plan(v.nx, v.ny, v.nz, cached_resident(k_mg_up<float, T, false>, &r_up0));
