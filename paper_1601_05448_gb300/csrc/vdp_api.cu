@@ -165,6 +165,7 @@ int configure_layout(vdp_ctx* c, int prec) {
   }
   d.rho32 = c->rho32;
   d.rho_lo = c->rho_lo;
+  d.g32 = d.form && prec == PREC_FP64 ? density_g32(c) : nullptr;
   d.dsc = c->dsc;
   d.ncell = c->n;
   d.bx = c->bx;
@@ -401,16 +402,17 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   const int nxt = spectral_nx(c);  // x transform length (twice the cells in the duct)
   const int m = nxt / 2;
   const bool fixed = c->opts.method == VDP_METHOD_FIXED_POINT;
-  a->in = c->r;
+  // density form: the stored residual is g = rho' r (fixed point) or r, z is unscaled and FP32, and
+  // the inverse is that of s L_h: no weights
+  const bool dens = density_form(c, prec);
+  const bool dens64 = dens && prec == PREC_FP64;
+  a->in = dens64 ? (const void*)density_g32(c) : c->r;
   // CG: z = W (-L_h)^-1 W rt, W = D^1/2.  Fixed point: with rt = D^-1/2 r the input weight
   // rho D^1/2 gives rho r, and z = damping D^1/2 (-L_h)^-1 (rho r) is the scaled form of the
   // paper's update p += damping L_h^-1 (rho r) (applied as p -= D^-1/2 x, x the sum of the z)
   a->out = c->za;
-  a->out_f32 = fixed || density_form(c, prec) ? 1 : 0;  // those sweeps read z as FP32
-  // density form: the stored residual is g = rho' r (FP32 fixed point) or r, z is unscaled and
-  // FP32, and the inverse is that of s L_h: no weights but rho' on the FP64 fixed point's r
-  const bool dens = density_form(c, prec);
-  a->omega_in = dens ? (fixed && prec == PREC_FP64 ? c->rho32 : nullptr) : fixed ? c->rho_w : c->omega;
+  a->f32 = (dens64 ? kInF32 : 0) | (fixed || dens ? kOutF32 : 0);  // those sweeps read z as FP32
+  a->omega_in = dens ? nullptr : fixed ? c->rho_w : c->omega;
   a->omega_out = dens ? nullptr : c->omega;
   a->spec = c->spec;
   a->tw = reinterpret_cast<const float2*>(c->sptab);
@@ -837,7 +839,7 @@ int vdp_inverse_laplacian(vdp_ctx* c, const double* g, double* out) {
   solve_spec_args(c, PREC_FP64, &a);
   a.in = g;
   a.out = out;
-  a.out_f32 = 0;
+  a.f32 = 0;
   a.omega_in = nullptr;
   a.omega_out = nullptr;
   a.scale = (float)(-1.0 / ((double)a.nx * c->ny * c->nz));  // L_h^-1, not (-L_h)^-1

@@ -104,6 +104,8 @@ int ensure_sinv(vdp_ctx* c);
 // its low part) is at hand.  A density that was set before the method or the precision was
 // selected is not: the solve then runs in the scaled form.
 bool density_form(const vdp_ctx* c, int prec);
+// FP64 density form: z is FP32, so the second half of its buffer holds X+'s FP32 input
+inline float* density_g32(const vdp_ctx* c) { return static_cast<float*>(c->za) + c->n; }
 // s of the density form: the power of 4 below hx^2
 inline double density_scale(const vdp_ctx* c) { return std::ldexp(1.0, 2 * std::ilogb(c->Lx / c->nx)); }
 // length of the x transform of the spectral passes: nx, or 2 nx in the duct (even extension)

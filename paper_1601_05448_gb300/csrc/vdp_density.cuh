@@ -316,13 +316,13 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
 // pair, the quotient by a Newton step and a corrected remainder, the differences of z exact, the
 // products by FMA with their rounding errors, the six terms summed with the errors carried along.
 // Only the update of the FP64 fields is FP64: three instructions per cell (fixed point), four
-// (CG).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
+// (CG).  The sweep also leaves rho' r in FP32 for the X+ pass, which read r and rho' and narrowed
+// the product itself: four bytes more here, eight fewer there, and X+ runs its FP32 form (256^3:
+// 75 -> 35 us).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
 // the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before.
 struct df {
   f2 h, l;
 };
-
-__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
 
 // h + l = a + b exactly
 __device__ __forceinline__ df two_sum(f2 a, f2 b) {
@@ -340,39 +340,49 @@ __device__ __forceinline__ df two_diff(f2 a, f2 b) {
   return r;
 }
 
-// c / (a + b), c = -(nch + ncl)
-__device__ __forceinline__ df face_df(f2 nch, f2 ncl, df a, df b) {
+// A face coefficient c / (a + b), c = ch + cl = -(nch + ncl): h and the negatives of both parts (the
+// paired instructions have no negated operands, and the products below want them).
+struct dface {
+  f2 h, nh, nl;
+};
+struct consts {
+  f2 ch, nch, cl;
+};
+__device__ __forceinline__ dface face_df(const consts& c, df a, df b) {
   df s = two_sum(a.h, b.h);
   s.l = add2(s.l, add2(a.l, b.l));
   const float2 v = up2(s.h);
   f2 y = pk(rcp_approx(-v.x), rcp_approx(-v.y));  // -1 / s
   y = fma2(y, fma2(s.h, y, pk(1.f, 1.f)), y);
-  df q;
-  q.h = mul2(nch, y);
-  const f2 t = add2(fma2(q.h, s.l, fma2(q.h, s.h, nch)), ncl);  // q s - c
-  q.l = mul2(t, y);
+  dface q;
+  q.h = mul2(c.nch, y);
+  q.nh = mul2(c.ch, y);
+  const f2 t = add2(fma2(q.nh, s.l, fma2(q.nh, s.h, c.ch)), c.cl);  // c - q s
+  q.nl = mul2(t, y);
   return q;
 }
 
-// -(b x difference) of a face as an unevaluated sum, from the exact difference d
-__device__ __forceinline__ df minus_flux(df b, df d) {
-  df f;
-  f.h = mul2(neg2(b.h), d.h);
-  const f2 e = fma2(b.l, d.h, fma2(b.h, d.l, fma2(b.h, d.h, f.h)));  // b d + f.h
-  f.l = neg2(e);
+// The flux b d through a face from the exact difference d, as h - nl
+struct dflux {
+  f2 h, nl;
+};
+__device__ __forceinline__ dflux flux_df(const dface& b, df d) {
+  dflux f;
+  f.h = mul2(b.h, d.h);
+  f.nl = fma2(b.nl, d.h, fma2(b.nh, d.l, fma2(b.nh, d.h, f.h)));  // f.h - b d
   return f;
 }
 
-// acc -= f
-__device__ __forceinline__ void accumulate_minus(df& acc, df f) {
-  const df s = two_diff(acc.h, f.h);
-  acc.h = s.h;
-  acc.l = add2(acc.l, sub2(s.l, f.l));
-}
-__device__ __forceinline__ void accumulate_plus(df& acc, df f) {
+// acc += f, acc -= f
+__device__ __forceinline__ void accumulate_plus(df& acc, const dflux& f) {
   const df s = two_sum(acc.h, f.h);
   acc.h = s.h;
-  acc.l = add2(acc.l, add2(s.l, f.l));
+  acc.l = add2(acc.l, sub2(s.l, f.nl));
+}
+__device__ __forceinline__ void accumulate_minus(df& acc, const dflux& f) {
+  const df s = two_diff(acc.h, f.h);
+  acc.h = s.h;
+  acc.l = add2(acc.l, add2(s.l, f.nl));
 }
 
 enum Stream64 { T_UP, T_UA, T_UB, T_HP, T_HA, T_HB, T_LP, T_LA, T_LB, T_P0, T_P1, T_Q0, T_Q1, kStreams64 };
@@ -399,11 +409,12 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
   const bool row_start = x0 == 0, row_end = x0 + kV == nx;
   const bool left_load = lane == 0 || row_start, right_load = lane == 31 || row_end;
   const bool wall_l = I.duct && row_start, wall_r = I.duct && row_end;
-  f2 nch[3], ncl[3];
+  consts cf[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    nch[d] = pk(-I.ch[d], -I.ch[d]);
-    ncl[d] = pk(-I.cl[d], -I.cl[d]);
+    cf[d].ch = pk(I.ch[d], I.ch[d]);
+    cf[d].nch = pk(-I.ch[d], -I.ch[d]);
+    cf[d].cl = pk(I.cl[d], I.cl[d]);
   }
   const double beta = st.beta;
   const bool first = st.inner_iters == 0;  // no X (fixed point), no history (CG) yet
@@ -451,7 +462,9 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
   fetch(0, z0, o);
   fetch_commit();
   f2 u[2];
-  df r[2], bzl[2], fz[2];  // fz: minus the flux through the lower z face
+  df r[2];
+  f2 bzl[2];    // lower z face: its coefficient (leading part) and flux b (z - z below)
+  dflux fz[2];
   {
     const long long om = z0 == 0 ? o + dz_last : o - plane;
     f2 um[2];
@@ -464,8 +477,9 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
     ldg2(rlo + o, r[0].l, r[1].l);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      bzl[h] = face_df(nch[2], ncl[2], rm[h], r[h]);
-      fz[h] = minus_flux(bzl[h], two_diff(u[h], um[h]));
+      const dface b = face_df(cf[2], rm[h], r[h]);
+      bzl[h] = b.h;
+      fz[h] = flux_df(b, two_diff(u[h], um[h]));
     }
   }
   double sum = 0.0;
@@ -492,24 +506,24 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
         hr = __ldg(rhi + o + dxr);
         lr = __ldg(rlo + o + dxr);
       }
-      df b01 = face_df(nch[0], ncl[0], df{pk(hl, h01.x), pk(ll, l01.x)}, r[0]);
-      const df b23 = face_df(nch[0], ncl[0], df{pk(h01.y, h23.x), pk(l01.y, l23.x)}, r[1]);
-      df b44 = face_df(nch[0], ncl[0], df{pk(h23.y, h23.y), pk(l23.y, l23.y)}, df{pk(hr, hr), pk(lr, lr)});
+      dface b01 = face_df(cf[0], df{pk(hl, h01.x), pk(ll, l01.x)}, r[0]);
+      const dface b23 = face_df(cf[0], df{pk(h01.y, h23.x), pk(l01.y, l23.x)}, r[1]);
+      dface b44 = face_df(cf[0], df{pk(h23.y, h23.y), pk(l23.y, l23.y)}, df{pk(hr, hr), pk(lr, lr)});
       if (wall_l) {
         b01.h = pk(0.f, up2(b01.h).y);
-        b01.l = pk(0.f, up2(b01.l).y);
+        b01.nh = pk(0.f, up2(b01.nh).y);
+        b01.nl = pk(0.f, up2(b01.nl).y);
       }
-      if (wall_r) b44.h = b44.l = 0ull;
-      const df f01 = minus_flux(b01, two_diff(u[0], pk(ul, u01.x)));
-      const df f23 = minus_flux(b23, two_diff(u[1], pk(u01.y, u23.x)));
-      const df f44 = minus_flux(b44, two_diff(pk(ur, ur), pk(u23.y, u23.y)));
-      const float2 fh01 = up2(f01.h), fh23 = up2(f23.h), fl01 = up2(f01.l), fl23 = up2(f23.l);
-      const df f12 = {pk(fh01.y, fh23.x), pk(fl01.y, fl23.x)};
-      const df f34 = {pk(fh23.y, up2(f44.h).x), pk(fl23.y, up2(f44.l).x)};
-      acc[0] = f01;  // A' z = sum of (upper flux - lower flux); f holds minus the flux
-      acc[1] = f23;
-      accumulate_minus(acc[0], f12);
-      accumulate_minus(acc[1], f34);
+      if (wall_r) b44.h = b44.nh = b44.nl = 0ull;
+      // fluxes b (u_k - u_{k-1}); A' z = sum of (upper flux - lower flux)
+      const dflux f01 = flux_df(b01, two_diff(u[0], pk(ul, u01.x)));
+      const dflux f23 = flux_df(b23, two_diff(u[1], pk(u01.y, u23.x)));
+      const dflux f44 = flux_df(b44, two_diff(pk(ur, ur), pk(u23.y, u23.y)));
+      const float2 fh01 = up2(f01.h), fh23 = up2(f23.h), fl01 = up2(f01.nl), fl23 = up2(f23.nl);
+      acc[0] = df{pk(fh01.y, fh23.x), sub2(0ull, pk(fl01.y, fl23.x))};
+      acc[1] = df{pk(fh23.y, up2(f44.h).x), sub2(0ull, pk(fl23.y, up2(f44.nl).x))};
+      accumulate_minus(acc[0], f01);
+      accumulate_minus(acc[1], f23);
       if (FIXED) {
         const float2 bh01 = up2(b01.h), bh23 = up2(b23.h);
         D[0] = add2(b01.h, pk(bh01.y, bh23.x));
@@ -524,13 +538,13 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
     const df rn[2] = {{t.x, t2.x}, {t.y, t2.y}};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const df bz = face_df(nch[2], ncl[2], r[h], rn[h]);
-      const df f = minus_flux(bz, two_diff(un[h], u[h]));
-      accumulate_plus(acc[h], fz[h]);
-      accumulate_minus(acc[h], f);
+      const dface bz = face_df(cf[2], r[h], rn[h]);
+      const dflux f = flux_df(bz, two_diff(un[h], u[h]));
+      accumulate_plus(acc[h], f);
+      accumulate_minus(acc[h], fz[h]);
       fz[h] = f;
-      if (FIXED) D[h] = add2(D[h], add2(bzl[h].h, bz.h));
-      bzl[h] = bz;
+      if (FIXED) D[h] = add2(D[h], add2(bzl[h], bz.h));
+      bzl[h] = bz.h;
     }
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
@@ -541,8 +555,8 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
       const df rv[2] = {{t.x, tl.x}, {t.y, tl.y}};
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const df by = face_df(nch[1], ncl[1], rv[h], r[h]);
-        accumulate_minus(acc[h], minus_flux(by, two_diff(v[h], u[h])));
+        const dface by = face_df(cf[1], rv[h], r[h]);
+        accumulate_plus(acc[h], flux_df(by, two_diff(v[h], u[h])));
         if (FIXED) D[h] = add2(D[h], by.h);
       }
     }
@@ -561,8 +575,9 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
           qo.x += qv.x;
           qo.y += qv.y;
         }
-        const float2 d = up2(D[h]);
+        const float2 d = up2(D[h]), rho = up2(r[h].h);
         const float rx = narrow(po.x), ry = narrow(po.y);
+        if (active) *reinterpret_cast<float2*>(I.g32 + o + 2 * h) = make_float2(rho.x * rx, rho.y * ry);
         sumf = fmaf(rx * rcp_approx(d.x), rx, sumf);
         sumf = fmaf(ry * rcp_approx(d.y), ry, sumf);
       } else {

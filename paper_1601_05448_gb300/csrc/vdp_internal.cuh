@@ -112,6 +112,8 @@ struct InstDesc {
   const void* sd;      // BF16 only: diagonal correction of the stored inner operator
   const float* rho32;  // density form: rho / 2^e0 in FP32
   const float* rho_lo; // density form, FP64: rho / 2^e0 - rho32
+  float* g32;          // density form, FP64: the X+ pass's input in FP32 (rho' r, CG: r), written by
+                       // every sweep that writes r
   const double* dsc;   // density form: kappa = 2^e0 s (the inner operator is kappa A)
   void* x;             // inner solution (correction), inner type
   void* r;             // inner residual

@@ -86,7 +86,7 @@ __device__ __forceinline__ int rows_each(int rows, int most) {
 // one body held them all in 128 registers with kilobytes of spills and took minutes to compile.
 // The mirrored row transforms serve both boundary conditions: without the mirror no pair lies in a
 // second half.
-template <class T, int M1, int M2>
+template <int M1, int M2>
 __device__ __noinline__ void x_forward(const SpecArgs& a, const Tables& tb, float2* buf) {
   constexpr int RY = rows_per_block<M1, M2>(), SX = x_row_stride<M1, M2>();
   const int rows = a.ny * a.nz, per = rows_each(rows, RY);
@@ -95,7 +95,7 @@ __device__ __noinline__ void x_forward(const SpecArgs& a, const Tables& tb, floa
     const long long row = (long long)g * per + r;
     const bool live = r < per && row < rows;
     float2* out = a.spec + row * a.nxp;
-    x_fwd_rows<T, M1, M2, true>(a, tb, buf + (r < RY ? r : 0) * SX, row, live, t,
+    x_fwd_rows<float, M1, M2, true>(a, tb, buf + (r < RY ? r : 0) * SX, row, live, t,
                                   [&](int k, float2 X) { out[k] = X; });
     __syncthreads();
   }
@@ -224,17 +224,16 @@ __device__ __noinline__ void lines(const SpecArgs& a, const Tables& tb, const fl
   }
 }
 
-template <class T>
 __device__ __forceinline__ void x_forward_any(const SpecArgs& a, const Tables& tb, float2* buf) {
   switch (a.nx / 2) {
-    case 16: x_forward<T, 4, 4>(a, tb, buf); break;
-    case 24: x_forward<T, 4, 6>(a, tb, buf); break;
-    case 32: x_forward<T, 4, 8>(a, tb, buf); break;
-    case 48: x_forward<T, 6, 8>(a, tb, buf); break;
-    case 64: x_forward<T, 8, 8>(a, tb, buf); break;
-    case 96: x_forward<T, 8, 12>(a, tb, buf); break;
-    case 128: x_forward<T, 8, 16>(a, tb, buf); break;
-    default: x_forward<T, 16, 16>(a, tb, buf); break;
+    case 16: x_forward<4, 4>(a, tb, buf); break;
+    case 24: x_forward<4, 6>(a, tb, buf); break;
+    case 32: x_forward<4, 8>(a, tb, buf); break;
+    case 48: x_forward<6, 8>(a, tb, buf); break;
+    case 64: x_forward<8, 8>(a, tb, buf); break;
+    case 96: x_forward<8, 12>(a, tb, buf); break;
+    case 128: x_forward<8, 16>(a, tb, buf); break;
+    default: x_forward<16, 16>(a, tb, buf); break;
   }
 }
 
@@ -393,7 +392,7 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
     int nparts = I.nunits;
     bool applied = false;  // the preconditioner's sweep was part of this round
     if (DENS && phase == PH_SPEC) {
-      x_forward_any<T>(spec, tb, work);
+      x_forward_any(spec, tb, work);
       if (!(ok = bar.sync())) break;
       lines_any<0>(spec.ny, spec, tb, wy, nullptr, work, slots);
       if (!(ok = bar.sync())) break;

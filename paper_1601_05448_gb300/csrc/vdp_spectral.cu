@@ -401,7 +401,9 @@ int line_index(int n) {
 std::vector<std::pair<SpecKernel, int>> g_x_per_sm[kMaxDevices];
 constexpr int kXHalfLengths[] = {16, 24, 32, 48, 64, 96, 128, 256};  // nx / 2
 
-bool x_f64(int prec, bool inv, const SpecArgs& a) { return prec == PREC_FP64 && !(inv && a.out_f32); }
+bool x_f64(int prec, bool inv, const SpecArgs& a) {
+  return prec == PREC_FP64 && !(a.f32 & (inv ? kOutF32 : kInF32));
+}
 
 SpecKernel x_pass_kernel(int prec, bool inv, const SpecArgs& a, int* threads) {
   const int m = a.nx / 2;

@@ -246,6 +246,8 @@ __device__ void sweep_update(const InstDesc& I, const InstState* st, long long c
       }
       VecIO<T, V>::st(x + c, xv[u]);
       VecIO<T, V>::st(rt + c, rv[u]);
+      if constexpr (sizeof(T) == 8)
+        if (I.g32) *reinterpret_cast<float2*>(I.g32 + c) = make_float2(narrow(rv[u][0]), narrow(rv[u][1]));
     }
   }
   T tot = 0;
@@ -612,7 +614,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       double2 si = make_double2(0.0, 0.0);
       float2 rh = make_float2(1.f, 1.f);
       if (!DENS) si = *reinterpret_cast<const double2*>(I.sinv + o);
-      if (DENS && dr.fixed && !IsF64<T>::value) rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o));
+      if (DENS && dr.fixed) rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o));
       const double l0 = h == 0 ? left : pc[h - 1];
       const double r1 = h + 2 == VR ? right : pc[h + 2];
       const double br1 = h + 2 == VR ? bxr : I.bx[o + 2];
@@ -658,6 +660,8 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       if (active) {
         rt[o] = t0;
         rt[o + 1] = t1;
+        if constexpr (DENS && IsF64<T>::value)
+          *reinterpret_cast<float2*>(I.g32 + o) = make_float2(rh.x * r0f, rh.y * r1f);
         a0 = fmaf(r0f, r0f, fmaf(r1f, r1f, a0));
         a1 = DENS ? a1 + (t0f + t1f) : fmaf(t0f, t0f, fmaf(t1f, t1f, a1));
         if (FIRST) {
@@ -711,13 +715,14 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
           const float r0 = narrow(f0), r1 = narrow(f1);
           float2 rh = make_float2(1.f, 1.f), d = make_float2(1.f, 1.f);
           if (dr.fixed) {
-            if (!IsF64<T>::value) rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o + h));
+            rh = __ldg(reinterpret_cast<const float2*>(dr.rho + o + h));
             const double2 D = *reinterpret_cast<const double2*>(I.dg + o + h);
             d = make_float2(dr.inv_diag(D.x), dr.inv_diag(D.y));
           }
           if constexpr (IsF64<T>::value) {
             rt[o + h] = f0;
             rt[o + h + 1] = f1;
+            *reinterpret_cast<float2*>(I.g32 + o + h) = make_float2(rh.x * r0, rh.y * r1);
           } else {
             rt[o + h] = rh.x * r0;
             rt[o + h + 1] = rh.y * r1;
