@@ -20,8 +20,9 @@
 // long-scoreboard, 47 % of the DRAM rate): each thread therefore fetches its operands of the next
 // plane by cp.async into slots of shared memory that only it reads, so no barrier is needed, no
 // registers are held while they fly, and the arithmetic of one plane covers the latency of the
-// next.  Sums, products and Newton steps of the four cells run as paired FP32 instructions, and
-// the fluxes through the x faces and the upper z face are computed once for both cells.
+// next.  The x neighbours at row and warp ends come the same way (loaded at their use, they cost
+// every plane a trip to L2).  Sums, products and Newton steps of the four cells run as paired FP32
+// instructions, and the fluxes through the x faces and the upper z face are computed once for both cells.
 #pragma once
 
 #include "vdp_device.cuh"
@@ -94,6 +95,12 @@ __device__ __forceinline__ void fetch16_once(void* smem, const float* g) {  // L
                "l"(g)
                : "memory");
 }
+__device__ __forceinline__ void fetch4(void* smem, const float* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(smem)),
+               "l"(g)
+               : "memory");
+}
 __device__ __forceinline__ void fetch_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // this thread's own copies: all but the newest group have landed
 __device__ __forceinline__ void fetch_wait_previous() {
@@ -149,7 +156,22 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
   const long long dz_last = plane * (nz - 1);  // from plane nz - 1 back to plane 0
   // stream k of stage b of this thread
   auto slot = [&](int b, int k) { return slots + (b * NS + k) * blockDim.x + threadIdx.x; };
+  // x neighbours beyond the warp or the row: value k (z, rho', d_old), side 0 left and 1 right
+  float* edges = reinterpret_cast<float*>(slots + kStages * NS * blockDim.x);
+  auto edge = [&](int b, int k, int side) {
+    return edges + ((b * 3 + k) * 2 + side) * blockDim.x + threadIdx.x;
+  };
   auto fetch = [&](int b, int z, long long o) {  // the operands of plane z (cells at o)
+    if (left_load) {
+      fetch4(edge(b, 0, 0), src + o + dxl);
+      fetch4(edge(b, 1, 0), rho + o + dxl);
+      if (kOld) fetch4(edge(b, 2, 0), dold + o + dxl);
+    }
+    if (right_load) {
+      fetch4(edge(b, 0, 1), src + o + dxr);
+      fetch4(edge(b, 1, 1), rho + o + dxr);
+      if (kOld) fetch4(edge(b, 2, 1), dold + o + dxr);
+    }
     const long long op = z == nz - 1 ? o - dz_last : o + plane;
     fetch16(slot(b, S_UP), src + op);
     fetch16(slot(b, S_UA), src + o + dym);
@@ -172,9 +194,6 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
     const ulonglong2 t = NC ? __ldg(v) : *v;
     a = t.x;
     b = t.y;
-  };
-  auto field1 = [&](long long o) -> float {
-    return kOld ? fmaf(beta, ro1<NC>(dold + o), ro1<NC>(src + o)) : ro1<NC>(src + o);
   };
   long long o = (long long)z0 * plane + cell0;
   fetch(0, z0, o);
@@ -209,17 +228,18 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
   for (int z = z0; z < z1; ++z) {
     if (z + 1 < z1) fetch(b ^ 1, z + 1, o + plane);
     fetch_commit();
-    // x neighbours: adjacent lanes, or a load at row ends and warp ends
+    fetch_wait_previous();
+    // x neighbours: adjacent lanes, or what was fetched at row ends and warp ends
     const float2 u01 = up2(u[0]), u23 = up2(u[1]), r01 = up2(r[0]), r23 = up2(r[1]);
     float ul = __shfl_up_sync(0xffffffffu, u23.y, 1), ur = __shfl_down_sync(0xffffffffu, u01.x, 1);
     float rl = __shfl_up_sync(0xffffffffu, r23.y, 1), rr = __shfl_down_sync(0xffffffffu, r01.x, 1);
     if (left_load) {
-      ul = field1(o + dxl);
-      rl = __ldg(rho + o + dxl);
+      ul = kOld ? fmaf(beta, *edge(b, 2, 0), *edge(b, 0, 0)) : *edge(b, 0, 0);
+      rl = *edge(b, 1, 0);
     }
     if (right_load) {
-      ur = field1(o + dxr);
-      rr = __ldg(rho + o + dxr);
+      ur = kOld ? fmaf(beta, *edge(b, 2, 1), *edge(b, 0, 1)) : *edge(b, 0, 1);
+      rr = *edge(b, 1, 1);
     }
     // faces and fluxes b (u_k - u_{k-1}) through the five x faces of the four cells
     const float b0 = wall_l ? 0.f : face(nx1, rl, r01.x), b1 = face(nx1, r01.x, r01.y);
@@ -229,7 +249,6 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
     const float f3 = b3 * (u23.y - u23.x), f4 = b4 * (ur - u23.y);
     f2 a[2] = {pk(f1 - f0, fm - f1), pk(f3 - fm, f4 - f3)};  // A' u, accumulated
     f2 D[2] = {pk(b0 + b1, b1 + b2), pk(b2 + b3, b3 + b4)};
-    fetch_wait_previous();
     ulonglong2 t = *slot(b, S_UP);
     f2 un[2] = {t.x, t.y};
     if (kOld) {
@@ -432,7 +451,22 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
   const long long cell0 = (long long)y * nx + x0;
   const long long dz_last = plane * (nz - 1);
   auto slot = [&](int b, int k) { return slots + (b * kStreams64 + k) * blockDim.x + threadIdx.x; };
+  // x neighbours beyond the warp or the row: value k (z, rho' high and low), side 0 left, 1 right
+  float* edges = reinterpret_cast<float*>(slots + kStages * kStreams64 * blockDim.x);
+  auto edge = [&](int b, int k, int side) {
+    return edges + ((b * 3 + k) * 2 + side) * blockDim.x + threadIdx.x;
+  };
   auto fetch = [&](int b, int z, long long o) {
+    if (left_load) {
+      fetch4(edge(b, 0, 0), src + o + dxl);
+      fetch4(edge(b, 1, 0), rhi + o + dxl);
+      fetch4(edge(b, 2, 0), rlo + o + dxl);
+    }
+    if (right_load) {
+      fetch4(edge(b, 0, 1), src + o + dxr);
+      fetch4(edge(b, 1, 1), rhi + o + dxr);
+      fetch4(edge(b, 2, 1), rlo + o + dxr);
+    }
     const long long op = z == nz - 1 ? o - dz_last : o + plane;
     fetch16(slot(b, T_UP), src + op);
     fetch16(slot(b, T_UA), src + o + dym);
@@ -488,6 +522,7 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
   for (int z = z0; z < z1; ++z) {
     if (z + 1 < z1) fetch(b ^ 1, z + 1, o + plane);
     fetch_commit();
+    fetch_wait_previous();
     df acc[2];
     f2 D[2];
     {  // x: faces 0 .. 4 of the four cells, as pairs (0, 1), (2, 3) and 4
@@ -497,14 +532,14 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
       float hl = __shfl_up_sync(0xffffffffu, h23.y, 1), hr = __shfl_down_sync(0xffffffffu, h01.x, 1);
       float ll = __shfl_up_sync(0xffffffffu, l23.y, 1), lr = __shfl_down_sync(0xffffffffu, l01.x, 1);
       if (left_load) {
-        ul = ro1<NC>(src + o + dxl);
-        hl = __ldg(rhi + o + dxl);
-        ll = __ldg(rlo + o + dxl);
+        ul = *edge(b, 0, 0);
+        hl = *edge(b, 1, 0);
+        ll = *edge(b, 2, 0);
       }
       if (right_load) {
-        ur = ro1<NC>(src + o + dxr);
-        hr = __ldg(rhi + o + dxr);
-        lr = __ldg(rlo + o + dxr);
+        ur = *edge(b, 0, 1);
+        hr = *edge(b, 1, 1);
+        lr = *edge(b, 2, 1);
       }
       dface b01 = face_df(cf[0], df{pk(hl, h01.x), pk(ll, l01.x)}, r[0]);
       const dface b23 = face_df(cf[0], df{pk(h01.y, h23.x), pk(l01.y, l23.x)}, r[1]);
@@ -530,7 +565,6 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
         D[1] = add2(b23.h, pk(bh23.y, up2(b44.h).x));
       }
     }
-    fetch_wait_previous();
     ulonglong2 t = *slot(b, T_UP);
     const f2 un[2] = {t.x, t.y};
     t = *slot(b, T_HP);
@@ -607,15 +641,15 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
   part = active ? (FIXED ? (double)sumf : sum) : 0.0;
 }
 
-inline size_t density_smem(bool fixed, int threads) {
+inline size_t density_smem(bool fixed, int threads) {  // operand slots and x edges
   const int streams = fixed ? Streams<0>::kCount : Streams<2>::kCount;
-  return sizeof(ulonglong2) * (size_t)kStages * streams * threads;
+  return (sizeof(ulonglong2) * streams + 6 * sizeof(float)) * (size_t)kStages * threads;
 }
 
 constexpr int kDensity64Threads = kDirectThreads / 2;  // four cells per thread, the FP64 layout has two
 
 inline size_t density64_smem(int threads) {
-  return sizeof(ulonglong2) * (size_t)kStages * kStreams64 * threads;
+  return (sizeof(ulonglong2) * kStreams64 + 6 * sizeof(float)) * (size_t)kStages * threads;
 }
 
 }  // namespace vdp
