@@ -111,9 +111,10 @@ __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>())
   }
 }
 
-// Whether X+ of FP32 rows also runs on a persistent grid (measured at 512^3, see the X+ forms:
-// it does not; X+ of FP64 rows and X- always do).
-constexpr bool kXFwdF32Persistent = false;
+// Whether X+ of FP32 rows (nx = 2 m) also runs on a persistent grid, as X+ of FP64 rows and X- always
+// do: us a pass at 256^3 37 against 42, duct 256 x 128 x 128 (512-point rows aside) 24 against 26;
+// rows of 512 the other way round, 275 against 204 at 512^3 (80 registers: fewer loads in flight).
+constexpr bool x_fwd_f32_persistent(int m) { return m <= 128; }
 
 // ---- Y and Z: tiles of TX consecutive kx columns, whole lines -----------------------------------
 
@@ -334,7 +335,7 @@ SpecKernel x_kernel(int m, bool inverse, bool mirror, bool weight, int* threads)
     if (inverse)                                                                            \
       return mirror ? k_spec_x_inv_persistent<T, M1, M2, true, false>                       \
                     : k_spec_x_inv_persistent<T, M1, M2, false, false>;                     \
-    if constexpr (sizeof(T) == 8 || kXFwdF32Persistent)                                     \
+    if constexpr (sizeof(T) == 8 || x_fwd_f32_persistent(M1 * M2))                                   \
       return mirror ? k_spec_x_fwd_persistent<T, M1, M2, true>                              \
                     : k_spec_x_fwd_persistent<T, M1, M2, false>;                            \
     else                                                                                    \
@@ -419,7 +420,7 @@ long long x_grid(int prec, bool inv, const SpecArgs& a, long long rows) {
   const SpecKernel k = x_pass_kernel(prec, inv, a, &threads);
   const int dev = current_device(), ry = x_rows_per_block(a.nx / 2, inv);
   if (!k || dev < 0 || ry <= 0) return 0;
-  const bool persistent = inv || x_f64(prec, inv, a) || kXFwdF32Persistent;
+  const bool persistent = inv || x_f64(prec, inv, a) || x_fwd_f32_persistent(a.nx / 2);
   if (!persistent) return (rows + ry - 1) / ry;
   int per_sm = 0;
   for (const auto& e : g_x_per_sm[dev])
