@@ -3,8 +3,6 @@
 // X+ and X-, and the tile layout of the Y and Z lines.  Internal to libvdp.
 #pragma once
 
-#include <cmath>
-
 #include "vdp_device.cuh"
 #include "vdp_internal.cuh"
 #include "vdp_spectral.h"
@@ -12,19 +10,6 @@
 namespace vdp {
 
 // ---- complex arithmetic and small DFTs in registers ---------------------------------------------
-
-// exp(-2 pi i k / 96): the roots of unity of every register DFT size used here (all divide 96).
-static __constant__ float2 c_w96[96];  // filled in each translation unit by upload_roots()
-
-// c_w96 of this translation unit, on the current device
-static inline cudaError_t upload_roots() {
-  float2 w[96];
-  for (int k = 0; k < 96; ++k) {
-    const double ang = -2.0 * M_PI * (double)k / 96.0;
-    w[k] = make_float2((float)std::cos(ang), (float)std::sin(ang));
-  }
-  return cudaMemcpyToSymbol(c_w96, w, sizeof(w));
-}
 
 // Complex sums, differences and real scalings as one paired FP32 instruction (add / sub / mul
 // .rn.f32x2: both lanes rounded as the scalar operation would round them); the FFT butterflies
@@ -57,8 +42,31 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
 }
 
+// exp(-2 pi i k / 96), 0 <= k < 96: the roots of unity of every register DFT size used here (all
+// divide 96).  k is a constant after unrolling, so each root is an immediate operand (from a table in
+// constant memory the Z pass ran 128^3 in 13.1 us instead of 12.5).
+__device__ __forceinline__ float quarter_cos(int j) {  // cos(2 pi j / 96), j = 0 .. 24
+  switch (j) {
+    case 0: return 1.0f; case 1: return 0.997858942f; case 2: return 0.991444886f;
+    case 3: return 0.980785251f; case 4: return 0.965925813f; case 5: return 0.94693011f;
+    case 6: return 0.923879504f; case 7: return 0.896872759f; case 8: return 0.866025388f;
+    case 9: return 0.831469595f; case 10: return 0.793353319f; case 11: return 0.751839817f;
+    case 12: return 0.707106769f; case 13: return 0.659345806f; case 14: return 0.60876143f;
+    case 15: return 0.555570245f; case 16: return 0.5f; case 17: return 0.442288697f;
+    case 18: return 0.382683426f; case 19: return 0.321439475f; case 20: return 0.258819044f;
+    case 21: return 0.195090324f; case 22: return 0.130526185f; case 23: return 0.0654031262f;
+    case 24: return 0.0f;
+  }
+  return 0.f;
+}
+__device__ __forceinline__ float cos96(int k) {
+  const int j = k > 48 ? 96 - k : k;
+  return j <= 24 ? quarter_cos(j) : -quarter_cos(48 - j);
+}
+__device__ __forceinline__ float2 root96(int k) { return make_float2(cos96(k), -cos96((k + 72) % 96)); }
+
 // v * W_M^k with W = exp(-2 pi i / M) (INV: the conjugate root).  k and M are constants after
-// unrolling, so the trivial roots cost nothing and the others are constant-bank operands.
+// unrolling, so the trivial roots cost nothing and the others are immediates.
 template <bool INV>
 __device__ __forceinline__ float2 rot(float2 v, int k, int M) {
   k %= M;
@@ -66,7 +74,7 @@ __device__ __forceinline__ float2 rot(float2 v, int k, int M) {
   if (2 * k == M) return make_float2(-v.x, -v.y);
   if (4 * k == M) return INV ? make_float2(-v.y, v.x) : make_float2(v.y, -v.x);
   if (4 * k == 3 * M) return INV ? make_float2(v.y, -v.x) : make_float2(-v.y, v.x);
-  const float2 w = c_w96[(96 / M) * k];
+  const float2 w = root96((96 / M) * k);
   return cmul(v, INV ? cconj(w) : w);
 }
 
@@ -204,20 +212,31 @@ constexpr int inv_rows_per_block() {
 template <int M1>
 __device__ __forceinline__ int ex(int k2, int j1) { return k2 * (M1 + 1) + j1; }
 
+// 16-byte asynchronous copy global -> shared (cached in L2 only), and its group wait: the copies
+// hold no registers while in flight, so a block can fetch its next tile while it finishes this
+// one.  wait_group is a hardware wait for this thread's own copies (no spin loop).
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 // ---- X+ : real rows -> half spectrum -----------------------------------------------------------
 
 // The X+ transform of RY rows (one per group of M1 threads: t = lane in the row, r = row in the
 // group), row `row` of the grid in thread group r; `ra` is the row's shared buffer of SX values
-// (the exchange, then the transformed row).  store(k, X) receives bin k of the row's half
-// spectrum for k < nxp (zero beyond nx/2).  Every thread of the block calls it (barriers).
-template <class T, int M1, int M2, bool MIRROR, class Store>
-__device__ __forceinline__ void x_fwd_rows(const SpecArgs& a, const Tables& tb, float2* ra,
-                                           long long row, bool live, int t, Store&& store) {
+// (the exchange, then the transformed row); `in` its cells (global or shared memory).  store(k, X)
+// receives bin k of the row's half spectrum for k < nxp (zero beyond nx/2); read() is called once
+// every thread of the block has read its part of `in`.  Every thread of the block calls it
+// (barriers).
+template <class T, int M1, int M2, bool MIRROR, class Store, class Read>
+__device__ __forceinline__ void x_fwd_rows(const SpecArgs& a, const Tables& tb, float2* ra, const T* in,
+                                           long long row, bool live, int t, Store&& store, Read&& read) {
   constexpr int m = M1 * M2;
   float2* rb = ra;
   // step A: M2-point DFTs over j2 of z[t + M1 j2] = (x[2j], x[2j+1]) * W
   if (live) {
-    const T* in = static_cast<const T*>(a.in) + row * a.nxd;
     const float* om = a.omega_in ? a.omega_in + row * a.nxd : nullptr;
     float2 v[M2], y[M2];
 #pragma unroll
@@ -240,6 +259,7 @@ __device__ __forceinline__ void x_fwd_rows(const SpecArgs& a, const Tables& tb, 
       ra[ex<M1>(k2, t)] = k2 == 0 || t == 0 ? y[k2] : cmul(y[k2], tb.wm[t * k2]);
   }
   __syncthreads();
+  read();
   // step B: M1-point DFTs over j1 -> Z[k2 + M2 k1]; the exchange is read completely before the
   // transformed row overwrites it
   constexpr int R = (M2 + M1 - 1) / M1;
@@ -268,19 +288,20 @@ __device__ __forceinline__ void x_fwd_rows(const SpecArgs& a, const Tables& tb, 
     }
   }
   __syncthreads();
-  // unpack: X[k] = E[k] + W_nx^k O[k], E = (Z[k] + conj Z[m-k]) / 2, O = (Z[k] - conj Z[m-k]) / 2i
+  // unpack: X[k] = E + W_nx^k O, X[m - k] = conj(E - W_nx^k O) with E = (Z[k] + conj Z[m-k]) / 2,
+  // O = (Z[k] - conj Z[m-k]) / 2i: both bins of a pair from one pair of values
   if (live) {
-    for (int k = t; k < a.nxp; k += M1) {
-      float2 X = make_float2(0.f, 0.f);
-      if (k <= m) {
-        const float2 p = rb[k == m ? 0 : k], q = cconj(rb[k == 0 ? 0 : m - k]);
-        const float2 e = cscale(cadd(p, q), 0.5f);
-        const float2 d = csub(p, q);
-        const float2 o = make_float2(0.5f * d.y, -0.5f * d.x);
-        X = cadd(e, cmul(tb.wr[k], o));
-      }
-      store(k, X);
-    }
+    auto bins = [&](int k) {
+      const float2 p = rb[k], q = cconj(rb[k == 0 ? 0 : m - k]);
+      const float2 e = cscale(cadd(p, q), 0.5f), d = cscale(csub(p, q), 0.5f);
+      const float2 o = cmul(tb.wr[k], make_float2(d.y, -d.x));
+      store(k, cadd(e, o));
+      if (k != m / 2) store(m - k, cconj(csub(e, o)));
+    };
+#pragma unroll
+    for (int i = 0; i < M2 / 2; ++i) bins(t + M1 * i);
+    if (t == 0) bins(m / 2);
+    for (int k = m + 1 + t; k < a.nxp; k += M1) store(k, make_float2(0.f, 0.f));
   }
 }
 
@@ -301,10 +322,12 @@ __device__ __forceinline__ Tables x_tables_shared(const SpecArgs& a, float2* st)
 
 // The X- transform of one row per group of M1 threads: `src` is the row of the half spectrum
 // (global or shared memory), `rb` the group's shared exchange buffer; z = W x is stored to row
-// `row` of a.out.  Every thread of the block calls it (barrier).
-template <class T, int M1, int M2, bool MIRROR, bool WEIGHT>
+// `row` of a.out; read() is called once every thread of the block has read its part of src.
+// Every thread of the block calls it (barrier).
+template <class T, int M1, int M2, bool MIRROR, bool WEIGHT, class Read>
 __device__ __forceinline__ void x_inv_rows(const SpecArgs& a, const Tables& tb, float2* rb,
-                                           const float2* src, long long row, bool live, int t) {
+                                           const float2* src, long long row, bool live, int t,
+                                           Read&& read) {
   constexpr int m = M1 * M2;
   // the output weights of this thread's cells are loaded first, so that their latency overlaps
   // the transforms (cells 2l, 2l + 1 with l = k2 + M2 k1, k2 = t, t + M1, ...)
@@ -349,6 +372,7 @@ __device__ __forceinline__ void x_inv_rows(const SpecArgs& a, const Tables& tb, 
       rb[ex<M1>(k2, t)] = k2 == 0 || t == 0 ? y[k2] : cmulc(y[k2], tb.wm[t * k2]);
   }
   __syncthreads();
+  read();
   if (live) {
     T* out = static_cast<T*>(a.out) + row * a.nxd;
 #pragma unroll
@@ -380,16 +404,6 @@ template <int G>
 __device__ __forceinline__ int tx(int group, int e, int c) {
   return group * pad_stride(G * kTX) + e * kTX + c;
 }
-
-// 16-byte asynchronous copy global -> shared (cached in L2 only), and its group wait: the copies
-// hold no registers while in flight, so a block can fetch its next tile while it finishes this
-// one.  wait_group is a hardware wait for this thread's own copies (no spin loop).
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // Tiles of the Y and Z passes: nz (or ny) line elements of kTX columns.  Element e = t + M1 j2 of
 // column c is copied to slot (j2, t, c) of the tile buffer, the layout step A reads; step A

@@ -279,7 +279,7 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
   }
   if (zc > nz) zc = nz;
   if (zc < 1) zc = 1;
-  long long nf = ncell / 4096;
+  long long nf = ncell / 8192;
   const long long nf_small = ncell / 1024 < 2LL * kSMs ? ncell / 1024 : 2LL * kSMs;
   if (nf < nf_small) nf = nf_small;
   if (nf > kSMs * 8) nf = kSMs * 8;

@@ -95,8 +95,9 @@ __device__ __noinline__ void x_forward(const SpecArgs& a, const Tables& tb, floa
     const long long row = (long long)g * per + r;
     const bool live = r < per && row < rows;
     float2* out = a.spec + row * a.nxp;
-    x_fwd_rows<float, M1, M2, true>(a, tb, buf + (r < RY ? r : 0) * SX, row, live, t,
-                                  [&](int k, float2 X) { out[k] = X; });
+    x_fwd_rows<float, M1, M2, true>(a, tb, buf + (r < RY ? r : 0) * SX,
+                                  static_cast<const float*>(a.in) + row * a.nxd, row, live, t,
+                                  [&](int k, float2 X) { out[k] = X; }, [] {});
     __syncthreads();
   }
 }
@@ -110,7 +111,7 @@ __device__ __noinline__ void x_inverse(const SpecArgs& a, const Tables& tb, floa
     const long long row = (long long)g * per + r;
     const bool live = r < per && row < rows;
     x_inv_rows<float, M1, M2, true, false>(a, tb, buf + (r < RY ? r : 0) * SB,
-                                             a.spec + (live ? row : 0) * a.nxp, row, live, t);
+                                             a.spec + (live ? row : 0) * a.nxp, row, live, t, [] {});
     __syncthreads();
   }
 }
@@ -513,7 +514,6 @@ cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, c
     std::lock_guard<std::mutex> lk(mu);
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (sms[dev] == 0) {
-      if ((e = upload_roots()) != cudaSuccess) return e;
       for (int p : {PREC_FP64, PREC_MIXED})
         for (int q : {R_FIXED, R_SPECTRAL})
           if ((e = cudaFuncSetAttribute((const void*)resident_kernel(p, q),

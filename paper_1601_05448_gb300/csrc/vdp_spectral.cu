@@ -40,28 +40,10 @@
 
 namespace vdp {
 
-// X+ of FP32 rows: one group of RY rows per block, tables read through L1.  The 512^3 mixed solve
-// takes 33.6 ms with it against 34.4 ms with the persistent form below for FP32 rows too (whose
-// loop needs 80 registers: one block per SM less for the loads in flight).
-template <class T, int M1, int M2, bool MIRROR>
-__global__ void __launch_bounds__(M1 * rows_per_block<M1, M2>(), 1024 / (M1 * rows_per_block<M1, M2>()))
-    k_spec_x_fwd(SpecArgs a) {
-  constexpr int RY = rows_per_block<M1, M2>();
-  constexpr int SX = x_row_stride<M1, M2>();
-  __shared__ float2 sx[RY * SX];  // per row: the exchange, then the transformed row
-  if (!spec_active(a)) return;
-  const Tables tb = tables(a);
-  const int t = threadIdx.x % M1, r = threadIdx.x / M1;
-  const long long row = (long long)a.z0 * a.ny + (long long)blockIdx.x * RY + r;
-  const bool live = row < (long long)a.z1 * a.ny;
-  float2* out = a.spec + row * a.nxp;
-  x_fwd_rows<T, M1, M2, MIRROR>(a, tb, sx + r * SX, row, live, t,
-                                 [&](int k, float2 X) { out[k] = X; });
-}
-
 // X+ of FP64 rows on a persistent grid: groups of RY rows (group = block, block + grid, ...) of
 // the planes [z0, z1), tables in shared memory; at least 768 resident threads per SM (80
-// registers a thread).  The 512^3 FP64 solve: 47.3 ms against 49.2 ms with the form above.
+// registers a thread).  The 512^3 FP64 solve: 47.3 ms against 49.2 ms with one group of rows
+// per block and the tables read through L1.
 template <class T, int M1, int M2, bool MIRROR>
 __global__ void __launch_bounds__(M1 * rows_per_block<M1, M2>(), 768 / (M1 * rows_per_block<M1, M2>()))
     k_spec_x_fwd_persistent(SpecArgs a) {
@@ -77,9 +59,47 @@ __global__ void __launch_bounds__(M1 * rows_per_block<M1, M2>(), 768 / (M1 * row
     const long long row = (long long)a.z0 * a.ny + g * RY + r;
     const bool live = g * RY + r < rows;
     float2* out = a.spec + row * a.nxp;
-    x_fwd_rows<T, M1, M2, MIRROR>(a, tb, sx + r * SX, row, live, t,
-                                   [&](int k, float2 X) { out[k] = X; });
+    x_fwd_rows<T, M1, M2, MIRROR>(a, tb, sx + r * SX, static_cast<const T*>(a.in) + row * a.nxd, row, live,
+                                   t, [&](int k, float2 X) { out[k] = X; }, [] {});
     __syncthreads();  // the row buffers are reused by the next group
+  }
+}
+
+// X+ of FP32 rows on a persistent grid, the group's rows copied to shared memory while the group
+// before is transformed.
+template <int M1, int M2, bool MIRROR>
+__global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>()) k_spec_x_fwd_staged(SpecArgs a) {
+  constexpr int RY = inv_rows_per_block<M1, M2>();
+  constexpr int SX = x_row_stride<M1, M2>();
+  constexpr int m = M1 * M2, SR = pad_stride(m);
+  __shared__ float2 sx[RY * SX];                // per row: the exchange, then the transformed row
+  __shared__ __align__(16) float2 sr[RY * SR];  // the group's rows, fetched ahead
+  __shared__ float2 stab[2 * m + 1];
+  const long long rows = (long long)(a.z1 - a.z0) * a.ny, first = (long long)a.z0 * a.ny;
+  const int pieces = a.nxd / 4;
+  auto fetch = [&](long long g) {
+    const int n = (int)(rows - g * RY < RY ? rows - g * RY : RY);
+    const float* src = static_cast<const float*>(a.in) + (first + g * RY) * a.nxd;
+    for (int q = threadIdx.x; q < n * pieces; q += M1 * RY) {  // the rows follow one another
+      const int r = q / pieces;
+      cp_async16(sr + r * SR + 2 * (q - r * pieces), src + 4 * (long long)q);
+    }
+    cp_async_commit();
+  };
+  long long g = blockIdx.x;
+  if (g * RY < rows) fetch(g);
+  const Tables tb = x_tables_shared<M1, M2>(a, stab);
+  if (!spec_active(a)) return cp_async_wait_all();
+  const int t = threadIdx.x % M1, r = threadIdx.x / M1;
+  for (; g * RY < rows; g += gridDim.x) {
+    const long long row = first + g * RY + r;
+    float2* out = a.spec + row * a.nxp;
+    cp_async_wait_all();
+    __syncthreads();  // the rows are there, and the row buffers of the group before have been read
+    x_fwd_rows<float, M1, M2, MIRROR>(
+        a, tb, sx + r * SX, reinterpret_cast<const float*>(sr + r * SR), row, g * RY + r < rows, t,
+        [&](int k, float2 X) { out[k] = X; },
+        [&] { if ((g + gridDim.x) * RY < rows) fetch(g + gridDim.x); });
   }
 }
 
@@ -92,17 +112,31 @@ __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>())
     k_spec_x_inv_persistent(SpecArgs a) {
   constexpr int RY = inv_rows_per_block<M1, M2>();
   constexpr int SB = pad_stride(M2 * (M1 + 1));
-  __shared__ float2 sb[RY * SB];
-  __shared__ float2 stab[2 * M1 * M2 + 1];
-  if (!spec_active(a)) return;
+  constexpr int m = M1 * M2, SR = pad_stride(m + 1), kPieces = m / 2 + 1;
+  __shared__ float2 sb[RY * SB];                 // the exchange
+  __shared__ __align__(16) float2 sr[RY * SR];   // the group's rows, fetched ahead
+  __shared__ float2 stab[2 * m + 1];
+  const long long rows = (long long)(a.z1 - a.z0) * a.ny, first = (long long)a.z0 * a.ny;
+  auto fetch = [&](long long g) {
+    const int n = (int)(rows - g * RY < RY ? rows - g * RY : RY);
+    const float2* src = a.spec + (first + g * RY) * a.nxp;
+    for (int q = threadIdx.x; q < n * kPieces; q += M1 * RY) {
+      const int r = q / kPieces, p = 2 * (q - r * kPieces);
+      cp_async16(sr + r * SR + p, src + (long long)r * a.nxp + p);
+    }
+    cp_async_commit();
+  };
+  long long g = blockIdx.x;
+  if (g * RY < rows) fetch(g);
   const Tables tb = x_tables_shared<M1, M2>(a, stab);
+  if (!spec_active(a)) return cp_async_wait_all();
   const int t = threadIdx.x % M1, r = threadIdx.x / M1;
-  const long long rows = (long long)(a.z1 - a.z0) * a.ny;
-  for (long long g = blockIdx.x; g * RY < rows; g += gridDim.x) {
-    const long long row = (long long)a.z0 * a.ny + g * RY + r;
+  for (; g * RY < rows; g += gridDim.x) {
+    cp_async_wait_all();
+    __syncthreads();  // the rows are there, and the exchange of the group before has been read
     const bool live = g * RY + r < rows;
-    x_inv_rows<T, M1, M2, MIRROR, WEIGHT>(a, tb, sb + r * SB, a.spec + row * a.nxp, row, live, t);
-    __syncthreads();  // the exchange buffers are reused by the next group
+    x_inv_rows<T, M1, M2, MIRROR, WEIGHT>(a, tb, sb + r * SB, sr + r * SR, first + g * RY + r, live, t,
+                                            [&] { if ((g + gridDim.x) * RY < rows) fetch(g + gridDim.x); });
   }
   if (a.st) {  // the solve: the last block of the application's X- launches completes the
                // preconditioner sweep, with <rt, z> from the partial sums the Z pass stored
@@ -110,11 +144,6 @@ __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>())
     finish_sweep(I, I.st, PH_SPEC, a.xunits, a.zunits);
   }
 }
-
-// Whether X+ of FP32 rows (nx = 2 m) also runs on a persistent grid, as X+ of FP64 rows and X- always
-// do: us a pass at 256^3 37 against 42, duct 256 x 128 x 128 (512-point rows aside) 24 against 26;
-// rows of 512 the other way round, 275 against 204 at 512^3 (80 registers: fewer loads in flight).
-constexpr bool x_fwd_f32_persistent(int m) { return m <= 128; }
 
 // ---- Y and Z: tiles of TX consecutive kx columns, whole lines -----------------------------------
 
@@ -142,7 +171,6 @@ __global__ void __launch_bounds__(M1 * kTX, LineOcc<M1>::kMinBlocks) k_spec_y(Sp
   extern __shared__ __align__(16) float2 ybuf[];
   float2* sm = ybuf;                          // the tile
   float2* wy = ybuf + line_buffer<M1, M2>();  // W_ny^k, k < ny
-  if (!spec_active(a)) return;
   const Tables tb = tables(a);
   const int c = threadIdx.x % kTX, t = threadIdx.x / kTX;
   const int tiles = a.nxp / kTX;
@@ -154,6 +182,7 @@ __global__ void __launch_bounds__(M1 * kTX, LineOcc<M1>::kMinBlocks) k_spec_y(Sp
   int tile = blockIdx.x;
   if (tile < ntile) fetch_tile<M1, M2>(sm, base(tile), es);
   for (int k = threadIdx.x; k < n; k += M1 * kTX) wy[k] = tb.wy[k];
+  if (!spec_active(a)) return cp_async_wait_all();
   for (; tile < ntile; tile += gridDim.x) {
     cp_async_wait_all();  // this thread's copies of the tile have landed
     __syncthreads();      // ... and every other thread's (and the twiddles are in place)
@@ -222,7 +251,6 @@ __global__ void __launch_bounds__(M1 * kTX, ZOcc<M1>::kMinBlocks) k_spec_z(SpecA
   float2* sm = zbuf;                         // the tile
   float2* wz = zbuf + line_buffer<M1, M2>();  // W_nz^k, k < nz
   float* lz = reinterpret_cast<float*>(wz + n);
-  if (!spec_active(a)) return;
   const Tables tb = tables(a);
   const int c = threadIdx.x % kTX, t = threadIdx.x / kTX;
   const int tiles = a.nxp / kTX;
@@ -238,6 +266,7 @@ __global__ void __launch_bounds__(M1 * kTX, ZOcc<M1>::kMinBlocks) k_spec_z(SpecA
     wz[k] = tb.wz[k];
     lz[k] = tb.lz[k];
   }
+  if (!spec_active(a)) return cp_async_wait_all();
   double energy_sum = 0.0;
   for (; tile < ntile; tile += gridDim.x) {
     cp_async_wait_all();  // this thread's copies of the tile have landed
@@ -328,18 +357,19 @@ SpecKernel x_kernel(int m, bool inverse, bool mirror, bool weight, int* threads)
   factor(m, &m1, &m2);
 #define VDP_X(M1, M2)                                                                       \
   if (m1 == M1 && m2 == M2) {                                                               \
-    *threads = M1 * (inverse ? inv_rows_per_block<M1, M2>() : rows_per_block<M1, M2>());     \
+    *threads = M1 * (inverse || sizeof(T) == 4 ? inv_rows_per_block<M1, M2>()                \
+                                               : rows_per_block<M1, M2>());                  \
     if (inverse && weight)                                                                  \
       return mirror ? k_spec_x_inv_persistent<T, M1, M2, true, true>                        \
                     : k_spec_x_inv_persistent<T, M1, M2, false, true>;                      \
     if (inverse)                                                                            \
       return mirror ? k_spec_x_inv_persistent<T, M1, M2, true, false>                       \
                     : k_spec_x_inv_persistent<T, M1, M2, false, false>;                     \
-    if constexpr (sizeof(T) == 8 || x_fwd_f32_persistent(M1 * M2))                                   \
+    if constexpr (sizeof(T) == 8)                                                           \
       return mirror ? k_spec_x_fwd_persistent<T, M1, M2, true>                              \
                     : k_spec_x_fwd_persistent<T, M1, M2, false>;                            \
     else                                                                                    \
-      return mirror ? k_spec_x_fwd<T, M1, M2, true> : k_spec_x_fwd<T, M1, M2, false>;     \
+      return mirror ? k_spec_x_fwd_staged<M1, M2, true> : k_spec_x_fwd_staged<M1, M2, false>; \
   }
   VDP_X(4, 4) VDP_X(4, 6) VDP_X(4, 8) VDP_X(6, 8) VDP_X(8, 8) VDP_X(8, 12) VDP_X(8, 16)
   VDP_X(16, 16)
@@ -347,11 +377,11 @@ SpecKernel x_kernel(int m, bool inverse, bool mirror, bool weight, int* threads)
   return nullptr;
 }
 
-int x_rows_per_block(int m, bool inverse) {
+int x_rows_per_block(int m, bool half) {
   int m1, m2;
   factor(m, &m1, &m2);
 #define VDP_R(M1, M2) \
-  if (m1 == M1 && m2 == M2) return inverse ? inv_rows_per_block<M1, M2>() : rows_per_block<M1, M2>();
+  if (m1 == M1 && m2 == M2) return half ? inv_rows_per_block<M1, M2>() : rows_per_block<M1, M2>();
   VDP_R(4, 4) VDP_R(4, 6) VDP_R(4, 8) VDP_R(6, 8) VDP_R(8, 8) VDP_R(8, 12) VDP_R(8, 16)
   VDP_R(16, 16)
 #undef VDP_R
@@ -418,10 +448,8 @@ SpecKernel x_pass_kernel(int prec, bool inv, const SpecArgs& a, int* threads) {
 long long x_grid(int prec, bool inv, const SpecArgs& a, long long rows) {
   int threads = 0;
   const SpecKernel k = x_pass_kernel(prec, inv, a, &threads);
-  const int dev = current_device(), ry = x_rows_per_block(a.nx / 2, inv);
+  const int dev = current_device(), ry = x_rows_per_block(a.nx / 2, inv || !x_f64(prec, inv, a));
   if (!k || dev < 0 || ry <= 0) return 0;
-  const bool persistent = inv || x_f64(prec, inv, a) || x_fwd_f32_persistent(a.nx / 2);
-  if (!persistent) return (rows + ry - 1) / ry;
   int per_sm = 0;
   for (const auto& e : g_x_per_sm[dev])
     if (e.first == k) per_sm = e.second;
@@ -491,9 +519,9 @@ void spectral_tables(int nx, int ny, int nz, double hx, double hy, double hz,
 }
 
 cudaError_t spectral_upload_roots() {
-  cudaError_t e = upload_roots();
+  cudaError_t e = cudaSuccess;
   const int dev = current_device();
-  if (e == cudaSuccess && dev < 0) e = cudaErrorInvalidDevice;
+  if (dev < 0) e = cudaErrorInvalidDevice;
   // the Y and Z passes' tile buffer and tables: dynamic shared memory (37 and 41 KB for lines
   // of 512), then the resident blocks per SM that size their persistent grids
   for (int which = 0; which < 3 && e == cudaSuccess; ++which)
