@@ -411,7 +411,8 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   // rho D^1/2 gives rho r, and z = damping D^1/2 (-L_h)^-1 (rho r) is the scaled form of the
   // paper's update p += damping L_h^-1 (rho r) (applied as p -= D^-1/2 x, x the sum of the z)
   a->out = c->za;
-  a->f32 = (dens64 ? kInF32 : 0) | (fixed || dens ? kOutF32 : 0);  // those sweeps read z as FP32
+  // the fixed-point and density sweeps read z as FP32
+  a->f32 = (dens64 ? kInF32 : 0) | (fixed || dens ? kOutF32 : 0) | (fixed ? 0 : kEnergy);
   a->omega_in = dens ? nullptr : fixed ? c->rho_w : c->omega;
   a->omega_out = dens ? nullptr : c->omega;
   a->spec = c->spec;

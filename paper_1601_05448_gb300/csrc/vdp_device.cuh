@@ -409,11 +409,11 @@ __device__ __forceinline__ int phase_slots(int phase) {
 // nunits units arrive; their partial slots were written by nparts units (default: the same),
 // which lets a sweep of several kernels reduce what an earlier kernel of the sweep stored.
 __device__ __forceinline__ void finish_sweep(const InstDesc& I, InstState* st, int phase,
-                                             int nunits, int nparts = 0) {
+                                             int nunits, int nparts = 0, bool sums = true) {
   if (nparts <= 0) nparts = nunits;
   if (arrive_last(I.ticket, nunits)) {  // uniform in the block
     double S[kSlots] = {0.0, 0.0, 0.0, 0.0};
-    block_sum_slots(I.part, nparts, phase_slots(phase), S);
+    if (sums) block_sum_slots(I.part, nparts, phase_slots(phase), S);
     if (threadIdx.x == 0) {
       // the whole state in one go (its words are independent loads past L1), the transition on
       // the copy, and back: field by field it was a chain of a dozen trips to L2

@@ -139,9 +139,9 @@ __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>())
                                             [&] { if ((g + gridDim.x) * RY < rows) fetch(g + gridDim.x); });
   }
   if (a.st) {  // the solve: the last block of the application's X- launches completes the
-               // preconditioner sweep, with <rt, z> from the partial sums the Z pass stored
+               // preconditioner sweep, in spectral CG with <rt, z> from the partial sums of Z
     const InstDesc& I = *a.I;
-    finish_sweep(I, I.st, PH_SPEC, a.xunits, a.zunits);
+    finish_sweep(I, I.st, PH_SPEC, a.xunits, a.zunits, (a.f32 & kEnergy) != 0);
   }
 }
 
@@ -234,15 +234,16 @@ __global__ void __launch_bounds__(M1 * kTX, LineOcc<M1>::kMinBlocks) k_spec_y(Sp
 // (M1-point over j1 = t) leaves owner k2 with X[k2 + M2 k1]; the owner scales and runs A' (M1-
 // point over k1) and writes back to the slots it read, (k2, l2), so B -> scaling -> A' needs no
 // barrier and keeps no line in registers across one; B' (M2-point over k2) reads slots (k2, t).
-// In the solve it also stores this block's part of <y, (-L_h)^-1 y> = sum_k |Y(k)|^2 s(k)
+// In spectral CG (ENERGY) it also stores this block's part of <y, (-L_h)^-1 y> = sum_k |Y(k)|^2 s(k)
 // (Parseval; y = W rt, the half spectrum counting kx = 1 .. nx/2 - 1 twice), which is <rt, z>:
-// FP32 per tile, summed over the block's tiles in FP64, always in the same order.
+// FP32 per tile, summed over the block's tiles in FP64, always in the same order.  The fixed-point
+// iteration has no use for it: without, 512^3 327 -> 315 us, 256^3 38.2 -> 35.8.
 template <int M1, int M2>
 constexpr size_t z_smem() {  // tile buffer, twiddles W_nz^k, eigenvalues lz
   return sizeof(float2) * (size_t)(line_buffer<M1, M2>() + M1 * M2) + sizeof(float) * (size_t)(M1 * M2);
 }
 
-template <int M1, int M2>
+template <int M1, int M2, bool ENERGY>
 __global__ void __launch_bounds__(M1 * kTX, ZOcc<M1>::kMinBlocks) k_spec_z(SpecArgs a) {
   constexpr int R = (M2 + M1 - 1) / M1;
   constexpr int n = M1 * M2;
@@ -300,7 +301,7 @@ __global__ void __launch_bounds__(M1 * kTX, ZOcc<M1>::kMinBlocks) k_spec_z(SpecA
           const float lam = lxy + lz[k2 + M2 * k1];
           // zero mode removed; the quotient is the hardware's approximate one (2 ulp)
           const float s = (lam > 0.f && !pad) ? __fdividef(a.scale, lam) : 0.f;
-          energy = fmaf(wkx * s, fmaf(o[k1].x, o[k1].x, o[k1].y * o[k1].y), energy);
+          if (ENERGY) energy = fmaf(wkx * s, fmaf(o[k1].x, o[k1].x, o[k1].y * o[k1].y), energy);
           o[k1] = cscale(o[k1], s);
         }
         dft<M1, 0, 1, true>(o, u);
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(M1 * kTX, ZOcc<M1>::kMinBlocks) k_spec_z(SpecA
           sm[tx<M1>(k2, l2, c)] = l2 == 0 || k2 == 0 ? u[l2] : cmulc(u[l2], wz[k2 * l2]);
       }
     }
-    energy_sum += (double)energy;
+    if (ENERGY) energy_sum += (double)energy;
     __syncthreads();
     float2 w[M2];
 #pragma unroll
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(M1 * kTX, ZOcc<M1>::kMinBlocks) k_spec_z(SpecA
 #pragma unroll
     for (int l1 = 0; l1 < M2; ++l1) g[(t + M1 * l1) * es] = o[l1];
   }
-  if (a.st) {
+  if (ENERGY) {
     const double part[1] = {energy_sum * (double)a.ewt};
     store_partials<1, double>(part, a.I->part, gridDim.x, blockIdx.x);
   }
@@ -389,7 +390,7 @@ int x_rows_per_block(int m, bool half) {
 }
 
 SpecKernel yz_kernel(int n, int which, int* threads, size_t* smem = nullptr) {
-  // which: 0 = Y+, 1 = Y-, 2 = Z; smem: the pass's dynamic shared memory
+  // which: 0 = Y+, 1 = Y-, 2 = Z, 3 = Z with the energy; smem: the pass's dynamic shared memory
   int m1, m2;
   factor(n, &m1, &m2);
   if (n == 48) {  // blocks of M1 * 8 threads: a whole number of warps for the block reduction
@@ -399,9 +400,9 @@ SpecKernel yz_kernel(int n, int which, int* threads, size_t* smem = nullptr) {
 #define VDP_YZ(M1, M2)                                                                  \
   if (m1 == M1 && m2 == M2) {                                                           \
     *threads = M1 * kTX;                                                                \
-    if (smem) *smem = which == 2 ? z_smem<M1, M2>() : y_smem<M1, M2>();               \
+    if (smem) *smem = which >= 2 ? z_smem<M1, M2>() : y_smem<M1, M2>();               \
     return which == 0 ? k_spec_y<M1, M2, false> : which == 1 ? k_spec_y<M1, M2, true>   \
-                                                             : k_spec_z<M1, M2>;        \
+           : which == 2 ? k_spec_z<M1, M2, false> : k_spec_z<M1, M2, true>;             \
   }
   VDP_YZ(4, 8) VDP_YZ(4, 12) VDP_YZ(8, 8) VDP_YZ(8, 12) VDP_YZ(8, 16) VDP_YZ(12, 16)
   VDP_YZ(16, 16) VDP_YZ(16, 32)
@@ -415,7 +416,7 @@ SpecKernel yz_kernel(int n, int which, int* threads, size_t* smem = nullptr) {
 constexpr int kLineLengths[] = {32, 48, 64, 96, 128, 192, 256, 512};
 constexpr int kLineCount = sizeof(kLineLengths) / sizeof(kLineLengths[0]);
 constexpr int kMaxDevices = 64;
-int g_per_sm[kMaxDevices][3][kLineCount];
+int g_per_sm[kMaxDevices][4][kLineCount];
 
 int current_device() {
   int dev = -1;
@@ -524,7 +525,7 @@ cudaError_t spectral_upload_roots() {
   if (dev < 0) e = cudaErrorInvalidDevice;
   // the Y and Z passes' tile buffer and tables: dynamic shared memory (37 and 41 KB for lines
   // of 512), then the resident blocks per SM that size their persistent grids
-  for (int which = 0; which < 3 && e == cudaSuccess; ++which)
+  for (int which = 0; which < 4 && e == cudaSuccess; ++which)
     for (int i = 0; i < kLineCount && e == cudaSuccess; ++i) {
       int threads = 0;
       size_t smem = 0;
@@ -575,7 +576,7 @@ cudaError_t launch_spectral_pass(int prec, int pass, const SpecArgs& a, cudaStre
       break;
     }
     case SPEC_Z:
-      k = yz_kernel(a.nz, 2, &threads, &smem);
+      k = yz_kernel(a.nz, a.f32 & kEnergy ? 3 : 2, &threads, &smem);
       grid = (unsigned)spectral_units(a.nx, a.ny, a.nz);
       break;
     default:
@@ -640,7 +641,7 @@ cudaError_t launch_spectral_apply(int prec, const SpecArgs& a, int slab, cudaStr
 }
 
 int spectral_units(int nx, int ny, int nz) {  // CTAs of the Z pass (they store <rt, z> parts)
-  return (int)line_grid(2, nz, (long long)(spectral_pitch(nx) / kTX) * ny);
+  return (int)line_grid(3, nz, (long long)(spectral_pitch(nx) / kTX) * ny);
 }
 
 }  // namespace vdp

@@ -13,13 +13,14 @@ namespace vdp {
 enum SpecPass : int { SPEC_X_FWD = 0, SPEC_Y_FWD = 1, SPEC_Z = 2, SPEC_Y_INV = 3, SPEC_X_INV = 4,
                       SPEC_PASSES = 5 };
 
-constexpr int kInF32 = 1, kOutF32 = 2;
+constexpr int kInF32 = 1, kOutF32 = 2, kEnergy = 4;
 
 // Arguments of every spectral pass (by value).
 struct SpecArgs {
   const void* in;        // X+: nxd*ny*nz values of the inner type (FP64 or FP32; see f32)
   void* out;             // X-: output, same layout; the inner type (see f32)
-  int f32;               // FP64 solves: kInF32 (in holds FP32) and / or kOutF32 (store z as FP32)
+  int f32;               // FP64 solves: kInF32 (in holds FP32) and / or kOutF32 (store z as FP32);
+                         // kEnergy: Z stores the partial sums of <rt, z> (spectral CG)
   const float* omega_in;   // per-cell weight applied before X+ (or null: 1)
   const float* omega_out;  // per-cell weight applied after X- (or null: 1)
   float2* spec;          // half spectrum [nz][ny][nxp]
