@@ -72,15 +72,34 @@ L2_BYTES = 129e6
 #   spec_x : X+ reads rt, W, writes S; X- reads S, W, rt, writes z   -> (3T + 8 + 2S) / 2 per launch
 #   spec_y : read and write S                                        -> 2S
 #   spec_z : read and write S (forward FFT, division, inverse FFT)   -> 2S
+#   Density form (dens; mixed and FP64 solves by the spectral inverse whose density was set after the
+#   options): unscaled variables, coefficients computed in the sweep from an FP32 density (FP64 solve:
+#   a pair of FP32 numbers), no weights:
+#   fixed-point sweep, mixed: read z, rho, g = rho r, x; write g, x     -> 24 B
+#            FP64: read z (4), rho (8), r, x; write r, x, g (FP32)      -> 48 B; A z in FP32 pairs,
+#            3 FP64 additions (x += z, r -= A z in two parts) -> 3 FP64 ops and flops
+#   stencil: mixed: read z, rho, d_old; write d, q -> 20 B; FP64: z (4), rho (8), d_old, q_old; d, q
+#            -> 44 B, 4 FP64 ops, 6 flop (two FMA).  update, FP64: also writes g (FP32) -> 6T + 4
+#   res64  : read p, f - <f>, D, 3 FP64 coefficients, fixed point: rho; write r or g (FP64: both)
+#            -> 48 + T (+4 fixed) (+4 FP64); 14 flop, 7 FP64 ops; the first: f (fixed: D, rho), write
+#            f - <f>, r or g -> 16 + T (+12 fixed) (+4 FP64); 3 flop, 2 FP64 ops
+#   spec_x : X+ reads FP32, X- writes FP32, no weights -> (8 + 2S) / 2 per launch
 #   When the half spectrum fits in L2 (256^3: 71 MB) the S bytes never reach HBM: the HBM bytes
 #   of a spectral pass are then only its rt / W / z traffic, and Y and Z have none (their roof
 #   is the L2 bandwidth, reported as plain GB/s without an HBM fraction).
 SIZES = {"fp64": (8, 8, False), "mixed": (4, 4, False), "mixed_bf16": (4, 2, True)}
 KERNEL_NAMES = {"res64": "k_res64_direct", "stencil": "k_stencil_direct", "cheb": "k_stencil_direct",
-                "update": "k_flat", "other": "k_flat", "spec_x": "k_spec_x_fwd(_persistent) / k_spec_x_inv_persistent",
+                "update": "k_flat", "other": "k_flat",
+                "spec_x": "k_spec_x_fwd_staged (FP64 input: _persistent) / k_spec_x_inv_persistent",
                 "spec_y": "k_spec_y", "spec_z": "k_spec_z",
                 "mg": "k_mg_down / k_mg_restrict / k_mg_coarse / k_mg_prolong / k_mg_up"}
 FP64_PIPE_OPS = {"stencil_fixed": 8.0, "res64": 8.0, "res64_first": 4.0}  # FP64 inner type
+DENSITY_FP64_OPS = {"stencil_fixed": 3.0, "stencil": 4.0, "res64": 7.0, "res64_first": 2.0}
+
+
+def density_form(prec: str, precond: str) -> bool:
+    """Whether the library runs this solve in the density form (see above)."""
+    return prec in ("mixed", "fp64") and precond in ("fixed_point", "spectral")
 
 
 def fixed_inner_tol(workload: str, prec: str) -> float:
@@ -105,21 +124,15 @@ def spectrum_bytes(nx: int) -> float:
 
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu capture of the
-# kernel at this precision and grid (192^3 captures, fixed-point method, FP64), keyed (precision,
-# sweep, grid, fixed-point); 256^3 entries scale by the cell count 256^3 / 192^3.  A changed
-# kernel drops its entries until it is re-captured, and the residual is left out (the capture
-# holds the residual from p = 0 only, the table averages both kinds).
-_SCALE_256 = (256 / 192) ** 3
-_TRAFFIC_192 = {("fp64", "stencil", True): 317.8e6 + 85.3e6}
-TRAFFIC = {(p, k, 192, f): v for (p, k, f), v in _TRAFFIC_192.items()}
-TRAFFIC.update({(p, k, 256, f): v * _SCALE_256 for (p, k, f), v in _TRAFFIC_192.items()})
-# the fused FP32 sweep of the mixed fixed-point solve: captured at 256^3 (a launch with x read and
-# written), scaled to 512^3 by the cell count
-TRAFFIC[("mixed", "stencil", 256, True)] = 343.2e6 + 107.0e6
-TRAFFIC[("mixed", "stencil", 512, True)] = (343.2e6 + 107.0e6) * 8
+# kernel at this precision and grid, keyed (precision, sweep, grid, fixed-point): the fixed-point
+# sweeps in the density form captured at 256^3 (a launch with x read and written), scaled to 512^3
+# by the cell count.  A changed kernel drops its entries until it is re-captured.
+_TRAFFIC_256 = {("mixed", "stencil", True): 400e6, ("fp64", "stencil", True): 800e6}
+TRAFFIC = {(p, k, 256, f): v for (p, k, f), v in _TRAFFIC_256.items()}
+TRAFFIC.update({(p, k, 512, f): v * 8 for (p, k, f), v in _TRAFFIC_256.items()})
 
 
-def spec_bytes(prec: str, kind: str, nx: int, ncell: int, slabbed: bool, fixed: bool):
+def spec_bytes(prec: str, kind: str, nx: int, ncell: int, slabbed: bool, fixed: bool, dens: bool = False):
     """(operand bytes, HBM bytes) per cell of the spectral passes of kind spec_x (X+ and X-),
     spec_y (Y+ and Y-) or spec_z over one application.  X+ reads rt (T) and its weight (4) and
     writes the half spectrum (S per cell); Y+ / Y- read and write it; Z reads and writes it; X-
@@ -127,13 +140,14 @@ def spec_bytes(prec: str, kind: str, nx: int, ncell: int, slabbed: bool, fixed: 
     whole spectrum fits in L2 (256^3: 71 MB) no S byte reaches HBM; when the passes run slab by
     slab (512^3) X+ hands its slab to Y+ and Y- to X- through L2, so only Y+'s write and Y-'s
     read of S reach HBM."""
-    T = SIZES[prec][0]
+    T = 4 if dens else SIZES[prec][0]  # density form: an FP32 input, no weights, z in FP32
     zT = 4 if fixed else T
+    W = 0 if dens else 4
     S = spectrum_bytes(nx)
     whole_l2 = S * ncell <= 0.6 * L2_BYTES
     if kind == "spec_x":
-        alg = T + 4 + S + S + 4 + zT
-        hbm = T + 4 + 4 + zT + (0 if (whole_l2 or slabbed) else 2 * S)
+        alg = T + W + S + S + W + zT
+        hbm = T + W + W + zT + (0 if (whole_l2 or slabbed) else 2 * S)
     elif kind == "spec_y":
         alg = 4 * S
         hbm = 0 if whole_l2 else (2 * S if slabbed else 4 * S)
@@ -143,11 +157,21 @@ def spec_bytes(prec: str, kind: str, nx: int, ncell: int, slabbed: bool, fixed: 
     return alg, hbm
 
 
-def sweep_cost(prec: str, kind: str, cheb_k: int = 1, nx: int = 256, fixed: bool = False, ncell: int = 0):
+def sweep_cost(prec: str, kind: str, cheb_k: int = 1, nx: int = 256, fixed: bool = False, ncell: int = 0,
+               dens: bool = False):
     """(bytes, flops, hbm_bytes) per cell of one launch of sweep `kind`, or None (the spectral
     passes: see spec_bytes, per application)."""
     T, B, diag = SIZES[prec]
     Bd = B if diag else 0
+    if dens and kind in ("stencil", "update", "res64", "res64_first"):
+        f64 = prec == "fp64"
+        g = 4 if f64 else 0  # the FP32 copy of the residual for X+
+        b, fl = {"stencil": ((48, 3.0) if f64 else (24, 14.0)) if fixed
+                 else ((44, 6.0) if f64 else (20, 16.0)),
+                 "update": (6 * T + g, 6.0),
+                 "res64": (48 + T + g + (4 if fixed else 0), 14.0),
+                 "res64_first": (16 + T + g + (12 if fixed else 0), 3.0)}[kind]
+        return b, fl, b
     if fixed and kind == "stencil":
         b = 4 + 4 * T + 3 * B + Bd
         return b, 14.0 + (2.0 if diag else 0.0), b
@@ -177,35 +201,40 @@ def sweep_cost(prec: str, kind: str, cheb_k: int = 1, nx: int = 256, fixed: bool
 
 
 def algorithmic(prec: str, ncell: int, iters: int, outer: int, spectral: bool = False, nx: int = 256,
-                fixed: bool = False, slabbed: bool = False):
+                fixed: bool = False, slabbed: bool = False, dens: bool = False):
     """Algorithmic HBM bytes of a whole solve (the roofline of the step as a whole)."""
     T = SIZES[prec][0]
-    spec = sum(spec_bytes(prec, k, nx, ncell, slabbed, fixed)[1] for k in ("spec_x", "spec_y", "spec_z"))
+    spec = sum(spec_bytes(prec, k, nx, ncell, slabbed, fixed, dens)[1] for k in ("spec_x", "spec_y", "spec_z"))
     if fixed:  # per update: one application and the fused sweep
-        per_iter = spec + sweep_cost(prec, "stencil", fixed=True)[2]
+        per_iter = spec + sweep_cost(prec, "stencil", fixed=True, dens=dens)[2]
     else:
-        per_iter = sweep_cost(prec, "stencil")[2] + sweep_cost(prec, "update")[2] + (spec if spectral else 0)
-    res = sweep_cost(prec, "res64")[2] * max(outer - 1, 0) + sweep_cost(prec, "res64_first")[2]
+        per_iter = (sweep_cost(prec, "stencil", dens=dens)[2] + sweep_cost(prec, "update", dens=dens)[2]
+                    + (spec if spectral else 0))
+    res = (sweep_cost(prec, "res64", fixed=fixed, dens=dens)[2] * max(outer - 1, 0)
+           + sweep_cost(prec, "res64_first", fixed=fixed, dens=dens)[2])
     return (iters * per_iter + res + max(outer - 1, 0) * (24 + T) + 32) * ncell
 
 
 def kernel_table(prec: str, ncell: int, kinds: dict, peaks: dict, grid: int, cheb_k: int = 1, nx: int = 256,
-                 fixed: bool = False, slabbed: bool = False):
+                 fixed: bool = False, slabbed: bool = False, dens: bool = False):
     """Per sweep kind: launches, mean/min duration (CUDA events around each launch), share of the
     summed kernel time, algorithmic GB/s (all operand bytes), the HBM fraction of the bytes that
     reach HBM, and for FP64 sweeps the FP64 TFLOP/s and its fraction of the measured FP64 peak.
     Spectral kinds are counted per application (their launches may be slabs)."""
     total = sum(k["ms"] for k in kinds.values()) or 1.0
     apps = max(kinds.get("spec_z", {}).get("launches", 0), 1)
+    fp64_ops = DENSITY_FP64_OPS if dens else FP64_PIPE_OPS
     out = {}
     for name, k in kinds.items():
         if not k["launches"]:
             continue
         row = {"kernel": KERNEL_NAMES[name], "launches": k["launches"], "mean_us": 1e3 * k["ms_mean"],
                "min_us": 1e3 * k["ms_min"], "share": k["ms"] / total}
+        if dens and name == "stencil":
+            row["kernel"] = "k_density64" if prec == "fp64" else "k_density"
         t_all = k["ms"] / 1e3
         if name.startswith("spec_"):
-            alg, hbm = spec_bytes(prec, name, nx, ncell, slabbed, fixed)
+            alg, hbm = spec_bytes(prec, name, nx, ncell, slabbed, fixed, dens)
             row["us_per_application"] = 1e6 * t_all / apps
             row["alg_bytes_per_launch"] = alg * ncell * apps / k["launches"]
             row["gbs"] = alg * ncell * apps / t_all / 1e9
@@ -218,14 +247,14 @@ def kernel_table(prec: str, ncell: int, kinds: dict, peaks: dict, grid: int, che
             row["traffic"] = None
             out[name] = row
             continue
-        cost = sweep_cost(prec, name, cheb_k, nx, fixed, ncell)
-        ops = FP64_PIPE_OPS.get("stencil_fixed" if (fixed and name == "stencil") else name)
+        cost = sweep_cost(prec, name, cheb_k, nx, fixed, ncell, dens)
+        ops = fp64_ops.get("stencil_fixed" if (fixed and name == "stencil") else name)
         if name == "res64" and k["launches"] > 0:
             # every benchmarked solve starts from p = 0: one of its residual launches is the
             # short first one; the row averages over the launches (bytes, flops, FP64 ops)
-            n, first = k["launches"], sweep_cost(prec, "res64_first")
+            n, first = k["launches"], sweep_cost(prec, "res64_first", fixed=fixed, dens=dens)
             cost = tuple(((n - 1) * c + f) / n for c, f in zip(cost, first))
-            ops = ((n - 1) * ops + FP64_PIPE_OPS["res64_first"]) / n
+            ops = ((n - 1) * ops + fp64_ops["res64_first"]) / n
         if cost is not None:
             t = k["ms_mean"] / 1e3
             row["alg_bytes_per_launch"] = cost[0] * ncell
@@ -854,9 +883,10 @@ def main():
     assert st_t.iters == iters and torch.equal(pt, p), "instrumented solve differs from the timed solves"
     del pt
     slabbed = solver.spectral_slabs() > 1
-    table = kernel_table(prec, ncell, kinds, peaks, nx, nx=nx, fixed=fixed, slabbed=slabbed)
+    dens = density_form(prec, args.precond)
+    table = kernel_table(prec, ncell, kinds, peaks, nx, nx=nx, fixed=fixed, slabbed=slabbed, dens=dens)
     roof = roofline(prec, table, peaks)
-    b_solve = algorithmic(prec, ncell, iters, outer, args.precond == "spectral", nx, fixed, slabbed)
+    b_solve = algorithmic(prec, ncell, iters, outer, args.precond == "spectral", nx, fixed, slabbed, dens)
     dtype = {"fp64": "f64", "mixed": "f32 inner, f64 outer",
              "mixed_bf16": "f32 inner (bf16 coefficients), f64 outer"}[prec]
     line = {
@@ -911,7 +941,7 @@ def main():
                 el64, st64 = timed(torch, s64, f, p64, prob.tol, args.steps, args.warmup, stream, barrier)
                 _, k64 = s64.solve_timed(f, p64, prob.tol)
                 sl64 = s64.spectral_slabs() > 1
-            tab = kernel_table("fp64", ncell, k64, peaks, nx, nx=nx, fixed=True, slabbed=sl64)
+            tab = kernel_table("fp64", ncell, k64, peaks, nx, nx=nx, fixed=True, slabbed=sl64, dens=True)
             return {"solves_per_s": args.steps / el64, "ms_per_step": 1e3 * el64 / args.steps,
                     "iters": st64[-1].iters, "outer": st64[-1].outer_iters, "rel_res": st64[-1].rel_res,
                     "roofline": roofline("fp64", tab, peaks),
@@ -994,7 +1024,7 @@ def run_c1(torch, vdp, dev, prob, stream, peaks, args, barrier):
         s.set_density(rho)
         el, st = timed(torch, s, f, p, 1e-10, args.steps, args.warmup, stream, barrier)
         _, kinds = s.solve_timed(f, p, 1e-10)
-    tab = kernel_table("fp64", ncell, kinds, peaks, nx, nx=nx, fixed=True)
+    tab = kernel_table("fp64", ncell, kinds, peaks, nx, nx=nx, fixed=True, dens=True)
     out = {"workload": WORKLOAD_C1, "solves_per_s": args.steps / el, "ms_per_step": 1e3 * el / args.steps,
            "iters": st[-1].iters, "outer": st[-1].outer_iters, "rel_res": st[-1].rel_res,
            "roofline": roofline("fp64", tab, peaks), "kernels": tab}
@@ -1036,7 +1066,8 @@ def run_c1_variants(torch, vdp, dev, prob, stream, peaks):
             pp = torch.empty_like(f)
             best = best_of(s2, f, pp, 1e-8)
             _, kk = s2.solve_timed(f, pp, 1e-8, check=False)
-            tab = kernel_table(prec, ncell, kk, peaks, nx, cheb_k=k, nx=nx, fixed=pc == "fixed_point")
+            tab = kernel_table(prec, ncell, kk, peaks, nx, cheb_k=k, nx=nx, fixed=pc == "fixed_point",
+                               dens=density_form(prec, pc))
             paths[label] = solve_summary(vdp, best, {
                 "oracle_rel_res": oracle.relative_residual(prob.rho, prob.L, prob.f, pp.cpu().numpy()),
                 "kernels": {n: {x: r[x] for x in ("mean_us", "share", "gbs", "hbm_frac") if x in r}

@@ -88,7 +88,8 @@ typedef enum {
                              max(rho)/min(rho) for any grid size.  Each of nx, ny, nz must be one
                              of 32, 48, 64, 96, 128, 192, 256, 512; direct stencil sweep only;
                              batch members only in batches of ordinary launches (persistent =
-                             0).  Extra memory: about 16 bytes per cell */
+                             0).  Extra memory: about 16 bytes per cell (24 where the density was
+                             set before this option) and the half spectrum */
   VDP_PRECOND_MG = 3      /* a geometric multigrid V-cycle (no counterpart in the paper; the
                              standard mesh-independent alternative to its FFT solve): cell-
                              centred, periodic, FP32; levels halve every size while all are even
@@ -137,8 +138,9 @@ typedef struct {
   int units;           /* work units (thread blocks) per sweep (0 = automatic) */
   int stages;          /* shared-memory pipeline stages of the stencil sweep, 4..8 (0 = auto) */
   int threads;         /* threads per stencil work unit, 128..512, multiple of 32 (0 = auto) */
-  int steps_per_sync;  /* 0 (default): each solve is one graph launch whose device-side loop
-                          stops when the solve is done; > 0: replay graphs of that many rounds
+  int steps_per_sync;  /* 0 (default): each solve is one cooperative launch (small grids) or one
+                          graph launch whose device-side loop stops when the solve is done;
+                          > 0: replay graphs of that many rounds
                           with a host check of the state after each (same results) */
   int method;          /* vdp_method (default VDP_METHOD_CG) */
   double damping;      /* VDP_METHOD_FIXED_POINT: scale of each update, 0 < damping <= 2
@@ -346,7 +348,9 @@ int vdp_solve_timed(vdp_ctx *ctx, const double *rhs, double *p, double tol, vdp_
  * vdp_solve on that context alone.  persistent = 1 runs each vdp_batch_run as one cooperative
  * persistent kernel looping over all members with grid-wide barriers (bounded waits);
  * persistent = 0 as the equivalent sequence of ordinary launches; either is captured into a
- * CUDA graph that is re-captured only when membership changes.  Work is ordered on `stream`
+ * CUDA graph that is re-captured only when membership changes.  Members with a preconditioner of
+ * several passes (spectral, fixed point, multigrid) run in a persistent = 0 batch as they do
+ * alone, several at a time on streams of the batch.  Work is ordered on `stream`
  * (NULL = legacy default stream).  A batch does not own its contexts.
  */
 typedef struct vdp_batch vdp_batch;

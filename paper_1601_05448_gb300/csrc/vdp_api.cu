@@ -370,12 +370,12 @@ int ensure_spectral(vdp_ctx* c) {
   if (!spectral_supported(spectral_nx(c), c->ny, c->nz)) return VDP_EINVAL;
   if (c->spec && c->sptab && c->za) return VDP_OK;
   static std::mutex mu;
-  static std::vector<int> uploaded;  // devices whose register-DFT roots are in place
+  static std::vector<int> prepared;  // devices whose spectral kernels are prepared
   {
     std::lock_guard<std::mutex> lk(mu);
-    if (std::find(uploaded.begin(), uploaded.end(), c->device) == uploaded.end()) {
-      VDP_CK(spectral_upload_roots());
-      uploaded.push_back(c->device);
+    if (std::find(prepared.begin(), prepared.end(), c->device) == prepared.end()) {
+      VDP_CK(spectral_prepare());
+      prepared.push_back(c->device);
     }
   }
   std::vector<float> tab;

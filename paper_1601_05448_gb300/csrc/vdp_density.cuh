@@ -8,7 +8,8 @@
 //     rho' = rho / 2^e0 (e0 the exponent of the first cell),  s = 2^(2 m), m the exponent of hx,
 //     A' = kappa A, kappa = 2^e0 s:  face values (2 s / h_d^2) / (rho'_l + rho'_r),
 // an inner solve of (-A') X = r gives the correction p -= kappa X, whatever the units of rho and
-// of the box; kappa is a power of two, so the scaling rounds nothing.  Per cell and iteration of the FP32 fixed-point solve this moves
+// of the box; kappa is a power of two, so the scaling rounds nothing.  Per cell and iteration of the
+// FP32 fixed-point solve this moves
 //     X+  g 4            (weights and rt: 8)        X-  z 4            (z and weight: 8)
 //     sweep  z, rho', g, X read, g, X written: 24   (z, three coefficients, rt, x: 32)
 // besides the half spectrum: 32 bytes instead of 48.  Fixed point: g = rho' r is the stored
@@ -22,7 +23,10 @@
 // registers are held while they fly, and the arithmetic of one plane covers the latency of the
 // next.  The x neighbours at row and warp ends come the same way (loaded at their use, they cost
 // every plane a trip to L2).  Sums, products and Newton steps of the four cells run as paired FP32
-// instructions, and the fluxes through the x faces and the upper z face are computed once for both cells.
+// instructions, and the fluxes through the x faces and the upper z face are computed once for both
+// cells.  The fused fixed-point sweep (scaled form with stored coefficients / plain loads / cp.async /
+// cp.async with the x neighbours): 512^3 662 / 595 / 555 / 514 us, 256^3 110 / 103 / 92 / 87; 24 bytes
+// a cell in 514 us are 0.92 of the copy bandwidth.
 #pragma once
 
 #include "vdp_device.cuh"
@@ -330,7 +334,7 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
 // ---- the FP64 inner solve ------------------------------------------------------------------------
 // z comes out of the FP32 transforms, so it is an FP32 field in this solve too; r, X, d and q are
 // FP64.  The product A' z in FP64 instructions bounds the sweep by the FP64 pipe (8 instructions
-// per cell at 2 per clock and SM: 282 us at 256^3, where its bytes take 109).  Here coefficients
+// per cell at 2 per clock and SM: 282 us at 256^3, where its bytes take 118).  Here coefficients
 // and product are pairs of FP32 numbers (unevaluated sums hi + lo, about 47 bits): rho' as such a
 // pair, the quotient by a Newton step and a corrected remainder, the differences of z exact, the
 // products by FMA with their rounding errors, the six terms summed with the errors carried along.
@@ -338,7 +342,10 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
 // (CG).  The sweep also leaves rho' r in FP32 for the X+ pass, which read r and rho' and narrowed
 // the product itself: four bytes more here, eight fewer there, and X+ runs its FP32 form (256^3:
 // 75 -> 35 us).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
-// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before.
+// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before.  The fused
+// sweep takes 215 us at 256^3 and 75 on the 256 x 128 x 128 duct (95 in the scaled form), CG's 44 at
+// 128^3 (64): bound by instruction issue and latency at three blocks of 128 threads per SM (two 270,
+// four 289 us).
 struct df {
   f2 h, l;
 };

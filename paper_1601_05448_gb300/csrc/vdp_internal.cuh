@@ -207,12 +207,14 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 // to the sweep's final sum, so small grids want few units, large ones enough for several waves
 // (sweep and residual, us: 112 x 100 x 90 FP64 46.5 and 68 with 1824 units, 34.8 and 45 with 456;
 // 96^3 FP32 26.2 and 56 against 19.4 and 42; 256^3 FP32 93.6 and 265 with 1824, 89.9 and 246 with
-// 1368; 512^3 550 with 1824, 598 with 456).
+// 1368; 512^3 550 with 1824, 598 with 456).  Grids that the resident solve takes get 304 units, one
+// for each of its blocks.
 // mode 1 (TMA pipeline): FP64 512-thread units with about 2048 cells per plane, FP32/BF16 256
 // threads with about 1024; the row tile shrinks until four pipeline stages fit; stages default to
 // what fits (at most 6), or to 4 when that lets two units share an SM; about four waves.
-// Both: stencil units = row tiles x z chunks (chunk-major); flat units of 4096+ cells
-// (at most 8 per SM), on small grids down to 1024 for two units per SM.  In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
+// Both: stencil units = row tiles x z chunks (chunk-major); flat units of 8192+ cells (at most 8 per
+// SM; 160^3 update 25.7 us with 4096, 23.4 with 8192), on small grids down to 1024 for two units
+// per SM.  In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
 // Returns false when the configuration cannot run (rows too long, bad counts).
 inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, int units,
                         int stages, int threads, Layout* L) {

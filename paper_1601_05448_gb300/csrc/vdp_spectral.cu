@@ -11,22 +11,25 @@
 // preconditioned condition number is at most the density ratio, whatever the grid size.
 //
 // Five passes over a half spectrum S[kz][ky][kx] (kx = 0 .. nx/2, complex FP32, row pitch nxp):
-//   X+  each row of nx reals is read as nx/2 complex pairs, weighted by W, transformed by a
-//       complex FFT of length nx/2 and unpacked into the nx/2 + 1 bins of the real transform;
+//   X+  each row of nx reals is read as nx/2 complex pairs (in the scaled form weighted by W; the
+//       density form, vdp_density.cuh, has no weights), transformed by a complex FFT of length
+//       nx/2 and unpacked into the nx/2 + 1 bins of the real transform;
 //   Y+  complex FFTs along y of tiles of 8 consecutive kx columns;
 //   Z   FFT along z, division by the eigenvalue (and by nx ny nz), inverse FFT along z: the
 //       whole z line is in the block, so the solve costs one pass;
 //   Y-  inverse FFTs along y;
-//   X-  the real inverse transform of each row, weighted by W, stored as z; in the solve this
-//       pass also sums <rt, z> and, as the last unit to finish, moves the solve to its next
-//       phase (the same fixed-order reduction as every other sweep).
+//   X-  the real inverse transform of each row, (weighted by W and) stored as z; in the solve the
+//       last unit to finish also sums the <rt, z> partials of Z (spectral CG) and moves the solve
+//       to its next phase (the same fixed-order reduction as every other sweep).
 // Every line FFT is a four-step factorisation n = M1 x M2 (both products of 2 and 3, at most
 // 32): M2-point DFTs in registers, twiddles W_n^(j1 k2), an exchange through shared memory,
 // M1-point DFTs in registers.  Global accesses are coalesced: rows are contiguous in the X
 // passes and the Y/Z tiles read 8 consecutive complex values (64 bytes) per line element.
-// One application moves about 49 bytes per cell for the FP32 inner solve; at 512^3 the X and Y
-// passes run at 0.85-0.91 of the copy bandwidth and Z, which does two transforms per element,
-// is bound by its instruction issue.
+// One application moves about 41 bytes per cell (FP32 input, no weights).  At 512^3 X takes 185 us a
+// launch, Y 191 (0.87 of the copy bandwidth each) and Z, which does two transforms per element, 315
+// (0.53).  At 256^3 the spectrum stays in L2 and nothing is saturated (ncu: issue 42-58 %, shared
+// memory 28-54 %, DRAM 28-43 %; 15-20 warps per SM): X 33, Y 26, Z 36 us.  In every pass the
+// first tile's copies and the tables are under way while the solve's phase is read.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -66,7 +69,9 @@ __global__ void __launch_bounds__(M1 * rows_per_block<M1, M2>(), 768 / (M1 * row
 }
 
 // X+ of FP32 rows on a persistent grid, the group's rows copied to shared memory while the group
-// before is transformed.
+// before is transformed (an FP32 row of the solve's own fields starts on a 16-byte boundary; FP64 rows
+// may be a caller's).  Loading them at their use, 512^3 took 204 us, the 256 x 128 x 128 duct 24;
+// now 185 and 20.
 template <int M1, int M2, bool MIRROR>
 __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>()) k_spec_x_fwd_staged(SpecArgs a) {
   constexpr int RY = inv_rows_per_block<M1, M2>();
@@ -104,9 +109,9 @@ __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>()) k_spec_x_fw
 }
 
 // X- on a persistent grid: groups of RY rows (group = block, block + grid, ...), tables in
-// shared memory.  The 512^3 mixed solve: 33.6 ms against 34.1 ms with one row group per block
-// and the tables read through L1; and a launch in another phase of the solve exits after 3 us
-// instead of 29 us.
+// shared memory, the group's rows copied there while the group before is transformed: each bin is
+// read twice (k and nx/2 - k), which through L1 cost 76 % of its rate and left 8 stall cycles per
+// issue on the loads (256^3: 35 us, now 33; 512^3 201 and 185).
 template <class T, int M1, int M2, bool MIRROR, bool WEIGHT>
 __global__ void __launch_bounds__(M1 * inv_rows_per_block<M1, M2>())
     k_spec_x_inv_persistent(SpecArgs a) {
@@ -519,7 +524,7 @@ void spectral_tables(int nx, int ny, int nz, double hx, double hy, double hz,
   eig(nz, nz, hz);
 }
 
-cudaError_t spectral_upload_roots() {
+cudaError_t spectral_prepare() {
   cudaError_t e = cudaSuccess;
   const int dev = current_device();
   if (dev < 0) e = cudaErrorInvalidDevice;

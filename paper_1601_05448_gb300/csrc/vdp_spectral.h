@@ -57,7 +57,7 @@ size_t spectral_table_floats(int nx, int ny, int nz);
 // 4 sin^2(pi k / n_d) / h_d^2 for kx = 0..m, ky, kz; computed in double, stored as float
 void spectral_tables(int nx, int ny, int nz, double hx, double hy, double hz,
                      std::vector<float>& out);
-cudaError_t spectral_upload_roots();               // the register-DFT roots, once per device
+cudaError_t spectral_prepare();                    // kernel attributes and resident blocks, once per device
 cudaError_t launch_spectral_pass(int prec, int pass, const SpecArgs& a, cudaStream_t s);
 int spectral_units(int nx, int ny, int nz);        // CTAs of the Z pass (partial slots)
 // Planes per slab of one application: req (vdp_opts.spec_slab) when positive and below nz, else
