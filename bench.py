@@ -108,8 +108,8 @@ def fixed_inner_tol(workload: str, prec: str) -> float:
     The paper's iteration reduces the residual by about 0.18 per iteration on the 512^3 input
     whatever the precision, so it needs 12 iterations to 1e-8; the inner target only decides how
     many FP64 residuals (and corrections) the mixed solve spends on the way.  Measured at 512^3
-    (FP32 inner): 1e-4 -> 12 iterations and 4 FP64 residuals (31.7 ms); 5e-5 and 3e-5 -> 12 and 3
-    (29.3 ms, final residual 9.2e-9); 2e-5 -> 13 and 3; 1e-5 -> 14 and 3 (the first inner solve,
+    (FP32 inner, before the density form): 1e-4 -> 12 iterations and 4 FP64 residuals (31.7 ms); 5e-5
+    and 3e-5 -> 12 and 3 (29.3 ms, final residual 9.2e-9; now 24.6 ms); 2e-5 -> 13 and 3; 1e-5 -> 14 and 3 (the first inner solve,
     from the largest residual, stalls near FP32 rounding).  With BF16 coefficients 1e-4 is best
     (19 iterations against 21 at 5e-5).  Elsewhere the library default 1e-4."""
     if workload == "c2" and prec == "mixed":
@@ -127,7 +127,7 @@ def spectrum_bytes(nx: int) -> float:
 # kernel at this precision and grid, keyed (precision, sweep, grid, fixed-point): the fixed-point
 # sweeps in the density form captured at 256^3 (a launch with x read and written), scaled to 512^3
 # by the cell count.  A changed kernel drops its entries until it is re-captured.
-_TRAFFIC_256 = {("mixed", "stencil", True): 400e6, ("fp64", "stencil", True): 800e6}
+_TRAFFIC_256 = {("mixed", "stencil", True): 269.6e6 + 94.5e6, ("fp64", "stencil", True): 482.8e6 + 282.1e6}
 TRAFFIC = {(p, k, 256, f): v for (p, k, f), v in _TRAFFIC_256.items()}
 TRAFFIC.update({(p, k, 512, f): v * 8 for (p, k, f), v in _TRAFFIC_256.items()})
 
