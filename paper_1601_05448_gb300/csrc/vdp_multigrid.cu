@@ -19,7 +19,8 @@
 // spectral preconditioner.
 //
 // Per level and cycle four launches: pre-smoothing + residual (down), restriction, prolongation
-// + pre-smoothed iterate, post-smoothing (up); one launch solves the coarsest level.  The level
+// + pre-smoothed iterate, post-smoothing (up); the levels of up to 4096 cells and the coarsest take
+// one launch of one block.  The level
 // sweeps are z-marching column kernels (one-wave work-item plan); the z-neighbours are carried in
 // registers.  All launches return at once unless the solve is in its preconditioner phase.
 #include <cuda_runtime.h>
@@ -35,6 +36,11 @@ namespace vdp {
 namespace {
 
 constexpr int kMgThreads = kMarchTx * kMarchTy;  // 1-D blocks of 256 (tile 32 x 8)
+// Levels that one block takes (k_mg_tail): up to 4096 cells.  CG solves, mixed, to 1e-9, with no such
+// levels / up to 1024 / 4096 / 8192 / 32768 cells, ms: 32^3 0.83 / 0.74 / 0.75 / 0.75 / 0.75, 40^3 1.00
+// / 0.92 / 0.92 / 1.03 / 1.03, 96^3 1.54 / 1.44 / 1.38 / 1.38 / 1.67, 128^3 2.21 / 2.12 / 2.14 / 2.14 /
+// 2.99, 160^3 3.43 / 3.35 / 3.35 / 3.51 / 3.51, 256 x 128 x 128 5.72 / 5.44 / 5.44 / 5.70 / 5.70.
+constexpr int kMgTailThreads = 1024, kMgTailLevels = 6, kMgTailCells = 4096;
 
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(double v) { return narrow(v); }
@@ -280,13 +286,12 @@ __global__ void __launch_bounds__(kMgThreads, 4)
 // products in sequence took 13 us for 125 cells).
 constexpr int kCoarseRows = 4 * (kMgThreads / 32);  // rows of a block
 
-__global__ void __launch_bounds__(kMgThreads)
-    k_mg_coarse(MgLevel lv, const float* __restrict__ pinv, int n, const InstState* st) {
-  if (!mg_active(st)) return;
-  const int lane = threadIdx.x & 31, i0 = blockIdx.x * kCoarseRows + (threadIdx.x >> 5) * 4;
+// Rows i0 .. i0 + 3 of x = pinv r by one warp.
+__device__ __forceinline__ void coarse_rows(const MgLevel& lv, const float* __restrict__ pinv, int n,
+                                            int i0, int lane) {
   float s[4] = {0.f, 0.f, 0.f, 0.f};
   for (int j = lane; j < n; j += 32) {
-    const float r = __ldg(lv.r + j);
+    const float r = lv.r[j];
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       if (i0 + q < n) s[q] = fmaf(__ldg(pinv + (long long)(i0 + q) * n + j), r, s[q]);
@@ -296,6 +301,117 @@ __global__ void __launch_bounds__(kMgThreads)
     const float v = warp_sum(s[q]);
     if (lane == 0 && i0 + q < n) lv.x[i0 + q] = v;
   }
+}
+
+__global__ void __launch_bounds__(kMgThreads)
+    k_mg_coarse(MgLevel lv, const float* __restrict__ pinv, int n, const InstState* st) {
+  if (!mg_active(st)) return;
+  coarse_rows(lv, pinv, n, blockIdx.x * kCoarseRows + (threadIdx.x >> 5) * 4, threadIdx.x & 31);
+}
+
+// The coarse levels of a cycle in one block: down, restriction, ..., coarsest, ..., prolongation and up
+// of every level from h.lev[0] on, separated by block barriers.  A level of a few thousand cells is a
+// microsecond or two of work for one block (trips to L2), and a launch of its own per step took three to
+// four.  Same operations per cell, in the same order, as the kernels above; fields that
+// this kernel writes are read by plain loads.
+struct MgTail {
+  MgLevel lev[kMgTailLevels];
+  int nlev;  // the last one is the coarsest
+  const float* pinv;
+  int ncoarse, wall_x;
+};
+
+__global__ void __launch_bounds__(kMgTailThreads) k_mg_tail(const __grid_constant__ MgTail h,
+                                                            const InstState* st) {
+  if (!mg_active(st)) return;
+  const float w = kMgOmega;
+  const int tid = threadIdx.x, lane = tid & 31;
+  // the sum of the six neighbours' bt v around cell c, added to s
+  auto neighbour_sum = [&](const MgLevel& lv, const float* v, int c, float s, bool up) {
+    const int nx = lv.nx, ny = lv.ny, nz = lv.nz, plane = nx * ny;
+    const int z = c / plane, y = (c - z * plane) / nx, x = c - z * plane - y * nx;
+    const int xm = x == 0 ? c + nx - 1 : c - 1, xp = x == nx - 1 ? c - (nx - 1) : c + 1;
+    const int ym = y == 0 ? c + (ny - 1) * nx : c - nx, yp = y == ny - 1 ? c - (ny - 1) * nx : c + nx;
+    const int zm = z == 0 ? c + (nz - 1) * plane : c - plane, zp = z == nz - 1 ? c - (nz - 1) * plane : c + plane;
+    s = up ? fmaf(__ldg(lv.bx + c), v[xm], s) : __ldg(lv.bx + c) * v[xm];
+    s = fmaf(__ldg(lv.bx + xp), v[xp], s);
+    s = fmaf(__ldg(lv.by + c), v[ym], s);
+    s = fmaf(__ldg(lv.by + yp), v[yp], s);
+    s = fmaf(__ldg(lv.bz + c), v[zm], s);
+    return fmaf(__ldg(lv.bz + zp), v[zp], s);
+  };
+  for (int l = 0; l < h.nlev - 1; ++l) {
+    const MgLevel &f = h.lev[l], &cv = h.lev[l + 1];
+    for (int c = tid; c < (int)f.n; c += kMgTailThreads) {
+      const float r = f.r[c];
+      f.t[c] = __ldg(f.om + c) * fmaf(1.f - w, r, w * neighbour_sum(f, f.r, c, 0.f, false));
+    }
+    __syncthreads();
+    const int nx = f.nx, ny = f.ny, nz = f.nz, cx = cv.nx, cy = cv.ny;
+    for (int C = tid; C < (int)cv.n; C += kMgTailThreads) {
+      const int K = C / (cx * cy), J = (C - K * cx * cy) / cx, I = C - K * cx * cy - J * cx;
+      const int xl = I == 0 ? nx - 1 : 2 * I - 1, xr = 2 * I + 2 == nx ? 0 : 2 * I + 2;
+      float s[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {  // fine planes 2K - 1 .. 2K + 2
+        const int k = 2 * K - 1 + a, kk = k < 0 ? k + nz : k == nz ? 0 : k;
+        float sum = 0.f;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const int j = 2 * J - 1 + b, jj = j < 0 ? j + ny : j == ny ? 0 : j;
+          const float* row = f.t + (kk * ny + jj) * nx;
+          const float2 v = *reinterpret_cast<const float2*>(row + 2 * I);
+          const float left = h.wall_x && I == 0 ? v.x : row[xl];
+          const float right = h.wall_x && I == cx - 1 ? v.y : row[xr];
+          const float rs = fmaf(0.25f, left + right, 0.75f * (v.x + v.y));
+          sum = fmaf(b == 0 || b == 3 ? 0.25f : 0.75f, rs, sum);
+        }
+        s[a] = sum;
+      }
+      const float v = fmaf(0.25f, s[0] + s[3], 0.75f * (s[1] + s[2]));
+      cv.r[C] = l + 1 < h.nlev - 1 ? __ldg(cv.oinv + C) * v : v;
+    }
+    __syncthreads();
+  }
+  const MgLevel& last = h.lev[h.nlev - 1];
+  for (int i0 = (tid >> 5) * 4; i0 < h.ncoarse; i0 += kMgTailThreads / 32 * 4)
+    coarse_rows(last, h.pinv, h.ncoarse, i0, lane);
+  __syncthreads();
+  for (int l = h.nlev - 2; l >= 0; --l) {
+    const MgLevel &f = h.lev[l], &cv = h.lev[l + 1];
+    const int nx = f.nx, ny = f.ny, cx = cv.nx, cy = cv.ny, cz = cv.nz;
+    for (int q = tid; q < (int)(f.n / 2); q += kMgTailThreads) {  // two cells of a row
+      const int z = q / (cx * ny), y = (q - z * cx * ny) / cx, I = q - z * cx * ny - y * cx;
+      const int K = z >> 1, Kn = z & 1 ? (K + 1 == cz ? 0 : K + 1) : (K == 0 ? cz - 1 : K - 1);
+      const int J0 = y >> 1;
+      const int Im = I == 0 ? (h.wall_x ? I : cx - 1) : I - 1, Ip = I + 1 == cx ? (h.wall_x ? I : 0) : I + 1;
+      const int J1 = (y & 1) ? (J0 + 1 == cy ? 0 : J0 + 1) : (J0 == 0 ? cy - 1 : J0 - 1);
+      auto L = [&](int k) {
+        const float *p0 = cv.x + (k * cy + J0) * cx, *p1 = cv.x + (k * cy + J1) * cx;
+        const float al = fmaf(0.75f, p0[I], 0.25f * p0[Im]), bl = fmaf(0.75f, p1[I], 0.25f * p1[Im]);
+        const float ah = fmaf(0.75f, p0[I], 0.25f * p0[Ip]), bh = fmaf(0.75f, p1[I], 0.25f * p1[Ip]);
+        return make_float2(fmaf(0.75f, al, 0.25f * bl), fmaf(0.75f, ah, 0.25f * bh));
+      };
+      const float2 Lc = L(K), Ln = L(Kn);
+      const int c = (z * ny + y) * nx + 2 * I;
+      const float2 r = *reinterpret_cast<const float2*>(f.r + c);
+      const float2 om = __ldg(reinterpret_cast<const float2*>(f.om + c));
+      *reinterpret_cast<float2*>(f.t + c) =
+          make_float2(fmaf(w, r.x, om.x * fmaf(0.75f, Lc.x, 0.25f * Ln.x)),
+                      fmaf(w, r.y, om.y * fmaf(0.75f, Lc.y, 0.25f * Ln.y)));
+    }
+    __syncthreads();
+    for (int c = tid; c < (int)f.n; c += kMgTailThreads)
+      f.x[c] = __ldg(f.oinv + c) * fmaf(1.f - w, f.t[c], w * neighbour_sum(f, f.t, c, f.r[c], true));
+    __syncthreads();
+  }
+}
+
+// First level of the tail, or 0: none.
+int tail_level(const MgHier& h) {
+  int l = h.nlev - 1;
+  while (l > 1 && h.nlev - l < kMgTailLevels && h.lev[l - 1].n <= kMgTailCells) --l;
+  return l < h.nlev - 1 ? l : 0;
 }
 
 // ---- set-up -------------------------------------------------------------------------------------
@@ -655,10 +771,11 @@ cudaError_t mg_setup(MgHier* h, const double* bx, const double* by, const double
   return launch_pinv(h->lev[h->nlev - 1], h->ncoarse, h->pinv, s);
 }
 
-int mg_launches(const MgHier& h, int prec) { return 4 * (h.nlev - 1) + 1 + (prec == PREC_FP64); }
+int mg_launches(const MgHier& h, int prec) {
+  const int tail = tail_level(h);
+  return 4 * (tail ? tail : h.nlev - 1) + 1 + (prec == PREC_FP64);
+}
 
-// One V-cycle; T is the type of the solve's rt and z.  An FP64 rt is rounded to FP32 once (into
-// level 0's r), so the level-0 sweeps read FP32 only.
 // One V-cycle; T is the type of the solve's rt and z.  An FP64 rt is rounded to FP32 once (into
 // level 0's r), so the level-0 sweeps read FP32 only.
 template <class T>
@@ -677,7 +794,8 @@ static cudaError_t vcycle(const MgHier& h, const MgArgs& a, cudaStream_t s) {
   T* out = static_cast<T*>(a.out);
   auto rhs = [&](int l) { return l == 0 ? in : static_cast<const float*>(h.lev[l].r); };
   auto wgt = [&](int l) { return l == 0 ? a.omega : static_cast<const float*>(h.lev[l].om); };
-  for (int l = 0; l < L - 1; ++l) {
+  const int tail = tail_level(h), top = tail ? tail : L - 1;  // levels 0 .. top - 1 by launches of their own
+  for (int l = 0; l < top; ++l) {
     const MgLevel& v = h.lev[l];
     const MgLevel& cv = h.lev[l + 1];
     const MarchPlan m = march_plan(v.nx, v.ny, v.nz, cached_resident(k_mg_down0<float>, &r_down));
@@ -686,8 +804,19 @@ static cudaError_t vcycle(const MgHier& h, const MgArgs& a, cudaStream_t s) {
     k_mg_restrict<<<mr.blocks, kMgThreads, 0, s>>>(v, cv, mr, l + 1 < L - 1 ? cv.oinv : nullptr,
                                                    h.wall_x, a.st);
   }
-  k_mg_coarse<<<(h.ncoarse + kCoarseRows - 1) / kCoarseRows, kMgThreads, 0, s>>>(h.lev[L - 1], h.pinv, h.ncoarse, a.st);
-  for (int l = L - 2; l >= 0; --l) {
+  if (tail) {
+    MgTail t = {};
+    for (int l = tail; l < L; ++l) t.lev[l - tail] = h.lev[l];
+    t.nlev = L - tail;
+    t.pinv = h.pinv;
+    t.ncoarse = h.ncoarse;
+    t.wall_x = h.wall_x;
+    k_mg_tail<<<1, kMgTailThreads, 0, s>>>(t, a.st);
+  } else {
+    k_mg_coarse<<<(h.ncoarse + kCoarseRows - 1) / kCoarseRows, kMgThreads, 0, s>>>(h.lev[L - 1], h.pinv,
+                                                                                   h.ncoarse, a.st);
+  }
+  for (int l = top - 1; l >= 0; --l) {
     const MgLevel& v = h.lev[l];
     const MgLevel& cv = h.lev[l + 1];
     const MarchPlan mp = march_plan(cv.nx, v.ny, cv.nz, cached_resident(k_mg_prolong, &r_pro));
