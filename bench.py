@@ -92,7 +92,7 @@ KERNEL_NAMES = {"res64": "k_res64_direct", "stencil": "k_stencil_direct", "cheb"
                 "update": "k_flat", "other": "k_flat",
                 "spec_x": "k_spec_x_fwd_staged (FP64 input: _persistent) / k_spec_x_inv_persistent",
                 "spec_y": "k_spec_y", "spec_z": "k_spec_z",
-                "mg": "k_mg_down / k_mg_restrict / k_mg_coarse / k_mg_prolong / k_mg_up"}
+                "mg": "k_mg_down0 / k_mg_restrict / k_mg_tail / k_mg_prolong / k_mg_up"}
 FP64_PIPE_OPS = {"stencil_fixed": 8.0, "res64": 8.0, "res64_first": 4.0}  # FP64 inner type
 DENSITY_FP64_OPS = {"stencil_fixed": 3.0, "stencil": 4.0, "res64": 7.0, "res64_first": 2.0}
 
