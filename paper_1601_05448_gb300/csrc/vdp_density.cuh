@@ -25,8 +25,8 @@
 // every plane a trip to L2).  Sums, products and Newton steps of the four cells run as paired FP32
 // instructions, and the fluxes through the x faces and the upper z face are computed once for both
 // cells.  The fused fixed-point sweep (scaled form with stored coefficients / plain loads / cp.async /
-// cp.async with the x neighbours): 512^3 662 / 595 / 555 / 514 us, 256^3 110 / 103 / 92 / 87; 24 bytes
-// a cell in 514 us are 0.92 of the copy bandwidth.
+// cp.async with the x neighbours / units in whole waves): 512^3 662 / 595 / 555 / 514 / 507 us, 256^3
+// 110 / 103 / 92 / 87 / 81; 24 bytes a cell in 507 us are 0.94 of the copy bandwidth.
 #pragma once
 
 #include "vdp_device.cuh"
@@ -343,7 +343,7 @@ __device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState
 // the product itself: four bytes more here, eight fewer there, and X+ runs its FP32 form (256^3:
 // 75 -> 35 us).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
 // the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before.  The fused
-// sweep takes 215 us at 256^3 and 75 on the 256 x 128 x 128 duct (95 in the scaled form), CG's 44 at
+// sweep takes 206 us at 256^3 and 64 on the 256 x 128 x 128 duct (95 in the scaled form), CG's 41 at
 // 128^3 (64): bound by instruction issue and latency at three blocks of 128 threads per SM (two 270,
 // four 289 us).
 struct df {

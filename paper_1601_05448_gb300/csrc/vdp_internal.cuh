@@ -202,13 +202,17 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 
 // Unit layout for an nx x ny x nz grid in precision `prec`; zero arguments pick the defaults.
 // mode 0 (direct, default): units of up to 256 threads (whole rows, whole warps), one thread per
-// 16-byte vector of a row tile of threads * V / nx rows (V = 4 FP32, 2 FP64); a unit per 12288
-// cells, at least 3 and at most 12 per SM.  A unit reloads two planes at its start and adds a slot
-// to the sweep's final sum, so small grids want few units, large ones enough for several waves
-// (sweep and residual, us: 112 x 100 x 90 FP64 46.5 and 68 with 1824 units, 34.8 and 45 with 456;
-// 96^3 FP32 26.2 and 56 against 19.4 and 42; 256^3 FP32 93.6 and 265 with 1824, 89.9 and 246 with
-// 1368; 512^3 550 with 1824, 598 with 456).  Grids that the resident solve takes get 304 units, one
-// for each of its blocks.
+// 16-byte vector of a row tile of threads * V / nx rows (V = 4 FP32, 2 FP64), at most 12 units per
+// SM.  The z chunks are chosen for the fewest plane steps in a row: waves of resident units times the
+// planes of a chunk and the two that it reloads.  In FP64 three units of all kernels are resident on an
+// SM, else two of the density form's sweep and of the residual, three of the scaled sweep: there the
+// sum of both, weighted 2 : 3.  The steps follow the measured times of sweep and residual (us): 256^3 FP64
+// 206 and 288 with 896 units (78 steps), 215 and 334 with 1024 (102), 216 and 338 with 1408 (104);
+// 256^3 mixed 81 and 198 with 896 (63 at two per SM), 87 and 216 with 1408 (70); 512^3 mixed 508 and
+// 1426 with 1792 (456), 528 and 1563 with 1536 (528); 128^3 FP64 41 and 36 with 448 (12), 44 and 38
+// with 288 (17); 160^3 mixed, scaled sweep, 48 and 71 with 280 (25 at three per SM), 38 and 87 with
+// 480 (28), 38 and 62 with 440 (17).  Grids that the resident solve takes
+// get 304 units, one for each of its blocks.
 // mode 1 (TMA pipeline): FP64 512-thread units with about 2048 cells per plane, FP32/BF16 256
 // threads with about 1024; the row tile shrinks until four pipeline stages fit; stages default to
 // what fits (at most 6), or to 4 when that lets two units share an SM; about four waves.
@@ -268,16 +272,26 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
   const int uy = (ny + ty - 1) / ty;
   const long long ncell = (long long)nx * ny * nz;
   long long want = units > 0 ? units : 2LL * kSMs * per_sm;
-  if (units <= 0 && mode == 0) {
-    const long long by_cells = ncell / 12288 > 3LL * kSMs ? ncell / 12288 : 3LL * kSMs;
-    if (by_cells < want) want = by_cells;
-  }
   long long zc = (want + uy - 1) / uy;
-  if (units <= 0 && mode == 0 && ncell <= kResidentCells) {
+  if (units <= 0 && mode == 0 && ncell <= (prec == PREC_FP64 ? kResidentCells / 2 : kResidentCells)) {
     // the resident solve's blocks (two per SM) take one unit each where the planes allow it
     want = 2LL * kSMs;
     zc = want / uy;
     if (zc > 0 && zc < nz) zc = (nz + (nz + zc - 1) / zc - 1) / ((nz + zc - 1) / zc);  // equal chunks
+  } else if (units <= 0 && mode == 0) {
+    auto steps = [&](long long k, long long resident) {
+      return (k * uy + resident - 1) / resident * ((nz + k - 1) / k + 2);
+    };
+    long long best = 0;
+    zc = 1;
+    for (long long k = 1; k <= nz && k * uy <= want; ++k) {
+      const long long cost = prec == PREC_FP64 ? steps(k, 3LL * kSMs)
+                                               : 2 * steps(k, 2LL * kSMs) + 3 * steps(k, 3LL * kSMs);
+      if (best == 0 || cost <= best) {
+        best = cost;
+        zc = k;
+      }
+    }
   }
   if (zc > nz) zc = nz;
   if (zc < 1) zc = 1;
