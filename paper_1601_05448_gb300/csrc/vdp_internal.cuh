@@ -202,7 +202,7 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 
 // Unit layout for an nx x ny x nz grid in precision `prec`; zero arguments pick the defaults.
 // mode 0 (direct, default): units of up to 256 threads (whole rows, whole warps), one thread per
-// 16-byte vector of a row tile of threads * V / nx rows (V = 4 FP32, 2 FP64), at most 12 units per
+// 16-byte vector of a row tile of threads * V / nx rows (V = 4 FP32, 2 FP64), about 12 units per
 // SM.  The z chunks are chosen for the fewest plane steps in a row: waves of resident units times the
 // planes of a chunk and the two that it reloads.  In FP64 three units of all kernels are resident on an
 // SM, else two of the density form's sweep and of the residual, three of the scaled sweep: there the
@@ -284,7 +284,7 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
     };
     long long best = 0;
     zc = 1;
-    for (long long k = 1; k <= nz && k * uy <= want; ++k) {
+    for (long long k = 1; k <= nz && (k - 1) * uy < want; ++k) {
       const long long cost = prec == PREC_FP64 ? steps(k, 3LL * kSMs)
                                                : 2 * steps(k, 2LL * kSMs) + 3 * steps(k, 3LL * kSMs);
       if (best == 0 || cost <= best) {
