@@ -165,7 +165,7 @@ int configure_layout(vdp_ctx* c, int prec) {
   }
   d.rho32 = c->rho32;
   d.rho_lo = c->rho_lo;
-  d.g32 = d.form && prec == PREC_FP64 ? density_g32(c) : nullptr;
+  d.g32 = d.form ? density_g32(c) : nullptr;
   d.dsc = c->dsc;
   d.ncell = c->n;
   d.bx = c->bx;
@@ -334,7 +334,7 @@ bool ensure_while_graph(vdp_ctx* c, int prec) {
 }
 
 bool density_form(const vdp_ctx* c, int prec) {
-  return (prec == PREC_MIXED || (prec == PREC_FP64 && c->rho_lo_valid)) && c->rho32_valid &&
+  return prec == PREC_FP64 && c->rho32_valid &&
          (c->opts.method == VDP_METHOD_FIXED_POINT || c->opts.precond == VDP_PRECOND_SPECTRAL);
 }
 
@@ -355,13 +355,16 @@ int ensure_scaled(vdp_ctx* c, int prec) {
   return VDP_OK;
 }
 
-// W = D^1/2 (the scaled spectral passes and the V-cycle)
-static int ensure_omega(vdp_ctx* c) {
-  if (c->omega_valid) return VDP_OK;
+// W = D^1/2 (the fixed-point iteration and the V-cycle; unit, for spectral CG: over the power of two
+// of the first cell's)
+static int ensure_omega(vdp_ctx* c, bool unit) {
+  if (c->omega_valid && c->omega_unit == unit) return VDP_OK;
   const int s = ensure_sinv(c);
   if (s != VDP_OK) return s;
   if (!c->omega) VDP_CK(cudaMalloc((void**)&c->omega, sizeof(float) * (size_t)c->n));
-  VDP_CK(launch_omega(c->dg, c->sinv, c->n, c->omega, c->stream));
+  VDP_CK(launch_weights(nullptr, c->dg, c->sinv, c->n, unit, c->omega, nullptr, nullptr, 0,
+                        c->stream));
+  c->omega_unit = unit;
   c->omega_valid = true;
   return VDP_OK;
 }
@@ -402,17 +405,16 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   const int nxt = spectral_nx(c);  // x transform length (twice the cells in the duct)
   const int m = nxt / 2;
   const bool fixed = c->opts.method == VDP_METHOD_FIXED_POINT;
-  // density form: the stored residual is g = rho' r (fixed point) or r, z is unscaled and FP32, and
+  // density form: the input is rho' r (fixed point) or r, kept in FP32, z is unscaled and FP32, and
   // the inverse is that of s L_h: no weights
   const bool dens = density_form(c, prec);
-  const bool dens64 = dens && prec == PREC_FP64;
-  a->in = dens64 ? (const void*)density_g32(c) : c->r;
+  a->in = dens ? (const void*)density_g32(c) : c->r;
   // CG: z = W (-L_h)^-1 W rt, W = D^1/2.  Fixed point: with rt = D^-1/2 r the input weight
   // rho D^1/2 gives rho r, and z = damping D^1/2 (-L_h)^-1 (rho r) is the scaled form of the
   // paper's update p += damping L_h^-1 (rho r) (applied as p -= D^-1/2 x, x the sum of the z)
   a->out = c->za;
   // the fixed-point and density sweeps read z as FP32
-  a->f32 = (dens64 ? kInF32 : 0) | (fixed || dens ? kOutF32 : 0) | (fixed ? 0 : kEnergy);
+  a->f32 = (dens ? kInF32 : 0) | (fixed || dens ? kOutF32 : 0) | (fixed ? 0 : kEnergy);
   a->omega_in = dens ? nullptr : fixed ? c->rho_w : c->omega;
   a->omega_out = dens ? nullptr : c->omega;
   a->spec = c->spec;
@@ -425,8 +427,9 @@ void solve_spec_args(const vdp_ctx* c, int prec, SpecArgs* a) {
   a->nxd = c->nx;
   a->mirror = c->bc_x == VDP_BC_DUCT;
   a->ewt = a->mirror ? 0.5f : 1.f;
+  // (CG: the inverse of s L_h in both forms, O(1) whatever the box's units)
   a->scale = (float)((fixed ? c->opts.damping : 1.0) / ((double)nxt * c->ny * c->nz) /
-                     (dens ? density_scale(c) : 1.0));
+                     (dens || !fixed ? density_scale(c) : 1.0));
   a->st = c->st;
   a->I = c->desc;
   a->zunits = spectral_units(nxt, c->ny, c->nz);
@@ -471,7 +474,7 @@ int prepare_spectral_solve(vdp_ctx* c) {
   int s;
   if (c->hdesc.pc == PC_MG) {
     if (!c->mg) return VDP_EINVAL;
-    if ((s = ensure_omega(c)) != VDP_OK) return s;
+    if ((s = ensure_omega(c, false)) != VDP_OK) return s;
     if (!c->mg_valid) {
       VDP_CK(mg_setup(c->mg, c->bx, c->by, c->bz, c->sinv, c->stream));
       c->mg_valid = true;
@@ -479,12 +482,12 @@ int prepare_spectral_solve(vdp_ctx* c) {
     return VDP_OK;
   }
   const bool fixed = c->hdesc.pc == PC_FIXED;
-  if (fixed && !c->rho32_valid) return VDP_EINVAL;
+  if (fixed && !c->rho32_valid && !c->rho_w_valid) return VDP_EINVAL;
   if (c->hdesc.form) return VDP_OK;
-  if ((s = ensure_omega(c)) != VDP_OK) return s;
+  if ((s = ensure_omega(c, !fixed)) != VDP_OK) return s;
   if (fixed && !c->rho_w_valid) {
     if (!c->rho_w) VDP_CK(cudaMalloc((void**)&c->rho_w, sizeof(float) * (size_t)c->n));
-    VDP_CK(launch_rho_weight(c->rho32, c->dsc, density_scale(c), c->dg, c->sinv, c->n, c->rho_w, c->stream));
+    VDP_CK(launch_rho_weight(c->rho32, c->rho_lo, c->dsc, density_scale(c), c->dg, c->sinv, c->n, c->rho_w, c->stream));
     c->rho_w_valid = true;
   }
   return VDP_OK;
@@ -636,25 +639,39 @@ int vdp_set_options(vdp_ctx* c, const vdp_opts* o) {
       return mres;
     }
   }
-  if ((o->method == VDP_METHOD_FIXED_POINT || o->precond == VDP_PRECOND_SPECTRAL) && !c->rho32) {
-    cudaError_t e = cudaMalloc((void**)&c->rho32, sizeof(float) * (size_t)c->n);
-    if (e == cudaSuccess && !c->dsc) e = cudaMalloc((void**)&c->dsc, sizeof(double));
-    if (e != cudaSuccess) {
-      if (c->rho32) cudaFree(c->rho32);
-      c->rho32 = nullptr;
-      c->opts = old;
-      return cuda_fail(e, "vdp_set_options (density weight)");
+  if (o->method == VDP_METHOD_FIXED_POINT || o->precond == VDP_PRECOND_SPECTRAL) {
+    // what the form of these solves keeps of the density: FP64 the density in two FP32 parts, FP32
+    // the weights of the scaled passes (both methods', so that the method may be changed later)
+    const size_t bytes = sizeof(float) * (size_t)c->n;
+    cudaError_t e = cudaSuccess;
+    if (o->precision == VDP_FP64) {
+      if (!c->rho32) {
+        c->rho32_valid = false;
+        e = cudaMalloc((void**)&c->rho32, bytes);
+      }
+      if (e == cudaSuccess && !c->rho_lo) e = cudaMalloc((void**)&c->rho_lo, bytes);
+      if (e == cudaSuccess && !c->dsc) e = cudaMalloc((void**)&c->dsc, sizeof(double));
+      if (e != cudaSuccess) {
+        for (float** b : {&c->rho32, &c->rho_lo}) {
+          if (*b) cudaFree(*b);
+          *b = nullptr;
+        }
+        c->rho32_valid = false;
+      }
+    } else {
+      if (!c->omega) {
+        c->omega_valid = false;
+        e = cudaMalloc((void**)&c->omega, bytes);
+      }
+      if (e == cudaSuccess && !c->rho_w) {
+        c->rho_w_valid = false;
+        e = cudaMalloc((void**)&c->rho_w, bytes);
+      }
     }
-    c->rho32_valid = false;
-  }
-  if (c->rho32 && o->precision == VDP_FP64 && !c->rho_lo) {
-    const cudaError_t e = cudaMalloc((void**)&c->rho_lo, sizeof(float) * (size_t)c->n);
     if (e != cudaSuccess) {
-      c->rho_lo = nullptr;
       c->opts = old;
       return cuda_fail(e, "vdp_set_options (density)");
     }
-    c->rho_lo_valid = false;
   }
   c->stream = (cudaStream_t)o->stream;
   c->layout_dirty = true;
@@ -679,33 +696,33 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
   // the check and everything built from rho are launched together; the kernels after the check
   // write nothing when it fails, and the host waits once
   const int gen = ++c->density_gen, prec = c->opts.precision;
-  const bool kept = c->rho32_valid, kept_lo = c->rho_lo_valid;
-  float* rho_lo = prec == PREC_FP64 ? c->rho_lo : nullptr;
-  c->rho32_valid = c->rho32 != nullptr;  // as they will be (density_form looks at them)
-  c->rho_lo_valid = rho_lo != nullptr;
+  const bool kept = c->rho32_valid;
+  c->rho32_valid = c->rho32 != nullptr;  // as it will be (density_form looks at it)
   const bool scaled = !density_form(c, prec);
   c->rho32_valid = kept;
-  c->rho_lo_valid = kept_lo;
   VDP_CK(launch_check_density(src, c->n, gen, c->flag, c->stream));
   VDP_CK(launch_build_coefficients(src, c->nx, c->ny, c->nz, c->Lx / c->nx, c->Ly / c->ny,
                                    c->Lz / c->nz, c->bc_x == VDP_BC_DUCT, c->bx, c->by, c->bz,
-                                   scaled ? c->sinv : nullptr, c->dg, c->rho32, rho_lo, c->dsc,
+                                   scaled ? c->sinv : nullptr, c->dg, c->rho32, c->rho_lo, c->dsc,
                                    density_scale(c), c->flag, gen, c->stream));
+  const bool weights = scaled && c->rho_w;  // rho W needs rho itself
+  const bool unit = c->opts.method != VDP_METHOD_FIXED_POINT && c->opts.precond == VDP_PRECOND_SPECTRAL;
   if (scaled)
     VDP_CK(launch_scaled(prec, c->bx, c->by, c->bz, c->sinv, c->nx, c->ny, c->nz, c->sx, c->sy,
                          c->sz, c->sd, c->flag, gen, c->stream));
+  if (weights)
+    VDP_CK(launch_weights(src, c->dg, c->sinv, c->n, unit, c->omega, c->rho_w, c->flag, gen, c->stream));
   VDP_CK(cudaMemcpyAsync(c->hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   VDP_CK(cudaStreamSynchronize(c->stream));
   if (*c->hflag == gen) return VDP_EDENSITY;
   c->scaled_prec = scaled ? prec : -1;
   c->sinv_valid = scaled;
-  c->omega_valid = false;
-  c->rho_w_valid = false;
+  c->omega_valid = weights && c->omega;
+  c->omega_unit = unit;
+  c->rho_w_valid = weights;
   c->rho32_valid = c->rho32 != nullptr;
-  c->rho_lo_valid = rho_lo != nullptr;
   c->mg_valid = false;
-  // the form may change with them
-  if (c->rho32_valid != kept || c->rho_lo_valid != kept_lo) c->layout_dirty = true;
+  if (c->rho32_valid != kept) c->layout_dirty = true;  // the form may change with it
   c->has_density = true;
   return VDP_OK;
 }
@@ -863,7 +880,7 @@ int vdp_mg_apply(vdp_ctx* c, const double* g, double* out) {
     return VDP_EINVAL;
   int s;
   if ((s = ensure_mg(c)) != VDP_OK) return s;
-  if ((s = ensure_omega(c)) != VDP_OK) return s;
+  if ((s = ensure_omega(c, false)) != VDP_OK) return s;
   if (!c->mg_valid) {
     VDP_CK(mg_setup(c->mg, c->bx, c->by, c->bz, c->sinv, c->stream));
     c->mg_valid = true;

@@ -47,14 +47,14 @@ struct vdp_ctx {
   float2* spec = nullptr;          // half spectrum
   float* omega = nullptr;          // D^1/2 per cell (FP32)
   float* sptab = nullptr;          // twiddle and eigenvalue tables
-  bool omega_valid = false;        // omega matches the current density
+  bool omega_valid = false;        // omega matches the current density ...
+  bool omega_unit = false;         // ... over a power of two (spectral CG), or itself
   float* rho_w = nullptr;          // scaled fixed-point iteration: rho D^1/2 per cell (FP32)
   bool rho_w_valid = false;        // rho_w was computed from the current density
-  float* rho32 = nullptr;          // rho / 2^e0 (FP32), kept once a spectral method is selected
-  float* rho_lo = nullptr;         // rho / 2^e0 - rho32 (FP64 solves)
-  bool rho_lo_valid = false;       // rho_lo holds the current density
+  float* rho32 = nullptr;          // rho / 2^e0 (FP32), kept once an FP64 spectral method is selected
+  float* rho_lo = nullptr;         // rho / 2^e0 - rho32
   double* dsc = nullptr;           // kappa = 2^e0 s
-  bool rho32_valid = false;        // rho32 and dsc hold the current density
+  bool rho32_valid = false;        // the three hold the current density
   bool sinv_valid = false;         // sinv was computed from the current density
   vdp::MgHier* mg = nullptr;       // multigrid levels (VDP_PRECOND_MG, vdp_mg_apply)
   bool mg_valid = false;           // the levels were built from the current density
@@ -99,12 +99,12 @@ namespace vdp {
 int configure_layout(vdp_ctx* c, int prec);
 int ensure_scaled(vdp_ctx* c, int prec);  // no-op in the density form, which has none
 int ensure_sinv(vdp_ctx* c);
-// The inner solve runs in the density form (vdp_density.cu): the spectral inverse is its
-// preconditioner or iteration, the coefficients are not BF16, and the FP32 density (for FP64 with
-// its low part) is at hand.  A density that was set before the method or the precision was
-// selected is not: the solve then runs in the scaled form.
+// The inner solve runs in the density form (vdp_density.cu): it is an FP64 one, the spectral inverse
+// is its preconditioner or iteration, and the density's two FP32 parts are at hand.  For a density
+// that was set before the method or the precision was selected they are not: the solve then runs
+// in the scaled form.
 bool density_form(const vdp_ctx* c, int prec);
-// FP64 density form: z is FP32, so the second half of its buffer holds X+'s FP32 input
+// Density form: z is FP32, so the second half of its buffer holds X+'s FP32 input
 inline float* density_g32(const vdp_ctx* c) { return static_cast<float*>(c->za) + c->n; }
 // s of the density form: the power of 4 below hx^2
 inline double density_scale(const vdp_ctx* c) { return std::ldexp(1.0, 2 * std::ilogb(c->Lx / c->nx)); }

@@ -1,32 +1,45 @@
-// vdp_density.cuh -- the density form of the inner iteration, used with the constant-coefficient
+// vdp_density.cuh -- the density form of the FP64 inner iteration, used with the constant-coefficient
 // inverse (the paper's fixed-point iteration and spectrally preconditioned CG).
 //
 // The Jacobi-scaled form of vdp_kernels.cu exists for preconditioners that need a unit diagonal.
 // The spectral inverse does not: in unscaled variables its passes need no weights, and the
 // operator's three face coefficients per cell are functions of one field, the density, so a sweep
-// that reads rho (4 bytes, the neighbours' values from L1 / L2) computes them.  With
+// that reads rho (its neighbours' values from L1 / L2) computes them.  With
 //     rho' = rho / 2^e0 (e0 the exponent of the first cell),  s = 2^(2 m), m the exponent of hx,
 //     A' = kappa A, kappa = 2^e0 s:  face values (2 s / h_d^2) / (rho'_l + rho'_r),
 // an inner solve of (-A') X = r gives the correction p -= kappa X, whatever the units of rho and
-// of the box; kappa is a power of two, so the scaling rounds nothing.  Per cell and iteration of the
-// FP32 fixed-point solve this moves
-//     X+  g 4            (weights and rt: 8)        X-  z 4            (z and weight: 8)
-//     sweep  z, rho', g, X read, g, X written: 24   (z, three coefficients, rt, x: 32)
-// besides the half spectrum: 32 bytes instead of 48.  Fixed point: g = rho' r is the stored
-// residual (the right side of the paper's L_h dp = rho r), so X+ reads one field.
+// of the box; kappa is a power of two, so the scaling rounds nothing.
+//
+// FP32 inner solves keep the scaled form.  The rounding of the FP32 product is part of what decides
+// where a mixed solve stops (the FP64 residual after an inner solve, and the targets drawn from
+// it): with the coefficients computed in FP32 the fixed-point iteration took another number of
+// iterations on 7 of 60 inputs of 256^3, on 1 of 40 of 192^3 and 1 of 5 of 512^3, and its pressures
+// moved by up to 1.2e-9.
+//
+// z comes out of the FP32 transforms, so it is an FP32 field in this solve too; r, X, d and q are
+// FP64.  The product A' z in FP64 instructions bounds the sweep by the FP64 pipe (8 instructions
+// per cell at 2 per clock and SM: 282 us at 256^3, where its bytes take 118).  Here coefficients
+// and product are pairs of FP32 numbers (unevaluated sums hi + lo, about 47 bits): rho' as such a
+// pair, the quotient by a Newton step and a corrected remainder, the differences of z exact, the
+// products by FMA with their rounding errors, the six terms summed with the errors carried along.
+// Only the update of the FP64 fields is FP64: three instructions per cell (fixed point), four
+// (CG).  The sweep also leaves rho' r in FP32 for the X+ pass, which read r and rho' and narrowed
+// the product itself: four bytes more here, eight fewer there, and X+ runs its FP32 form (256^3:
+// 75 -> 35 us).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
+// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before: over 484
+// spectral and 12 fixed-point inputs of 32^3 to 256^3 no pressure was further from the one in 64 bits
+// than with the FP64 product.
 //
 // The march is that of sweep_stencil_direct: a thread owns 16 bytes of one row and walks a z chunk,
-// x neighbours come by shuffle, the rows above and below and the plane above by loads.  Written
-// with plain loads the sweep waited for memory (ncu at 256^3: 8.2 of 13 stall cycles per issue on
-// long-scoreboard, 47 % of the DRAM rate): each thread therefore fetches its operands of the next
-// plane by cp.async into slots of shared memory that only it reads, so no barrier is needed, no
-// registers are held while they fly, and the arithmetic of one plane covers the latency of the
-// next.  The x neighbours at row and warp ends come the same way (loaded at their use, they cost
-// every plane a trip to L2).  Sums, products and Newton steps of the four cells run as paired FP32
-// instructions, and the fluxes through the x faces and the upper z face are computed once for both
-// cells.  The fused fixed-point sweep (scaled form with stored coefficients / plain loads / cp.async /
-// cp.async with the x neighbours / units in whole waves): 512^3 662 / 595 / 555 / 514 / 507 us, 256^3
-// 110 / 103 / 92 / 87 / 81; 24 bytes a cell in 507 us are 0.94 of the copy bandwidth.
+// x neighbours come by shuffle, the rows above and below and the plane above by loads.  Each thread
+// fetches its operands of the next plane by cp.async into slots of shared memory that only it
+// reads, so no barrier is needed, no registers are held while they fly, and the arithmetic of one
+// plane covers the latency of the next.  The x neighbours at row and warp ends come the same way
+// (loaded at their use, they cost every plane a trip to L2).  Sums, products and Newton steps of the
+// four cells run as paired FP32 instructions, and the fluxes through the x faces and the upper z face
+// are computed once for both cells.  The fused sweep takes 206 us at 256^3 and 64 on the 256 x 128 x
+// 128 duct (95 in the scaled form), CG's 41 at 128^3 (64): bound by instruction issue and latency at
+// three blocks of 128 threads per SM (two 270, four 289 us).
 #pragma once
 
 #include "vdp_device.cuh"
@@ -71,22 +84,6 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
   return r;
 }
 
-// c / (a + b) of a face: the approximate reciprocal and one Newton step (nc = -c; the reciprocal of
-// the negated sum leaves the residual 1 - s y as one FMA).  Symmetric in a and b, so the two cells
-// of a face compute the same value, and each lane of the paired form the scalar form's.
-__device__ __forceinline__ float face(float nc, float a, float b) {
-  const float s = a + b, y = rcp_approx(-s);
-  const float w = nc * y;
-  return fmaf(w, fmaf(s, y, 1.f), w);
-}
-__device__ __forceinline__ f2 face2(f2 nc, f2 a, f2 b) {
-  const f2 s = add2(a, b);
-  const float2 v = up2(s);
-  const f2 y = pk(rcp_approx(-v.x), rcp_approx(-v.y));
-  const f2 w = mul2(nc, y);
-  return fma2(w, fma2(s, y, pk(1.f, 1.f)), w);
-}
-
 __device__ __forceinline__ void fetch16(void* smem, const float* g) {  // through L1
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
                    (unsigned)__cvta_generic_to_shared(smem)),
@@ -111,241 +108,7 @@ __device__ __forceinline__ void fetch_wait_previous() {
   asm volatile("cp.async.wait_group 1;" ::: "memory");
 }
 
-// Operand streams of a plane z (16 bytes per thread each): z+1 and the rows above and below of the
-// marched field and of the density, then what the kind needs besides.
-enum Stream { S_UP, S_UA, S_UB, S_RP, S_RA, S_RB, S_0, S_1, S_2 };
-template <int KIND> struct Streams { static constexpr int kCount = KIND == 0 ? 8 : (KIND == 1 ? 6 : 9); };
-
-// NC: z and d_old are not written while the kernel runs (read-only loads).
-// KIND 0: the fixed-point iteration, z = damping (-L')^-1 g: X += z, g -= rho' (-A') z and the sum
-// of r^2 / D' (the norm of the scaled residual, which steers the inner stop).
-// KIND 1, 2: CG, d = z + beta d_old (1: first iteration, d = z), q = (-A') d and the sum of d q.
-template <int KIND, bool NC = true>
-__device__ __forceinline__ void sweep_density(const InstDesc& I, const InstState* st, int unit,
-                                              float& part, ulonglong2* slots) {
-  constexpr bool kFixed = KIND == 0, kOld = KIND == 2;
-  constexpr int NS = Streams<KIND>::kCount;
-  const int nx = I.nx, ny = I.ny, nz = I.nz;
-  const int tpr = nx / kV;
-  const int tile = unit % I.uy, chunk = unit / I.uy;
-  const int row = threadIdx.x / tpr;
-  const int x0 = (threadIdx.x - row * tpr) * kV;
-  const int yr = tile * I.ty + row;
-  const bool active = row < I.ty && yr < ny;
-  const int y = active ? yr : ny - 1;  // idle threads follow a valid row (shuffles need them)
-  const int z0 = (int)((long long)chunk * nz / I.zc), z1 = (int)((long long)(chunk + 1) * nz / I.zc);
-  part = 0.f;
-  if (z0 >= z1 || !__any_sync(0xffffffffu, active)) return;  // (no block barrier below)
-  const int lane = threadIdx.x & 31;
-  const bool row_start = x0 == 0, row_end = x0 + kV == nx;
-  const bool left_load = lane == 0 || row_start, right_load = lane == 31 || row_end;
-  const bool wall_l = I.duct && row_start, wall_r = I.duct && row_end;
-  const float nx1 = -I.ch[0];
-  const f2 ny2 = pk(-I.ch[1], -I.ch[1]), nz2 = pk(-I.ch[2], -I.ch[2]);
-  const float beta = (float)st->beta;
-  const f2 beta2 = pk(beta, beta);
-  const bool first = st->inner_iters == 0;
-  const float* rho = I.rho32;
-  const float* src = static_cast<const float*>(I.za);
-  const float* dold = static_cast<const float*>(st->parity ? I.d1 : I.d0);
-  float* dnew = static_cast<float*>(st->parity ? I.d0 : I.d1);
-  float* q = static_cast<float*>(I.q);
-  float* g = static_cast<float*>(I.r);
-  float* X = static_cast<float*>(I.x);
-  const long long plane = (long long)nx * ny;
-  const long long dym = y == 0 ? (long long)(ny - 1) * nx : -(long long)nx;
-  const long long dyp = y == ny - 1 ? -(long long)(ny - 1) * nx : (long long)nx;
-  const int dxl = row_start ? nx - 1 : -1, dxr = row_end ? -x0 : kV;
-  const long long cell0 = (long long)y * nx + x0;
-  const long long dz_last = plane * (nz - 1);  // from plane nz - 1 back to plane 0
-  // stream k of stage b of this thread
-  auto slot = [&](int b, int k) { return slots + (b * NS + k) * blockDim.x + threadIdx.x; };
-  // x neighbours beyond the warp or the row: value k (z, rho', d_old), side 0 left and 1 right
-  float* edges = reinterpret_cast<float*>(slots + kStages * NS * blockDim.x);
-  auto edge = [&](int b, int k, int side) {
-    return edges + ((b * 3 + k) * 2 + side) * blockDim.x + threadIdx.x;
-  };
-  auto fetch = [&](int b, int z, long long o) {  // the operands of plane z (cells at o)
-    if (left_load) {
-      fetch4(edge(b, 0, 0), src + o + dxl);
-      fetch4(edge(b, 1, 0), rho + o + dxl);
-      if (kOld) fetch4(edge(b, 2, 0), dold + o + dxl);
-    }
-    if (right_load) {
-      fetch4(edge(b, 0, 1), src + o + dxr);
-      fetch4(edge(b, 1, 1), rho + o + dxr);
-      if (kOld) fetch4(edge(b, 2, 1), dold + o + dxr);
-    }
-    const long long op = z == nz - 1 ? o - dz_last : o + plane;
-    fetch16(slot(b, S_UP), src + op);
-    fetch16(slot(b, S_UA), src + o + dym);
-    fetch16(slot(b, S_UB), src + o + dyp);
-    fetch16(slot(b, S_RP), rho + op);
-    fetch16(slot(b, S_RA), rho + o + dym);
-    fetch16(slot(b, S_RB), rho + o + dyp);
-    if (kFixed) {  // rewritten by this thread only, after this plane's copies have landed
-      fetch16_once(slot(b, S_0), g + o);
-      if (!first) fetch16_once(slot(b, S_1), X + o);
-    }
-    if (kOld) {
-      fetch16(slot(b, S_0), dold + op);
-      fetch16(slot(b, S_1), dold + o + dym);
-      fetch16(slot(b, S_2), dold + o + dyp);
-    }
-  };
-  auto ldg2 = [](const float* p, f2& a, f2& b) {
-    const ulonglong2* v = reinterpret_cast<const ulonglong2*>(p);
-    const ulonglong2 t = NC ? __ldg(v) : *v;
-    a = t.x;
-    b = t.y;
-  };
-  long long o = (long long)z0 * plane + cell0;
-  fetch(0, z0, o);
-  fetch_commit();
-  // the field and the density of planes z0 - 1 and z0; the flux through the face between them
-  f2 u[2], r[2], bzl[2], fz[2];
-  {
-    const long long om = z0 == 0 ? o + dz_last : o - plane;
-    f2 um[2], rm[2];
-    ldg2(src + om, um[0], um[1]);
-    ldg2(src + o, u[0], u[1]);
-    ldg2(rho + om, rm[0], rm[1]);
-    ldg2(rho + o, r[0], r[1]);
-    if (kOld) {
-      f2 dm[2], dc[2];
-      ldg2(dold + om, dm[0], dm[1]);
-      ldg2(dold + o, dc[0], dc[1]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        um[h] = fma2(beta2, dm[h], um[h]);
-        u[h] = fma2(beta2, dc[h], u[h]);
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      bzl[h] = face2(nz2, rm[h], r[h]);
-      fz[h] = mul2(bzl[h], sub2(u[h], um[h]));
-    }
-  }
-  f2 sum[2] = {0ull, 0ull};
-  int b = 0;
-  for (int z = z0; z < z1; ++z) {
-    if (z + 1 < z1) fetch(b ^ 1, z + 1, o + plane);
-    fetch_commit();
-    fetch_wait_previous();
-    // x neighbours: adjacent lanes, or what was fetched at row ends and warp ends
-    const float2 u01 = up2(u[0]), u23 = up2(u[1]), r01 = up2(r[0]), r23 = up2(r[1]);
-    float ul = __shfl_up_sync(0xffffffffu, u23.y, 1), ur = __shfl_down_sync(0xffffffffu, u01.x, 1);
-    float rl = __shfl_up_sync(0xffffffffu, r23.y, 1), rr = __shfl_down_sync(0xffffffffu, r01.x, 1);
-    if (left_load) {
-      ul = kOld ? fmaf(beta, *edge(b, 2, 0), *edge(b, 0, 0)) : *edge(b, 0, 0);
-      rl = *edge(b, 1, 0);
-    }
-    if (right_load) {
-      ur = kOld ? fmaf(beta, *edge(b, 2, 1), *edge(b, 0, 1)) : *edge(b, 0, 1);
-      rr = *edge(b, 1, 1);
-    }
-    // faces and fluxes b (u_k - u_{k-1}) through the five x faces of the four cells
-    const float b0 = wall_l ? 0.f : face(nx1, rl, r01.x), b1 = face(nx1, r01.x, r01.y);
-    const float b2 = face(nx1, r01.y, r23.x), b3 = face(nx1, r23.x, r23.y);
-    const float b4 = wall_r ? 0.f : face(nx1, r23.y, rr);
-    const float f0 = b0 * (u01.x - ul), f1 = b1 * (u01.y - u01.x), fm = b2 * (u23.x - u01.y);
-    const float f3 = b3 * (u23.y - u23.x), f4 = b4 * (ur - u23.y);
-    f2 a[2] = {pk(f1 - f0, fm - f1), pk(f3 - fm, f4 - f3)};  // A' u, accumulated
-    f2 D[2] = {pk(b0 + b1, b1 + b2), pk(b2 + b3, b3 + b4)};
-    ulonglong2 t = *slot(b, S_UP);
-    f2 un[2] = {t.x, t.y};
-    if (kOld) {
-      t = *slot(b, S_0);
-      un[0] = fma2(beta2, t.x, un[0]);
-      un[1] = fma2(beta2, t.y, un[1]);
-    }
-    t = *slot(b, S_RP);
-    const f2 rn[2] = {t.x, t.y};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {  // upper z face: its flux is the next plane's lower one
-      const f2 bz = face2(nz2, r[h], rn[h]);
-      const f2 f = mul2(bz, sub2(un[h], u[h]));
-      a[h] = add2(a[h], sub2(f, fz[h]));
-      fz[h] = f;
-      if (kFixed) D[h] = add2(D[h], add2(bzl[h], bz));
-      bzl[h] = bz;
-    }
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {  // the rows above and below
-      t = *slot(b, side ? S_UB : S_UA);
-      f2 v[2] = {t.x, t.y};
-      if (kOld) {
-        t = *slot(b, side ? S_2 : S_1);
-        v[0] = fma2(beta2, t.x, v[0]);
-        v[1] = fma2(beta2, t.y, v[1]);
-      }
-      t = *slot(b, side ? S_RB : S_RA);
-      const f2 rv[2] = {t.x, t.y};
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const f2 by = face2(ny2, rv[h], r[h]);
-        a[h] = fma2(by, sub2(v[h], u[h]), a[h]);
-        if (kFixed) D[h] = add2(D[h], by);
-      }
-    }
-    if constexpr (kFixed) {
-      t = *slot(b, S_0);
-      f2 gv[2] = {t.x, t.y}, xv[2] = {u[0], u[1]};
-      if (!first) {
-        t = *slot(b, S_1);
-        xv[0] = add2(t.x, u[0]);
-        xv[1] = add2(t.y, u[1]);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        gv[h] = fma2(r[h], a[h], gv[h]);
-        const float2 d = up2(D[h]), rv = up2(r[h]);
-        const f2 w = mul2(gv[h], pk(rcp_approx(rv.x), rcp_approx(rv.y)));
-        sum[h] = fma2(mul2(w, w), pk(rcp_approx(d.x), rcp_approx(d.y)), sum[h]);
-      }
-      if (active) {
-        *reinterpret_cast<ulonglong2*>(g + o) = make_ulonglong2(gv[0], gv[1]);
-        *reinterpret_cast<ulonglong2*>(X + o) = make_ulonglong2(xv[0], xv[1]);
-      }
-    } else {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        a[h] = sub2(0ull, a[h]);
-        sum[h] = fma2(u[h], a[h], sum[h]);
-      }
-      if (active) {
-        *reinterpret_cast<ulonglong2*>(dnew + o) = make_ulonglong2(u[0], u[1]);
-        *reinterpret_cast<ulonglong2*>(q + o) = make_ulonglong2(a[0], a[1]);
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      u[h] = un[h];
-      r[h] = rn[h];
-    }
-    o += plane;
-    b ^= 1;
-  }
-  const float2 s = up2(add2(sum[0], sum[1]));
-  part = active ? s.x + s.y : 0.f;
-}
-
-// ---- the FP64 inner solve ------------------------------------------------------------------------
-// z comes out of the FP32 transforms, so it is an FP32 field in this solve too; r, X, d and q are
-// FP64.  The product A' z in FP64 instructions bounds the sweep by the FP64 pipe (8 instructions
-// per cell at 2 per clock and SM: 282 us at 256^3, where its bytes take 118).  Here coefficients
-// and product are pairs of FP32 numbers (unevaluated sums hi + lo, about 47 bits): rho' as such a
-// pair, the quotient by a Newton step and a corrected remainder, the differences of z exact, the
-// products by FMA with their rounding errors, the six terms summed with the errors carried along.
-// Only the update of the FP64 fields is FP64: three instructions per cell (fixed point), four
-// (CG).  The sweep also leaves rho' r in FP32 for the X+ pass, which read r and rho' and narrowed
-// the product itself: four bytes more here, eight fewer there, and X+ runs its FP32 form (256^3:
-// 75 -> 35 us).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
-// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before.  The fused
-// sweep takes 206 us at 256^3 and 64 on the 256 x 128 x 128 duct (95 in the scaled form), CG's 41 at
-// 128^3 (64): bound by instruction issue and latency at three blocks of 128 threads per SM (two 270,
-// four 289 us).
+// An unevaluated sum h + l
 struct df {
   f2 h, l;
 };
@@ -411,8 +174,11 @@ __device__ __forceinline__ void accumulate_minus(df& acc, const dflux& f) {
   acc.l = add2(acc.l, add2(s.l, f.nl));
 }
 
+// Operands of a plane z (16 bytes per thread each): z + 1 and the rows above and below of z and of both
+// parts of the density, then the two FP64 fields.
 enum Stream64 { T_UP, T_UA, T_UB, T_HP, T_HA, T_HB, T_LP, T_LA, T_LB, T_P0, T_P1, T_Q0, T_Q1, kStreams64 };
 
+// NC: z is not written while the kernel runs (read-only loads).
 // thread: this thread's place in the unit (a block may hold two units).
 // FIXED: X += z, r -= (-A') z and the sum of r^2 / D' (FP32, steers the inner stop).
 // CG: d = z + beta d_old, q = (-A') z + beta q_old, and the sum of d q.
@@ -648,14 +414,9 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
   part = active ? (FIXED ? (double)sumf : sum) : 0.0;
 }
 
-inline size_t density_smem(bool fixed, int threads) {  // operand slots and x edges
-  const int streams = fixed ? Streams<0>::kCount : Streams<2>::kCount;
-  return (sizeof(ulonglong2) * streams + 6 * sizeof(float)) * (size_t)kStages * threads;
-}
-
 constexpr int kDensity64Threads = kDirectThreads / 2;  // four cells per thread, the FP64 layout has two
 
-inline size_t density64_smem(int threads) {
+inline size_t density64_smem(int threads) {  // operand slots and x edges
   return (sizeof(ulonglong2) * kStreams64 + 6 * sizeof(float)) * (size_t)kStages * threads;
 }
 

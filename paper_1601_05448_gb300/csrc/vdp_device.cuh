@@ -40,6 +40,14 @@ __device__ __forceinline__ float narrow_pow2(double v, int p) {
   return __uint_as_float(bits);
 }
 
+// v times 2^p to binary64 (results in the normal range)
+__device__ __forceinline__ double widen_scaled(float v, int p) {
+  const unsigned b = __float_as_uint(v);
+  const unsigned sign = b & 0x80000000u, e = (b >> 23) & 0xffu, frac = b & 0x7fffffu;
+  const unsigned hi = e == 0 ? sign : (sign | ((e + 1023u - 127u + (unsigned)p) << 20) | (frac >> 3));
+  return __hiloint2double((int)hi, (int)(e == 0 ? 0u : frac << 29));
+}
+
 // approximate reciprocal (1 ulp)
 __device__ __forceinline__ float rcp_approx(float s) {
   float y;
@@ -215,6 +223,18 @@ __device__ __forceinline__ double quotient(double c, double s) {
   return fma(w, fma(e, e, e), w);
 }
 
+// The power of two for the FP32 inner variables when the mean square of rt = D^-1/2 r, summed in FP32
+// (rrt), lies where an inner solve's reductions or its largest cells would take it out of the FP32
+// range: what brings the root mean square to about one, from ||f - <f>||^2 (fn2, an FP64 sum) and the
+// first cell's D.  0: none (any magnitude that a solve in ordinary units has; a power of two would not
+// change its results either, but the repeated sweep costs time).
+__device__ __forceinline__ int inner_scale(const InstDesc& I, const InstState* st, double fn2, double rrt) {
+  const double n = (double)I.ncell;
+  if (st->precision == PREC_FP64 || I.mode != 0 || !(fn2 > 0.0) || !isfinite(fn2)) return 0;
+  if (rrt > 0x1p-60 * n && rrt < 0x1p80 * n) return 0;
+  return (ilogb(I.dg[0]) - ilogb(fn2 / n)) / 2;
+}
+
 // ---- phase transitions (run by thread 0 of the last unit) -------------------------------------
 
 static __device__ __noinline__ void transition(const InstDesc& I, InstState* st, int phase,
@@ -234,6 +254,7 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
       break;
     case PH_RES64: {
       const double rr64 = S[0], rrt = S[1];
+      const bool first = st->first_res != 0;
       if (st->first_res) st->sum_p = S[2];  // later: summed by the correction sweep
       if (st->first_res) {
         st->fn2 = S[3];
@@ -245,6 +266,13 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
         st->zero_sol = 1;
         st->rel_res = 0.0;
         st->phase = PH_FINAL;
+        break;
+      }
+      if (first && st->texp == 0 && inner_scale(I, st, fn2, rrt) != 0) {
+        // the sweep is repeated with the scaled variables (p, and what it adds, are as they were)
+        st->texp = inner_scale(I, st, fn2, rrt);
+        st->first_res = 1;
+        st->outer -= 1;
         break;
       }
       const double rel = sqrt(rr64 / fn2);

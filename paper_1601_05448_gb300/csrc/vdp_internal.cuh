@@ -61,6 +61,8 @@ struct __align__(16) InstState {
   int precision;
   int fault;           // a unit's bounded wait expired (reported as VDP_ETIMEOUT)
   int cheb_j;          // Chebyshev sweep index (1 .. cheb_k - 1)
+  int texp;            // FP32 inner solve, direct sweeps: the inner variables are 2^texp times D^-1/2 r
+                       // and its corrections; 0 unless <rt, rt> would leave the FP32 range
   int p_set;           // p holds an iterate: the caller's guess, or a correction was applied
                        // (from p = 0 the first correction writes p without reading it)
   double rz;           // <rt, z> (preconditioned inner product; = <rt, rt> for Jacobi)
@@ -93,7 +95,7 @@ struct InstDesc {
   int nunits_f;        // flat work units per sweep
   int zc;              // z chunks: stencil unit u = (row tile u % uy, z chunk u / uy)
   int mode;            // stencil sweep: 0 = direct register march, 1 = TMA-staged pipeline
-  int form;            // inner variables: 0 = Jacobi-scaled, 1 = density form (vdp_density.cu)
+  int form;            // inner variables: 0 = Jacobi-scaled, 1 = density form (vdp_density.cu; FP64)
   int duct;            // density form: the faces at the x ends carry no coefficient
   float ch[3], cl[3];  // density form: face factors 2 s / h_d^2 as FP32 pairs hi + lo
   long long ncell;
@@ -111,8 +113,8 @@ struct InstDesc {
   const void* sz;
   const void* sd;      // BF16 only: diagonal correction of the stored inner operator
   const float* rho32;  // density form: rho / 2^e0 in FP32
-  const float* rho_lo; // density form, FP64: rho / 2^e0 - rho32
-  float* g32;          // density form, FP64: the X+ pass's input in FP32 (rho' r, CG: r), written by
+  const float* rho_lo; // density form: rho / 2^e0 - rho32
+  float* g32;          // density form: the X+ pass's input in FP32 (rho' r, CG: r), written by
                        // every sweep that writes r
   const double* dsc;   // density form: kappa = 2^e0 s (the inner operator is kappa A)
   void* x;             // inner solution (correction), inner type
@@ -177,9 +179,8 @@ constexpr int kSMs = 152;                 // GB300
 constexpr size_t kSmemPerSM = 227 * 1024; // shared memory per SM available to CTAs
 constexpr size_t kSmemBudget = 225 * 1024;
 
-// Largest grid that one resident launch solves (vdp_resident.cu; resident_supported() has the line
-// for each kind of solve).
-constexpr long long kResidentCells = 2500000;
+// Largest grid that one resident launch solves (vdp_resident.cu; figures at resident_supported()).
+constexpr long long kResidentCells = 1250000;
 
 struct Layout {
   int mode;            // stencil sweep variant (0 direct, 1 TMA pipeline)
@@ -273,7 +274,7 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
   const long long ncell = (long long)nx * ny * nz;
   long long want = units > 0 ? units : 2LL * kSMs * per_sm;
   long long zc = (want + uy - 1) / uy;
-  if (units <= 0 && mode == 0 && ncell <= (prec == PREC_FP64 ? kResidentCells / 2 : kResidentCells)) {
+  if (units <= 0 && mode == 0 && ncell <= kResidentCells) {
     // the resident solve's blocks (two per SM) take one unit each where the planes allow it
     want = 2LL * kSMs;
     zc = want / uy;

@@ -506,10 +506,10 @@ __device__ __forceinline__ void flat_kind_unit(const InstDesc& I, int unit) {
     }
     case PH_CORRECT: {
       double ps[1] = {0.0};
-      if (I.form)
-        sweep_correct<T, true>(I, c0, c1, sn.p_set == 0, ps[0]);
+      if (sizeof(T) == 8 && I.form)
+        sweep_correct<T, sizeof(T) == 8>(I, c0, c1, sn.p_set == 0, sn.texp, ps[0]);
       else
-        sweep_correct<T, false>(I, c0, c1, sn.p_set == 0, ps[0]);
+        sweep_correct<T, false>(I, c0, c1, sn.p_set == 0, sn.texp, ps[0]);
       store_partials<1, double>(ps, I.part, I.nunits_f, unit);
       break;
     }
@@ -548,9 +548,8 @@ __global__ void __launch_bounds__(kDirectThreads, Res64Occ<T>::kMinBlocks) k_res
   stencil_kind_unit<T, T, 0, 2>(insts[ur.inst], ur.unit, nullptr);
 }
 
-// The same for the instances in the density form.
-template <class T>
-__global__ void __launch_bounds__(kDirectThreads, Res64Occ<T>::kMinBlocks) k_res64_density(
+// The same for the instances in the density form (FP64).
+__global__ void __launch_bounds__(kDirectThreads, Res64Occ<double>::kMinBlocks) k_res64_density(
     const InstDesc* __restrict__ insts, const UnitRef* __restrict__ units) {
   const UnitRef ur = units[blockIdx.x];
   const InstDesc& I = insts[ur.inst];
@@ -558,7 +557,7 @@ __global__ void __launch_bounds__(kDirectThreads, Res64Occ<T>::kMinBlocks) k_res
   const InstState& sn = block_state(st);
   if (sn.phase != PH_RES64 || I.form == 0) return;
   double acc[kSlots] = {0.0, 0.0, 0.0, 0.0};
-  sweep_res64_direct<T, true>(I, &sn, ur.unit, acc);
+  sweep_res64_direct<double, true>(I, &sn, ur.unit, acc);
   store_partials<kSlots, double>(acc, I.part, I.nunits, ur.unit);
   finish_sweep(I, st, PH_RES64, I.nunits);
 }
@@ -739,10 +738,8 @@ cudaError_t prepare_step(int prec, int mode, size_t smem_bytes) {
 
 cudaError_t launch_res64(int prec, int form, const InstDesc* desc, const UnitRef* units, int nunits,
                          int threads, cudaStream_t s) {
-  if (form && prec == PREC_FP64)
-    k_res64_density<double><<<nunits, threads, 0, s>>>(desc, units);
-  else if (form)
-    k_res64_density<float><<<nunits, threads, 0, s>>>(desc, units);
+  if (form)
+    k_res64_density<<<nunits, threads, 0, s>>>(desc, units);
   else if (prec == PREC_FP64)
     k_res64_direct<double><<<nunits, threads, 0, s>>>(desc, units);
   else
@@ -753,7 +750,7 @@ cudaError_t launch_res64(int prec, int form, const InstDesc* desc, const UnitRef
 cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
                            const UnitRef* units, int nunits, int threads, size_t smem_bytes,
                            cudaStream_t s) {
-  if (kind >= kSweepDensityCg) return launch_density(prec, kind, desc, units, nunits, threads, s);
+  if (kind >= kSweepDensityCg) return launch_density(kind, desc, units, nunits, threads, s);
   void* fn = stencil_fn(prec, mode, kind);
   void* args[] = {(void*)&desc, (void*)&units};
   return cudaLaunchKernel(fn, dim3(nunits), dim3(threads), args, smem_bytes, s);

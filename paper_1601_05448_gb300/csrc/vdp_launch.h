@@ -12,8 +12,8 @@ namespace vdp {
 // that take (bad, gen) then write nothing (null: not gated).
 cudaError_t launch_check_density(const double* rho, long long n, int gen, int* bad, cudaStream_t s);
 // face coefficients on the low faces (spacings h_d; duct: no flux through the x ends) and D; with
-// sinv also D^-1/2, with rho32 the density form's FP32 density (with rho_lo what it rounds off)
-// and dsc[0] = kappa = 2^e0 s
+// sinv also D^-1/2, with rho32 the density form's FP32 density, what it rounds off (rho_lo) and
+// dsc[0] = kappa = 2^e0 s
 cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
                                       double hy, double hz, int duct, double* bx, double* by,
                                       double* bz, double* sinv, double* dg, float* rho32,
@@ -23,11 +23,13 @@ cudaError_t launch_sinv(const double* dg, long long n, double* sinv, cudaStream_
 cudaError_t launch_scaled(int prec, const double* bx, const double* by, const double* bz,
                           const double* sinv, int nx, int ny, int nz, void* sx, void* sy, void* sz,
                           void* sd, const int* bad, int gen, cudaStream_t s);
-// W = D^1/2, and rho W (the scaled fixed-point iteration's input weight) from rho32 and kappa
-cudaError_t launch_omega(const double* dg, const double* sinv, long long n, float* omega,
-                         cudaStream_t s);
-cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double s2, const double* dg,
-                              const double* sinv, long long n, float* out, cudaStream_t s);
+// W = D^1/2 (omega; unit: over the first cell's power of two) and rho W (rho_w, the scaled fixed-point iteration's input weight); null: not
+// stored.  launch_rho_weight takes rho from the density form's fields instead.
+cudaError_t launch_weights(const double* rho, const double* dg, const double* sinv, long long n,
+                           bool unit, float* omega, float* rho_w, const int* bad, int gen, cudaStream_t s);
+cudaError_t launch_rho_weight(const float* rho32, const float* rho_lo, const double* dsc, double s2,
+                              const double* dg, const double* sinv, long long n, float* rho_w,
+                              cudaStream_t s);
 cudaError_t launch_apply(const double* bx, const double* by, const double* bz, const double* p,
                          int nx, int ny, int nz, double* out, cudaStream_t s);
 // ctl: also the control words of a resident solve (or null)
@@ -48,7 +50,7 @@ inline int stencil_kind(const InstDesc& d) {
   return d.pc == PC_FIXED ? 2 : (d.pc == PC_CHEB ? 1 : 0);
 }
 cudaError_t prepare_density();  // shared-memory limits on the current device
-cudaError_t launch_density(int prec, int kind, const InstDesc* desc, const UnitRef* units, int nunits,
+cudaError_t launch_density(int kind, const InstDesc* desc, const UnitRef* units, int nunits,
                            int threads, cudaStream_t s);
 cudaError_t launch_stencil(int prec, int mode, int kind, const InstDesc* desc,
                            const UnitRef* units, int nunits, int threads, size_t smem_bytes,

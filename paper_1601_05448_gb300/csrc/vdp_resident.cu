@@ -102,7 +102,7 @@ __device__ __noinline__ void x_forward(const SpecArgs& a, const Tables& tb, floa
   }
 }
 
-template <int M1, int M2>
+template <int M1, int M2, bool WEIGHT>
 __device__ __noinline__ void x_inverse(const SpecArgs& a, const Tables& tb, float2* buf) {
   constexpr int RY = inv_rows_per_block<M1, M2>(), SB = pad_stride(M2 * (M1 + 1));
   const int rows = a.ny * a.nz, per = rows_each(rows, RY);
@@ -110,7 +110,7 @@ __device__ __noinline__ void x_inverse(const SpecArgs& a, const Tables& tb, floa
   for (int g = blockIdx.x; (long long)g * per < rows; g += gridDim.x) {
     const long long row = (long long)g * per + r;
     const bool live = r < per && row < rows;
-    x_inv_rows<float, M1, M2, true, false>(a, tb, buf + (r < RY ? r : 0) * SB,
+    x_inv_rows<float, M1, M2, true, WEIGHT>(a, tb, buf + (r < RY ? r : 0) * SB,
                                              a.spec + (live ? row : 0) * a.nxp, row, live, t, [] {});
     __syncthreads();
   }
@@ -238,16 +238,17 @@ __device__ __forceinline__ void x_forward_any(const SpecArgs& a, const Tables& t
   }
 }
 
+template <bool WEIGHT>
 __device__ __forceinline__ void x_inverse_any(const SpecArgs& a, const Tables& tb, float2* buf) {
   switch (a.nx / 2) {
-    case 16: x_inverse<4, 4>(a, tb, buf); break;
-    case 24: x_inverse<4, 6>(a, tb, buf); break;
-    case 32: x_inverse<4, 8>(a, tb, buf); break;
-    case 48: x_inverse<6, 8>(a, tb, buf); break;
-    case 64: x_inverse<8, 8>(a, tb, buf); break;
-    case 96: x_inverse<8, 12>(a, tb, buf); break;
-    case 128: x_inverse<8, 16>(a, tb, buf); break;
-    default: x_inverse<16, 16>(a, tb, buf); break;
+    case 16: x_inverse<4, 4, WEIGHT>(a, tb, buf); break;
+    case 24: x_inverse<4, 6, WEIGHT>(a, tb, buf); break;
+    case 32: x_inverse<4, 8, WEIGHT>(a, tb, buf); break;
+    case 48: x_inverse<6, 8, WEIGHT>(a, tb, buf); break;
+    case 64: x_inverse<8, 8, WEIGHT>(a, tb, buf); break;
+    case 96: x_inverse<8, 12, WEIGHT>(a, tb, buf); break;
+    case 128: x_inverse<8, 16, WEIGHT>(a, tb, buf); break;
+    default: x_inverse<16, 16, WEIGHT>(a, tb, buf); break;
   }
 }
 
@@ -292,8 +293,8 @@ size_t table_bytes(int nx, int ny, int nz) {
 
 // ---- the solve ------------------------------------------------------------------------------------
 
-// What the instance runs: Jacobi CG in the scaled form, or in the density form the fixed-point
-// iteration or spectral CG.
+// What the instance runs: Jacobi CG, the fixed-point iteration or spectral CG.  The last two run in the
+// density form in FP64 and in the scaled form in FP32, Jacobi CG always in the scaled form.
 enum ResidentKind { R_JACOBI = 0, R_FIXED = 1, R_SPECTRAL = 2 };
 
 template <class T, bool DENS>
@@ -305,16 +306,10 @@ __device__ __noinline__ void unit_res64(const InstDesc& I, const InstState& sn, 
 }
 
 template <class T, int KIND>
-__device__ __noinline__ void unit_stencil(const InstDesc& I, const InstState& sn, int u,
-                                          ulonglong2* stages, double* slots) {
+__device__ __noinline__ void unit_stencil(const InstDesc& I, const InstState& sn, int u, double* slots) {
   T part[1] = {0};
   if constexpr (KIND == R_FIXED) {
-    sweep_density<0, false>(I, &sn, u, part[0], stages);
-  } else if constexpr (KIND == R_SPECTRAL) {
-    if (sn.inner_iters > 0)
-      sweep_density<2, false>(I, &sn, u, part[0], stages);
-    else
-      sweep_density<1, false>(I, &sn, u, part[0], stages);
+    sweep_stencil_direct<T, T, false, 2, false>(I, &sn, u, part[0]);
   } else {
     if (sn.inner_iters > 0)
       sweep_stencil_direct<T, T, false, 1, false>(I, &sn, u, part[0]);
@@ -358,7 +353,7 @@ __device__ __noinline__ void unit_flat(const InstDesc& I, const InstState& sn, i
     if (phase == PH_MEANF)
       sweep_meanf(I, c0, c1, sum[0]);
     else
-      sweep_correct<T, DENS>(I, c0, c1, sn.p_set == 0, sum[0]);
+      sweep_correct<T, DENS>(I, c0, c1, sn.p_set == 0, sn.texp, sum[0]);
     store_partials<1, double>(sum, slots, I.nunits_f, u);
   }
 }
@@ -367,7 +362,7 @@ template <class T, int KIND>
 __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOBI ? 1 : 2)
     k_resident(const InstDesc* desc, const __grid_constant__ SpecArgs spec, ResidentCtl* ctl,
                unsigned max_sweeps) {
-  constexpr bool DENS = KIND != R_JACOBI;
+  constexpr bool SPEC = KIND != R_JACOBI, DENS = SPEC && sizeof(T) == 8;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(16) unsigned char desc_bytes[sizeof(InstDesc)];
   for (int k = threadIdx.x; k < (int)(sizeof(InstDesc) / 4); k += blockDim.x)
@@ -381,7 +376,7 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
   const float2 *wy = nullptr, *wz = nullptr;
   const float* lz = nullptr;
   float2* work = reinterpret_cast<float2*>(smem);
-  if constexpr (DENS) tb = shared_tables(spec, reinterpret_cast<float2*>(smem), wy, wz, lz, work);
+  if constexpr (SPEC) tb = shared_tables(spec, reinterpret_cast<float2*>(smem), wy, wz, lz, work);
   ulonglong2* stages = reinterpret_cast<ulonglong2*>(work);
   __syncthreads();
   GridBarrier bar{ctl, 0u};
@@ -392,7 +387,7 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
     double* slots = I.part + (done & 1u) * kResidentSlots;
     int nparts = I.nunits;
     bool applied = false;  // the preconditioner's sweep was part of this round
-    if (DENS && phase == PH_SPEC) {
+    if (SPEC && phase == PH_SPEC) {
       x_forward_any(spec, tb, work);
       if (!(ok = bar.sync())) break;
       lines_any<0>(spec.ny, spec, tb, wy, nullptr, work, slots);
@@ -401,7 +396,7 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
       if (!(ok = bar.sync())) break;
       lines_any<1>(spec.ny, spec, tb, wy, nullptr, work, slots);
       if (!(ok = bar.sync())) break;
-      x_inverse_any(spec, tb, work);
+      x_inverse_any<!DENS>(spec, tb, work);  // scaled form: z = W x
       if (KIND == R_FIXED) {  // always followed by the sweep: one transition for both
         if (!(ok = bar.sync())) break;
         applied = true;
@@ -413,13 +408,13 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
     if (phase == PH_RES64) {
       for (int u = blockIdx.x; u < I.nunits; u += gridDim.x) unit_res64<T, DENS>(I, sn, u, slots);
     } else if (phase == PH_STENCIL) {
-      if constexpr (DENS && sizeof(T) == 8) {
+      if constexpr (DENS) {
         for (int u = blockIdx.x; u < I.nunits; u += 2 * gridDim.x)
           two_units_density64<KIND == R_FIXED>(I, sn, u, u + gridDim.x < I.nunits ? u + gridDim.x : -1,
                                                stages, slots);
       } else {
         for (int u = blockIdx.x; u < I.nunits; u += gridDim.x)
-          unit_stencil<T, KIND>(I, sn, u, stages, slots);
+          unit_stencil<T, KIND>(I, sn, u, slots);
       }
     } else if (phase != PH_SPEC) {
       nparts = I.nunits_f;
@@ -477,26 +472,25 @@ size_t resident_smem(int prec, int kind, const SpecArgs& a) {
   size_t b = 40960;
   for (int n : {a.ny, a.nz})
     if (line_bytes(n) > b) b = line_bytes(n);
-  const size_t d = prec == PREC_FP64 ? density64_smem(kResThreads) : density_smem(kind == R_FIXED, kResThreads);
-  return table_bytes(a.nx, a.ny, a.nz) + (d > b ? d : b);
+  if (prec == PREC_FP64 && density64_smem(kResThreads) > b) b = density64_smem(kResThreads);
+  return table_bytes(a.nx, a.ny, a.nz) + b;
 }
 
 constexpr int kMaxDevices = 64;
 
 }  // namespace
 
-// Where the line lies (us a solve to 1e-9, resident and in a graph of launches): FP32 fixed point
-// 96^3 481 and 723, 128^3 702 and 881, 96 x 128 x 192 920 and 959, 128 x 128 x 192 1088 and 1088;
-// FP64 fixed point 96^3 685 and 846, 128^3 1090 and 1113; spectral CG FP64 96^3 1407 and 1534,
-// 128^3 2537 and 2236; FP64 Jacobi 112 x 100 x 100 22450 and 23160, FP32 128^3 20770 and 18960: the
-// FP32 fixed-point iteration up to kResidentCells, the others up to half of that.
+// Where the line lies (us a solve to 1e-9, resident and in a graph of launches): FP32 fixed point 64^3
+// 440 and 554, 96^3 640 and 643, 128 x 96 x 96 672 and 683, 128 x 128 x 96 850 and 803, 128^3 980 and
+// 925; FP64 fixed point 64^3 390 and 506, 96^3 750 and 728, 128 x 96 x 96 784 and 751; spectral CG FP32
+// 96^3 1314 and 1343, 128 x 96 x 96 1452 and 1427, FP64 64^3 860 and 1073, 96^3 1589 and 1526; Jacobi FP32
+// 96^3 9918 and 12437, 128 x 96 x 96 12559 and 14297, FP64 17367 and 18645, 24908 and 24921.
 bool resident_supported(const InstDesc& d, int prec) {
-  const bool fixed32 = d.pc == PC_FIXED && prec == PREC_MIXED;
-  if (prec == PREC_MIXED_BF16 || d.mode != 0 || d.ncell > (fixed32 ? kResidentCells : kResidentCells / 2) ||
+  if (prec == PREC_MIXED_BF16 || d.mode != 0 || d.ncell > kResidentCells ||
       kSlots * d.nunits > kResidentSlots || d.nunits_f > kResidentSlots)
     return false;
   if (d.pc == PC_JACOBI) return d.form == 0;
-  return d.form == 1 && (d.pc == PC_FIXED || d.pc == PC_SPECTRAL) && d.ny <= kMaxLine && d.nz <= kMaxLine;
+  return d.form == (prec == PREC_FP64 ? 1 : 0) && (d.pc == PC_FIXED || d.pc == PC_SPECTRAL) && d.ny <= kMaxLine && d.nz <= kMaxLine;
 }
 
 cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, const SpecArgs& spec,

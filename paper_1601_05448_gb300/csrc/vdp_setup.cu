@@ -1,7 +1,7 @@
 // vdp_setup.cu -- what vdp_set_density builds from rho: the FP64 face coefficients
 // b_d = 2 / (rho_l + rho_r) / h_d^2 on the low faces, the diagonal D (sum of the six faces of a
-// cell), the Jacobi scaling D^-1/2, the scaled inner coefficients, and the FP32 density of the
-// density-form sweeps (vdp_density.cu).
+// cell), the Jacobi scaling D^-1/2, the scaled inner coefficients, the weights of the scaled spectral
+// passes, and the density as two FP32 numbers for the FP64 density-form sweeps (vdp_density.cu).
 //
 // What bounds these kernels.  The FP64 pipe of this GPU issues 2 FMA per clock and SM, 1/64 of the
 // FP32 rate: an IEEE double division costs about ten such instructions and a reciprocal square
@@ -134,7 +134,7 @@ __global__ void k_check_density(const double* __restrict__ rho, long long n, int
 }
 
 // b_d[c] = 2 / (rho[c - e_d] + rho[c]) / h_d^2 on the low d-face of every cell; with rho32 also the
-// FP32 density, scaled by the power of two of the first cell's (2^-e0), with rho_lo what that
+// FP32 density, scaled by the power of two of the first cell's (2^-e0), rho_lo what that
 // rounds off, and dsc[0] = 2^e0 s2, the factor between the density-form operator and A
 // (vdp_density.cu).
 // duct: the face at the x ends (slot x = 0, shared by x = 0 and x = Lx) carries no flux.
@@ -174,10 +174,9 @@ __global__ void __launch_bounds__(kSetupThreads)
     if (rho32) {
       const float2 h = make_float2(narrow_rn_pow2(r.x, -e0), narrow_rn_pow2(r.y, -e0));
       *reinterpret_cast<float2*>(rho32 + c) = h;
-      if (rho_lo)
-        *reinterpret_cast<float2*>(rho_lo + c) =
-            make_float2(narrow_rn_pow2(r.x - widen_pow2(h.x, e0), -e0),
-                        narrow_rn_pow2(r.y - widen_pow2(h.y, e0), -e0));
+      *reinterpret_cast<float2*>(rho_lo + c) =
+          make_float2(narrow_rn_pow2(r.x - widen_pow2(h.x, e0), -e0),
+                      narrow_rn_pow2(r.y - widen_pow2(h.y, e0), -e0));
     }
     lo = r;
   }
@@ -298,21 +297,26 @@ __global__ void k_diag_correction(const __nv_bfloat16* __restrict__ sx,
   }
 }
 
-// W = D^1/2 = D D^-1/2 per cell (FP32), and the fixed-point iteration's weight rho W
-__global__ void k_omega(const double* __restrict__ dg, const double* __restrict__ sinv,
-                        long long n, float* __restrict__ omega) {
+// W = D^1/2 = D D^-1/2 per cell (FP32; unit: over the power of two of the first cell's, so that the
+// preconditioner, which CG knows up to a factor only, stays in the FP32 range), and with rho the scaled fixed-point iteration's weight rho W
+// (each null: not stored).  rho comes from the density itself, or where a context was set up for the
+// density form from the two FP32 parts kept there (48 bits; kappa / s = 2^e0).
+__global__ void k_weights(const double* __restrict__ rho, const float* __restrict__ rho32,
+                          const float* __restrict__ rho_lo, const double* __restrict__ dsc, double is2,
+                          const double* __restrict__ dg, const double* __restrict__ sinv, long long n, bool unit,
+                          float* __restrict__ omega, float* __restrict__ rho_w, const int* bad, int gen) {
+  if (rejected(bad, gen)) return;
+  const double one = unit ? ldexp(1.0, -(ilogb(dg[0]) / 2)) : 1.0;
+  const double scale = rho || !rho_w ? 1.0 : dsc[0] * is2;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x)
-    omega[c] = __double2float_rn(dg[c] * sinv[c]);
-}
-
-__global__ void k_rho_weight(const float* __restrict__ rho32, const double* __restrict__ dsc,
-                             double is2, const double* __restrict__ dg,
-                             const double* __restrict__ sinv, long long n, float* __restrict__ out) {
-  const double scale = dsc[0] * is2;  // 2^e0
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n;
-       c += (long long)gridDim.x * blockDim.x)
-    out[c] = __double2float_rn((double)rho32[c] * scale * (dg[c] * sinv[c]));
+       c += (long long)gridDim.x * blockDim.x) {
+    const double w = dg[c] * sinv[c];
+    if (omega) omega[c] = __double2float_rn(w * one);
+    if (rho_w) {
+      const double r = rho ? rho[c] : ((double)rho32[c] + (double)rho_lo[c]) * scale;
+      rho_w[c] = __double2float_rn(r * w);
+    }
+  }
 }
 
 // ---- host launchers ---------------------------------------------------------------------------
@@ -389,15 +393,18 @@ cudaError_t launch_scaled(int prec, const double* bx, const double* by, const do
   return cudaGetLastError();
 }
 
-cudaError_t launch_omega(const double* dg, const double* sinv, long long n, float* omega,
-                         cudaStream_t s) {
-  k_omega<<<flat_grid(n), 256, 0, s>>>(dg, sinv, n, omega);
+cudaError_t launch_weights(const double* rho, const double* dg, const double* sinv, long long n,
+                           bool unit, float* omega, float* rho_w, const int* bad, int gen, cudaStream_t s) {
+  k_weights<<<flat_grid(n), 256, 0, s>>>(rho, nullptr, nullptr, nullptr, 1.0, dg, sinv, n, unit, omega,
+                                          rho_w, bad, gen);
   return cudaGetLastError();
 }
 
-cudaError_t launch_rho_weight(const float* rho32, const double* dsc, double s2, const double* dg,
-                              const double* sinv, long long n, float* out, cudaStream_t s) {
-  k_rho_weight<<<flat_grid(n), 256, 0, s>>>(rho32, dsc, 1.0 / s2, dg, sinv, n, out);
+cudaError_t launch_rho_weight(const float* rho32, const float* rho_lo, const double* dsc, double s2,
+                              const double* dg, const double* sinv, long long n, float* rho_w,
+                              cudaStream_t s) {
+  k_weights<<<flat_grid(n), 256, 0, s>>>(nullptr, rho32, rho_lo, dsc, 1.0 / s2, dg, sinv, n, false,
+                                          nullptr, rho_w, nullptr, 0);
   return cudaGetLastError();
 }
 

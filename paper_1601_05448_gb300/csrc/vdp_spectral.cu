@@ -43,6 +43,25 @@
 
 namespace vdp {
 
+// X+ with one group of RY rows per block, everything loaded at its use: the weighted FP32 rows whose
+// transform has 512 values.  512^3: 261 us; with the rows staged as below, their weights then waited for
+// behind a few large blocks, 293 (256^3: 45.5 and 36 the other way round).
+template <class T, int M1, int M2, bool MIRROR>
+__global__ void __launch_bounds__(M1 * rows_per_block<M1, M2>(), 1024 / (M1 * rows_per_block<M1, M2>()))
+    k_spec_x_fwd(SpecArgs a) {
+  constexpr int RY = rows_per_block<M1, M2>();
+  constexpr int SX = x_row_stride<M1, M2>();
+  __shared__ float2 sx[RY * SX];  // per row: the exchange, then the transformed row
+  if (!spec_active(a)) return;
+  const Tables tb = tables(a);
+  const int t = threadIdx.x % M1, r = threadIdx.x / M1;
+  const long long row = (long long)a.z0 * a.ny + (long long)blockIdx.x * RY + r;
+  const bool live = row < (long long)a.z1 * a.ny;
+  float2* out = a.spec + row * a.nxp;
+  x_fwd_rows<T, M1, M2, MIRROR>(a, tb, sx + r * SX, static_cast<const T*>(a.in) + row * a.nxd, row, live, t,
+                                 [&](int k, float2 X) { out[k] = X; }, [] {});
+}
+
 // X+ of FP64 rows on a persistent grid: groups of RY rows (group = block, block + grid, ...) of
 // the planes [z0, z1), tables in shared memory; at least 768 resident threads per SM (80
 // registers a thread).  The 512^3 FP64 solve: 47.3 ms against 49.2 ms with one group of rows
@@ -357,6 +376,8 @@ void factor(int n, int* m1, int* m2) {
 
 using SpecKernel = void (*)(SpecArgs);
 
+constexpr int kXDirect = 256;  // nx / 2 of the weighted FP32 rows that k_spec_x_fwd transforms
+
 template <class T>
 SpecKernel x_kernel(int m, bool inverse, bool mirror, bool weight, int* threads) {
   int m1, m2;
@@ -371,6 +392,11 @@ SpecKernel x_kernel(int m, bool inverse, bool mirror, bool weight, int* threads)
     if (inverse)                                                                            \
       return mirror ? k_spec_x_inv_persistent<T, M1, M2, true, false>                       \
                     : k_spec_x_inv_persistent<T, M1, M2, false, false>;                     \
+    if constexpr (sizeof(T) == 4 && M1 * M2 == kXDirect)                                    \
+      if (weight) {                                                                         \
+        *threads = M1 * rows_per_block<M1, M2>();                                           \
+        return mirror ? k_spec_x_fwd<T, M1, M2, true> : k_spec_x_fwd<T, M1, M2, false>;     \
+      }                                                                                     \
     if constexpr (sizeof(T) == 8)                                                           \
       return mirror ? k_spec_x_fwd_persistent<T, M1, M2, true>                              \
                     : k_spec_x_fwd_persistent<T, M1, M2, false>;                            \
@@ -444,7 +470,7 @@ bool x_f64(int prec, bool inv, const SpecArgs& a) {
 
 SpecKernel x_pass_kernel(int prec, bool inv, const SpecArgs& a, int* threads) {
   const int m = a.nx / 2;
-  const bool weight = inv && a.omega_out;
+  const bool weight = inv ? a.omega_out != nullptr : a.omega_in != nullptr;
   return x_f64(prec, inv, a) ? x_kernel<double>(m, inv, a.mirror != 0, weight, threads)
                              : x_kernel<float>(m, inv, a.mirror != 0, weight, threads);
 }
@@ -453,6 +479,10 @@ SpecKernel x_pass_kernel(int prec, bool inv, const SpecArgs& a, int* threads) {
 // prepared), else one block per group of rows.
 long long x_grid(int prec, bool inv, const SpecArgs& a, long long rows) {
   int threads = 0;
+  if (!inv && a.omega_in && a.nx / 2 == kXDirect && !x_f64(prec, inv, a)) {
+    const int ry = x_rows_per_block(kXDirect, false);
+    return (rows + ry - 1) / ry;
+  }
   const SpecKernel k = x_pass_kernel(prec, inv, a, &threads);
   const int dev = current_device(), ry = x_rows_per_block(a.nx / 2, inv || !x_f64(prec, inv, a));
   if (!k || dev < 0 || ry <= 0) return 0;

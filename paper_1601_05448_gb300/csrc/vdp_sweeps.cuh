@@ -126,8 +126,8 @@ __device__ __forceinline__ long long flat_begin(const InstDesc& I, int u) {
 // before the first use (one vector per thread per round left these sweeps latency bound).
 constexpr int kFlatU = 4;
 
-__device__ __forceinline__ double widen_t(float v) { return widen(v); }
-__device__ __forceinline__ double widen_t(double v) { return v; }
+__device__ __forceinline__ double widen_t(float v, int p) { return widen_scaled(v, p); }
+__device__ __forceinline__ double widen_t(double v, int) { return v; }
 
 // <f>, ||f||^2; p := 0 unless p is the caller's initial guess.
 static __device__ void sweep_meanf(const InstDesc& I, long long c0, long long c1, double& sum) {
@@ -152,12 +152,12 @@ static __device__ void sweep_meanf(const InstDesc& I, long long c0, long long c1
   sum = s[0] + s[1];
 }
 
-// p -= D^-1/2 x (x in the inner type; DENS, the density form: p -= kappa x); sums the new p (the
-// final gauge needs its mean).  fresh: p is still the zero start (never written), so it is not
-// read.
-template <class T, bool DENS>
+// p -= D^-1/2 x (x in the inner type, FP32 with the factor 2^texp; DENS, the density form: p -=
+// kappa x); sums the new p (the final gauge needs its mean).  fresh: p is still the zero start (never
+// written), so it is not read.
+template <class T, bool DENS = false>
 __device__ void sweep_correct(const InstDesc& I, long long c0, long long c1, bool fresh,
-                              double& psum) {
+                              int texp, double& psum) {
   const T* x = static_cast<const T*>(I.x);
   const double kappa = DENS ? I.dsc[0] : 0.0;
   double s = 0.0;
@@ -181,8 +181,8 @@ __device__ void sweep_correct(const InstDesc& I, long long c0, long long c1, boo
       const long long c = cb + u * step;
       if (c < c1) {
         double2 p = pv[u];
-        p.x = fma(-sv[u].x, widen_t(xa[u]), p.x);
-        p.y = fma(-sv[u].y, widen_t(xb[u]), p.y);
+        p.x = fma(-sv[u].x, widen_t(xa[u], -texp), p.x);
+        p.y = fma(-sv[u].y, widen_t(xb[u], -texp), p.y);
         *reinterpret_cast<double2*>(I.p + c) = p;
         s += p.x + p.y;
       }
@@ -535,9 +535,9 @@ __device__ void sweep_stencil_direct(const InstDesc& I, const InstState* st, int
 // diagonal form r = (f - <f>) + D p_c - sum of b_face p_neighbour (D stored per cell): one FMA
 // per term, 8 FP64 operations per cell against 13 for the face-difference form; in the mixed
 // precisions the scaling rt = D^-1/2 r is an FP32 product; the norms are summed in FP32.
-// What the residual sweep hands to the inner solve in the density form (DENS), from the FP64
-// residual of a cell: fixed point g = rho' r (FP64 inner type: r) and r^2 / D' (D' = kappa D), CG r
-// and r^2.
+// What the residual sweep hands to the inner solve in the density form (DENS, FP64): r, X+'s FP32
+// input (fixed point rho' r, CG r), and the norm's terms: fixed point r^2 / D' (D' = kappa D), CG
+// r^2.
 struct DensityResidual {
   bool fixed;
   int ek;      // kappa = 2^ek x mk
@@ -558,6 +558,7 @@ struct DensityResidual {
 template <class T, bool FIRST, bool DENS, bool F0 = false>
 __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* st, int unit,
                                             double (&acc)[kSlots]) {
+  static_assert(!DENS || IsF64<T>::value, "the density form is an FP64 one");
   constexpr int VR = VecW<T>::V;  // cells per thread (4 for FP32 inner, 2 for FP64)
   const int nx = I.nx, ny = I.ny, nz = I.nz;
   const int tpr = nx / VR;
@@ -574,6 +575,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
   const bool row_start = x0 == 0, row_end = x0 + VR == nx;
   const int xl = row_start ? nx - 1 : x0 - 1, xr = row_end ? 0 : x0 + VR;
   const double mu = st->mu_f;
+  const int texp = st->texp;
   const double* p = I.p;
   T* rt = static_cast<T*>(I.r);
   const DensityResidual dr = DENS ? DensityResidual(I) : DensityResidual();
@@ -646,13 +648,8 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       T t0, t1;
       float r0f = narrow(res0), r1f = narrow(res1), t0f, t1f;
       if constexpr (DENS) {
-        if constexpr (IsF64<T>::value) {  // r itself
-          t0 = res0;
-          t1 = res1;
-        } else {
-          t0 = rh.x * r0f;
-          t1 = rh.y * r1f;
-        }
+        t0 = res0;
+        t1 = res1;
         t0f = dr.fixed ? r0f * r0f * dr.inv_diag(dg.x) : r0f * r0f;  // the norm's terms
         t1f = dr.fixed ? r1f * r1f * dr.inv_diag(dg.y) : r1f * r1f;
       } else if constexpr (IsF64<T>::value) {
@@ -662,12 +659,12 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
         t1f = narrow(t1);
       } else {  // the inner residual in FP32: D^-1/2 r from the FP32 factors (the inner solve's
                 // own rounding), no FP64 multiply
-        t0 = t0f = narrow(si.x) * r0f;
-        t1 = t1f = narrow(si.y) * r1f;
+        t0 = t0f = narrow_pow2(si.x, texp) * r0f;
+        t1 = t1f = narrow_pow2(si.y, texp) * r1f;
       }
       if (active) {
         store2(rt + o, t0, t1);
-        if constexpr (DENS && IsF64<T>::value)
+        if constexpr (DENS)
           *reinterpret_cast<float2*>(I.g32 + o) = make_float2(rh.x * r0f, rh.y * r1f);
         a0 = fmaf(r0f, r0f, fmaf(r1f, r1f, a0));
         a1 = DENS ? a1 + (t0f + t1f) : fmaf(t0f, t0f, fmaf(t1f, t1f, a1));
@@ -703,6 +700,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
   const int yr = tile * I.ty + row;
   const int z0 = (int)((long long)chunk * nz / I.zc), z1 = (int)((long long)(chunk + 1) * nz / I.zc);
   const double mu = st->mu_f;
+  const int texp = st->texp;
   T* rt = static_cast<T*>(I.r);
   const DensityResidual dr = DENS ? DensityResidual(I) : DensityResidual();
   double a0 = 0;
@@ -735,12 +733,8 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
         const float2 rh = diag ? c.rho[h / 2] : make_float2(1.f, 1.f);
         float2 d = make_float2(1.f, 1.f);
         if (diag) d = make_float2(dr.inv_diag(c.w[h / 2].x), dr.inv_diag(c.w[h / 2].y));
-        if constexpr (IsF64<T>::value) {
-          store2(rt + o + h, f0, f1);
-          *reinterpret_cast<float2*>(I.g32 + o + h) = make_float2(rh.x * r0, rh.y * r1);
-        } else {
-          store2(rt + o + h, rh.x * r0, rh.y * r1);
-        }
+        store2(rt + o + h, f0, f1);
+        *reinterpret_cast<float2*>(I.g32 + o + h) = make_float2(rh.x * r0, rh.y * r1);
         a0 = fma(f0, f0, fma(f1, f1, a0));
         a1f = fmaf(r0 * d.x, r0, fmaf(r1 * d.y, r1, a1f));
       } else if constexpr (IsF64<T>::value) {
@@ -753,7 +747,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
                 // factors; ||f - <f>||^2, the denominator of every relative residual of the
                 // solve, stays an FP64 sum (any magnitude of f)
         const double2 si = c.w[h / 2];
-        const float t0 = narrow(si.x) * narrow(f0), t1 = narrow(si.y) * narrow(f1);
+        const float t0 = narrow_pow2(si.x, texp) * narrow(f0), t1 = narrow_pow2(si.y, texp) * narrow(f1);
         store2(rt + o + h, t0, t1);
         a0 = fma(f0, f0, fma(f1, f1, a0));
         a1 = fmaf(t0, t0, fmaf(t1, t1, a1));
