@@ -44,6 +44,8 @@ __device__ __forceinline__ double face_quotient(const FaceFactor& f, double s) {
   if (f.e == kSlow || !mid_range(s)) return f.c / s;
   const unsigned lo = (unsigned)__double2loint(s);
   const int E = exponent_of(s) - 1023;
+  // each factor may be far out while the quotient is itself near the ends of the range, or past them
+  if ((unsigned)(f.e - E + 1000) > 2000u) return f.c / s;
   const float sh = mantissa_f(s);
   const float sl = (__uint_as_float(0x3f800000u | ((lo & 0x1fffffffu) >> 6)) - 1.f) * 0x1p-23f;
   const float y = rcp_approx(sh);
