@@ -360,7 +360,8 @@ void vdp_batch_destroy(vdp_batch *batch);   /* NULL-safe */
 /*
  * Queue a solve of ctx (after vdp_set_density; options precision equal to the batch's):
  * A p = rhs - <rhs> to relative residual tol, as vdp_solve.  rhs and p: device pointers, 16-byte
- * aligned, valid until the member is done.  VDP_EINVAL if ctx is already a member.
+ * aligned, valid until the member is done.  VDP_EINVAL if ctx is already a member.  The solve runs
+ * with the options that ctx has now: options set while it is queued apply to later solves.
  */
 int vdp_batch_add(vdp_batch *batch, vdp_ctx *ctx, const double *rhs, double *p, double tol);
 

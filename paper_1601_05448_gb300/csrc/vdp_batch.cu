@@ -38,7 +38,12 @@ struct Member {
   double* p;
   double tol;
   bool done;
-  bool alone;  // runs by itself, not in the shared launches
+  // how it runs, and what that takes, as the context's options were when it was added: they may be
+  // changed while the member is queued
+  enum How { SHARED, LOOP, RESIDENT } how;  // in the shared launches, or by itself in one of two forms
+  InstDesc desc;
+  SpecArgs spec;  // of members with the spectral passes
+  int slab;
 };
 
 }  // namespace
@@ -95,11 +100,11 @@ int grow(X** ptr, long long* cap, long long need) {
   return VDP_OK;
 }
 
-// Whether a member runs by itself (see above) instead of in the shared launches.
-bool runs_alone(vdp_batch* b, const Member& m) {
-  vdp_ctx* c = m.ctx;
-  return !b->persistent && c->hdesc.pc >= PC_SPECTRAL &&
-         (resident_solve(c, b->prec) || ensure_while_graph(c, b->prec));
+// How a new member runs (see above).
+Member::How how_to_run(vdp_batch* b, vdp_ctx* c) {
+  if (b->persistent || c->hdesc.pc < PC_SPECTRAL) return Member::SHARED;
+  if (resident_solve(c, b->prec)) return Member::RESIDENT;
+  return ensure_while_graph(c, b->prec) ? Member::LOOP : Member::SHARED;
 }
 
 int rebuild(vdp_batch* b) {
@@ -108,7 +113,6 @@ int rebuild(vdp_batch* b) {
     if (!b->members[i].done) b->active.push_back((int)i);
   const int n = (int)b->active.size();
   b->nshared = 0;
-  for (int k : b->active) b->members[k].alone = runs_alone(b, b->members[k]);
   long long cd = b->cap_desc;
   int s;
   if ((s = grow(&b->d_desc, &cd, std::max(n, 1))) != VDP_OK) return s;
@@ -127,12 +131,12 @@ int rebuild(vdp_batch* b) {
   std::vector<UnitRef> su, fu;
   for (int k = 0; k < n; ++k) {
     const Member& m = b->members[b->active[k]];
-    InstDesc d = m.ctx->hdesc;
+    InstDesc d = m.desc;
     d.rhs = m.rhs;
     d.p = m.p;
-    d.remaining = &b->d_ctl->remaining;
+    d.remaining = m.how == Member::SHARED ? &b->d_ctl->remaining : nullptr;
     desc[k] = d;
-    if (m.alone) continue;
+    if (m.how != Member::SHARED) continue;
     ++b->nshared;
     for (int u = 0; u < d.nunits; ++u) su.push_back(UnitRef{k, u});
     for (int u = 0; u < d.nunits_f; ++u) fu.push_back(UnitRef{k, u});
@@ -178,8 +182,8 @@ int capture(vdp_batch* b, int pairs) {
     // residual and sweep kernels (each kernel leaves the other forms' units alone)
     int nscaled = 0, nfixed = 0, ncheb = 0, ndfixed = 0, ndcg = 0;
     for (int k : b->active) {
-      if (b->members[k].alone) continue;
-      const InstDesc& d = b->members[k].ctx->hdesc;
+      if (b->members[k].how != Member::SHARED) continue;
+      const InstDesc& d = b->members[k].desc;
       if (d.form) {
         ++(d.pc == PC_FIXED ? ndfixed : ndcg);
         continue;
@@ -202,23 +206,22 @@ int capture(vdp_batch* b, int pairs) {
       // runs concurrently (small grids alone would leave most SMs idle).
       int nspec = 0;
       for (int k : b->active)
-        nspec += !b->members[k].alone && b->members[k].ctx->hdesc.pc >= PC_SPECTRAL;
+        nspec += b->members[k].how == Member::SHARED && b->members[k].desc.pc >= PC_SPECTRAL;
       const int nb = std::min(nspec, (int)vdp_batch::kBranches);
       if (nb > 0 && e == cudaSuccess) e = cudaEventRecord(b->fork, b->cap);
       for (int j = 0; j < nb && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(b->aux[j], b->fork, 0);
       int slot = 0;
       for (size_t k = 0; k < b->active.size() && e == cudaSuccess; ++k) {
-        const vdp_ctx* c = b->members[b->active[k]].ctx;
-        if (b->members[b->active[k]].alone || c->hdesc.pc < PC_SPECTRAL) continue;
+        const Member& m = b->members[b->active[k]];
+        const vdp_ctx* c = m.ctx;
+        if (m.how != Member::SHARED || m.desc.pc < PC_SPECTRAL) continue;
         cudaStream_t br = b->aux[slot++ % nb];
-        if (c->hdesc.pc == PC_MG) {
+        if (m.desc.pc == PC_MG) {
           const MgArgs a{c->r, c->za, c->omega, c->st, c->desc};
           e = launch_mg_vcycle(*c->mg, b->prec, a, br);
           continue;
         }
-        SpecArgs a;
-        solve_spec_args(c, b->prec, &a);
-        e = launch_spectral_apply(b->prec, a, spec_slab(c), br);
+        e = launch_spectral_apply(b->prec, m.spec, m.slab, br);
       }
       for (int j = 0; j < nb && e == cudaSuccess; ++j) {
         e = cudaEventRecord(b->join[j], b->aux[j]);
@@ -247,28 +250,30 @@ int capture(vdp_batch* b, int pairs) {
 // Launch the members that run by themselves, each for up to `pairs` rounds, on the branch streams
 // (largest first, to the stream with the fewest cells), between two points of the batch's stream.
 int launch_alone(vdp_batch* b, int pairs) {
-  std::vector<int> own;
-  for (int k : b->active)
-    if (b->members[k].alone) own.push_back(k);
+  std::vector<int> own;  // places in b->active, and in the device tables
+  auto member = [&](int k) -> const Member& { return b->members[b->active[k]]; };
+  for (int k = 0; k < (int)b->active.size(); ++k)
+    if (member(k).how != Member::SHARED) own.push_back(k);
   if (own.empty()) return VDP_OK;
   std::sort(own.begin(), own.end(), [&](int i, int j) {
-    return b->members[i].ctx->n != b->members[j].ctx->n ? b->members[i].ctx->n > b->members[j].ctx->n : i < j;
+    return member(i).ctx->n != member(j).ctx->n ? member(i).ctx->n > member(j).ctx->n : i < j;
   });
   const int nb = std::min((int)own.size(), (int)vdp_batch::kBranches);
   long long load[vdp_batch::kBranches] = {};
   VDP_CK(cudaEventRecord(b->fork, b->stream));
   for (int j = 0; j < nb; ++j) VDP_CK(cudaStreamWaitEvent(b->aux[j], b->fork, 0));
   for (int k : own) {
-    vdp_ctx* c = b->members[k].ctx;
+    const Member& m = member(k);
+    vdp_ctx* c = m.ctx;
     const int j = (int)(std::min_element(load, load + nb) - load);
     load[j] += c->n;
-    if (resident_solve(c, b->prec)) {
-      SpecArgs a;
-      solve_spec_args(c, b->prec, &a);
+    if (m.how == Member::RESIDENT) {
       VDP_CK(cudaMemsetAsync(c->rctl, 0, sizeof(ResidentCtl), b->aux[j]));
       // a round is at most two sweeps; side by side, each member takes its share of the blocks
-      VDP_CK(launch_resident(b->prec, c->hdesc, c->desc, a, c->rctl, 2u * (unsigned)pairs,
+      VDP_CK(launch_resident(b->prec, m.desc, b->d_desc + k, m.spec, c->rctl, 2u * (unsigned)pairs,
                              2 * kSMs / nb, b->aux[j]));
+    } else if (!c->wexec || !c->d_rounds) {  // the context has been set up anew meanwhile
+      return VDP_EINVAL;
     } else {
       VDP_CK(launch_start_rounds(c->d_rounds, (unsigned)((pairs + kWhileRounds - 1) / kWhileRounds), b->aux[j]));
       VDP_CK(cudaGraphLaunch(c->wexec, b->aux[j]));
@@ -362,7 +367,12 @@ int vdp_batch_add(vdp_batch* b, vdp_ctx* c, const double* rhs, double* p, double
   VDP_CK(cudaStreamSynchronize(c->stream));
   VDP_CK(launch_init(c->desc, rhs, p, tol, c->opts.inner_tol, c->opts.max_iter, c->opts.max_iter,
                      c->opts.use_guess ? 1 : 0, b->prec, nullptr, b->stream));
-  b->members.push_back(Member{c, rhs, p, tol, false, false});
+  Member m{c, rhs, p, tol, false, how_to_run(b, c), c->hdesc, {}, 0};
+  if (m.desc.pc == PC_SPECTRAL || m.desc.pc == PC_FIXED) {
+    solve_spec_args(c, b->prec, &m.spec);
+    m.slab = spec_slab(c);
+  }
+  b->members.push_back(m);
   b->dirty = true;
   return VDP_OK;
 }
