@@ -601,14 +601,15 @@ class Batch:
         return vdp_batch_size(self.handle)
 
     def set_wait_limit(self, seconds: float) -> None:
-        """Bound on each grid-barrier wait of the persistent kernel (an expired wait raises
-        VdpError(VDP_ETIMEOUT) from run(); the members stay usable)."""
+        """Bound on each grid-barrier wait of the persistent kernel and of members that run as one
+        cooperative launch (an expired wait raises VdpError(VDP_ETIMEOUT) from run(); the members
+        stay usable)."""
         st = vdp_batch_set_wait_limit(self.handle, seconds)
         if st != VDP_OK:
             raise VdpError(st, "vdp_batch_set_wait_limit")
 
     def inject_lost_arrival(self) -> None:
-        """Failure injection for tests: the next persistent run waits for a block that never
+        """Failure injection for tests: the next run waits at its grid barriers for a block that never
         arrives, so its bounded grid-barrier wait expires."""
         st = vdp_batch_inject_lost_arrival(self.handle)
         if st != VDP_OK:

@@ -44,6 +44,7 @@ struct Member {
   InstDesc desc;
   SpecArgs spec;  // of members with the spectral passes
   int slab;
+  vdp_opts opts;
 };
 
 }  // namespace
@@ -249,7 +250,7 @@ int capture(vdp_batch* b, int pairs) {
 
 // Launch the members that run by themselves, each for up to `pairs` rounds, on the branch streams
 // (largest first, to the stream with the fewest cells), between two points of the batch's stream.
-int launch_alone(vdp_batch* b, int pairs) {
+int launch_alone(vdp_batch* b, int pairs, bool inject) {
   std::vector<int> own;  // places in b->active, and in the device tables
   auto member = [&](int k) -> const Member& { return b->members[b->active[k]]; };
   for (int k = 0; k < (int)b->active.size(); ++k)
@@ -268,7 +269,7 @@ int launch_alone(vdp_batch* b, int pairs) {
     const int j = (int)(std::min_element(load, load + nb) - load);
     load[j] += c->n;
     if (m.how == Member::RESIDENT) {
-      VDP_CK(cudaMemsetAsync(c->rctl, 0, sizeof(ResidentCtl), b->aux[j]));
+      VDP_CK(launch_start_resident(c->rctl, inject ? 1u : 0u, (unsigned long long)(b->wait_limit_s * 1e9), b->aux[j]));
       // a round is at most two sweeps; side by side, each member takes its share of the blocks
       VDP_CK(launch_resident(b->prec, m.desc, b->d_desc + k, m.spec, c->rctl, 2u * (unsigned)pairs,
                              2 * kSMs / nb, b->aux[j]));
@@ -367,7 +368,7 @@ int vdp_batch_add(vdp_batch* b, vdp_ctx* c, const double* rhs, double* p, double
   VDP_CK(cudaStreamSynchronize(c->stream));
   VDP_CK(launch_init(c->desc, rhs, p, tol, c->opts.inner_tol, c->opts.max_iter, c->opts.max_iter,
                      c->opts.use_guess ? 1 : 0, b->prec, nullptr, b->stream));
-  Member m{c, rhs, p, tol, false, how_to_run(b, c), c->hdesc, {}, 0};
+  Member m{c, rhs, p, tol, false, how_to_run(b, c), c->hdesc, {}, 0, c->opts};
   if (m.desc.pc == PC_SPECTRAL || m.desc.pc == PC_FIXED) {
     solve_spec_args(c, b->prec, &m.spec);
     m.slab = spec_slab(c);
@@ -389,17 +390,18 @@ int vdp_batch_run(vdp_batch* b, int max_pairs, int* active_out) {
   if (b->nshared > 0 && (!b->gexec || b->g_pairs != max_pairs)) {
     if ((s = capture(b, max_pairs)) != VDP_OK) return s;
   }
+  const bool inject = b->inject;
   if (b->ctl_stale || b->inject) {  // fresh barrier words (after an expired wait, or to inject)
     BatchCtl ctl{};
     ctl.remaining = n;
     ctl.limit_ns = (unsigned long long)(b->wait_limit_s * 1e9);
-    ctl.extra = b->inject ? 1u : 0u;
+    ctl.extra = inject ? 1u : 0u;
     *b->h_ctl = ctl;
     VDP_CK(cudaMemcpyAsync(b->d_ctl, b->h_ctl, sizeof(BatchCtl), cudaMemcpyHostToDevice, b->stream));
     b->ctl_stale = b->inject;  // an injected run leaves words to reset
     b->inject = false;
   }
-  if ((s = launch_alone(b, max_pairs)) != VDP_OK) return s;
+  if ((s = launch_alone(b, max_pairs, inject)) != VDP_OK) return s;
   if (b->nshared > 0) VDP_CK(cudaGraphLaunch(b->gexec, b->stream));
   VDP_CK(launch_gather(b->d_desc, n, b->d_states, b->stream));
   VDP_CK(cudaMemcpyAsync(b->h_states, b->d_states, sizeof(InstState) * n, cudaMemcpyDeviceToHost,
@@ -407,10 +409,18 @@ int vdp_batch_run(vdp_batch* b, int max_pairs, int* active_out) {
   VDP_CK(cudaMemcpyAsync(b->h_ctl, b->d_ctl, sizeof(BatchCtl), cudaMemcpyDeviceToHost, b->stream));
   VDP_CK(cudaStreamSynchronize(b->stream));
   int remaining = 0;
+  bool expired = b->h_ctl->fault != 0;
   for (int k = 0; k < n; ++k) {
     Member& m = b->members[b->active[k]];
     const InstState& h = b->h_states[k];
-    if (h.phase >= PH_DONE) {
+    if (m.how == Member::RESIDENT && h.phase >= PH_DONE && h.status == VDP_ETIMEOUT) {
+      // a sweep of the resident launch was left incomplete: the solve starts again at the next run
+      // (from what p holds, where p was its initial guess)
+      VDP_CK(launch_init(b->d_desc + k, m.rhs, m.p, m.tol, m.opts.inner_tol, m.opts.max_iter, m.opts.max_iter,
+                         m.opts.use_guess ? 1 : 0, b->prec, nullptr, b->stream));
+      expired = true;
+      ++remaining;
+    } else if (h.phase >= PH_DONE) {
       m.done = true;
       b->dirty = true;  // retire it from the device tables at the next run
       vdp_stats& st = m.ctx->stats;
@@ -427,10 +437,8 @@ int vdp_batch_run(vdp_batch* b, int max_pairs, int* active_out) {
     }
   }
   if (active_out) *active_out = remaining;
-  if (b->h_ctl->fault) {
-    b->ctl_stale = true;  // the members stay usable: their last completed sweeps are consistent
-    return VDP_ETIMEOUT;
-  }
+  if (b->h_ctl->fault) b->ctl_stale = true;  // the members stay usable: their last completed sweeps are consistent
+  if (expired) return VDP_ETIMEOUT;
   return VDP_OK;
 }
 
@@ -442,7 +450,10 @@ int vdp_batch_set_wait_limit(vdp_batch* b, double seconds) {
 }
 
 int vdp_batch_inject_lost_arrival(vdp_batch* b) {
-  if (!b || !b->persistent) return VDP_EINVAL;
+  if (!b) return VDP_EINVAL;
+  bool waits = b->persistent != 0;  // has a grid barrier
+  for (const Member& m : b->members) waits = waits || (!m.done && m.how == Member::RESIDENT);
+  if (!waits) return VDP_EINVAL;
   b->inject = true;
   return VDP_OK;
 }

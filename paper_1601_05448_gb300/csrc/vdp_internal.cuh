@@ -146,13 +146,16 @@ struct BatchCtl {
   unsigned long long limit_ns;  // bound on one grid barrier wait
 };
 
-// Control words of a resident solve (vdp_resident.cu), a cache line each; zero at launch.
+// Control words of a resident solve (vdp_resident.cu), the arrivals in a cache line of their own.
 struct ResidentCtl {
-  unsigned count;      // barrier arrivals
+  unsigned count;      // barrier arrivals (0 at launch)
   unsigned pad0[31];
-  int fault;           // a wait expired
-  unsigned pad1[31];
+  int fault;           // a wait expired (0 at launch)
+  unsigned extra;      // arrivals that the first barrier expects beyond the grid (failure injection)
+  unsigned long long limit_ns;  // bound on one wait
+  unsigned pad1[28];
 };
+constexpr unsigned long long kResidentWaitNs = 2000000000ull;  // of a solve alone
 
 struct UnitRef {
   int inst;            // index into the batch's InstDesc table

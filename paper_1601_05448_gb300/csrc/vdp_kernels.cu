@@ -665,6 +665,8 @@ __global__ void k_init(InstDesc* desc, const double* rhs, double* p, double tol,
   if (ctl) {
     ctl->count = 0u;
     ctl->fault = 0;
+    ctl->extra = 0u;
+    ctl->limit_ns = kResidentWaitNs;
   }
 }
 
@@ -808,6 +810,18 @@ __global__ void k_continue(const InstState* st, cudaGraphConditionalHandle handl
 __global__ void k_start_rounds(unsigned* rounds, unsigned limit) {
   rounds[0] = 0u;
   rounds[1] = limit;
+}
+
+__global__ void k_start_resident(ResidentCtl* ctl, unsigned extra, unsigned long long limit_ns) {
+  ctl->count = 0u;
+  ctl->fault = 0;
+  ctl->extra = extra;
+  ctl->limit_ns = limit_ns;
+}
+
+cudaError_t launch_start_resident(ResidentCtl* ctl, unsigned extra, unsigned long long limit_ns, cudaStream_t s) {
+  k_start_resident<<<1, 1, 0, s>>>(ctl, extra, limit_ns);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_start_rounds(unsigned* rounds, unsigned limit, cudaStream_t s) {

@@ -60,7 +60,8 @@ cudaError_t launch_flat(int prec, const InstDesc* desc, const UnitRef* units, in
 
 // vdp_resident.cu: the whole solve in one cooperative launch, for grids of at most kResidentCells
 // cells.  spec: the solve's spectral arguments (unused by Jacobi CG); stops after max_sweeps sweeps;
-// at most max_blocks blocks (0: as many as are resident).  ctl must be zero.
+// at most max_blocks blocks (0: as many as are resident).  The control words are set before, by
+// launch_init or launch_start_resident.
 struct SpecArgs;
 bool resident_supported(const InstDesc& d, int prec);
 cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, const SpecArgs& spec,
@@ -71,6 +72,7 @@ cudaError_t launch_persistent(int prec, const InstDesc* desc, const UnitRef* sun
                               const UnitRef* funits, int nf, int pairs, BatchCtl* ctl, int grid,
                               cudaStream_t s);
 cudaError_t launch_gather(const InstDesc* desc, int n, InstState* out, cudaStream_t s);
+cudaError_t launch_start_resident(ResidentCtl* ctl, unsigned extra, unsigned long long limit_ns, cudaStream_t s);
 // before a device-side loop: rounds = {0, limit} (limit 0: none)
 cudaError_t launch_start_rounds(unsigned* rounds, unsigned limit, cudaStream_t s);
 // device-side solve loop: sets the WHILE condition `handle` to continue while the instance is

@@ -17,8 +17,8 @@
 // Units, partial slots, the order of the sums and the arithmetic of every sweep are those of the
 // separate kernels (vdp_sweeps.cuh, vdp_density.cuh, vdp_fft.cuh), so the result is the same bit
 // for bit; data that other blocks wrote are read by plain loads, never through the read-only path.
-// All waits are bounded: one that expires sets the fault word and ends the launch, and the host
-// reports VDP_ETIMEOUT.
+// All waits are bounded: one that expires sets the fault word, which the other waits look at too, and
+// ends the launch; the host reports VDP_ETIMEOUT, and a batch starts the member again.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -42,6 +42,7 @@ constexpr int kResidentSlots = kSlots * kSMs * 8;  // half of the smallest parti
 struct GridBarrier {
   ResidentCtl* ctl;
   unsigned target;  // arrivals of all barriers so far, this one included
+  unsigned long long limit_ns;
 
   __device__ __forceinline__ static unsigned load_acquire(const unsigned* p) {
     unsigned v;
@@ -62,7 +63,7 @@ struct GridBarrier {
         if ((++polls & 255u) == 0) {
           const uint64_t now = global_ns();
           if (t0 == 0) t0 = now;
-          if (now - t0 > 2000000000ull) {
+          if (now - t0 > limit_ns || __ldcg(&ctl->fault) != 0) {
             atomicExch(&ctl->fault, 1);
             ok = false;
             break;
@@ -379,7 +380,7 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
   if constexpr (SPEC) tb = shared_tables(spec, reinterpret_cast<float2*>(smem), wy, wz, lz, work);
   ulonglong2* stages = reinterpret_cast<ulonglong2*>(work);
   __syncthreads();
-  GridBarrier bar{ctl, 0u};
+  GridBarrier bar{ctl, __ldcg(&ctl->extra), __ldcg(&ctl->limit_ns)};
   bool ok = true;
   for (unsigned done = 0; ok && done < max_sweeps; ++done) {
     int phase = sn.phase;
