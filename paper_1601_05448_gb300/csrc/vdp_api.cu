@@ -776,8 +776,9 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   if (resident) {
     SpecArgs a{};
     if (c->hdesc.pc != PC_JACOBI) solve_spec_args(c, prec, &a);
-    // two sweeps per iteration and the outer phases; the state machine stops at max_iter itself
-    const long long bound = 3LL * c->opts.max_iter + 4096;
+    // at most two rounds an iteration (its update and a correction end one each) and the outer phases;
+    // the state machine stops at max_iter itself
+    const long long bound = 4LL * c->opts.max_iter + 4096;
     VDP_CK(launch_resident(prec, c->hdesc, c->desc, a, c->rctl,
                            (unsigned)std::min<long long>(bound, 0x7fffffffLL), 0, c->stream));
     VDP_CK(cudaMemcpyAsync(&c->hstate[0], c->st, sizeof(InstState), cudaMemcpyDeviceToHost,

@@ -270,8 +270,8 @@ int launch_alone(vdp_batch* b, int pairs, bool inject) {
     load[j] += c->n;
     if (m.how == Member::RESIDENT) {
       VDP_CK(launch_start_resident(c->rctl, inject ? 1u : 0u, (unsigned long long)(b->wait_limit_s * 1e9), b->aux[j]));
-      // a round is at most two sweeps; side by side, each member takes its share of the blocks
-      VDP_CK(launch_resident(b->prec, m.desc, b->d_desc + k, m.spec, c->rctl, 2u * (unsigned)pairs,
+      // side by side, each member takes its share of the blocks
+      VDP_CK(launch_resident(b->prec, m.desc, b->d_desc + k, m.spec, c->rctl, (unsigned)pairs,
                              2 * kSMs / nb, b->aux[j]));
     } else if (!c->wexec || !c->d_rounds) {  // the context has been set up anew meanwhile
       return VDP_EINVAL;

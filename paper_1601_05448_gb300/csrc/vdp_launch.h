@@ -59,13 +59,14 @@ cudaError_t launch_flat(int prec, const InstDesc* desc, const UnitRef* units, in
                         cudaStream_t s);
 
 // vdp_resident.cu: the whole solve in one cooperative launch, for grids of at most kResidentCells
-// cells.  spec: the solve's spectral arguments (unused by Jacobi CG); stops after max_sweeps sweeps;
+// cells.  spec: the solve's spectral arguments (unused by Jacobi CG); stops after max_rounds rounds, a
+// round being what one pass of the separate launches (residual, preconditioner, stencil, flat) advances;
 // at most max_blocks blocks (0: as many as are resident).  The control words are set before, by
 // launch_init or launch_start_resident.
 struct SpecArgs;
 bool resident_supported(const InstDesc& d, int prec);
 cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, const SpecArgs& spec,
-                            ResidentCtl* ctl, unsigned max_sweeps, int max_blocks, cudaStream_t s);
+                            ResidentCtl* ctl, unsigned max_rounds, int max_blocks, cudaStream_t s);
 
 cudaError_t persistent_grid(int prec, int* grid);
 cudaError_t launch_persistent(int prec, const InstDesc* desc, const UnitRef* sunits, int ns,

@@ -359,10 +359,15 @@ __device__ __noinline__ void unit_flat(const InstDesc& I, const InstState& sn, i
   }
 }
 
+// Place of a phase in a round of the separate launches: residual, preconditioner, stencil, flat sweeps.
+__device__ __forceinline__ int round_place(int phase) {
+  return phase == PH_RES64 ? 0 : phase == PH_SPEC ? 1 : phase == PH_STENCIL ? 2 : 3;
+}
+
 template <class T, int KIND>
 __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOBI ? 1 : 2)
     k_resident(const InstDesc* desc, const __grid_constant__ SpecArgs spec, ResidentCtl* ctl,
-               unsigned max_sweeps) {
+               unsigned max_rounds) {
   constexpr bool SPEC = KIND != R_JACOBI, DENS = SPEC && sizeof(T) == 8;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(16) unsigned char desc_bytes[sizeof(InstDesc)];
@@ -382,9 +387,13 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
   __syncthreads();
   GridBarrier bar{ctl, __ldcg(&ctl->extra), __ldcg(&ctl->limit_ns)};
   bool ok = true;
-  for (unsigned done = 0; ok && done < max_sweeps; ++done) {
+  unsigned rounds = 0;
+  int place = 3;
+  for (unsigned done = 0; ok; ++done) {
     int phase = sn.phase;
     if (phase >= PH_DONE) break;
+    if (round_place(phase) <= place && rounds++ == max_rounds) break;
+    place = round_place(phase);
     double* slots = I.part + (done & 1u) * kResidentSlots;
     int nparts = I.nunits;
     bool applied = false;  // the preconditioner's sweep was part of this round
@@ -402,6 +411,7 @@ __global__ void __launch_bounds__(kResThreads, sizeof(T) == 8 && KIND != R_JACOB
         if (!(ok = bar.sync())) break;
         applied = true;
         phase = PH_STENCIL;
+        place = round_place(phase);
       } else {
         nparts = spec.zunits;
       }
@@ -495,7 +505,7 @@ bool resident_supported(const InstDesc& d, int prec) {
 }
 
 cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, const SpecArgs& spec,
-                            ResidentCtl* ctl, unsigned max_sweeps, int max_blocks, cudaStream_t s) {
+                            ResidentCtl* ctl, unsigned max_rounds, int max_blocks, cudaStream_t s) {
   const int kind = resident_kind(d);
   if (kind != R_JACOBI && spec.zunits > kResidentSlots) return cudaErrorInvalidValue;
   const ResidentKernel k = resident_kernel(prec, kind);
@@ -542,7 +552,7 @@ cudaError_t launch_resident(int prec, const InstDesc& d, const InstDesc* desc, c
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  void* args[] = {(void*)&desc, (void*)&spec, (void*)&ctl, (void*)&max_sweeps};
+  void* args[] = {(void*)&desc, (void*)&spec, (void*)&ctl, (void*)&max_rounds};
   return cudaLaunchKernelExC(&cfg, (const void*)k, args);
 }
 
