@@ -209,6 +209,7 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
     cf[d].cl = pk(I.cl[d], I.cl[d]);
   }
   const double beta = st.beta;
+  const int rexp = st.rexp;
   const bool first = st.inner_iters == 0;  // no X (fixed point), no history (CG) yet
   const float* rhi = I.rho32;
   const float* rlo = I.rho_lo;
@@ -374,24 +375,24 @@ __device__ __forceinline__ void sweep_density64(const InstDesc& I, const InstSta
       const double2 qv = *reinterpret_cast<const double2*>(slot(b, h ? T_Q1 : T_Q0));
       double2 po, qo;
       if constexpr (FIXED) {
-        po.x = (pv.x + widen(ah.x)) + widen(al.x);
-        po.y = (pv.y + widen(ah.y)) + widen(al.y);
-        qo.x = widen(uu.x);
-        qo.y = widen(uu.y);
+        po.x = (pv.x + widen_scaled(ah.x, -rexp)) + widen_scaled(al.x, -rexp);
+        po.y = (pv.y + widen_scaled(ah.y, -rexp)) + widen_scaled(al.y, -rexp);
+        qo.x = widen_scaled(uu.x, -rexp);
+        qo.y = widen_scaled(uu.y, -rexp);
         if (!first) {
           qo.x += qv.x;
           qo.y += qv.y;
         }
         const float2 d = up2(D[h]), rho = up2(r[h].h);
-        const float rx = narrow(po.x), ry = narrow(po.y);
+        const float rx = narrow_pow2(po.x, rexp), ry = narrow_pow2(po.y, rexp);
         if (active) *reinterpret_cast<float2*>(I.g32 + o + 2 * h) = make_float2(rho.x * rx, rho.y * ry);
         sumf = fmaf(rx * rcp_approx(d.x), rx, sumf);
         sumf = fmaf(ry * rcp_approx(d.y), ry, sumf);
       } else {
-        po.x = widen(uu.x);
-        po.y = widen(uu.y);
-        qo.x = -(widen(ah.x) + widen(al.x));
-        qo.y = -(widen(ah.y) + widen(al.y));
+        po.x = widen_scaled(uu.x, -rexp);
+        po.y = widen_scaled(uu.y, -rexp);
+        qo.x = -(widen_scaled(ah.x, -rexp) + widen_scaled(al.x, -rexp));
+        qo.y = -(widen_scaled(ah.y, -rexp) + widen_scaled(al.y, -rexp));
         if (!first) {
           po.x = fma(beta, pv.x, po.x);
           po.y = fma(beta, pv.y, po.y);

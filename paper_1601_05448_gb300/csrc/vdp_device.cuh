@@ -223,16 +223,20 @@ __device__ __forceinline__ double quotient(double c, double s) {
   return fma(w, fma(e, e, e), w);
 }
 
-// The power of two for the FP32 inner variables when the mean square of rt = D^-1/2 r, summed in FP32
-// (rrt), lies where an inner solve's reductions or its largest cells would take it out of the FP32
-// range: what brings the root mean square to about one, from ||f - <f>||^2 (fn2, an FP64 sum) and the
-// first cell's D.  0: none (any magnitude that a solve in ordinary units has; a power of two would not
-// change its results either, but the repeated sweep costs time).
-__device__ __forceinline__ int inner_scale(const InstDesc& I, const InstState* st, double fn2, double rrt) {
+// Powers of two for what FP32 holds, where the root mean square of f - <f> (fn2: an FP64 sum), or of
+// rt = D^-1/2 r of an FP32 inner solve (rrt, summed in FP32), lies so far out that squares, or what an
+// inner solve leaves of them, would leave the FP32 range: both are then brought to about one (D from the
+// first cell).  false: none.  Solves in ordinary units have none; a power of two would not change their
+// results either, but the repeated residual costs time.
+__device__ __forceinline__ bool set_scales(const InstDesc& I, InstState* st, double fn2, double rrt) {
   const double n = (double)I.ncell;
-  if (st->precision == PREC_FP64 || I.mode != 0 || !(fn2 > 0.0) || !isfinite(fn2)) return 0;
-  if (rrt > 0x1p-60 * n && rrt < 0x1p80 * n) return 0;
-  return (ilogb(I.dg[0]) - ilogb(fn2 / n)) / 2;
+  if (I.mode != 0 || !(fn2 > 0.0) || !isfinite(fn2)) return false;
+  const int e = ilogb(fn2 / n) / 2;
+  const bool fp32 = st->precision != PREC_FP64;
+  if (e >= -30 && e <= 40 && (!fp32 || (rrt > 0x1p-60 * n && rrt < 0x1p80 * n))) return false;
+  st->rexp = -e;
+  if (fp32) st->texp = ilogb(I.dg[0]) / 2 - e;
+  return st->rexp != 0 || st->texp != 0;
 }
 
 // ---- phase transitions (run by thread 0 of the last unit) -------------------------------------
@@ -253,7 +257,7 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
       st->phase = PH_RES64;
       break;
     case PH_RES64: {
-      const double rr64 = S[0], rrt = S[1];
+      const double rr64 = st->rexp ? ldexp(S[0], -2 * st->rexp) : S[0], rrt = S[1];
       const bool first = st->first_res != 0;
       if (st->first_res) st->sum_p = S[2];  // later: summed by the correction sweep
       if (st->first_res) {
@@ -268,9 +272,8 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
         st->phase = PH_FINAL;
         break;
       }
-      if (first && st->texp == 0 && inner_scale(I, st, fn2, rrt) != 0) {
+      if (first && st->rexp == 0 && st->texp == 0 && set_scales(I, st, fn2, rrt)) {
         // the sweep is repeated with the scaled variables (p, and what it adds, are as they were)
-        st->texp = inner_scale(I, st, fn2, rrt);
         st->first_res = 1;
         st->outer -= 1;
         break;
@@ -371,7 +374,7 @@ static __device__ __noinline__ void transition(const InstDesc& I, InstState* st,
         st->cheb_j += 1;
         break;
       }
-      const double rz = S[0];
+      const double rz = I.form && st->rexp ? ldexp(S[0], -2 * st->rexp) : S[0];
       if (!(rz > 0.0) || !isfinite(rz)) {  // the preconditioner must stay positive definite
         if (st->inner_iters > 0) {
           st->inner_ratio = sqrt(st->rr / st->rr0);

@@ -61,8 +61,9 @@ struct __align__(16) InstState {
   int precision;
   int fault;           // a unit's bounded wait expired (reported as VDP_ETIMEOUT)
   int cheb_j;          // Chebyshev sweep index (1 .. cheb_k - 1)
-  int texp;            // FP32 inner solve, direct sweeps: the inner variables are 2^texp times D^-1/2 r
-                       // and its corrections; 0 unless <rt, rt> would leave the FP32 range
+  int rexp, texp;      // direct sweeps: what FP32 holds of r (its norms; the density form's X+ input and
+                       // z) is 2^rexp times that, an FP32 inner solve's variables are 2^texp times D^-1/2 r
+                       // and its corrections; 0 unless a norm would leave the FP32 range
   int p_set;           // p holds an iterate: the caller's guess, or a correction was applied
                        // (from p = 0 the first correction writes p without reading it)
   double rz;           // <rt, z> (preconditioned inner product; = <rt, rt> for Jacobi)

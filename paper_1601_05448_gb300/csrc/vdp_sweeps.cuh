@@ -255,7 +255,7 @@ __device__ void sweep_update(const InstDesc& I, const InstState* st, long long c
       VecIO<T, V>::st(x + c, xv[u]);
       VecIO<T, V>::st(rt + c, rv[u]);
       if constexpr (sizeof(T) == 8)
-        if (I.g32) *reinterpret_cast<float2*>(I.g32 + c) = make_float2(narrow(rv[u][0]), narrow(rv[u][1]));
+        if (I.g32) *reinterpret_cast<float2*>(I.g32 + c) = make_float2(narrow_pow2(rv[u][0], st->rexp), narrow_pow2(rv[u][1], st->rexp));
     }
   }
   T tot = 0;
@@ -575,7 +575,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
   const bool row_start = x0 == 0, row_end = x0 + VR == nx;
   const int xl = row_start ? nx - 1 : x0 - 1, xr = row_end ? 0 : x0 + VR;
   const double mu = st->mu_f;
-  const int texp = st->texp;
+  const int rexp = st->rexp, sexp = st->texp - st->rexp;
   const double* p = I.p;
   T* rt = static_cast<T*>(I.r);
   const DensityResidual dr = DENS ? DensityResidual(I) : DensityResidual();
@@ -646,7 +646,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
       res0 = fma(-bzp.x, pp[h], res0);
       res1 = fma(-bzp.y, pp[h + 1], res1);
       T t0, t1;
-      float r0f = narrow(res0), r1f = narrow(res1), t0f, t1f;
+      float r0f = narrow_pow2(res0, rexp), r1f = narrow_pow2(res1, rexp), t0f, t1f;
       if constexpr (DENS) {
         t0 = res0;
         t1 = res1;
@@ -659,8 +659,8 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
         t1f = narrow(t1);
       } else {  // the inner residual in FP32: D^-1/2 r from the FP32 factors (the inner solve's
                 // own rounding), no FP64 multiply
-        t0 = t0f = narrow_pow2(si.x, texp) * r0f;
-        t1 = t1f = narrow_pow2(si.y, texp) * r1f;
+        t0 = t0f = narrow_pow2(si.x, sexp) * r0f;
+        t1 = t1f = narrow_pow2(si.y, sexp) * r1f;
       }
       if (active) {
         store2(rt + o, t0, t1);
@@ -683,6 +683,7 @@ __device__ __forceinline__ void res64_march(const InstDesc& I, const InstState* 
   }
   acc[0] = (double)a0;
   acc[1] = (double)a1;
+  if (DENS && !dr.fixed && rexp) acc[1] = ldexp(acc[1], -2 * rexp);  // CG's norms are FP64
   acc[2] = a2;
   acc[3] = a3;
 }
@@ -700,7 +701,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
   const int yr = tile * I.ty + row;
   const int z0 = (int)((long long)chunk * nz / I.zc), z1 = (int)((long long)(chunk + 1) * nz / I.zc);
   const double mu = st->mu_f;
-  const int texp = st->texp;
+  const int rexp = st->rexp, sexp = st->texp - st->rexp;
   T* rt = static_cast<T*>(I.r);
   const DensityResidual dr = DENS ? DensityResidual(I) : DensityResidual();
   double a0 = 0;
@@ -729,7 +730,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
       const double f0 = c.f[h / 2].x - mu, f1 = c.f[h / 2].y - mu;
       if (I.f0) *reinterpret_cast<double2*>(I.f0 + o + h) = make_double2(f0, f1);
       if constexpr (DENS) {
-        const float r0 = narrow(f0), r1 = narrow(f1);
+        const float r0 = narrow_pow2(f0, rexp), r1 = narrow_pow2(f1, rexp);
         const float2 rh = diag ? c.rho[h / 2] : make_float2(1.f, 1.f);
         float2 d = make_float2(1.f, 1.f);
         if (diag) d = make_float2(dr.inv_diag(c.w[h / 2].x), dr.inv_diag(c.w[h / 2].y));
@@ -747,7 +748,8 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
                 // factors; ||f - <f>||^2, the denominator of every relative residual of the
                 // solve, stays an FP64 sum (any magnitude of f)
         const double2 si = c.w[h / 2];
-        const float t0 = narrow_pow2(si.x, texp) * narrow(f0), t1 = narrow_pow2(si.y, texp) * narrow(f1);
+        const float t0 = narrow_pow2(si.x, sexp) * narrow_pow2(f0, rexp);
+        const float t1 = narrow_pow2(si.y, sexp) * narrow_pow2(f1, rexp);
         store2(rt + o + h, t0, t1);
         a0 = fma(f0, f0, fma(f1, f1, a0));
         a1 = fmaf(t0, t0, fmaf(t1, t1, a1));
@@ -763,7 +765,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
       if (z + 1 < z1) store(z + 1, c[1]);
     }
   }
-  acc[0] = a0;          // ||r||^2
+  acc[0] = rexp ? ldexp(a0, 2 * rexp) : a0;  // ||r||^2, in the units of the later sweeps' sums
   acc[1] = DENS ? (dr.fixed ? (double)a1f : a0) : (double)a1;  // ||rt||^2 (density form: see above)
   acc[2] = 0.0;         // sum of p
   acc[3] = a0;          // ||f - <f>||^2 (this is the first residual)
