@@ -551,22 +551,22 @@ int vdp_create_bc(int nx, int ny, int nz, double Lx, double Ly, double Lz, int b
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->st, sizeof(InstState));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->desc, sizeof(InstDesc));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->units, sizeof(UnitRef) * (maxunits + kSMs * 8));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->flag, sizeof(int));
-  // pinned: two states and the density verdict
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hstate, 2 * sizeof(InstState) + sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->flag, 2 * sizeof(int));
+  // pinned: two states and the density's two verdicts
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hstate, 2 * sizeof(InstState) + 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->evs[0], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->evs[1], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaMemset(c->ticket, 0, sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMemset(c->flag, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(c->flag, 0, 2 * sizeof(int));
   if (e != cudaSuccess) {
     int s = cuda_fail(e, "vdp_create");
     free_ctx(c);
     return s;
   }
-  std::memset(c->hstate, 0, 2 * sizeof(InstState) + sizeof(int));
+  std::memset(c->hstate, 0, 2 * sizeof(InstState) + 2 * sizeof(int));
   c->hflag = reinterpret_cast<int*>(c->hstate + 2);
   Layout lay;
   if (choose_layout(c, c->opts.precision, &lay) != VDP_OK) {  // rows too long for any stage
@@ -704,7 +704,7 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
   VDP_CK(launch_build_coefficients(src, c->nx, c->ny, c->nz, c->Lx / c->nx, c->Ly / c->ny,
                                    c->Lz / c->nz, c->bc_x == VDP_BC_DUCT, c->bx, c->by, c->bz,
                                    scaled ? c->sinv : nullptr, c->dg, c->rho32, c->rho_lo, c->dsc,
-                                   density_scale(c), c->flag, gen, c->stream));
+                                   density_scale(c), c->flag, c->flag + 1, gen, c->stream));
   const bool weights = scaled && c->rho_w;  // rho W needs rho itself
   const bool unit = c->opts.method != VDP_METHOD_FIXED_POINT && c->opts.precond == VDP_PRECOND_SPECTRAL;
   if (scaled)
@@ -712,16 +712,25 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
                          c->sz, c->sd, c->flag, gen, c->stream));
   if (weights)
     VDP_CK(launch_weights(src, c->dg, c->sinv, c->n, unit, c->omega, c->rho_w, c->flag, gen, c->stream));
-  VDP_CK(cudaMemcpyAsync(c->hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  VDP_CK(cudaMemcpyAsync(c->hflag, c->flag, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   VDP_CK(cudaStreamSynchronize(c->stream));
-  if (*c->hflag == gen) return VDP_EDENSITY;
+  if (c->hflag[0] == gen) return VDP_EDENSITY;
+  const bool wide = c->rho32 && c->hflag[1] == gen;
   c->scaled_prec = scaled ? prec : -1;
   c->sinv_valid = scaled;
   c->omega_valid = weights && c->omega;
   c->omega_unit = unit;
   c->rho_w_valid = weights;
-  c->rho32_valid = c->rho32 != nullptr;
+  c->rho32_valid = c->rho32 && !wide;
   c->mg_valid = false;
+  if (wide && !weights) {  // the scaled form's weight of rho, while rho is at hand
+    const int s = ensure_sinv(c);
+    if (s != VDP_OK) return s;
+    if (!c->rho_w) VDP_CK(cudaMalloc((void**)&c->rho_w, sizeof(float) * (size_t)c->n));
+    VDP_CK(launch_weights(src, c->dg, c->sinv, c->n, false, nullptr, c->rho_w, nullptr, 0, c->stream));
+    VDP_CK(cudaStreamSynchronize(c->stream));
+    c->rho_w_valid = true;
+  }
   if (c->rho32_valid != kept) c->layout_dirty = true;  // the form may change with it
   c->has_density = true;
   return VDP_OK;

@@ -70,7 +70,7 @@ struct vdp_ctx {
   double *stage_a = nullptr, *stage_b = nullptr;  // staging for host pointers
   double* proj_f = nullptr;        // vdp_project: the assembled Poisson right side
   vdp::InstState* hstate = nullptr;     // pinned, 2 entries
-  int* hflag = nullptr;            // pinned: the verdict of the last density check
+  int* hflag = nullptr;            // pinned: the verdicts of the last density: refused, outside the density form's range
   int density_gen = 0;             // number of the last vdp_set_density call (the failed check's mark)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, evs[2] = {nullptr, nullptr};
   // layout

@@ -13,12 +13,12 @@ namespace vdp {
 cudaError_t launch_check_density(const double* rho, long long n, int gen, int* bad, cudaStream_t s);
 // face coefficients on the low faces (spacings h_d; duct: no flux through the x ends) and D; with
 // sinv also D^-1/2, with rho32 the density form's FP32 density, what it rounds off (rho_lo) and
-// dsc[0] = kappa = 2^e0 s
+// dsc[0] = kappa = 2^e0 s, and far[0] = gen where these do not hold the density
 cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz, double hx,
                                       double hy, double hz, int duct, double* bx, double* by,
                                       double* bz, double* sinv, double* dg, float* rho32,
                                       float* rho_lo, double* dsc, double s2, const int* bad,
-                                      int gen, cudaStream_t s);
+                                      int* far, int gen, cudaStream_t s);
 cudaError_t launch_sinv(const double* dg, long long n, double* sinv, cudaStream_t s);
 cudaError_t launch_scaled(int prec, const double* bx, const double* by, const double* bz,
                           const double* sinv, int nx, int ny, int nz, void* sx, void* sy, void* sz,

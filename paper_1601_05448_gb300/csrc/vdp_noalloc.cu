@@ -199,7 +199,7 @@ extern "C" int vdp_solve_noalloc(int nx, int ny, int nz, double L, const double*
   if (bad) return VDP_EDENSITY;
   double* dg = f64[12];
   NA_CK(launch_build_coefficients(rho, nx, ny, nz, L / nx, L / ny, L / nz, 0, bx, by, bz, sinv, dg,
-                                  nullptr, nullptr, nullptr, 1.0, nullptr, 0, s));
+                                  nullptr, nullptr, nullptr, 1.0, nullptr, nullptr, 0, s));
   NA_CK(launch_scaled(precision, bx, by, bz, sinv, nx, ny, nz, sx, sy, sz, sd, nullptr, 0, s));
 
   // the default unit layout of vdp_solve

@@ -138,13 +138,14 @@ __global__ void k_check_density(const double* __restrict__ rho, long long n, int
 // b_d[c] = 2 / (rho[c - e_d] + rho[c]) / h_d^2 on the low d-face of every cell; with rho32 also the
 // FP32 density, scaled by the power of two of the first cell's (2^-e0), rho_lo what that
 // rounds off, and dsc[0] = 2^e0 s2, the factor between the density-form operator and A
-// (vdp_density.cu).
+// (vdp_density.cu).  far[0] = gen when a density is more than 2^60 from the first cell's, or below the
+// normal range: the density form's FP32 fields and coefficients do not hold that, the scaled form's do.
 // duct: the face at the x ends (slot x = 0, shared by x = 0 and x = Lx) carries no flux.
 __global__ void __launch_bounds__(kSetupThreads)
     k_faces(const double* __restrict__ rho, int nx, int ny, int nz, FaceFactor cx, FaceFactor cy, FaceFactor cz,
             int duct, double* __restrict__ bx, double* __restrict__ by, double* __restrict__ bz,
             float* __restrict__ rho32, float* __restrict__ rho_lo, double* dsc, double s2,
-            const int* bad, int gen) {
+            const int* bad, int* far, int gen) {
   if (rejected(bad, gen)) return;
   const PairMarch m = pair_march(nx, ny, nz);
   const int e0 = exponent_of(__ldg(rho)) - 1023;
@@ -174,6 +175,8 @@ __global__ void __launch_bounds__(kSetupThreads)
     *reinterpret_cast<double2*>(by + c) = vy;
     *reinterpret_cast<double2*>(bz + c) = vz;
     if (rho32) {
+      const unsigned ex = (unsigned)exponent_of(r.x), ey = (unsigned)exponent_of(r.y);
+      if (ex - (unsigned)(e0 + 963) > 120u || ey - (unsigned)(e0 + 963) > 120u || ex == 0u || ey == 0u) *far = gen;
       const float2 h = make_float2(narrow_rn_pow2(r.x, -e0), narrow_rn_pow2(r.y, -e0));
       *reinterpret_cast<float2*>(rho32 + c) = h;
       *reinterpret_cast<float2*>(rho_lo + c) =
@@ -350,7 +353,7 @@ cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz,
                                       double hy, double hz, int duct, double* bx, double* by,
                                       double* bz, double* sinv, double* dg, float* rho32,
                                       float* rho_lo, double* dsc, double s2, const int* bad,
-                                      int gen, cudaStream_t s) {
+                                      int* far, int gen, cudaStream_t s) {
   const dim3 g = pair_grid(nx, ny, nz);
   auto factor = [](double h) {
     FaceFactor f;
@@ -364,7 +367,7 @@ cudaError_t launch_build_coefficients(const double* rho, int nx, int ny, int nz,
     return f;
   };
   k_faces<<<g, kSetupThreads, 0, s>>>(rho, nx, ny, nz, factor(hx), factor(hy), factor(hz), duct, bx,
-                                      by, bz, rho32, rho_lo, dsc, s2, bad, gen);
+                                      by, bz, rho32, rho_lo, dsc, s2, bad, far, gen);
   k_diag<<<g, kSetupThreads, 0, s>>>(bx, by, bz, nx, ny, nz, sinv, dg, bad, gen);
   return cudaGetLastError();
 }

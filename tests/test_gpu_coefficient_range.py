@@ -1,5 +1,6 @@
-"""Face coefficients near and past the ends of the binary64 range: spacings and densities that the
-seeded quotient takes one by one, whose quotient it does not."""
+"""Densities and boxes at the ends of what is accepted: face coefficients near and past the ends of the
+binary64 range (spacings and densities that the seeded quotient takes one by one, whose quotient it does
+not), and densities whose cells the FP32 density of the FP64 solves does not hold together."""
 import numpy as np
 import pytest
 
@@ -36,3 +37,33 @@ def test_operator_near_the_ends_of_the_range(L, scale):
     # coefficients within 3 roundings, six products and eleven additions of the magnitudes; below the
     # normal range a rounding is half of 2^-1074, six coefficients' times |p| differences below 8
     assert np.all(abs(out.cpu().numpy() - ref) <= 20 * 2.0 ** -53 * mag + np.longdouble(2.0) ** -1074 * 64)
+
+
+SPECTRAL = {"precond": vdp.VDP_PRECOND_SPECTRAL}
+
+
+def relative_residual(s, f, p):
+    a = torch.empty_like(p)
+    s.apply(p, a)
+    return float((f - a).norm() / f.norm())
+
+
+# factor of one cell's density, and the cell: the first one sets the scale of the FP32 density.  A light
+# cell is one more isolated eigenvalue of the preconditioned operator, so CG takes a few more iterations
+@pytest.mark.parametrize("cell", [(0, 0, 0), (31, 17, 5)])
+@pytest.mark.parametrize("factor", [1e-12, 1e-17, 1e-18, 1e-19, 1e-30, 1e-36, 1e-40, 1e-60, 1e-300])
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_one_cell_of_another_density(factor, cell, precision):
+    rng = np.random.default_rng(6)
+    base = np.exp(rng.uniform(-0.5, 0.5, (32, 32, 32)))
+    rho = base.copy()
+    rho[cell] *= factor
+    f = torch.from_numpy(rng.standard_normal(rho.shape)).to(DEV)
+    f -= f.mean()
+    p = torch.empty_like(f)
+    with vdp.Solver(32, 32, 32, 1.0, precision=precision, **SPECTRAL) as s:
+        for r in (rho, base, rho):  # and from one form to the other
+            s.set_density(torch.from_numpy(r).to(DEV))
+            st = s.solve(f, p, 1e-8)
+            # 1 %: the check's own rounding, here of coefficients near 2e3 in all but one cell
+            assert st.iters < 40 and relative_residual(s, f, p) <= 1.01e-8
