@@ -464,6 +464,17 @@ int ensure_mg(vdp_ctx* c) {
   return VDP_OK;
 }
 
+// The verdict of the levels' set-up: an error for coefficients that FP32 does not hold.  Waits for the
+// stream, so it is asked for where a result is given out or has broken down.
+static int check_mg(vdp_ctx* c) {
+  int bad = 0;
+  VDP_CK(cudaMemcpyAsync(&bad, c->mg->bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  VDP_CK(cudaStreamSynchronize(c->stream));
+  if (!bad) return VDP_OK;
+  c->mg_valid = false;
+  return cuda_fail(cudaErrorInvalidValue, "multigrid levels");
+}
+
 int precond_launches(const vdp_ctx* c) {
   if (c->hdesc.pc == PC_MG) return c->mg ? mg_launches(*c->mg, c->opts.precision) : 0;
   return c->hdesc.pc >= PC_SPECTRAL ? SPEC_PASSES : 0;
@@ -811,6 +822,7 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
     VDP_CK(cudaStreamSynchronize(c->stream));
     set_stats(c, c->hstate[0], c->hstate[0].phase >= PH_DONE,
               (int)(1 + (long long)loops * (per_round * kWhileRounds + 1)));
+    if (c->stats.status == VDP_EBREAKDOWN && c->hdesc.pc == PC_MG && (s = check_mg(c)) != VDP_OK) return s;
     return c->stats.status;
   }
   // Polling schedule: graphs of m rounds, two in flight, the host checks the state after each.
@@ -841,6 +853,7 @@ int vdp_solve(vdp_ctx* c, const double* rhs, double* p, double tol) {
   if (host_p) VDP_CK(cudaMemcpyAsync(p, dp, bytes, cudaMemcpyDeviceToHost, c->stream));
   VDP_CK(cudaStreamSynchronize(c->stream));
   set_stats(c, c->hstate[(checked - 1) & 1], done, (int)(1 + issued * per_round * m));
+  if (c->stats.status == VDP_EBREAKDOWN && c->hdesc.pc == PC_MG && (s = check_mg(c)) != VDP_OK) return s;
   return c->stats.status;
 }
 
@@ -902,8 +915,7 @@ int vdp_mg_apply(vdp_ctx* c, const double* g, double* out) {
   const MgArgs a{rt, z, c->omega, nullptr, nullptr};
   VDP_CK(launch_mg_vcycle(*c->mg, PREC_FP64, a, c->stream));
   VDP_CK(launch_mg_scale(z, c->sinv, c->n, out, c->stream));
-  VDP_CK(cudaStreamSynchronize(c->stream));
-  return VDP_OK;
+  return check_mg(c);
 }
 
 int vdp_apply(vdp_ctx* c, const double* p, double* out) {

@@ -522,7 +522,7 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(kPinvThreads) k_mg_pinv(MgLevel lv, int n, float* __restrict__ pinv) {
+__global__ void __launch_bounds__(kPinvThreads) k_mg_pinv(MgLevel lv, int n, float* __restrict__ pinv, int* bad) {
   extern __shared__ double rows[];  // this block's rows: rank, rank + 16, ...
   __shared__ double pivot[2][kMgMaxCoarsest];  // published pivot rows (even and odd steps)
   __shared__ double prow[kMgMaxCoarsest];
@@ -579,7 +579,8 @@ __global__ void __launch_bounds__(kPinvThreads) k_mg_pinv(MgLevel lv, int n, flo
   // the owner of row k scales and publishes it; every thread of that block calls it
   auto publish = [&](int k) {
     double* row = rows + k / kPinvBlocks * n;
-    const double inv = quotient(1.0, row[k]);
+    const double d = row[k], inv = quotient(1.0, d);
+    if (t == 0 && !(d > 0.0 && isfinite(d))) *bad = 1;
     __syncthreads();
     for (int j = t; j < n; j += kPinvThreads) {
       const double v = j == k ? inv : row[j] * inv;
@@ -625,7 +626,7 @@ __global__ void __launch_bounds__(kPinvThreads) k_mg_pinv(MgLevel lv, int n, flo
       pinv[(long long)(rank + kPinvBlocks * r) * n + j] = (float)(rows[r * n + j] - 1.0 / (a * n));
 }
 
-cudaError_t launch_pinv(const MgLevel& lv, int n, float* pinv, cudaStream_t s) {
+cudaError_t launch_pinv(const MgLevel& lv, int n, float* pinv, int* bad, cudaStream_t s) {
   const size_t smem = sizeof(double) * (size_t)((n + kPinvBlocks - 1) / kPinvBlocks) * n;
   // (per call: the limits belong to the current device's copy of the kernel)
   cudaError_t e = cudaFuncSetAttribute(k_mg_pinv, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -644,7 +645,7 @@ cudaError_t launch_pinv(const MgLevel& lv, int n, float* pinv, cudaStream_t s) {
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_mg_pinv, lv, n, pinv);
+  return cudaLaunchKernelEx(&cfg, k_mg_pinv, lv, n, pinv, bad);
 }
 
 // out = in rounded to FP32 (the FP64 solve's scaled residual, read by the level-0 sweeps)
@@ -739,6 +740,7 @@ cudaError_t mg_alloc(MgHier* h, int nx, int ny, int nz, int wall_x) {
   }
   hh.ncoarse = (int)hh.lev[L - 1].n;
   hh.pinv = take((size_t)hh.ncoarse * hh.ncoarse);
+  hh.bad = reinterpret_cast<int*>(take(1));
   hh.mem = mem;
   hh.bytes = bytes;
   *h = hh;
@@ -768,7 +770,9 @@ cudaError_t mg_setup(MgHier* h, const double* bx, const double* by, const double
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_pinv(h->lev[h->nlev - 1], h->ncoarse, h->pinv, s);
+  const cudaError_t e2 = cudaMemsetAsync(h->bad, 0, sizeof(int), s);
+  if (e2 != cudaSuccess) return e2;
+  return launch_pinv(h->lev[h->nlev - 1], h->ncoarse, h->pinv, h->bad, s);
 }
 
 int mg_launches(const MgHier& h, int prec) {

@@ -35,6 +35,7 @@ struct MgHier {
   MgLevel lev[kMgMaxLevels] = {};
   float* pinv = nullptr;  // ncoarse x ncoarse pseudo-inverse of -A on the coarsest level
   int ncoarse = 0;
+  int* bad = nullptr;     // the coarsest matrix of the last set-up was not positive definite (or not finite)
   void* mem = nullptr;    // one allocation holds every array
   size_t bytes = 0;
 };
@@ -51,7 +52,7 @@ cudaError_t mg_alloc(MgHier* h, int nx, int ny, int nz, int wall_x);
 void mg_free(MgHier* h);
 // Build every level's coefficients from the FP64 face coefficients of the grid (level 0 scaled
 // by sinv = D^-1/2 on both sides) and the coarsest level's pseudo-inverse (double precision), on
-// stream s.
+// stream s; *h->bad is its verdict.
 cudaError_t mg_setup(MgHier* h, const double* bx, const double* by, const double* bz,
                      const double* sinv, cudaStream_t s);
 // out = in * sinv (n doubles)
