@@ -350,7 +350,7 @@ int vdp_solve_timed(vdp_ctx *ctx, const double *rhs, double *p, double tol, vdp_
  * persistent = 0 as the equivalent sequence of ordinary launches; either is captured into a
  * CUDA graph that is re-captured only when membership changes.  Members with a preconditioner of
  * several passes (spectral, fixed point, multigrid) run in a persistent = 0 batch as they do
- * alone, several at a time on streams of the batch.  Work is ordered on `stream`
+ * alone, several at a time on streams of the batch (with steps_per_sync > 0: in the launches).  Work is ordered on `stream`
  * (NULL = legacy default stream).  A batch does not own its contexts.
  */
 typedef struct vdp_batch vdp_batch;

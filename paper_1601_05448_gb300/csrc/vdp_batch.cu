@@ -9,8 +9,8 @@
 // membership and replayed.  Members can be added and retired between runs (continuous batching):
 // the device tables are rebuilt and the graph re-captured only when membership changes.
 //
-// A batch of ordinary launches shares launches among its Jacobi and Chebyshev members only.  The
-// others (spectral passes, V-cycle) have chains of kernels of their own anyway, so each runs as it
+// A batch of ordinary launches shares launches among its Jacobi and Chebyshev members (and any member
+// that is not to run, or cannot, without the host).  The others (spectral passes, V-cycle) have chains of kernels of their own anyway, so each runs as it
 // does alone -- one resident launch, or the context's device-side loop, both kept with the context
 // -- with a limit on its rounds, on one of a few streams side by side.  Capturing 64 rounds of
 // every member's passes took longer than running them, and rounds past a member's end were idle
@@ -75,8 +75,8 @@ struct vdp_batch {
   bool inject = false;        // next persistent run: one arrival more than the grid (tests)
   bool ctl_stale = false;     // the control words must be reset before the next run
   int nshared = 0;            // active members in the shared launches
-  // streams for the members that run by themselves (and graph branches for such members' passes
-  // where the driver has no device-side loops)
+  // streams for the members that run by themselves, and graph branches for such members' passes in the
+  // shared launches
   static constexpr int kBranches = 8;  // that batch of 8: 8.9, 8.6 and 7.5 ms with 2, 4 and 8
   cudaStream_t aux[kBranches] = {};
   cudaEvent_t fork = nullptr, join[kBranches] = {};
@@ -101,9 +101,10 @@ int grow(X** ptr, long long* cap, long long need) {
   return VDP_OK;
 }
 
-// How a new member runs (see above).
+// How a new member runs (see above).  One that asked for the host-polled schedule (steps_per_sync) gets
+// it: the shared launches.
 Member::How how_to_run(vdp_batch* b, vdp_ctx* c) {
-  if (b->persistent || c->hdesc.pc < PC_SPECTRAL) return Member::SHARED;
+  if (b->persistent || c->hdesc.pc < PC_SPECTRAL || c->opts.steps_per_sync > 0) return Member::SHARED;
   if (resident_solve(c, b->prec)) return Member::RESIDENT;
   return ensure_while_graph(c, b->prec) ? Member::LOOP : Member::SHARED;
 }
@@ -203,7 +204,7 @@ int capture(vdp_batch* b, int pairs) {
         e = launch_res64(b->prec, 1, b->d_desc, b->d_units, b->ns, kDirectThreads, b->cap);
       // members with the spectral passes or the V-cycle: their kernels (each gated on its own
       // member's phase), between the residual and the stencil sweeps as in a solve alone.  The
-      // members' chains are independent, so they go to up to four graph branches that the GPU
+      // members' chains are independent, so they go to a few graph branches that the GPU
       // runs concurrently (small grids alone would leave most SMs idle).
       int nspec = 0;
       for (int k : b->active)
