@@ -27,8 +27,8 @@ using namespace vdp;
 namespace {
 
 constexpr long long kMaxCells = VDP_NOALLOC_MAX_CELLS;
-// stencil units (3 per SM and one more row of tiles, of at least 256 cells each: below 1000) plus
-// flat units (<= 64); the size of the scratch array is part of the interface
+// room for stencil and flat units; plan_layout gives grids of this size far fewer (two stencil units per
+// SM and 64 flat ones), which is checked; the size of the scratch array is part of the interface
 constexpr int kMaxUnits = kMaxCells / 8 + 16;
 constexpr size_t kAlign = 256;
 
@@ -206,6 +206,7 @@ extern "C" int vdp_solve_noalloc(int nx, int ny, int nz, double L, const double*
   Layout lay;
   if (!plan_layout(nx, ny, nz, precision, 0, 0, 0, 0, 0, &lay)) return VDP_EINVAL;
   const int nunits = lay.nunits, nunits_f = lay.nunits_f;
+  if (nunits + nunits_f > kMaxUnits) return VDP_EINVAL;
 
   UnitRef hu[kMaxUnits];
   for (int i = 0; i < nunits; ++i) hu[i] = UnitRef{0, i};
