@@ -222,8 +222,10 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 // threads with about 1024; the row tile shrinks until four pipeline stages fit; stages default to
 // what fits (at most 6), or to 4 when that lets two units share an SM; about four waves.
 // Both: stencil units = row tiles x z chunks (chunk-major); flat units of 8192+ cells (at most 8 per
-// SM; 160^3 update 25.7 us with 4096, 23.4 with 8192), on small grids down to 1024 for two units
-// per SM.  In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
+// SM; 160^3 update 25.7 us with 4096, 23.4 with 8192), on small grids down to 4096 for two units
+// per SM.  Still smaller ones suit a solve alone (Jacobi CG, 4096 / 2048 / 1024 cells: 40 x 37 x 29 FP64
+// 2.42 / 2.10 / 1.91 ms, 64^3 mixed 3.92 / 3.59 / 3.48) and not a batch, whose members have the units of
+// their solves alone (32 of 64^3 mixed: launches 45 / 47 / 52 ms, persistent 79 / 89 / 109).  In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
 // Returns false when the configuration cannot run (rows too long, bad counts).
 inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, int units,
                         int stages, int threads, Layout* L) {
@@ -301,7 +303,7 @@ inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, 
   if (zc > nz) zc = nz;
   if (zc < 1) zc = 1;
   long long nf = ncell / 8192;
-  const long long nf_small = ncell / 1024 < 2LL * kSMs ? ncell / 1024 : 2LL * kSMs;
+  const long long nf_small = ncell / 4096 < 2LL * kSMs ? ncell / 4096 : 2LL * kSMs;
   if (nf < nf_small) nf = nf_small;
   if (nf > kSMs * 8) nf = kSMs * 8;
   if (nf < 1) nf = 1;

@@ -439,11 +439,16 @@ __device__ void sweep_res64(const InstDesc& I, const InstState* st, int unit,
 // KIND (direct form): 0 = CG sweeps only (the Chebyshev sweep compiled out, so the kernel keeps
 // the register budget of the plain stencil sweep), 1 = CG and Chebyshev sweeps, 2 = the
 // fixed-point iteration's sweep only.  The persistent batch kernel uses 1.
-template <class T, class BT, int MODE, int WHICH = 0, int KIND = 1>
+// PERSIST: that kernel's units, in which every thread reads the state words that it needs: a block runs
+// units one after the other there, and handing the state on through shared memory cost each of them two
+// barriers (64 grids of 32^3 mixed 12.3 ms, now 11.8, FP64 24.4 and 23.4; 32 of 64^3 79.0 and 75.7).
+template <class T, class BT, int MODE, int WHICH = 0, int KIND = 1, bool PERSIST = false>
 __device__ __forceinline__ void stencil_kind_unit(const InstDesc& I, int unit,
                                                   unsigned char* smem_raw) {
   InstState* st = I.st;
-  const InstState& sn = block_state(st);
+  InstState own;
+  if (PERSIST) load_state(st, own);
+  const InstState& sn = PERSIST ? own : block_state(st);
   const int phase = sn.phase;  // decides whether this unit has work
   if (phase != PH_RES64 && phase != PH_STENCIL && phase != PH_CHEB) return;
   if ((WHICH == 1 && phase == PH_RES64) || (WHICH == 2 && phase != PH_RES64)) return;
@@ -484,10 +489,12 @@ __device__ __forceinline__ void stencil_kind_unit(const InstDesc& I, int unit,
 }
 
 // One flat-kind unit (MEANF, UPDATE, CORRECT or FINAL phase) of instance I.
-template <class T>
+template <class T, bool PERSIST = false>
 __device__ __forceinline__ void flat_kind_unit(const InstDesc& I, int unit) {
   InstState* st = I.st;
-  const InstState& sn = block_state(st);
+  InstState own;
+  if (PERSIST) load_state(st, own);
+  const InstState& sn = PERSIST ? own : block_state(st);
   const int phase = sn.phase;
   if (phase != PH_MEANF && phase != PH_UPDATE && phase != PH_CORRECT && phase != PH_FINAL) return;
   const long long c0 = flat_begin(I, unit), c1 = flat_begin(I, unit + 1);
@@ -623,12 +630,12 @@ __global__ void __launch_bounds__(kDirectThreads, VDP_DIRECT_MIN_BLOCKS)
     if (*(volatile int*)&ctl->remaining <= 0) break;
     for (int u = blockIdx.x; u < ns; u += gridDim.x) {
       const UnitRef ur = sunits[u];
-      stencil_kind_unit<T, BT, 0>(insts[ur.inst], ur.unit, nullptr);
+      stencil_kind_unit<T, BT, 0, 0, 1, true>(insts[ur.inst], ur.unit, nullptr);
     }
     if (!grid_sync(ctl)) return;
     for (int u = blockIdx.x; u < nf; u += gridDim.x) {
       const UnitRef ur = funits[u];
-      flat_kind_unit<T>(insts[ur.inst], ur.unit);
+      flat_kind_unit<T, true>(insts[ur.inst], ur.unit);
     }
     if (!grid_sync(ctl)) return;
   }
