@@ -72,17 +72,16 @@ L2_BYTES = 129e6
 #   spec_x : X+ reads rt, W, writes S; X- reads S, W, rt, writes z   -> (3T + 8 + 2S) / 2 per launch
 #   spec_y : read and write S                                        -> 2S
 #   spec_z : read and write S (forward FFT, division, inverse FFT)   -> 2S
-#   Density form (dens; mixed and FP64 solves by the spectral inverse whose density was set after the
-#   options): unscaled variables, coefficients computed in the sweep from an FP32 density (FP64 solve:
-#   a pair of FP32 numbers), no weights:
-#   fixed-point sweep, mixed: read z, rho, g = rho r, x; write g, x     -> 24 B
-#            FP64: read z (4), rho (8), r, x; write r, x, g (FP32)      -> 48 B; A z in FP32 pairs,
+#   Density form (dens; FP64 solves by the spectral inverse whose density was set after the options):
+#   unscaled variables, coefficients computed in the sweep from the density as a pair of FP32 numbers,
+#   no weights:
+#   fixed-point sweep: read z (4), rho (8), r, x; write r, x, g = rho r (FP32) -> 48 B; A z in FP32 pairs,
 #            3 FP64 additions (x += z, r -= A z in two parts) -> 3 FP64 ops and flops
-#   stencil: mixed: read z, rho, d_old; write d, q -> 20 B; FP64: z (4), rho (8), d_old, q_old; d, q
-#            -> 44 B, 4 FP64 ops, 6 flop (two FMA).  update, FP64: also writes g (FP32) -> 6T + 4
-#   res64  : read p, f - <f>, D, 3 FP64 coefficients, fixed point: rho; write r or g (FP64: both)
-#            -> 48 + T (+4 fixed) (+4 FP64); 14 flop, 7 FP64 ops; the first: f (fixed: D, rho), write
-#            f - <f>, r or g -> 16 + T (+12 fixed) (+4 FP64); 3 flop, 2 FP64 ops
+#   stencil: read z (4), rho (8), d_old, q_old; write d, q -> 44 B, 4 FP64 ops, 6 flop (two FMA).
+#            update: also writes g -> 6T + 4
+#   res64  : read p, f - <f>, D, 3 FP64 coefficients, fixed point: rho; write r and g -> 60 (+4 fixed);
+#            14 flop, 7 FP64 ops; the first: f (fixed: D, rho), write f - <f>, r and g
+#            -> 28 (+12 fixed); 3 flop, 2 FP64 ops
 #   spec_x : X+ reads FP32, X- writes FP32, no weights -> (8 + 2S) / 2 per launch
 #   When the half spectrum fits in L2 (256^3: 71 MB) the S bytes never reach HBM: the HBM bytes
 #   of a spectral pass are then only its rt / W / z traffic, and Y and Z have none (their roof
@@ -99,7 +98,7 @@ DENSITY_FP64_OPS = {"stencil_fixed": 3.0, "stencil": 4.0, "res64": 7.0, "res64_f
 
 def density_form(prec: str, precond: str) -> bool:
     """Whether the library runs this solve in the density form (see above)."""
-    return prec in ("mixed", "fp64") and precond in ("fixed_point", "spectral")
+    return prec == "fp64" and precond in ("fixed_point", "spectral")
 
 
 def fixed_inner_tol(workload: str, prec: str) -> float:
@@ -125,9 +124,9 @@ def spectrum_bytes(nx: int) -> float:
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu capture of the
 # kernel at this precision and grid, keyed (precision, sweep, grid, fixed-point): the fixed-point
-# sweeps in the density form captured at 256^3 (a launch with x read and written), scaled to 512^3
+# sweeps (FP64: the density form's) captured at 256^3 (a launch with x read and written), scaled to 512^3
 # by the cell count.  A changed kernel drops its entries until it is re-captured.
-_TRAFFIC_256 = {("mixed", "stencil", True): 269.6e6 + 94.5e6, ("fp64", "stencil", True): 482.8e6 + 282.1e6}
+_TRAFFIC_256 = {("mixed", "stencil", True): 343.2e6 + 107.0e6, ("fp64", "stencil", True): 482.8e6 + 282.1e6}
 TRAFFIC = {(p, k, 256, f): v for (p, k, f), v in _TRAFFIC_256.items()}
 TRAFFIC.update({(p, k, 512, f): v * 8 for (p, k, f), v in _TRAFFIC_256.items()})
 
@@ -164,13 +163,9 @@ def sweep_cost(prec: str, kind: str, cheb_k: int = 1, nx: int = 256, fixed: bool
     T, B, diag = SIZES[prec]
     Bd = B if diag else 0
     if dens and kind in ("stencil", "update", "res64", "res64_first"):
-        f64 = prec == "fp64"
-        g = 4 if f64 else 0  # the FP32 copy of the residual for X+
-        b, fl = {"stencil": ((48, 3.0) if f64 else (24, 14.0)) if fixed
-                 else ((44, 6.0) if f64 else (20, 16.0)),
-                 "update": (6 * T + g, 6.0),
-                 "res64": (48 + T + g + (4 if fixed else 0), 14.0),
-                 "res64_first": (16 + T + g + (12 if fixed else 0), 3.0)}[kind]
+        b, fl = {"stencil": (48, 3.0) if fixed else (44, 6.0), "update": (6 * T + 4, 6.0),
+                 "res64": (60 + (4 if fixed else 0), 14.0),
+                 "res64_first": (28 + (12 if fixed else 0), 3.0)}[kind]
         return b, fl, b
     if fixed and kind == "stencil":
         b = 4 + 4 * T + 3 * B + Bd
@@ -231,7 +226,7 @@ def kernel_table(prec: str, ncell: int, kinds: dict, peaks: dict, grid: int, che
         row = {"kernel": KERNEL_NAMES[name], "launches": k["launches"], "mean_us": 1e3 * k["ms_mean"],
                "min_us": 1e3 * k["ms_min"], "share": k["ms"] / total}
         if dens and name == "stencil":
-            row["kernel"] = "k_density64" if prec == "fp64" else "k_density"
+            row["kernel"] = "k_density64"
         t_all = k["ms"] / 1e3
         if name.startswith("spec_"):
             alg, hbm = spec_bytes(prec, name, nx, ncell, slabbed, fixed, dens)
@@ -391,6 +386,23 @@ def max_over_ranks(x: float, dist=None, device=None) -> float:
     t = torch.tensor([float(x)], dtype=torch.float64, device=device)
     dist.all_reduce(t, op=dist.ReduceOp.MAX)
     return float(t.item())
+
+
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "iterations",
+            "outer_iterations", "rel_res", "solve_ms_median", "solve_hbm_frac", "roofline", "cpu_baseline", "summary")
+
+
+def headline(line: dict) -> dict:
+    """The line for standard output: the headline with its end-to-end figure, roofline and the extras'
+    summary, short enough (some 2 KB) for a reader that keeps the end of the output only.  The tables go
+    to standard error."""
+    def short(v):
+        return {k: short(x) for k, x in v.items() if k not in ("timing", "sample", "wall_s", "sample_s")} \
+            if isinstance(v, dict) else float(f"{v:.6g}") if isinstance(v, float) else v
+    out = {k: line[k] if k in ("value", "ms_per_step") else short(line[k]) for k in HEADLINE if k in line}
+    failed = sorted(k for k, v in line.items() if isinstance(v, dict) and "error" in v)
+    return dict(out, failed=failed) if failed else out
 
 
 def replica_rate(world: int, steps: int, elapsed: float) -> float:
@@ -1004,7 +1016,8 @@ def main():
     line["summary"] = dict(summary, headline_solves_per_s=value, headline_iters=iters,
                            roofline_frac=roof["frac"], roofline_kernel=roof["kernel"])
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)  # every table
+        print(json.dumps(headline(line)), flush=True)
     if pg is not None:
         pg.destroy_process_group()
     return 0
