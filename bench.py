@@ -126,7 +126,7 @@ def spectrum_bytes(nx: int) -> float:
 # kernel at this precision and grid, keyed (precision, sweep, grid, fixed-point): the fixed-point
 # sweeps (FP64: the density form's) captured at 256^3 (a launch with x read and written), scaled to 512^3
 # by the cell count.  A changed kernel drops its entries until it is re-captured.
-_TRAFFIC_256 = {("mixed", "stencil", True): 343.2e6 + 107.0e6, ("fp64", "stencil", True): 482.8e6 + 282.1e6}
+_TRAFFIC_256 = {("mixed", "stencil", True): 345.9e6 + 105.4e6, ("fp64", "stencil", True): 479.9e6 + 284.5e6}
 TRAFFIC = {(p, k, 256, f): v for (p, k, f), v in _TRAFFIC_256.items()}
 TRAFFIC.update({(p, k, 512, f): v * 8 for (p, k, f), v in _TRAFFIC_256.items()})
 

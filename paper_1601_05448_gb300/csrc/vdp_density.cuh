@@ -26,8 +26,8 @@
 // (CG).  The sweep also leaves rho' r in FP32 for the X+ pass, which read r and rho' and narrowed
 // the product itself: four bytes more here, eight fewer there, and X+ runs its FP32 form (256^3:
 // 75 -> 35 us).  The 47 bits act on differences of z across a face, not on z D as in the scaled form, and
-// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before: over 484
-// spectral and 12 fixed-point inputs of 32^3 to 256^3 no pressure was further from the one in 64 bits
+// the refinement's FP64 residual is evaluated from p with the FP64 coefficients as before: over 242
+// spectral and 242 fixed-point inputs of 32^3 to 256^3 no pressure was further from the one in 64 bits
 // than with the FP64 product.
 //
 // The march is that of sweep_stencil_direct: a thread owns 16 bytes of one row and walks a z chunk,

@@ -193,9 +193,6 @@ static __device__ __noinline__ void block_sum_slots(const double* part, int nuni
     for (int k = 0; k < ns; ++k) S[k] = (wsum[k][0] + wsum[k][1]) + (wsum[k][2] + wsum[k][3]);
 }
 
-// c / s in FP64 for s > 0 in the middle of the binary64 range: the FP32 approximation of 1/s as the
-// seed Y, e = 1 - s Y (|e| < 2^-21.4), c/s = w (1 + e + e^2), w = c Y; relative error below
-// 2^-52.  Five FP64 instructions; the division takes more than ten, each 64 cycles after the other.
 __device__ __forceinline__ int exponent_of(double v) {  // biased exponent field
   return (__double2hiint(v) >> 20) & 0x7ff;
 }
@@ -215,6 +212,9 @@ __device__ __forceinline__ bool mid_range(double v) {
   const int e = exponent_of(v);
   return e > 200 && e < 1846;
 }
+// c / s in FP64 for s > 0 in the middle of the binary64 range: the FP32 approximation of 1/s as the
+// seed Y, e = 1 - s Y (|e| < 2^-21.4), c/s = w (1 + e + e^2), w = c Y; relative error below
+// 2^-52.  Five FP64 instructions; the division takes more than ten, each 64 cycles after the other.
 __device__ __forceinline__ double quotient(double c, double s) {
   if (!mid_range(s)) return c / s;
   const double Y = widen_pow2(rcp_approx(mantissa_f(s)), 1023 - exponent_of(s));

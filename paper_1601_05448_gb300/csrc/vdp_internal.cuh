@@ -210,14 +210,13 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 // 16-byte vector of a row tile of threads * V / nx rows (V = 4 FP32, 2 FP64), about 12 units per
 // SM.  The z chunks are chosen for the fewest plane steps in a row: waves of resident units times the
 // planes of a chunk and the two that it reloads.  In FP64 three units of all kernels are resident on an
-// SM, else two of the density form's sweep and of the residual, three of the scaled sweep: there the
-// sum of both, weighted 2 : 3.  The steps follow the measured times of sweep and residual (us): 256^3 FP64
-// 206 and 288 with 896 units (78 steps), 215 and 334 with 1024 (102), 216 and 338 with 1408 (104);
-// 256^3 mixed 81 and 198 with 896 (63 at two per SM), 87 and 216 with 1408 (70); 512^3 mixed 508 and
-// 1426 with 1792 (456), 528 and 1563 with 1536 (528); 128^3 FP64 41 and 36 with 448 (12), 44 and 38
-// with 288 (17); 160^3 mixed, scaled sweep, 48 and 71 with 280 (25 at three per SM), 38 and 87 with
-// 480 (28), 38 and 62 with 440 (17).  Grids that the resident solve takes
-// get 304 units, one for each of its blocks.
+// SM, else two of the residual and three of the sweep: there the sum of both, weighted 2 : 3.  The
+// steps follow the measured times of sweep and residual (us): 256^3 FP64 206 and 288 with 896 units
+// (78 steps), 215 and 334 with 1024 (102), 216 and 338 with 1408 (104);
+// 256^3 mixed 99 and 240 with 896, 113 and 274 with 1024, 113 and 261 with 1408; 512^3 mixed 647 and
+// 1652 with 1792, 687 and 1827 with 1536; 128^3 FP64 41 and 36 with 448 (12), 44 and 38
+// with 288 (17); 160^3 mixed 48 and 71 with 280 (25 at three per SM), 38 and 87 with 480 (28), 38 and
+// 62 with 440 (17).  Grids that the resident solve takes get 304 units, one for each of its blocks.
 // mode 1 (TMA pipeline): FP64 512-thread units with about 2048 cells per plane, FP32/BF16 256
 // threads with about 1024; the row tile shrinks until four pipeline stages fit; stages default to
 // what fits (at most 6), or to 4 when that lets two units share an SM; about four waves.
@@ -225,7 +224,8 @@ inline void prec_sizes(int prec, int* ts, int* bs, bool* diag) {
 // SM; 160^3 update 25.7 us with 4096, 23.4 with 8192), on small grids down to 4096 for two units
 // per SM.  Still smaller ones suit a solve alone (Jacobi CG, 4096 / 2048 / 1024 cells: 40 x 37 x 29 FP64
 // 2.42 / 2.10 / 1.91 ms, 64^3 mixed 3.92 / 3.59 / 3.48) and not a batch, whose members have the units of
-// their solves alone (32 of 64^3 mixed: launches 45 / 47 / 52 ms, persistent 79 / 89 / 109).  In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
+// their solves alone (32 of 64^3 mixed: launches 45 / 47 / 52 ms, persistent 79 / 89 / 109).
+// In mode 1 the dynamic shared memory also covers the FP64 residual sweep's ring.
 // Returns false when the configuration cannot run (rows too long, bad counts).
 inline bool plan_layout(int nx, int ny, int nz, int prec, int mode, int tile_y, int units,
                         int stages, int threads, Layout* L) {

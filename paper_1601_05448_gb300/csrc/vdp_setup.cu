@@ -7,12 +7,12 @@
 // FP32 rate: an IEEE double division costs about ten such instructions and a reciprocal square
 // root more, so a set-up written with `/` and `sqrt` is bound by that pipe at several times the
 // HBM time (512^3: 16.3 ms against about 1 ms of traffic).  Here both start from the FP32
-// approximation instruction (relative error below 2^-22, on the mantissa alone, so the whole
-// binary64 range works).  The root takes one third-order Newton step in FP64.  The quotient is
+// approximation instruction (relative error below 2^-22, on the mantissa alone; where operands or quotient
+// leave the middle of the binary64 range, the division and the root themselves run).  The root takes one third-order Newton step in FP64.  The quotient is
 // refined in pairs of FP32 numbers to about 2^-44 and assembled into a double by integer
 // operations; its FP64 remainder then gives the last bits: three FP64 instructions a face (the sum
-// included) instead of more than ten.  512^3 in the density form: 16.3 -> 5.3 (five instructions a
-// face, Newton in FP64) -> 3.8 ms.
+// included) instead of more than ten.  512^3: 16.3 ms with both written out; now 4.0 in the density
+// form (FP64 solves), 8.5 with D^-1/2, the scaled coefficients and the weights (FP32).
 //
 // Layout: a thread owns two neighbouring cells of a row (16-byte accesses) and marches a z chunk,
 // so the plane below is in registers; the row above comes from L1 / L2.

@@ -25,10 +25,11 @@
 // 32): M2-point DFTs in registers, twiddles W_n^(j1 k2), an exchange through shared memory,
 // M1-point DFTs in registers.  Global accesses are coalesced: rows are contiguous in the X
 // passes and the Y/Z tiles read 8 consecutive complex values (64 bytes) per line element.
-// One application moves about 41 bytes per cell (FP32 input, no weights).  At 512^3 X takes 185 us a
-// launch, Y 191 (0.87 of the copy bandwidth each) and Z, which does two transforms per element, 315
+// One application moves about 41 bytes per cell (FP32 input, no weights; with weights 49).  At 512^3 X
+// takes 185 us a launch (with weights X+ 242, X- 256), Y 191 (0.87 of the copy bandwidth each) and Z, which does two transforms per element, 315
 // (0.53).  At 256^3 the spectrum stays in L2 and nothing is saturated (ncu: issue 42-58 %, shared
-// memory 28-54 %, DRAM 28-43 %; 15-20 warps per SM): X 33, Y 26, Z 36 us.  In every pass the
+// memory 28-54 %, DRAM 28-43 %; 15-20 warps per SM): X 33 (with
+// weights 36 and 40), Y 26, Z 36 us.  In every pass the
 // first tile's copies and the tables are under way while the solve's phase is read.
 #include <cuda_runtime.h>
 

@@ -708,7 +708,7 @@ __device__ void res64_zero_p(const InstDesc& I, const InstState* st, int unit,
   T a1 = 0;
   float a1f = 0.f;  // DENS
   // two planes' loads before the first plane's stores (which the compiler cannot move loads across):
-  // 512^3 density form 1012 -> 753 us (32 bytes a cell: 5.7 TB/s), 256^3 157 -> 126
+  // 512^3 mixed 730 -> 582 us (28 bytes a cell: 6.5 TB/s), 256^3 152 -> 96, FP64 157 -> 122
   struct Cells {
     double2 f[VR / 2], w[VR / 2];  // w: D (density form), else D^-1/2
     float2 rho[VR / 2];
