@@ -734,6 +734,8 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
   c->rho_w_valid = weights;
   c->rho32_valid = c->rho32 && !wide;
   c->mg_valid = false;
+  if (c->rho32_valid != kept) c->layout_dirty = true;  // the form may change with it
+  c->has_density = true;
   if (wide && !weights) {  // the scaled form's weight of rho, while rho is at hand
     const int s = ensure_sinv(c);
     if (s != VDP_OK) return s;
@@ -742,8 +744,6 @@ int vdp_set_density(vdp_ctx* c, const double* rho) {
     VDP_CK(cudaStreamSynchronize(c->stream));
     c->rho_w_valid = true;
   }
-  if (c->rho32_valid != kept) c->layout_dirty = true;  // the form may change with it
-  c->has_density = true;
   return VDP_OK;
 }
 

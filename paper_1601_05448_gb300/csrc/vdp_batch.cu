@@ -10,11 +10,12 @@
 // the device tables are rebuilt and the graph re-captured only when membership changes.
 //
 // A batch of ordinary launches shares launches among its Jacobi and Chebyshev members (and any member
-// that is not to run, or cannot, without the host).  The others (spectral passes, V-cycle) have chains of kernels of their own anyway, so each runs as it
-// does alone -- one resident launch, or the context's device-side loop, both kept with the context
-// -- with a limit on its rounds, on one of a few streams side by side.  Capturing 64 rounds of
-// every member's passes took longer than running them, and rounds past a member's end were idle
-// launches (8 grids of 64^3 to 192^3, mixed to 1e-8 with their densities set: 20.1 -> 7.5 ms).
+// that is not to run, or cannot, without the host).  The others (spectral passes, V-cycle) have
+// chains of kernels of their own anyway, so each runs as it does alone -- one resident launch, or the
+// context's device-side loop, both kept with the context -- with a limit on its rounds, on one of a
+// few streams side by side.  Capturing 64 rounds of every member's passes took longer than running
+// them, and rounds past a member's end were idle launches (8 grids of 64^3 to 192^3, mixed to 1e-8
+// with their densities set: 24.1 -> 8.4 ms).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -77,7 +78,7 @@ struct vdp_batch {
   int nshared = 0;            // active members in the shared launches
   // streams for the members that run by themselves, and graph branches for such members' passes in the
   // shared launches
-  static constexpr int kBranches = 8;  // that batch of 8: 8.9, 8.6 and 7.5 ms with 2, 4 and 8
+  static constexpr int kBranches = 8;  // that batch of 8: 8.9, 8.6 and 7.5 ms with 2, 4 and 8 (FP32 density form)
   cudaStream_t aux[kBranches] = {};
   cudaEvent_t fork = nullptr, join[kBranches] = {};
 };
